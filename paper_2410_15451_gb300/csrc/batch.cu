@@ -511,14 +511,56 @@ __global__ void k_ds_best(const uint64_t *pkey, const int64_t *pw, const int64_t
   }
 }
 
-// Warp per vertex with dE: neighbours of G^t become affected.
-__global__ void k_ds_expand_neighbours(const uint8_t *dE, int64_t n, const int64_t *off, const int32_t *deg,
-                                       const int32_t *col, uint8_t *dV) {
-  int lane = threadIdx.x & 31;
-  int64_t warp = ld_gtid() >> 5, nwarps = ld_gstride() >> 5;
-  for (int64_t i = warp; i < n; i += nwarps) {
-    if (!dE[i]) continue;
-    for (int64_t a = lane; a < deg[i]; a += 32) dV[col[off[i] + a]] = 1;
+// Neighbours of G^t of the vertices with dE become affected.  Rows by
+// windows of 32 per warp, the flagged ones flattened; flagged rows above
+// ROWS_BIG arcs are listed for the chunked kernel (a warp per vertex of the
+// graph spent its time on unflagged rows and on the longest hub: R-MAT 20,
+// 15,700 edges: 580 -> 19 us, and 14 us for the hubs' chunks).
+__global__ void __launch_bounds__(256) k_ds_expand_neighbours(const uint8_t *dE, int64_t n, const int64_t *off,
+                                                              const int32_t *deg, const int32_t *col, uint8_t *dV,
+                                                              int32_t *big, DevCounters *cnt) {
+  const int lane = threadIdx.x & 31;
+  int64_t warp = ld_gtid() >> 5, nw = ld_gstride() >> 5;
+  for (int64_t r = warp * 32; r < n; r += nw * 32) {  // warp-uniform
+    int64_t i = r + lane;
+    bool f = i < n && dE[i];
+    if (!__any_sync(LD_FULL, f)) continue;
+    int d = f ? deg[i] : 0;
+    if (d > ROWS_BIG) {
+      big[atomicAdd(&cnt->big_count, 1)] = (int32_t)i;
+      d = 0;
+    }
+    int e = ld_warp_incl_i32(d), s = e - d, total = __shfl_sync(LD_FULL, e, 31);
+    int64_t ab = (f ? off[i] : 0) - s;
+    for (int x0 = 0; x0 < total; x0 += 128) {  // warp-uniform
+      int k[4];
+      int32_t j[4];
+      ld_window_rows<4>(s, x0, lane, k);
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        int x = x0 + 32 * u + lane;
+        int64_t a = __shfl_sync(LD_FULL, ab, k[u]) + x;
+        j[u] = x < total ? col[a] : -1;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; u++)
+        if (j[u] >= 0) dV[j[u]] = 1;
+    }
+  }
+}
+__global__ void __launch_bounds__(256) k_ds_expand_big(const int32_t *big, const int64_t *ch_off, const int64_t *off,
+                                                       const int32_t *deg, const int32_t *col, uint8_t *dV,
+                                                       const DevCounters *cnt) {
+  const int64_t count = cnt->big_count;
+  if (count == 0) return;
+  const int64_t nch = ch_off[count];
+  for (int64_t t = blockIdx.x; t < nch; t += gridDim.x) {  // block-uniform
+    int64_t k = ld_chunk_item(ch_off, count, t);
+    int32_t i = big[k];
+    int64_t x0 = (t - ch_off[k]) * TABLE_CHUNK, b = off[i] + x0;
+    int len = (int)(deg[i] - x0 < TABLE_CHUNK ? deg[i] - x0 : TABLE_CHUNK);
+#pragma unroll 4
+    for (int x = threadIdx.x; x < len; x += 256) dV[col[b + x]] = 1;
   }
 }
 __global__ void k_ds_expand_communities(const uint8_t *dCf, const int32_t *C, int64_t n, uint8_t *dV) {
@@ -902,7 +944,12 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
         ld_note_launch(), k_ds_best<<<grid_for(ni, TB), TB, 0, s>>>(b.ds_ukey, b.ds_uw, b.pos + ni, vb, h->K, h->Sig, cnt, dV, h->dE,
                                                   h->dCf, h->gid0, h->gc.m2);
       }
-      ld_note_launch(), k_ds_expand_neighbours<<<grid_for(n * 32, TB), TB, 0, s>>>(h->dE, n, h->g_off, h->g_deg, h->g_col, dV);
+      cudaMemsetAsync(&cnt->big_count, 0, sizeof(int32_t), s);
+      ld_note_launch(), k_ds_expand_neighbours<<<grid_for(n, TB), TB, 0, s>>>(h->dE, n, h->g_off, h->g_deg, h->g_col,
+                                                                              dV, h->ibuf0, cnt);
+      launch_table_plan(h->ibuf0, &cnt->big_count, h->g_deg, nullptr, 1, h->lbuf0, h->lbuf1, s);
+      ld_note_launch(), k_ds_expand_big<<<h->sm_count * 8, TB, 0, s>>>(h->ibuf0, h->lbuf1, h->g_off, h->g_deg,
+                                                                       h->g_col, dV, cnt);
       ld_note_launch(), k_ds_expand_communities<<<grid_for(n, TB), TB, 0, s>>>(h->dCf, h->C, n, dV);
     }
   }

@@ -407,6 +407,78 @@ __device__ __forceinline__ int64_t ld_w(const W *w, int64_t a) {
   return (int64_t)w[a];
 }
 
+// ---------------------------------------------------------------- rows by windows
+// A warp takes the arcs of up to 32 rows as one flat range: lane i holds row
+// i's first flat position s (non-decreasing over the lanes) and arc(x) =
+// ab + x of that row, so that consecutive lanes read consecutive arcs
+// whatever the rows' lengths.  A warp per row leaves 31 lanes idle on a short
+// row and one warp alone on a hub; longer rows than ROWS_BIG are therefore
+// cut into chunks by the callers.
+constexpr int ROWS_BIG = 2048;
+
+// The row (lane) that holds flat position x: the last one with s <= x.  All
+// lanes call it; positions of one call rise with the lane, so when the first
+// and last fall into one row (a long row) the search is two ballots (and the
+// result true).
+template <int U>
+__device__ __forceinline__ bool ld_window_rows(int s, int x0, int lane, int *k) {
+  int first = 31 - __clz(__ballot_sync(LD_FULL, s <= x0));
+  int last = 31 - __clz(__ballot_sync(LD_FULL, s <= x0 + 32 * U - 1));
+#pragma unroll
+  for (int u = 0; u < U; u++) k[u] = first;
+  if (first == last) return true;  // warp-uniform
+#pragma unroll
+  for (int u = 0; u < U; u++) {
+    int x = x0 + 32 * u + lane, r = 0;
+#pragma unroll
+    for (int step = 16; step > 0; step >>= 1) {
+      int sc = __shfl_sync(LD_FULL, s, r + step);
+      if (sc <= x) r += step;
+    }
+    k[u] = r;
+  }
+  return false;
+}
+
+// Inclusive sum over the lanes.
+__device__ __forceinline__ int64_t ld_warp_incl_i64(int64_t v) {
+  int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    int64_t y = __shfl_up_sync(LD_FULL, v, o);
+    if (lane >= o) v += y;
+  }
+  return v;
+}
+__device__ __forceinline__ int ld_warp_incl_i32(int v) {
+  int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    int y = __shfl_up_sync(LD_FULL, v, o);
+    if (lane >= o) v += y;
+  }
+  return v;
+}
+
+// The part of each lane's row [s, e) in 32 flat positions xb .. xb + 31 that
+// hold one value per lane (v): the values summed over the overlap.
+__device__ __forceinline__ int64_t ld_window_part(int s, int e, int xb, int64_t v) {
+  int64_t p = ld_warp_incl_i64(v);
+  int lo = s > xb ? s - xb : 0, hi = e < xb + 32 ? e - xb : 32;  // [lo, hi) of the step
+  int64_t a = __shfl_sync(LD_FULL, p, (lo - 1) & 31), b = __shfl_sync(LD_FULL, p, (hi - 1) & 31);
+  return lo < hi ? b - (lo > 0 ? a : 0) : 0;
+}
+
+// Item k of a chunk plan (ch_off[k] <= t < ch_off[k+1]).
+__device__ __forceinline__ int64_t ld_chunk_item(const int64_t *ch_off, int64_t count, int64_t t) {
+  int64_t lo = 0, hi = count - 1;
+  while (lo < hi) {
+    int64_t mid = (lo + hi + 1) >> 1;
+    if (ch_off[mid] <= t) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
 // Grid-stride helpers.
 __device__ __forceinline__ int64_t ld_gtid() { return (int64_t)blockIdx.x * blockDim.x + threadIdx.x; }
 __device__ __forceinline__ int64_t ld_gstride() { return (int64_t)gridDim.x * blockDim.x; }

@@ -213,24 +213,100 @@ __global__ void k_sig_of(int64_t N, const int32_t *C, const int64_t *K, int64_t 
   }
 }
 // Batched handles (gid0 non-null) also sum per graph: sigg, sqg, m2g.
-__global__ void k_sigma_intra(int64_t N, const int64_t *off, const int32_t *deg, const int32_t *col, const int32_t *w,
-                              const int32_t *C, DevCounters *cnt, const int32_t *gid0, int64_t *sigg) {
-  int lane = threadIdx.x & 31;
+// Intra-community weight and (k_rowsum) row sums, rows by windows of 32 per
+// warp; rows above ROWS_BIG arcs are listed and their chunks summed by the
+// second kernel.  With a warp per row, the longest hub's warp was the kernel's
+// time (R-MAT 21: k_rowsum 412 -> 260 us).
+constexpr int ROW_UNROLL = 4;
+
+// The rows of a window: lane i's first flat position s, end e, row start minus
+// s (ab); rows above ROWS_BIG are listed instead.  Returns the flat length.
+__device__ __forceinline__ int window_of(int64_t i, int64_t N, const int64_t *off, const int32_t *deg, int32_t *big,
+                                         int32_t *nbig, int &s, int &e, int64_t &ab) {
+  int d = i < N ? deg[i] : 0;
+  int64_t b = i < N ? off[i] : 0;
+  if (d > ROWS_BIG) {
+    big[atomicAdd(nbig, 1)] = (int32_t)i;
+    d = 0;
+  }
+  e = ld_warp_incl_i32(d);
+  s = e - d;
+  ab = b - s;
+  return __shfl_sync(LD_FULL, e, 31);
+}
+
+__global__ void __launch_bounds__(256) k_sigma_intra(int64_t N, const int64_t *off, const int32_t *deg,
+                                                     const int32_t *col, const int32_t *w, const int32_t *C,
+                                                     DevCounters *cnt, const int32_t *gid0, int64_t *sigg,
+                                                     int32_t *big) {
+  const int lane = threadIdx.x & 31;
   int64_t warp = ld_gtid() >> 5, nw = ld_gstride() >> 5;
   int64_t acc = 0;
-  for (int64_t i = warp; i < N; i += nw) {
-    int32_t c = C[i];
-    int64_t b = off[i], d = deg[i], vi = 0;
-    for (int64_t a = lane; a < d; a += 32)
-      if (C[col[b + a]] == c) vi += w[b + a];
-    acc += vi;
-    if (gid0) {
-      vi = ld_warp_sum_i64(vi);
-      if (lane == 0 && vi) atomicAdd((unsigned long long *)&sigg[gid0[i]], (unsigned long long)vi);
+  for (int64_t r = warp * 32; r < N; r += nw * 32) {  // warp-uniform
+    int64_t i = r + lane, ab;
+    int s, e;
+    int total = window_of(i, N, off, deg, big, &cnt->big_count, s, e, ab);
+    int32_t c = i < N ? C[i] : -1, g = gid0 && i < N ? gid0[i] : 0;
+    int64_t here = 0;
+    // the usual window lies in one graph; one across a boundary adds each hit to its row's graph
+    int32_t g0 = __shfl_sync(LD_FULL, g, 0);
+    bool one = __all_sync(LD_FULL, g == g0 || i >= N);
+    for (int x0 = 0; x0 < total; x0 += 32 * ROW_UNROLL) {  // warp-uniform
+      int k[ROW_UNROLL];
+      int32_t j[ROW_UNROLL], wv[ROW_UNROLL], cj[ROW_UNROLL];
+      ld_window_rows<ROW_UNROLL>(s, x0, lane, k);
+#pragma unroll
+      for (int u = 0; u < ROW_UNROLL; u++) {
+        int x = x0 + 32 * u + lane;
+        int64_t a = __shfl_sync(LD_FULL, ab, k[u]) + x;
+        j[u] = x < total ? col[a] : -1;
+        wv[u] = x < total ? w[a] : 0;
+      }
+#pragma unroll
+      for (int u = 0; u < ROW_UNROLL; u++) cj[u] = j[u] >= 0 ? C[j[u]] : -2;
+#pragma unroll
+      for (int u = 0; u < ROW_UNROLL; u++) {
+        int32_t ci = __shfl_sync(LD_FULL, c, k[u]), gi = __shfl_sync(LD_FULL, g, k[u]);
+        if (ci != cj[u]) continue;
+        here += wv[u];
+        if (gid0 && !one) atomicAdd((unsigned long long *)&sigg[gi], (unsigned long long)wv[u]);
+      }
+    }
+    acc += here;
+    if (gid0 && one) {
+      here = ld_warp_sum_i64(here);
+      if (lane == 0 && here) atomicAdd((unsigned long long *)&sigg[g0], (unsigned long long)here);
     }
   }
   acc = ld_warp_sum_i64(acc);
   if (lane == 0 && acc) atomicAdd((unsigned long long *)&cnt->sigma_intra, (unsigned long long)acc);
+}
+
+__global__ void __launch_bounds__(256) k_sigma_intra_big(const int32_t *big, const int64_t *ch_off, const int64_t *off,
+                                                         const int32_t *deg, const int32_t *col, const int32_t *w,
+                                                         const int32_t *C, DevCounters *cnt, const int32_t *gid0,
+                                                         int64_t *sigg) {
+  const int64_t count = cnt->big_count;
+  if (count == 0) return;
+  const int64_t nch = ch_off[count];
+  int64_t acc = 0;
+  for (int64_t t = blockIdx.x; t < nch; t += gridDim.x) {  // block-uniform
+    int64_t k = ld_chunk_item(ch_off, count, t);
+    int32_t i = big[k], c = C[i];
+    int64_t x0 = (t - ch_off[k]) * TABLE_CHUNK, b = off[i] + x0;
+    int len = (int)(deg[i] - x0 < TABLE_CHUNK ? deg[i] - x0 : TABLE_CHUNK);
+    int64_t here = 0;
+#pragma unroll 4
+    for (int x = threadIdx.x; x < len; x += 256)
+      if (C[col[b + x]] == c) here += w[b + x];
+    acc += here;
+    if (gid0) {
+      here = ld_warp_sum_i64(here);
+      if ((threadIdx.x & 31) == 0 && here) atomicAdd((unsigned long long *)&sigg[gid0[i]], (unsigned long long)here);
+    }
+  }
+  acc = ld_warp_sum_i64(acc);
+  if ((threadIdx.x & 31) == 0 && acc) atomicAdd((unsigned long long *)&cnt->sigma_intra, (unsigned long long)acc);
 }
 __global__ void k_sq(int64_t N, const int64_t *Sig, DevCounters *cnt, const int32_t *gid0, unsigned long long *sqg) {
   i128 acc = 0;
@@ -246,20 +322,81 @@ __global__ void k_sq(int64_t N, const int64_t *Sig, DevCounters *cnt, const int3
   if ((threadIdx.x & 31) == 0) ld_atomic_add_i128(cnt->sq, acc);
 }
 
-__global__ void k_rowsum(int64_t N, const int64_t *off, const int32_t *deg, const int32_t *w, int64_t *K,
-                         DevCounters *cnt, const int32_t *gid0, int64_t *m2g) {
-  int lane = threadIdx.x & 31;
+// K of the rows up to ROWS_BIG arcs; a longer row's K is set to 0 and its
+// chunks are added by k_rowsum_big.  Steps inside one row are summed per lane
+// and reduced when the row changes; only steps across rows pay for a scan.
+constexpr int SUM_UNROLL = 8;
+__global__ void __launch_bounds__(256) k_rowsum(int64_t N, const int64_t *off, const int32_t *deg, const int32_t *w,
+                                                int64_t *K, DevCounters *cnt, const int32_t *gid0, int64_t *m2g,
+                                                int32_t *big) {
+  __shared__ unsigned long long bsum;
+  if (threadIdx.x == 0) bsum = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
   int64_t warp = ld_gtid() >> 5, nw = ld_gstride() >> 5;
   int64_t tot = 0;
-  for (int64_t i = warp; i < N; i += nw) {
-    int64_t b = off[i], d = deg[i], acc = 0;
-    for (int64_t a = lane; a < d; a += 32) acc += w[b + a];
-    acc = ld_warp_sum_i64(acc);
-    if (lane == 0) K[i] = acc;
-    if (lane == 0 && gid0 && acc) atomicAdd((unsigned long long *)&m2g[gid0[i]], (unsigned long long)acc);
-    tot += acc;
+  for (int64_t r = warp * 32; r < N; r += nw * 32) {  // warp-uniform
+    int64_t i = r + lane, ab, kw = 0, lacc = 0;
+    int s, e, cur = 0;
+    int total = window_of(i, N, off, deg, big, &cnt->big_count, s, e, ab);
+    for (int x0 = 0; x0 < total; x0 += 32 * SUM_UNROLL) {  // warp-uniform
+      int k[SUM_UNROLL];
+      int32_t wv[SUM_UNROLL];
+      bool inside = ld_window_rows<SUM_UNROLL>(s, x0, lane, k);
+#pragma unroll
+      for (int u = 0; u < SUM_UNROLL; u++) {
+        int x = x0 + 32 * u + lane;
+        int64_t a = __shfl_sync(LD_FULL, ab, k[u]) + x;
+        wv[u] = x < total ? w[a] : 0;
+      }
+      int kc = __shfl_sync(LD_FULL, k[0], 0);
+      if (!inside || kc != cur) {  // warp-uniform: the row summed so far is complete
+        lacc = ld_warp_sum_i64(lacc);
+        if (lane == cur) kw += lacc;
+        lacc = 0;
+        cur = kc;
+      }
+#pragma unroll
+      for (int u = 0; u < SUM_UNROLL; u++) {
+        if (inside) lacc += wv[u];
+        else kw += ld_window_part(s, e, x0 + 32 * u, wv[u]);
+      }
+    }
+    lacc = ld_warp_sum_i64(lacc);
+    if (lane == cur) kw += lacc;
+    if (i < N) {
+      K[i] = kw;
+      tot += kw;
+    }
+    if (gid0) ld_graph_add_i64(m2g, i < N, i < N ? gid0[i] : 0, kw);
   }
-  if (lane == 0 && tot) atomicAdd((unsigned long long *)&cnt->m2, (unsigned long long)tot);
+  tot = ld_warp_sum_i64(tot);
+  if (lane == 0 && tot) atomicAdd(&bsum, (unsigned long long)tot);
+  __syncthreads();
+  if (threadIdx.x == 0 && bsum) atomicAdd((unsigned long long *)&cnt->m2, bsum);
+}
+
+__global__ void __launch_bounds__(256) k_rowsum_big(const int32_t *big, const int64_t *ch_off, const int64_t *off,
+                                                    const int32_t *deg, const int32_t *w, int64_t *K, DevCounters *cnt,
+                                                    const int32_t *gid0, int64_t *m2g) {
+  const int64_t count = cnt->big_count;
+  if (count == 0) return;
+  const int64_t nch = ch_off[count];
+  for (int64_t t = blockIdx.x; t < nch; t += gridDim.x) {  // block-uniform
+    int64_t k = ld_chunk_item(ch_off, count, t);
+    int32_t i = big[k];
+    int64_t x0 = (t - ch_off[k]) * TABLE_CHUNK, b = off[i] + x0;
+    int len = (int)(deg[i] - x0 < TABLE_CHUNK ? deg[i] - x0 : TABLE_CHUNK);
+    int64_t acc = 0;
+#pragma unroll 4
+    for (int x = threadIdx.x; x < len; x += 256) acc += w[b + x];
+    acc = ld_warp_sum_i64(acc);
+    if ((threadIdx.x & 31) == 0 && acc) {
+      atomicAdd((unsigned long long *)&K[i], (unsigned long long)acc);
+      atomicAdd((unsigned long long *)&cnt->m2, (unsigned long long)acc);
+      if (gid0) atomicAdd((unsigned long long *)&m2g[gid0[i]], (unsigned long long)acc);
+    }
+  }
 }
 
 }  // namespace
@@ -313,8 +450,13 @@ void modularity_terms(leiden_handle *h, const int32_t *C) {
     cudaMemsetAsync(h->gc.sigma, 0, (size_t)h->G * sizeof(int64_t), s);
     cudaMemsetAsync(h->gc.sq, 0, (size_t)h->G * 2 * sizeof(unsigned long long), s);
   }
-  ld_note_launch(), k_sigma_intra<<<grid_for(N * 32, TB), TB, 0, s>>>(N, h->g_off, h->g_deg, h->g_col, h->g_w, C, h->dcnt,
-                                                                      h->gid0, h->gc.sigma);
+  int32_t *big = h->ibuf0;
+  cudaMemsetAsync(&h->dcnt->big_count, 0, sizeof(int32_t), s);
+  ld_note_launch(), k_sigma_intra<<<grid_for(N, TB), TB, 0, s>>>(N, h->g_off, h->g_deg, h->g_col, h->g_w, C, h->dcnt,
+                                                                 h->gid0, h->gc.sigma, big);
+  launch_table_plan(big, &h->dcnt->big_count, h->g_deg, nullptr, 1, h->lbuf2, h->lbuf3, s);
+  ld_note_launch(), k_sigma_intra_big<<<h->sm_count * 8, TB, 0, s>>>(big, h->lbuf3, h->g_off, h->g_deg, h->g_col,
+                                                                     h->g_w, C, h->dcnt, h->gid0, h->gc.sigma);
   ld_note_launch(), k_sq<<<grid_for(N, TB), TB, 0, s>>>(N, Sig, h->dcnt, h->gid0, h->gc.sq);
 }
 
@@ -330,8 +472,13 @@ void recompute_weights(leiden_handle *h) {
   cudaStream_t s = h->stream;
   cudaMemsetAsync(&h->dcnt->m2, 0, sizeof(int64_t), s);
   if (h->gid0) cudaMemsetAsync(h->gc.m2, 0, (size_t)h->G * sizeof(int64_t), s);
-  ld_note_launch(), k_rowsum<<<grid_for(h->n * 32, TB), TB, 0, s>>>(h->n, h->g_off, h->g_deg, h->g_w, h->K, h->dcnt,
-                                                                    h->gid0, h->gc.m2);
+  int32_t *big = h->ibuf0;
+  cudaMemsetAsync(&h->dcnt->big_count, 0, sizeof(int32_t), s);
+  ld_note_launch(), k_rowsum<<<grid_for(h->n, TB), TB, 0, s>>>(h->n, h->g_off, h->g_deg, h->g_w, h->K, h->dcnt,
+                                                               h->gid0, h->gc.m2, big);
+  launch_table_plan(big, &h->dcnt->big_count, h->g_deg, nullptr, 1, h->lbuf2, h->lbuf3, s);
+  ld_note_launch(), k_rowsum_big<<<h->sm_count * 8, TB, 0, s>>>(big, h->lbuf3, h->g_off, h->g_deg, h->g_w, h->K,
+                                                                h->dcnt, h->gid0, h->gc.m2);
 }
 
 LD_CHECK_WORD_READER(check_word_track)

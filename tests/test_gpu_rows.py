@@ -1,0 +1,84 @@
+"""Kernels that walk rows by windows of 32 and cut long rows into chunks
+(modularity, row sums, Delta-screening's neighbour expansion): rows of the
+lengths where a window, a step or a chunk ends, against the oracle."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2410_15451_gb300 import leiden as L
+from paper_2410_15451_gb300 import synth
+from tests.helpers import csr_from_edges
+
+pytestmark = pytest.mark.gpu
+
+LENGTHS = {
+    "short": [0, 1, 31, 32, 33, 0, 0, 127, 128, 129, 2, 0],
+    "chunk": [4095, 4096, 4097, 0, 8191, 8193, 1, 0],
+    "hub": [12289, 0, 5],
+    "single": [1],
+}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2410_15451_gb300 import _build
+
+    _build.build()
+    L.load()
+
+
+def stars(lengths, weighted):
+    """Hubs spread over the ids, each joined to its own number of leaves (shared
+    between the hubs), and isolated vertices at both ends."""
+    leaves = max(lengths) if lengths else 0
+    n = leaves + 3 * len(lengths) + 5
+    hubs = [2 + 3 * k for k in range(len(lengths))]
+    others = [v for v in range(2, n - 3) if v not in set(hubs)]
+    edges = [(min(h, v), max(h, v)) for h, k in zip(hubs, lengths) for v in others[:k]]
+    w = [(1 << 30) - 7 * i if weighted else 1 for i in range(len(edges))]
+    off, col, wt = csr_from_edges(n, edges, w)
+    return synth.Graph(n, off, col, wt.astype(np.int32))
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("name", sorted(LENGTHS))
+def test_modularity_and_row_sums(name, weighted):
+    import torch
+
+    g = stars(LENGTHS[name], weighted)
+    w64 = g.w.astype(np.int64)
+    h = L.Leiden(g.n, g.off, g.col, g.w)
+    d = [torch.from_numpy(x).cuda() for x in (g.off, g.col, g.w)]
+    rng = np.random.default_rng(3)
+    for C in (np.zeros(g.n, np.int32), np.arange(g.n, dtype=np.int32), rng.integers(0, min(7, g.n), g.n).astype(np.int32)):
+        q, _ = oracle.modularity(g.off, g.col, w64, C)
+        c = torch.from_numpy(C).cuda()
+        assert h.modularity(C) == q
+        assert L.leiden_modularity_noalloc(g.n, d[0], d[1], d[2], c) == q
+        if not weighted:
+            assert L.leiden_modularity_noalloc(g.n, d[0], d[1], None, c) == q
+    h.static()
+    st = h.state()
+    K = np.zeros(g.n, np.int64)
+    np.add.at(K, np.repeat(np.arange(g.n), np.diff(g.off)), w64)
+    assert np.array_equal(st["K"], K) and st["m2"] == int(w64.sum())
+
+
+@pytest.mark.parametrize("name", ["short", "chunk", "hub"])
+def test_screening_expands_rows_of_every_length(name):
+    g = stars(LENGTHS[name], False)
+    gpu = L.Leiden(g.n, g.off, g.col, g.w)
+    ref = oracle.Oracle(g.n, g.off, g.col, g.w, schedule=oracle.SYNC)
+    gpu.static(), ref.static()
+    # an edge of every hub deleted (its row is expanded), edges between leaves and isolated vertices inserted
+    dels = [(2 + 3 * k, int(g.col[g.off[2 + 3 * k]]), 1) for k in range(len(LENGTHS[name])) if LENGTHS[name][k]]
+    ins = [(0, 3, 1), (1, 4, 2), (g.n - 1, 3, 1)]
+    assert np.array_equal(gpu.update(dels, ins, L.LEIDEN_DS), ref.update(dels, ins, oracle.DS))
+    assert np.array_equal(gpu.affected(), ref.affected())
+    assert np.array_equal(gpu.state()["K"], ref.state()["K"])
