@@ -19,9 +19,9 @@ struct DevCounters {
   unsigned long long dq[2];       // sum of accepted gains g (int128, two's complement)
   int32_t bin_count[4];           // vertices in each degree bin of the current sub-sweep
   int32_t movers;                 // deferred moves of the current sub-sweep (SYNC)
+  int32_t big_movers;             // moved hubs whose neighbours are marked when the moves are applied
   int32_t accepted;               // refinement moves applied in this round
   int32_t cand_count[2];          // refinement candidate lists (ping-pong)
-  int32_t refined_any;            // a vertex lies in a refined bound
   int32_t error;                  // batch validation error (first offending arc + 1)
   int32_t overflow;               // a touched CSR row outgrew its capacity
   int32_t list_count;             // generic list length
@@ -45,6 +45,7 @@ struct DevCounters {
   int32_t large_count;            // batch apply: touched rows merged in chunks
   int32_t tr_occ;                 // tracking: filled slots of the pair table
   int32_t mid_count;              // batch apply: touched rows merged by one block each
+  int32_t hub_big;                // local moving: listed hubs whose tables are read in pieces
   int64_t arena_used;             // next free arc slot of G^t (relocated rows go here)
   int64_t bcounts[8];             // batch apply: unique deletions, unique insertions, new arcs,
                                   //   touched rows, merge-buffer arcs
@@ -158,106 +159,143 @@ __device__ __forceinline__ bool ld_group_leader(uint32_t peers) {
   return (__ffs(peers) - 1) == (int)(threadIdx.x & 31);
 }
 
-// Open-addressing insert into a global table (linear probing, key -1 =
-// empty) that records each slot it fills in `list` (count in *occ), so the
-// reader visits only filled slots and can empty them again afterwards.
-__device__ __forceinline__ void ld_gtable_insert(int32_t *keys, int64_t *vals, int32_t *list, int32_t *occ, int tmask,
-                                                 int32_t c, int64_t w) {
-  // A slot's key only goes from empty to a key while a table is in use, so
-  // a plain read from L2 decides every probe but the claim of an empty slot:
-  // a key already in the table costs a load and an add whose result is not
-  // waited for, instead of a compare-and-swap on a slot every warp touches.
-  uint32_t s = ld_hash32((uint32_t)c) & (uint32_t)tmask;
-  for (uint32_t probe = 0; ld_ok(probe <= (uint32_t)tmask, LD_CHK_PROBE); probe++) {
-    int32_t k = __ldcg(&keys[s]);
-    if (k == LD_EMPTY_KEY) {
-      k = atomicCAS(&keys[s], LD_EMPTY_KEY, c);
+// ---------------------------------------------------------------- sums by community
+// Tables of (community, weight sum).  NARROW tables hold 32-bit sums and are
+// used when the graph's total weight 2m is below 2^32, which bounds every sum
+// of arc weights; WIDE ones hold the low and the high halves apart, so that
+// the shared-memory adds are 32-bit in both (the high half is only touched by
+// a carry or a weight above 2^32; 64-bit shared atomics cost more than twice
+// as much).  The sums are exact in both.
+
+// The gain term m2 * kv - Ki * S as an exact 128-bit integer.  NARROW: all four
+// below 2^32, so each product is one 32 x 32 multiplication.
+template <bool WIDE>
+__device__ __forceinline__ i128 ld_gain(int64_t m2, int64_t kv, int64_t Ki, int64_t S) {
+  if (WIDE) return (i128)m2 * kv - (i128)Ki * S;
+  uint64_t a = (uint64_t)(uint32_t)m2 * (uint32_t)kv, b = (uint64_t)(uint32_t)Ki * (uint32_t)S;
+  return (i128)a - (i128)b;
+}
+
+// Lane holding the largest v among the lanes with c >= 0, ties to the
+// smallest c; -1 if there is none.  All lanes call it.  The warp's reduction
+// unit takes the value word by word (a butterfly of shuffles moves every
+// field of a candidate through every step).
+template <bool WIDE>
+__device__ __forceinline__ int ld_warp_argmax(i128 v, int32_t c) {
+  bool has = c >= 0;
+  if (!__any_sync(LD_FULL, has)) return -1;
+  // (every lane takes part in every reduction; `has` only selects its input)
+  if (WIDE) {
+    int32_t w3 = (int32_t)(v >> 96), m3 = __reduce_max_sync(LD_FULL, has ? w3 : INT32_MIN);
+    has = has && w3 == m3;
+    uint32_t w2 = (uint32_t)((u128)v >> 64), m2 = __reduce_max_sync(LD_FULL, has ? w2 : 0u);
+    has = has && w2 == m2;
+  } else {  // |v| < 2^64: the upper half is the sign
+    int32_t w2 = (int32_t)(v >> 64), m2 = __reduce_max_sync(LD_FULL, has ? w2 : INT32_MIN);
+    has = has && w2 == m2;
+  }
+  uint32_t w1 = (uint32_t)((u128)v >> 32), m1 = __reduce_max_sync(LD_FULL, has ? w1 : 0u);
+  has = has && w1 == m1;
+  uint32_t w0 = (uint32_t)(u128)v, m0 = __reduce_max_sync(LD_FULL, has ? w0 : 0u);
+  has = has && w0 == m0;
+  int32_t cm = __reduce_min_sync(LD_FULL, has ? c : INT32_MAX);
+  return __ffs(__ballot_sync(LD_FULL, has && c == cm)) - 1;
+}
+
+// Sum over the lanes of a warp of values whose total is a sum of arc weights.
+template <bool WIDE>
+__device__ __forceinline__ int64_t ld_warp_weight(int64_t v) {
+  if (WIDE) return ld_warp_sum_i64(v);
+  return (int64_t)__reduce_add_sync(LD_FULL, (uint32_t)v);
+}
+
+// A table in global memory (a vertex's or a community's slice of the handle's
+// table scratch): open addressing on the community id, or, when it has a slot
+// per community (dense), indexed by it.  Slots filled are listed (count in
+// *occ), so the reader visits only those and empties them again.  NARROW: key
+// + 1 and sum share one 64-bit word of `vals` (0 = empty), so an insertion
+// touches one sector (emission of the giant communities' tables, R-MAT 21
+// static: 2525 -> 570 us per launch, its loads four deep; chunked scan 2259 ->
+// 1438 us); WIDE: key in `keys` (-1 = empty), sum in `vals`.  Both
+// leave keys all -1 and vals all 0.
+struct GTable {
+  int32_t *keys;
+  int64_t *vals;
+  int32_t *list;
+  int32_t *occ;
+  int mask;
+  bool dense;
+};
+
+// Find or claim the slot of c and add w; the claimed slot if it was empty,
+// else -1.  A slot's key only goes from empty to a key while a table is in
+// use, so a plain read from L2 decides every probe but the claim of an empty
+// slot.
+template <bool WIDE>
+__device__ __forceinline__ int32_t gt_add(const GTable &T, int32_t c, int64_t w) {
+  uint32_t s = T.dense ? (uint32_t)c : ld_hash32((uint32_t)c) & (uint32_t)T.mask;
+  for (uint32_t probe = 0; ld_ok(probe <= (uint32_t)T.mask, LD_CHK_PROBE); probe++) {
+    if (WIDE) {
+      int32_t k = __ldcg(&T.keys[s]);
+      bool claimed = false;
       if (k == LD_EMPTY_KEY) {
-        list[atomicAdd(occ, 1)] = (int32_t)s;
-        k = c;
+        k = atomicCAS(&T.keys[s], LD_EMPTY_KEY, c);
+        claimed = k == LD_EMPTY_KEY;
+      }
+      if (claimed || k == c) {
+        atomicAdd((unsigned long long *)&T.vals[s], (unsigned long long)w);
+        return claimed ? (int32_t)s : -1;
+      }
+    } else {
+      unsigned long long *p = (unsigned long long *)&T.vals[s];
+      unsigned long long key = (unsigned long long)((uint32_t)c + 1u) << 32, x = __ldcg(p);
+      if (x == 0) {
+        x = atomicCAS(p, 0ull, key | (uint32_t)w);
+        if (x == 0) return (int32_t)s;
+      }
+      if ((x >> 32) == (key >> 32)) {
+        atomicAdd(p, (unsigned long long)(uint32_t)w);
+        return -1;
       }
     }
-    if (k == c) {
-      atomicAdd((unsigned long long *)&vals[s], (unsigned long long)w);
-      return;
-    }
-    s = (s + 1) & (uint32_t)tmask;
+    s = (s + 1) & (uint32_t)T.mask;
   }
+  return -1;
 }
 
-// The same for a table with a slot per key (slot = key): the key array
-// only marks the slots already listed.
-__device__ __forceinline__ void ld_gtable_add_direct(int32_t *keys, int64_t *vals, int32_t *list, int32_t *occ,
-                                                     int32_t c, int64_t w) {
-  if (__ldcg(&keys[c]) == LD_EMPTY_KEY && atomicCAS(&keys[c], LD_EMPTY_KEY, c) == LD_EMPTY_KEY)
-    list[atomicAdd(occ, 1)] = c;
-  atomicAdd((unsigned long long *)&vals[c], (unsigned long long)w);
+// One lane: add and list.
+template <bool WIDE>
+__device__ __forceinline__ void gt_insert(const GTable &T, int32_t c, int64_t w) {
+  int32_t s = gt_add<WIDE>(T, c, w);
+  if (s >= 0) T.list[atomicAdd(T.occ, 1)] = s;
 }
 
-// All 32 lanes, each with up to GT_KEYS keys (has[u]): add them to a global
-// table (`direct`: slot = key; otherwise open addressing as above).  A key's
-// slot is read first and claimed only when empty; the weight add is not
-// waited for; a collision probes on.  The slots claimed by the warp are
-// listed with one atomic on the fill count, which every warp flushing into
-// the same table would otherwise hit once per new key.  GT_KEYS is 1: with
-// more keys per lane in flight the loops' registers cost the hub scan more
-// occupancy than the overlapped reads gained.
-constexpr int GT_KEYS = 1;
-__device__ __forceinline__ void ld_gtable_add_warp(const bool *has, bool direct, int32_t *keys, int64_t *vals,
-                                                   int32_t *list, int32_t *occ, int tmask, const int32_t *c,
-                                                   const int64_t *w) {
+// All 32 lanes, each with at most one key: the slots claimed by the warp are
+// listed with one atomic on the fill count.
+template <bool WIDE>
+__device__ __forceinline__ void gt_insert_warp(const GTable &T, bool has, int32_t c, int64_t w) {
   int lane = threadIdx.x & 31;
-  uint32_t s[GT_KEYS];
-  int32_t k[GT_KEYS], claimed[GT_KEYS];
-#pragma unroll
-  for (int u = 0; u < GT_KEYS; u++) {
-    s[u] = direct ? (uint32_t)c[u] : ld_hash32((uint32_t)c[u]) & (uint32_t)tmask;
-    k[u] = has[u] ? __ldcg(&keys[s[u]]) : c[u];
-    claimed[u] = -1;
-  }
-#pragma unroll
-  for (int u = 0; u < GT_KEYS; u++) {
-    if (has[u] && k[u] == LD_EMPTY_KEY) {
-      k[u] = atomicCAS(&keys[s[u]], LD_EMPTY_KEY, c[u]);
-      if (k[u] == LD_EMPTY_KEY) {
-        claimed[u] = (int32_t)s[u];
-        k[u] = c[u];
-      }
-    }
-  }
-  int mine = 0;
-#pragma unroll
-  for (int u = 0; u < GT_KEYS; u++) {
-    if (!has[u]) continue;
-    // a collision (hash tables only: a direct slot holds its own key or none)
-    for (uint32_t probe = 1; k[u] != c[u] && ld_ok(probe <= (uint32_t)tmask, LD_CHK_PROBE); probe++) {
-      s[u] = (s[u] + 1) & (uint32_t)tmask;
-      k[u] = __ldcg(&keys[s[u]]);
-      if (k[u] == LD_EMPTY_KEY) {
-        k[u] = atomicCAS(&keys[s[u]], LD_EMPTY_KEY, c[u]);
-        if (k[u] == LD_EMPTY_KEY) {
-          claimed[u] = (int32_t)s[u];
-          k[u] = c[u];
-        }
-      }
-    }
-    if (k[u] == c[u]) atomicAdd((unsigned long long *)&vals[s[u]], (unsigned long long)w[u]);
-    mine += claimed[u] >= 0;
-  }
-  int incl = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int y = __shfl_up_sync(LD_FULL, incl, o);
-    if (lane >= o) incl += y;
-  }
-  int total = __shfl_sync(LD_FULL, incl, 31);
-  if (total == 0) return;  // warp-uniform
-  int32_t base = 0;
-  if (lane == 31) base = atomicAdd(occ, total);
-  base = __shfl_sync(LD_FULL, base, 31) + incl - mine;
-#pragma unroll
-  for (int u = 0; u < GT_KEYS; u++)
-    if (claimed[u] >= 0) list[base++] = claimed[u];
+  int32_t s = has ? gt_add<WIDE>(T, c, w) : -1;
+  uint32_t m = __ballot_sync(LD_FULL, s >= 0);
+  if (!m) return;
+  int leader = __ffs(m) - 1;
+  int32_t p0 = 0;
+  if (lane == leader) p0 = atomicAdd(T.occ, __popc(m));
+  p0 = __shfl_sync(LD_FULL, p0, leader);
+  if (s >= 0) T.list[p0 + __popc(m & ((1u << lane) - 1u))] = s;
+}
+
+// Read slot s; leave it empty.
+template <bool WIDE>
+__device__ __forceinline__ void gt_read(const GTable &T, int32_t s, int32_t &c, int64_t &w) {
+  int64_t x = T.vals[s];
+  c = WIDE ? T.keys[s] : (int32_t)((uint64_t)x >> 32) - 1;
+  w = WIDE ? x : (int64_t)(uint32_t)x;
+}
+template <bool WIDE>
+__device__ __forceinline__ void gt_empty(const GTable &T, int32_t s) {
+  if (WIDE) T.keys[s] = LD_EMPTY_KEY;
+  T.vals[s] = 0;
 }
 
 // Shared staging table of one block (local moving and refinement of the
@@ -265,93 +303,103 @@ __device__ __forceinline__ void ld_gtable_add_warp(const bool *has, bool direct,
 constexpr int STAGE_SLOTS = 2048;
 constexpr int STAGE_FILL = 1024;  // distinct keys per use at most (load <= 1/2)
 
-// Warp-private shared table: only the lanes of one warp touch it, so the
-// only contention on a slot is between lanes with the same key.  Flushed
+// Warp-private shared table: only the lanes of one warp touch it.  Flushed
 // into a global table before it passes half full.
 constexpr int WT_SLOTS = 256;
 constexpr int WT_LIMIT = WT_SLOTS / 2 - 32;  // flush above this many keys
-struct WarpTable {
-  int32_t keys[WT_SLOTS];
-  int64_t vals[WT_SLOTS];
-  int32_t list[WT_SLOTS / 2];
+
+// `hi` of a NARROW table is one unused word.
+template <bool WIDE, int SLOTS, int FILL, typename Slot>
+struct STable {
+  int32_t keys[SLOTS];
+  uint32_t lo[SLOTS];
+  uint32_t hi[WIDE ? SLOTS : 1];
+  Slot list[FILL];
+};
+template <bool WIDE>
+struct WarpTable : STable<WIDE, WT_SLOTS, WT_SLOTS / 2, uint8_t> {
   int32_t count;
 };
 
-__device__ __forceinline__ void wt_init(WarpTable &T) {
-  int lane = threadIdx.x & 31;
-  for (int s = lane; s < WT_SLOTS; s += 32) { T.keys[s] = LD_EMPTY_KEY; T.vals[s] = 0; }
-  if (lane == 0) T.count = 0;
-  __syncwarp();
+template <typename T>
+__device__ __forceinline__ void st_clear(T &t, int first, int stride, int slots) {
+  for (int s = first; s < slots; s += stride) {
+    t.keys[s] = LD_EMPTY_KEY;
+    t.lo[s] = 0;
+    if (sizeof(t.hi) > 4) t.hi[s] = 0;
+  }
 }
 
-// All 32 lanes call it; each lane with a pair adds it on its own with a
-// shared-memory atomic (lanes of one warp only, so the only contention is
-// between lanes with the same key, which the atomic unit serialises) -- no
-// key grouping and no shuffles.
-__device__ __forceinline__ void wt_insert_lanes(WarpTable &T, bool valid, int32_t c, int64_t w) {
-  if (valid) {
-    uint32_t s = ld_hash32((uint32_t)c) & (uint32_t)(WT_SLOTS - 1);
-    for (int probe = 0; ld_ok(probe < WT_SLOTS, LD_CHK_PROBE); probe++) {
-      int32_t k = T.keys[s];
-      if (k == LD_EMPTY_KEY) {
-        k = atomicCAS(&T.keys[s], LD_EMPTY_KEY, c);
-        if (k == LD_EMPTY_KEY) {
-          T.list[atomicAdd(&T.count, 1)] = (int32_t)s;
-          k = c;
-        }
-      }
-      if (k == c) {
-        atomicAdd((unsigned long long *)&T.vals[s], (unsigned long long)w);
-        break;
-      }
-      s = (s + 1) & (uint32_t)(WT_SLOTS - 1);
-    }
+template <bool WIDE, int SLOTS, int FILL, typename Slot>
+__device__ __forceinline__ void st_add(STable<WIDE, SLOTS, FILL, Slot> &t, uint32_t s, int64_t w) {
+  uint32_t a = (uint32_t)w;
+  if (!WIDE) {
+    atomicAdd(&t.lo[s], a);
+  } else {
+    uint32_t old = atomicAdd(&t.lo[s], a), h = (uint32_t)((uint64_t)w >> 32) + (old + a < old ? 1u : 0u);
+    if (h) atomicAdd(&t.hi[s], h);
   }
+}
+
+// Add (c, w); a newly filled slot is listed with the fill count *count.
+// Lanes of one warp or of one block may call it at once.
+template <bool WIDE, int SLOTS, int FILL, typename Slot>
+__device__ __forceinline__ void st_insert(STable<WIDE, SLOTS, FILL, Slot> &t, int32_t *count, int32_t c, int64_t w) {
+  uint32_t s = ld_hash32((uint32_t)c) & (uint32_t)(SLOTS - 1);
+  for (int probe = 0; ld_ok(probe < SLOTS, LD_CHK_PROBE); probe++) {
+    int32_t k = t.keys[s];
+    if (k == LD_EMPTY_KEY) {
+      k = atomicCAS(&t.keys[s], LD_EMPTY_KEY, c);
+      if (k == LD_EMPTY_KEY) {
+        t.list[atomicAdd(count, 1)] = (Slot)s;
+        k = c;
+      }
+    }
+    if (k == c) {
+      st_add(t, s, w);
+      return;
+    }
+    s = (s + 1) & (uint32_t)(SLOTS - 1);
+  }
+}
+
+// Read the listed slot q and leave it empty.
+template <bool WIDE, int SLOTS, int FILL, typename Slot>
+__device__ __forceinline__ void st_take(STable<WIDE, SLOTS, FILL, Slot> &t, int q, int32_t &c, int64_t &w) {
+  uint32_t s = t.list[q];
+  c = t.keys[s];
+  w = (int64_t)t.lo[s];
+  t.keys[s] = LD_EMPTY_KEY;
+  t.lo[s] = 0;
+  if (WIDE) {
+    w |= (int64_t)((uint64_t)t.hi[s] << 32);
+    t.hi[s] = 0;
+  }
+}
+
+template <bool WIDE>
+__device__ __forceinline__ void wt_init(WarpTable<WIDE> &T) {
+  st_clear(T, threadIdx.x & 31, 32, WT_SLOTS);
+  if ((threadIdx.x & 31) == 0) T.count = 0;
   __syncwarp();
 }
 
 // All 32 lanes: move the pairs into a global table and empty the warp table.
-__device__ __forceinline__ void wt_flush_to(WarpTable &T, bool direct, int32_t *gkeys, int64_t *gvals,
-                                            int32_t *glist, int32_t *gocc, int gmask) {
+template <bool WIDE>
+__device__ __forceinline__ void wt_flush(WarpTable<WIDE> &T, const GTable &G) {
   int lane = threadIdx.x & 31;
   __syncwarp();
   int n = T.count;
-  for (int q0 = 0; q0 < n; q0 += 32 * GT_KEYS) {  // warp-uniform
-    bool has[GT_KEYS];
-    int32_t sl[GT_KEYS], key[GT_KEYS];
-    int64_t v[GT_KEYS];
-#pragma unroll
-    for (int u = 0; u < GT_KEYS; u++) {
-      int q = q0 + 32 * u + lane;
-      has[u] = q < n;
-      sl[u] = has[u] ? T.list[q] : 0;
-      key[u] = has[u] ? T.keys[sl[u]] : 0;
-      v[u] = has[u] ? T.vals[sl[u]] : 0;
-    }
-    ld_gtable_add_warp(has, direct, gkeys, gvals, glist, gocc, gmask, key, v);
-#pragma unroll
-    for (int u = 0; u < GT_KEYS; u++) {
-      if (has[u]) {
-        T.keys[sl[u]] = LD_EMPTY_KEY;
-        T.vals[sl[u]] = 0;
-      }
-    }
+  for (int q0 = 0; q0 < n; q0 += 32) {  // warp-uniform
+    bool has = q0 + lane < n;
+    int32_t c = 0;
+    int64_t w = 0;
+    if (has) st_take(T, q0 + lane, c, w);
+    gt_insert_warp<WIDE>(G, has, c, w);
   }
   __syncwarp();
   if (lane == 0) T.count = 0;
   __syncwarp();
-}
-
-__device__ __forceinline__ void wt_flush(WarpTable &T, int32_t *gkeys, int64_t *gvals, int32_t *glist, int32_t *gocc,
-                                         int gmask) {
-  wt_flush_to(T, false, gkeys, gvals, glist, gocc, gmask);
-}
-
-// All 32 lanes: move the pairs into a directly indexed table (slot = key,
-// for keys below the table's size) and empty the warp table.
-__device__ __forceinline__ void wt_flush_dense(WarpTable &T, int32_t *gkeys, int64_t *gvals, int32_t *glist,
-                                               int32_t *gocc) {
-  wt_flush_to(T, true, gkeys, gvals, glist, gocc, 0);
 }
 
 // Per-graph sums of a batched handle: every lane of the warp calls these;

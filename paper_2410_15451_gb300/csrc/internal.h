@@ -278,10 +278,21 @@ void launch_fill_i64(int64_t *p, int64_t v, int64_t n, cudaStream_t s);
 void launch_iota_i32(int32_t *p, int64_t n, cudaStream_t s);
 // Per-item global tables and work chunks for the listed items (see prims.cu).
 constexpr int TABLE_CHUNK = 4096;
+// Of the listed items, those with more than BIG_KEYS filled slots (occ), whose
+// tables are read by a block per piece of BIG_PIECE slots.
+constexpr int BIG_KEYS = 512;
+constexpr int BIG_PIECE = 2048;
+struct BigTables {
+  int32_t *items = nullptr;   // list positions of those items
+  int32_t *count = nullptr;   // how many
+  int64_t *pieces = nullptr;  // their piece offsets, total at *count
+  int32_t *ticket = nullptr;  // by list position: pieces finished so far
+};
+void launch_piece_plan(const int32_t *count, const int32_t *occ, const BigTables &big, cudaStream_t s);
 // key_cap: the most distinct keys any item can have (tables take
-// pow2 >= 2*min(size, key_cap) slots).
+// pow2 >= 2*min(size, key_cap) slots).  occ: zeroed for the listed items.
 void launch_table_plan(const int32_t *list, const int32_t *count, const int32_t *deg32, const int64_t *off64,
-                       int64_t key_cap, int64_t *tab_off, int64_t *ch_off, cudaStream_t s);
+                       int64_t key_cap, int64_t *tab_off, int64_t *ch_off, cudaStream_t s, int32_t *occ = nullptr);
 int grid_for(int64_t n, int block, int max_blocks = 152 * 16);
 
 // ------------------------------------------------------------ batch.cu
@@ -296,6 +307,10 @@ inline int64_t spill_arena_size(int64_t used, int log2_min) { return used / 8 + 
 inline int lm_classes(const leiden_handle *h) {
   return h->p.deterministic ? h->p.classes : (h->p.classes > 16 ? h->p.classes : 16);
 }
+
+// Sums of arc weights need 64 bits (else the tables of sums by community hold
+// 32): every such sum is at most 2m.
+inline bool wide_sums(const leiden_handle *h) { return h->m2 >= ((int64_t)1 << 32); }
 
 // ------------------------------------------------------------ move.cu
 // One local-moving sub-sweep of class `cls` (0 .. classes-1).

@@ -14,7 +14,6 @@
 // move as soon as it is found.
 #include <algorithm>
 #include <atomic>
-#include <type_traits>
 
 #include "internal.h"
 
@@ -44,6 +43,7 @@ struct Args {
   uint32_t *unproc;      // bitmap
   const uint8_t *in_range;
   int32_t *movers, *mtarget;
+  int32_t *big_movers;   // moved hubs whose neighbours the apply kernel marks
   const int32_t *list;   // bin list
   const int32_t *count;  // bin count (device)
   const int32_t *list_tiny;   // bin 3 list (degree <= 8), used with bin 0
@@ -70,102 +70,6 @@ struct Args {
 
 // 2m of the graph vertex i belongs to.
 __device__ __forceinline__ int64_t m2_of(const Args &A, int64_t i) { return A.gid ? A.m2g[A.gid[i]] : A.m2; }
-
-__device__ __forceinline__ int next_pow2(int x) {
-  int p = 1;
-  while (p < x) p <<= 1;
-  return p;
-}
-
-__device__ __forceinline__ void table_insert(int32_t *keys, int64_t *vals, int tmask, int32_t c, int64_t w) {
-  uint32_t s = ld_hash32((uint32_t)c) & (uint32_t)tmask;
-  for (uint32_t probe = 0; ld_ok(probe <= (uint32_t)tmask, LD_CHK_PROBE); probe++) {
-    int32_t k = atomicCAS(&keys[s], LD_EMPTY_KEY, c);
-    if (k == LD_EMPTY_KEY || k == c) {
-      atomicAdd((unsigned long long *)&vals[s], (unsigned long long)w);
-      return;
-    }
-    s = (s + 1) & (uint32_t)tmask;
-  }
-}
-
-// Decision of one vertex once its table is complete: the best community c*
-// (other than the current d), K_{i->c*}, K_{i->d}.
-struct Best {
-  i128 v;
-  int32_t c;
-  int64_t kc;
-  int64_t kd;
-};
-
-__device__ __forceinline__ void best_merge(Best &a, const Best &b) {
-  if (ld_better(b.v, b.c, a.v, a.c)) { a.v = b.v; a.c = b.c; a.kc = b.kc; }
-  a.kd += b.kd;
-}
-
-__device__ __forceinline__ Best warp_best(Best b) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    Best t;
-    t.v = ld_shfl_xor_i128(b.v, o);
-    t.c = __shfl_xor_sync(LD_FULL, b.c, o);
-    t.kc = __shfl_xor_sync(LD_FULL, b.kc, o);
-    t.kd = __shfl_xor_sync(LD_FULL, b.kd, o);
-    best_merge(b, t);
-  }
-  return b;
-}
-
-// Scan arcs [lo, hi) of vertex i with `stride` threads starting at `t0`.
-template <typename W, int KIND>
-__device__ __forceinline__ void scan_arcs(const Args &A, int64_t i, int64_t base, int64_t dg, int t0, int stride,
-                                          int32_t *keys, int64_t *vals, int tmask) {
-  const W *w = (const W *)A.w;
-  int32_t bi = KIND == KIND_REFINE ? A.CB[i] : 0;
-  for (int64_t a = t0; a < dg; a += stride) {
-    int32_t j = A.col[base + a];
-    if (j == i) continue;
-    if (KIND == KIND_REFINE && A.CB[j] != bi) continue;
-    table_insert(keys, vals, tmask, A.C[j], (int64_t)w[base + a]);
-  }
-}
-
-// The decision and its effects, run by one thread (the group leader).
-// Returns the gain counted into dQ (0 if no move).
-template <int KIND>
-__device__ __forceinline__ i128 decide_leader(const Args &A, int64_t i, const Best &b) {
-  int32_t d = A.C[i];
-  int64_t Ki = A.K[i];
-  int64_t m2 = m2_of(A, i);
-  if (b.c < 0) return 0;
-  i128 g = (i128)m2 * (b.kc - b.kd) - (i128)Ki * ((i128)Ki + A.S[b.c] - A.S[d]);
-  if (g <= 0) return 0;
-  if (KIND == KIND_MOVE) {
-    if (A.size[d] == 1 && A.size[b.c] == 1 && b.c > d) return 0;
-    if (A.async_mode) {
-      A.C[i] = b.c;
-      atomicAdd((unsigned long long *)&A.S[d], (unsigned long long)(-Ki));
-      atomicAdd((unsigned long long *)&A.S[b.c], (unsigned long long)Ki);
-      atomicSub(&A.size[d], 1);
-      atomicAdd(&A.size[b.c], 1);
-    } else {
-      int32_t slot = atomicAdd(&A.cnt->movers, 1);
-      A.movers[slot] = (int32_t)i;
-      A.mtarget[slot] = b.c;
-      if (A.mgain) { A.mgain[2 * slot] = (int64_t)(u128)g; A.mgain[2 * slot + 1] = (int64_t)((u128)g >> 64); }
-    }
-    if (A.dynamic) A.dS[d] = 1;
-    return g;
-  } else {
-    // Refinement runs in proposal/accept rounds in both modes: an in-place
-    // CAS scheme (pin the target, then leave) never merges mutual best
-    // pairs, because both pin each other before either can leave, and such
-    // pairs are common since the gain of joining a singleton is symmetric.
-    if (A.C[b.c] != b.c) return 0;  // the representative of c* left it
-    A.prop[i] = b.c;
-    return g;
-  }
-}
 
 __device__ __forceinline__ void mark_neighbours(const Args &A, int64_t i, int64_t base, int64_t dg, int t0,
                                                 int stride) {
@@ -199,46 +103,78 @@ __device__ __forceinline__ void add_lmk(DevCounters *cnt, int k, int64_t visits,
 }
 
 // ---------------------------------------------------------------- bins 3 and 0: warp range
-// Candidate with the values the decision needs carried along, so that the
-// winner's Sigma and size are not loaded again after the reduction.
+// The best candidate community of a vertex with what its decision needs:
+// K_{i->c}, Sigma_c, and K_{i->d} of the vertex's own community.
 struct BestX {
   i128 v;
   int32_t c;
-  int32_t szc;  // size of c (local moving)
+  int32_t szc;  // size of c (local moving; read for the winner only)
   int64_t kc;
   int64_t kd;
   int64_t sc;   // Sigma of c
 };
 
 __device__ __forceinline__ void bestx_merge(BestX &a, const BestX &b) {
-  if (ld_better(b.v, b.c, a.v, a.c)) { a.v = b.v; a.c = b.c; a.kc = b.kc; a.sc = b.sc; a.szc = b.szc; }
+  if (ld_better(b.v, b.c, a.v, a.c)) { a.v = b.v; a.c = b.c; a.kc = b.kc; a.sc = b.sc; }
   a.kd += b.kd;
 }
 
-__device__ __forceinline__ int64_t shfl_xor_i64(int64_t v, int o) { return __shfl_xor_sync(LD_FULL, v, o); }
+// The warp's best candidate and summed K_{i->d}, in every lane.
+template <bool WIDE>
+__device__ __forceinline__ BestX warp_bestx(BestX b) {
+  b.kd = ld_warp_weight<WIDE>(b.kd);
+  int win = ld_warp_argmax<WIDE>(b.v, b.c);
+  int src = win < 0 ? 0 : win;
+  uint64_t lo = __shfl_sync(LD_FULL, (unsigned long long)(u128)b.v, src);
+  int64_t hi = __shfl_sync(LD_FULL, (long long)(b.v >> 64), src);
+  b.v = (i128)(((u128)(uint64_t)hi << 64) | lo);
+  b.c = __shfl_sync(LD_FULL, b.c, src);
+  b.kc = __shfl_sync(LD_FULL, b.kc, src);
+  b.sc = __shfl_sync(LD_FULL, b.sc, src);
+  if (win < 0) b.c = -1;
+  return b;
+}
 
-// Reduction over lanes that differ in the bits of `width` - 1 (width 8:
-// within aligned groups of 8 lanes; 32: the whole warp).
-template <int WIDTH>
-__device__ __forceinline__ BestX bestx_reduce(BestX b) {
+// The block's best and summed K_{i->d}, in every thread (sb: one per warp).
+template <bool WIDE>
+__device__ __forceinline__ BestX block_bestx(BestX b, BestX *sb) {
+  b = warp_bestx<WIDE>(b);
+  if ((threadIdx.x & 31) == 0) sb[threadIdx.x >> 5] = b;
+  __syncthreads();
+  BestX r = sb[0];
+  for (int q = 1; q < (int)(blockDim.x >> 5); q++) bestx_merge(r, sb[q]);
+  __syncthreads();
+  return r;
+}
+
+// The best over aligned groups of eight lanes, by a butterfly over (value,
+// community, lane); the other fields are read from the winner once.
+__device__ __forceinline__ BestX group_bestx(BestX b) {
+  i128 v = b.v;
+  int32_t c = b.c;
+  int at = threadIdx.x & 31;
 #pragma unroll
-  for (int o = WIDTH / 2; o > 0; o >>= 1) {
-    BestX t;
-    t.v = ld_shfl_xor_i128(b.v, o);
-    t.c = __shfl_xor_sync(LD_FULL, b.c, o);
-    t.szc = __shfl_xor_sync(LD_FULL, b.szc, o);
-    t.kc = shfl_xor_i64(b.kc, o);
-    t.kd = shfl_xor_i64(b.kd, o);
-    t.sc = shfl_xor_i64(b.sc, o);
-    bestx_merge(b, t);
+  for (int o = 4; o > 0; o >>= 1) {
+    i128 tv = ld_shfl_xor_i128(v, o);
+    int32_t tc = __shfl_xor_sync(LD_FULL, c, o);
+    int ta = __shfl_xor_sync(LD_FULL, at, o);
+    if (ld_better(tv, tc, v, c)) { v = tv; c = tc; at = ta; }
+    b.kd += __shfl_xor_sync(LD_FULL, b.kd, o);
   }
+  b.v = v;
+  b.c = c;
+  b.kc = __shfl_sync(LD_FULL, b.kc, at);
+  b.sc = __shfl_sync(LD_FULL, b.sc, at);
   return b;
 }
 
 // The decision of vertex i in community d (K_i, Sigma_d, size_d given) for
 // the reduced candidate b.  Returns the gain (Eq. 2 times 2m^2) when i moves
 // (local moving) or proposes (refinement), else 0; the caller records a
-// deferred move.
+// deferred move.  Refinement runs in proposal/accept rounds in both modes: an
+// in-place CAS scheme (pin the target, then leave) never merges mutual best
+// pairs, because both pin each other before either can leave, and such
+// pairs are common since the gain of joining a singleton is symmetric.
 template <int KIND>
 __device__ __forceinline__ i128 decide_x(const Args &A, int64_t i, int32_t d, int64_t Ki, int64_t Sd, int32_t szd,
                                          int64_t m2, BestX b) {
@@ -298,14 +234,25 @@ __device__ __forceinline__ void record_movers(const Args &A, bool mv, int32_t i,
   }
 }
 
+// One thread's deferred move.
+__device__ __forceinline__ void record_mover(const Args &A, int32_t i, int32_t c, i128 g) {
+  int32_t slot = atomicAdd(&A.cnt->movers, 1);
+  A.movers[slot] = i;
+  A.mtarget[slot] = c;
+  if (A.mgain) { A.mgain[2 * slot] = (int64_t)(u128)g; A.mgain[2 * slot + 1] = (int64_t)((u128)g >> 64); }
+}
+
 struct Tally {
   int64_t visits = 0, arcs = 0, moves = 0;
   i128 dq = 0;
 };
 
-// Per-block sums of the lanes' tallies, then one set of counter updates.
-template <typename W, int KIND>
-__device__ __forceinline__ void flush_tally(const Args &A, Tally t) {
+// Per-block sums of the lanes' tallies, then one set of counter updates; with
+// kt >= 0 also the work counters of that timed kernel (local moving;
+// algorithmic bytes: per visit the list entry, off, deg, C[i], K[i],
+// Sigma[C[i]], size[C[i]], 40 B; per arc col, C[j] and the weight).
+template <int KIND>
+__device__ __forceinline__ void flush_tally(const Args &A, Tally t, int kt = -1, int wbytes = 0) {
   __shared__ unsigned long long sacc[6];
   if (threadIdx.x < 6) sacc[threadIdx.x] = 0;
   __syncthreads();
@@ -323,11 +270,8 @@ __device__ __forceinline__ void flush_tally(const Args &A, Tally t) {
   if (threadIdx.x == 0 && sacc[0]) {
     i128 dq = (i128)(((u128)sacc[4] << 64) | (u128)sacc[3]);
     add_counters(A.cnt, KIND, (int64_t)sacc[0], (int64_t)sacc[1], (int64_t)sacc[2], dq);
-    if (KIND == KIND_MOVE) {
-      // algorithmic bytes: per visit the list entry, off, deg, C[i], K[i],
-      // Sigma[C[i]], size[C[i]] (40 B); per arc col, C[j] and the weight
-      add_lmk(A.cnt, KT_WARP, (int64_t)sacc[0], (int64_t)sacc[1], 40 * (int64_t)sacc[0] + (8 + (int64_t)sizeof(W)) * (int64_t)sacc[1]);
-    }
+    if (KIND == KIND_MOVE && kt >= 0)
+      add_lmk(A.cnt, kt, (int64_t)sacc[0], (int64_t)sacc[1], 40 * (int64_t)sacc[0] + (8 + wbytes) * (int64_t)sacc[1]);
   }
 }
 
@@ -336,7 +280,7 @@ constexpr int TINY_LANES = 8;  // lanes per vertex of degree <= BIN_TINY_MAX (on
 // Four vertices of degree <= 8 per warp, one arc per lane: lanes whose
 // neighbours share a community find each other with __match_any_sync, so
 // no table is built; each group's leader lanes hold K_{i->c} and Sigma_c.
-template <typename W, int KIND>
+template <typename W, int KIND, bool WIDE>
 __device__ __forceinline__ void tiny_step(const Args &A, int64_t item, int64_t ntiny, int lane, Tally &tl) {
   const W *w = (const W *)A.w;
   int grp = lane >> 3, sub = lane & 7, gl = lane & ~7;
@@ -378,12 +322,12 @@ __device__ __forceinline__ void tiny_step(const Args &A, int64_t item, int64_t n
       b.kd = kv;
     } else {
       b.sc = A.S[c];
-      b.v = (i128)m2 * kv - (i128)Ki * b.sc;
+      b.v = ld_gain<WIDE>(m2, kv, Ki, b.sc);
       b.c = c;
       b.kc = kv;
     }
   }
-  b = bestx_reduce<TINY_LANES>(b);
+  b = group_bestx(b);
   i128 g = 0;
   if (has && sub == 0) {
     // the winner's size matters only to the singleton rule (size_d == 1)
@@ -402,10 +346,26 @@ __device__ __forceinline__ void tiny_step(const Args &A, int64_t item, int64_t n
 // once per launch, not per vertex).  Every lane keeps its up to four arcs in
 // flight: their col, weight and C[j] loads are independent, and so are the
 // Sigma loads of the up to four candidates each lane reads back.
+//
+// Arcs into the vertex's own community and into one more community seen in
+// the first step (`hot`) are summed in registers: the neighbours of a vertex
+// fall mostly into a few communities, and every lane of the warp would add to
+// the same table slot, one after the other.  With the 32-bit sums and the
+// reduction by words, alone on the GPU: warp range 86 -> 72 us per launch
+// (R-MAT 20, all vertices), block bin 79 -> 58 us (30 -> 9 us on the web-like
+// graph).  Loading a segment's vertex records ahead of the rows was slower in
+// both (registers: 72 -> 75 and 58 -> 70 us).
 constexpr int WARP_UNROLL = BIN_WARP_MAX / 32;
 
-template <typename W, int KIND>
-__device__ __forceinline__ void warp_step(const Args &A, int32_t i, int lane, WarpTable &T, Tally &tl) {
+// A community other than d among the lanes' first arcs, or -1.
+__device__ __forceinline__ int32_t hot_community(bool valid, int32_t c, int32_t d) {
+  uint32_t m = __ballot_sync(LD_FULL, valid && c != d);
+  int32_t h = __shfl_sync(LD_FULL, c, m ? __ffs(m) - 1 : 0);
+  return m ? h : -1;
+}
+
+template <typename W, int KIND, bool WIDE>
+__device__ __forceinline__ void warp_step(const Args &A, int32_t i, int lane, WarpTable<WIDE> &T, Tally &tl) {
   const W *w = (const W *)A.w;
   int64_t base = A.off[i];
   int32_t dg = A.deg[i];
@@ -435,8 +395,17 @@ __device__ __forceinline__ void warp_step(const Args &A, int32_t i, int lane, Wa
     c[u] = v[u] ? A.C[j[u]] : 0;
     v[u] = v[u] && ld_ok((uint64_t)c[u] < (uint64_t)A.n, LD_CHK_COMM);
   }
+  BestX b{0, -1, 0, 0, 0, 0};
+  int32_t hot = hot_community(v[0], c[0], d);
+  int64_t sh = hot >= 0 ? A.S[hot] : 0, kh = 0;
 #pragma unroll
-  for (int u = 0; u < WARP_UNROLL; u++) wt_insert_lanes(T, v[u], c[u], wa[u]);
+  for (int u = 0; u < WARP_UNROLL; u++) {
+    if (!v[u]) continue;
+    if (c[u] == d) b.kd += wa[u];
+    else if (c[u] == hot) kh += wa[u];
+    else st_insert(T, &T.count, c[u], wa[u]);
+  }
+  __syncwarp();
   int n = T.count;
   int32_t cc[WARP_UNROLL];
   int64_t kv[WARP_UNROLL], sc[WARP_UNROLL];
@@ -445,28 +414,27 @@ __device__ __forceinline__ void warp_step(const Args &A, int32_t i, int lane, Wa
     int q = lane + 32 * u;
     cc[u] = -1;
     kv[u] = 0;
-    if (q < n) {
-      int32_t sl = T.list[q];
-      cc[u] = T.keys[sl];
-      kv[u] = T.vals[sl];
-      T.keys[sl] = LD_EMPTY_KEY;
-      T.vals[sl] = 0;
-    }
+    if (q < n) st_take(T, q, cc[u], kv[u]);
   }
   __syncwarp();
   if (lane == 0) T.count = 0;
   __syncwarp();
 #pragma unroll
-  for (int u = 0; u < WARP_UNROLL; u++) sc[u] = cc[u] >= 0 && cc[u] != d ? A.S[cc[u]] : 0;
-  BestX b{0, -1, 0, 0, 0, 0};
+  for (int u = 0; u < WARP_UNROLL; u++) sc[u] = cc[u] >= 0 ? A.S[cc[u]] : 0;
+  kh = ld_warp_weight<WIDE>(kh);
+  if (lane == 31 && hot >= 0) {  // the last lane has the fewest candidates of its own
+    b.v = ld_gain<WIDE>(m2, kh, Ki, sh);
+    b.c = hot;
+    b.kc = kh;
+    b.sc = sh;
+  }
 #pragma unroll
   for (int u = 0; u < WARP_UNROLL; u++) {
     if (cc[u] < 0) continue;
-    if (cc[u] == d) { b.kd += kv[u]; continue; }
-    i128 val = (i128)m2 * kv[u] - (i128)Ki * sc[u];
+    i128 val = ld_gain<WIDE>(m2, kv[u], Ki, sc[u]);
     if (ld_better(val, cc[u], b.v, b.c)) { b.v = val; b.c = cc[u]; b.kc = kv[u]; b.sc = sc[u]; }
   }
-  b = bestx_reduce<32>(b);
+  b = warp_bestx<WIDE>(b);
   i128 g = 0;
   if (lane == 0) {
     // the winner's size matters only to the singleton rule (size_d == 1)
@@ -476,45 +444,31 @@ __device__ __forceinline__ void warp_step(const Args &A, int32_t i, int lane, Wa
   bool mv = g > 0;
   if (KIND == KIND_MOVE && !A.async_mode) record_movers(A, mv, i, b.c, g);
   int moved = __shfl_sync(LD_FULL, mv ? 1 : 0, 0);
-  if (KIND == KIND_MOVE && moved) mark_neighbours(A, i, base, dg, lane, 32);
+  if (KIND == KIND_MOVE && moved) {
+#pragma unroll
+    for (int u = 0; u < WARP_UNROLL; u++)
+      if (j[u] != i && (!A.in_range || A.in_range[j[u]])) ld_bit_set(A.unproc, j[u]);
+  }
   if (lane == 0) { tl.visits++; tl.arcs += dg; tl.moves += mv; tl.dq += g; }
 }
 
 // Bins 3 (degree <= 8, groups of 8 lanes) and 0 (degree <= 128, a warp
 // each) in one launch: items [0, ceil(n3/4)) are groups of four tiny
 // vertices, the rest one warp-bin vertex each.
-template <typename W, int KIND>
+template <typename W, int KIND, bool WIDE>
 __global__ void __launch_bounds__(WARPS_PER_BLOCK * 32, 4) k_decide_warp(Args A) {
-  __shared__ WarpTable WT[WARPS_PER_BLOCK];
+  __shared__ WarpTable<WIDE> WT[WARPS_PER_BLOCK];
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  wt_init(WT[wid]);
   int64_t ntiny = *A.count_tiny, nwarp = *A.count;
   int64_t ngroups = (ntiny + 3) / 4, total = ngroups + nwarp;
   int64_t gw = (int64_t)blockIdx.x * WARPS_PER_BLOCK + wid, nw = (int64_t)gridDim.x * WARPS_PER_BLOCK;
+  wt_init(WT[wid]);
   Tally tl;
   for (int64_t t = gw; t < total; t += nw) {
-    if (t < ngroups) tiny_step<W, KIND>(A, t, ntiny, lane, tl);
-    else warp_step<W, KIND>(A, A.list[t - ngroups], lane, WT[wid], tl);
+    if (t < ngroups) tiny_step<W, KIND, WIDE>(A, t, ntiny, lane, tl);
+    else warp_step<W, KIND, WIDE>(A, A.list[t - ngroups], lane, WT[wid], tl);
   }
-  flush_tally<W, KIND>(A, tl);
-}
-
-// Block-wide merge of per-thread Best values (result valid in thread 0).
-__device__ __forceinline__ Best block_best(Best b) {
-  __shared__ Best sb[32];
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  b = warp_best(b);
-  if (lane == 0) sb[wid] = b;
-  __syncthreads();
-  if (wid == 0) {
-    Best x = lane < nw ? sb[lane] : Best{0, -1, 0, 0};
-    x = warp_best(x);
-    if (lane == 0) sb[0] = x;
-  }
-  __syncthreads();
-  Best r = sb[0];
-  __syncthreads();
-  return r;
+  flush_tally<KIND>(A, tl, KT_WARP, (int)sizeof(W));
 }
 
 // ---------------------------------------------------------------- bin 1: block, shared stage
@@ -532,40 +486,21 @@ __device__ __forceinline__ Best block_best(Best b) {
 // whose inserts begin after B2(k+1).  The slots read (and emptied) for
 // vertex k are all emptied before B2(k), so the inserts of vertex k+1 find
 // the stage empty.
+//
+// As in the warp bin, arcs into the vertex's own community and into one more
+// per warp are summed in registers (the second is added to the stage once).
 constexpr int BLOCK_UNROLL = 4;
-struct BlockStage {
-  int32_t keys[STAGE_SLOTS];
-  int64_t vals[STAGE_SLOTS];
-  int32_t list[STAGE_FILL];
+template <bool WIDE>
+struct BlockStage : STable<WIDE, STAGE_SLOTS, STAGE_FILL, uint16_t> {
   int32_t count[2];
 };
 
-__device__ __forceinline__ void bstage_insert(BlockStage &S, int32_t *count, bool valid, int32_t c, int64_t w) {
-  if (!valid) return;
-  uint32_t s = ld_hash32((uint32_t)c) & (uint32_t)(STAGE_SLOTS - 1);
-  for (int probe = 0; ld_ok(probe < STAGE_SLOTS, LD_CHK_PROBE); probe++) {
-    int32_t k = S.keys[s];
-    if (k == LD_EMPTY_KEY) {
-      k = atomicCAS(&S.keys[s], LD_EMPTY_KEY, c);
-      if (k == LD_EMPTY_KEY) {
-        S.list[atomicAdd(count, 1)] = (int32_t)s;
-        k = c;
-      }
-    }
-    if (k == c) {
-      atomicAdd((unsigned long long *)&S.vals[s], (unsigned long long)w);
-      return;
-    }
-    s = (s + 1) & (uint32_t)(STAGE_SLOTS - 1);
-  }
-}
-
-template <typename W, int KIND>
+template <typename W, int KIND, bool WIDE>
 __global__ void __launch_bounds__(BLOCK_THREADS) k_decide_block(Args A) {
-  __shared__ BlockStage S;
+  __shared__ BlockStage<WIDE> S;
   __shared__ BestX sb[BLOCK_THREADS / 32];
   __shared__ int moved_s;
-  for (int s = threadIdx.x; s < STAGE_SLOTS; s += BLOCK_THREADS) { S.keys[s] = LD_EMPTY_KEY; S.vals[s] = 0; }
+  st_clear(S, threadIdx.x, BLOCK_THREADS, STAGE_SLOTS);
   if (threadIdx.x < 2) S.count[threadIdx.x] = 0;
   __syncthreads();
   const W *w = (const W *)A.w;
@@ -585,6 +520,9 @@ __global__ void __launch_bounds__(BLOCK_THREADS) k_decide_block(Args A) {
     int32_t bi = KIND == KIND_REFINE ? A.CB[i] : 0;
     int64_t m2 = m2_of(A, i);
     int32_t *cnt = &S.count[par];
+    BestX b{0, -1, 0, 0, 0, 0};
+    int32_t hot = -1;
+    int64_t kh = 0;
     for (int r0 = 0; r0 < dg; r0 += BLOCK_THREADS * BLOCK_UNROLL) {
       int32_t j[BLOCK_UNROLL], c[BLOCK_UNROLL];
       int64_t wa[BLOCK_UNROLL];
@@ -606,12 +544,19 @@ __global__ void __launch_bounds__(BLOCK_THREADS) k_decide_block(Args A) {
         c[u] = v[u] ? A.C[j[u]] : 0;
         v[u] = v[u] && ld_ok((uint64_t)c[u] < (uint64_t)A.n, LD_CHK_COMM);
       }
+      if (r0 == 0) hot = hot_community(v[0], c[0], d);
 #pragma unroll
-      for (int u = 0; u < BLOCK_UNROLL; u++) bstage_insert(S, cnt, v[u], c[u], wa[u]);
+      for (int u = 0; u < BLOCK_UNROLL; u++) {
+        if (!v[u]) continue;
+        if (c[u] == d) b.kd += wa[u];
+        else if (c[u] == hot) kh += wa[u];
+        else st_insert(S, cnt, c[u], wa[u]);
+      }
     }
-    __syncthreads();  // B1: the stage holds K_{i->c} for every neighbour community c
+    kh = ld_warp_weight<WIDE>(kh);
+    if (lane == 0 && kh) st_insert(S, cnt, hot, kh);
+    __syncthreads();  // B1: the stage holds K_{i->c} for every neighbour community c but d
     int n = *cnt;
-    BestX b{0, -1, 0, 0, 0, 0};
     for (int q0 = 0; q0 < n; q0 += BLOCK_THREADS * BLOCK_UNROLL) {
       int32_t cc[BLOCK_UNROLL];
       int64_t kv[BLOCK_UNROLL], sc[BLOCK_UNROLL];
@@ -620,25 +565,18 @@ __global__ void __launch_bounds__(BLOCK_THREADS) k_decide_block(Args A) {
         int q = q0 + u * BLOCK_THREADS + tid;
         cc[u] = -1;
         kv[u] = 0;
-        if (q < n) {
-          int32_t sl = S.list[q];
-          cc[u] = S.keys[sl];
-          kv[u] = S.vals[sl];
-          S.keys[sl] = LD_EMPTY_KEY;
-          S.vals[sl] = 0;
-        }
+        if (q < n) st_take(S, q, cc[u], kv[u]);
       }
 #pragma unroll
-      for (int u = 0; u < BLOCK_UNROLL; u++) sc[u] = cc[u] >= 0 && cc[u] != d ? A.S[cc[u]] : 0;
+      for (int u = 0; u < BLOCK_UNROLL; u++) sc[u] = cc[u] >= 0 ? A.S[cc[u]] : 0;
 #pragma unroll
       for (int u = 0; u < BLOCK_UNROLL; u++) {
         if (cc[u] < 0) continue;
-        if (cc[u] == d) { b.kd += kv[u]; continue; }
-        i128 val = (i128)m2 * kv[u] - (i128)Ki * sc[u];
+        i128 val = ld_gain<WIDE>(m2, kv[u], Ki, sc[u]);
         if (ld_better(val, cc[u], b.v, b.c)) { b.v = val; b.c = cc[u]; b.kc = kv[u]; b.sc = sc[u]; }
       }
     }
-    b = bestx_reduce<32>(b);
+    b = warp_bestx<WIDE>(b);
     if (lane == 0) sb[wid] = b;
     __syncthreads();  // B2: every warp's best is posted, every read slot emptied
     if (tid == 0) S.count[par] = 0;
@@ -665,12 +603,7 @@ __global__ void __launch_bounds__(BLOCK_THREADS) k_decide_block(Args A) {
       i128 g = 0;
       if (tid == 0) {
         g = decide_x<KIND>(A, i, d, Ki, Sd, szd, m2, r);
-        if (KIND == KIND_MOVE && g > 0) {
-          int32_t slot = atomicAdd(&A.cnt->movers, 1);
-          A.movers[slot] = i;
-          A.mtarget[slot] = r.c;
-          if (A.mgain) { A.mgain[2 * slot] = (int64_t)(u128)g; A.mgain[2 * slot + 1] = (int64_t)((u128)g >> 64); }
-        }
+        if (KIND == KIND_MOVE && g > 0) record_mover(A, i, r.c, g);
         visits++; arcs += dg; moves += g > 0; dq += g;
       }
       mv = KIND == KIND_MOVE && would_move(d, Ki, Sd, szd, m2, r);
@@ -689,126 +622,48 @@ __global__ void __launch_bounds__(BLOCK_THREADS) k_decide_block(Args A) {
 constexpr int HUGE_CHUNK = TABLE_CHUNK;
 constexpr int HUGE_UNROLL = 4;
 
-// Global tables start clean (empty keys, zero values) and are cleaned again
-// by the kernel that reads them; each records the slots it fills in a list
-// (occ[k] entries at tab_off[k] in A.glist), so the decision visits only the
-// distinct communities instead of the whole table.
-__global__ void k_huge_zero_occ(const int32_t *count_p, int32_t *occ) {
-  for (int64_t k = ld_gtid(); k < *count_p; k += ld_gstride()) occ[k] = 0;
+// Global tables start clean and are cleaned again by the kernel that reads
+// them; each records the slots it fills in a list (occ[k] entries at
+// tab_off[k] in A.glist), so the decision visits only the distinct
+// communities instead of the whole table.
+__device__ __forceinline__ GTable hub_table(const Args &A, const int64_t *tab_off, int64_t k) {
+  int64_t o = tab_off[k];
+  return GTable{A.gkeys + o, A.gvals + o, A.glist + o, &A.gocc[k], (int)(tab_off[k + 1] - o - 1), false};
 }
 
-// Warp table with 32-bit sums, for 32-bit arc weights: 64-bit shared atomics
-// cost more than twice as much, and the smaller table and register footprint
-// leave room for more resident warps.  A lane whose add carries the slot past
-// 2^32 adds the carry straight into the vertex's global table, so the sums
-// stay exact for any weights (a weight below 2^31 carries at most once).
-struct WarpTable32 {
-  int32_t keys[WT_SLOTS];
-  uint32_t vals[WT_SLOTS];
-  int32_t list[WT_SLOTS / 2];
-  int32_t count;
-};
-
-__device__ __forceinline__ void wt_init(WarpTable32 &T) {
-  int lane = threadIdx.x & 31;
-  for (int s = lane; s < WT_SLOTS; s += 32) { T.keys[s] = LD_EMPTY_KEY; T.vals[s] = 0; }
-  if (lane == 0) T.count = 0;
-  __syncwarp();
-}
-
-__device__ __forceinline__ void wt_insert_lanes(WarpTable32 &T, bool valid, int32_t c, int64_t w, int32_t *gkeys,
-                                                int64_t *gvals, int32_t *glist, int32_t *gocc, int gmask) {
-  if (valid) {
-    uint32_t s = ld_hash32((uint32_t)c) & (uint32_t)(WT_SLOTS - 1);
-    for (int probe = 0; ld_ok(probe < WT_SLOTS, LD_CHK_PROBE); probe++) {
-      int32_t k = T.keys[s];
-      if (k == LD_EMPTY_KEY) {
-        k = atomicCAS(&T.keys[s], LD_EMPTY_KEY, c);
-        if (k == LD_EMPTY_KEY) {
-          T.list[atomicAdd(&T.count, 1)] = (int32_t)s;
-          k = c;
-        }
-      }
-      if (k == c) {
-        uint32_t add = (uint32_t)w;
-        uint32_t old = atomicAdd(&T.vals[s], add);
-        if (old + add < old) ld_gtable_insert(gkeys, gvals, glist, gocc, gmask, c, (int64_t)1 << 32);
-        break;
-      }
-      s = (s + 1) & (uint32_t)(WT_SLOTS - 1);
-    }
-  }
-  __syncwarp();
-}
-
-__device__ __forceinline__ void wt_flush(WarpTable32 &T, int32_t *gkeys, int64_t *gvals, int32_t *glist, int32_t *gocc,
-                                         int gmask) {
-  int lane = threadIdx.x & 31;
-  __syncwarp();
-  int n = T.count;
-  for (int q0 = 0; q0 < n; q0 += 32 * GT_KEYS) {  // warp-uniform
-    bool has[GT_KEYS];
-    int32_t sl[GT_KEYS], key[GT_KEYS];
-    int64_t v[GT_KEYS];
-#pragma unroll
-    for (int u = 0; u < GT_KEYS; u++) {
-      int q = q0 + 32 * u + lane;
-      has[u] = q < n;
-      sl[u] = has[u] ? T.list[q] : 0;
-      key[u] = has[u] ? T.keys[sl[u]] : 0;
-      v[u] = has[u] ? (int64_t)T.vals[sl[u]] : 0;
-    }
-    ld_gtable_add_warp(has, false, gkeys, gvals, glist, gocc, gmask, key, v);
-#pragma unroll
-    for (int u = 0; u < GT_KEYS; u++) {
-      if (has[u]) {
-        T.keys[sl[u]] = LD_EMPTY_KEY;
-        T.vals[sl[u]] = 0;
-      }
-    }
-  }
-  __syncwarp();
-  if (lane == 0) T.count = 0;
-  __syncwarp();
-}
-
-template <typename W, int KIND>
+template <typename W, int KIND, bool WIDE>
 __global__ void __launch_bounds__(256) k_huge_scan(Args A, const int64_t *tab_off, const int64_t *ch_off) {
   // Each warp sums its arcs per community in a private shared table first
   // (the neighbours of a hub fall into few communities), then each distinct
-  // community updates the vertex's global table once per flush.
-  using Table = typename std::conditional<sizeof(W) == 4, WarpTable32, WarpTable>::type;
-  __shared__ Table WT[8];
-  Table &T8 = WT[threadIdx.x >> 5];
+  // community updates the vertex's global table once per flush.  The hub's
+  // own community and one more are summed in registers, as in the other bins.
+  __shared__ WarpTable<WIDE> WT[8];
+  WarpTable<WIDE> &T8 = WT[threadIdx.x >> 5];
   wt_init(T8);
+  const int lane = threadIdx.x & 31;
   int64_t count = *A.count;
   int64_t nch = ch_off[count];
   for (int64_t t = blockIdx.x; t < nch; t += gridDim.x) {
-    int64_t lo = 0, hi = count - 1;  // vertex k with ch_off[k] <= t < ch_off[k+1]
-    while (lo < hi) {
-      int64_t mid = (lo + hi + 1) >> 1;
-      if (ch_off[mid] <= t) lo = mid; else hi = mid - 1;
-    }
+    int64_t lo = ld_chunk_item(ch_off, count, t);
     int64_t i = A.list[lo];
     int64_t first = (t - ch_off[lo]) * HUGE_CHUNK;
     int64_t full = A.deg[i];
     int64_t last = first + HUGE_CHUNK < full ? first + HUGE_CHUNK : full;
-    int64_t T = tab_off[lo + 1] - tab_off[lo];
+    GTable G = hub_table(A, tab_off, lo);
     const W *w = (const W *)A.w;
-    int64_t base = A.off[i] + first, len = last - first;
-    int32_t bi = KIND == KIND_REFINE ? A.CB[i] : 0;
-    int32_t *keys = A.gkeys + tab_off[lo], *list = A.glist + tab_off[lo];
-    int64_t *vals = A.gvals + tab_off[lo];
-    int lane = threadIdx.x & 31;
+    int64_t base = A.off[i] + first;
+    int len = (int)(last - first);
+    int32_t bi = KIND == KIND_REFINE ? A.CB[i] : 0, d = A.C[i], hot = -1;
+    int64_t kd = 0, kh = 0;
     // HUGE_UNROLL arcs per lane in flight: their col, weight and C[j] loads
     // are independent; the inserts follow one by one
-    for (int64_t a0 = threadIdx.x & ~31; a0 < len; a0 += (int64_t)blockDim.x * HUGE_UNROLL) {  // warp-uniform
+    for (int a0 = threadIdx.x & ~31; a0 < len; a0 += (int)blockDim.x * HUGE_UNROLL) {  // warp-uniform
       int32_t j[HUGE_UNROLL], c[HUGE_UNROLL];
       int64_t wa[HUGE_UNROLL];
       bool valid[HUGE_UNROLL];
 #pragma unroll
       for (int u = 0; u < HUGE_UNROLL; u++) {
-        int64_t a = a0 + (int64_t)u * blockDim.x + lane;
+        int a = a0 + u * (int)blockDim.x + lane;
         valid[u] = a < len;
         j[u] = valid[u] ? A.col[base + a] : (int32_t)i;
         wa[u] = valid[u] ? (int64_t)w[base + a] : 0;
@@ -823,59 +678,179 @@ __global__ void __launch_bounds__(256) k_huge_scan(Args A, const int64_t *tab_of
         c[u] = valid[u] ? A.C[j[u]] : 0;
         valid[u] = valid[u] && ld_ok((uint64_t)c[u] < (uint64_t)A.n, LD_CHK_COMM);
       }
+      if (hot < 0) hot = hot_community(valid[0], c[0], d);
 #pragma unroll
       for (int u = 0; u < HUGE_UNROLL; u++) {
-        if (T8.count > WT_LIMIT) wt_flush(T8, keys, vals, list, &A.gocc[lo], (int)(T - 1));
-        if constexpr (sizeof(W) == 4)
-          wt_insert_lanes(T8, valid[u], c[u], wa[u], keys, vals, list, &A.gocc[lo], (int)(T - 1));
-        else wt_insert_lanes(T8, valid[u], c[u], wa[u]);
+        if (T8.count > WT_LIMIT) wt_flush(T8, G);
+        if (valid[u]) {
+          if (c[u] == d) kd += wa[u];
+          else if (c[u] == hot) kh += wa[u];
+          else st_insert(T8, &T8.count, c[u], wa[u]);
+        }
+        __syncwarp();
       }
     }
-    wt_flush(T8, keys, vals, list, &A.gocc[lo], (int)(T - 1));
+    wt_flush(T8, G);
+    kd = ld_warp_weight<WIDE>(kd);
+    kh = ld_warp_weight<WIDE>(kh);
+    gt_insert_warp<WIDE>(G, lane == 0 ? kd != 0 : lane == 1 && kh != 0, lane == 0 ? d : hot, lane == 0 ? kd : kh);
     if (KIND == KIND_MOVE && threadIdx.x == 0)
       add_lmk(A.cnt, KT_HUGE_SCAN, first == 0 ? 1 : 0, len, (8 + (int64_t)sizeof(W)) * len);
   }
 }
 
+// Decisions of the hubs, from their tables: a warp per hub of at most BIG_KEYS
+// slots (a hub's decision is a chain of dependent loads; a block per hub has
+// an eighth as many of them in flight and waits at its barriers), a block per
+// piece of BIG_PIECE slots of the others, because at the first aggregated
+// level a hub has a slot per neighbour.  Each piece of several leaves its best
+// candidate behind the hub's slot list (which has at least twice as many
+// words as slots), and the block that finishes a hub's last piece decides.
+// R-MAT 21, static: 120 -> 89 us per launch (a block per hub, the moved hubs'
+// neighbours marked by their block).
+constexpr int PIECE_WORDS = 12;  // a BestX without szc, padded
+
+__device__ __forceinline__ void piece_put(volatile int32_t *p, const BestX &b) {
+  int32_t x[11] = {(int32_t)(uint32_t)(u128)b.v,
+                   (int32_t)(uint32_t)((u128)b.v >> 32),
+                   (int32_t)(uint32_t)((u128)b.v >> 64),
+                   (int32_t)(uint32_t)((u128)b.v >> 96),
+                   b.c,
+                   (int32_t)b.kc, (int32_t)(b.kc >> 32), (int32_t)b.kd, (int32_t)(b.kd >> 32),
+                   (int32_t)b.sc, (int32_t)(b.sc >> 32)};
+#pragma unroll
+  for (int q = 0; q < 11; q++) p[q] = x[q];
+}
+__device__ __forceinline__ int64_t join64(int32_t lo, int32_t hi) {
+  return (int64_t)(((uint64_t)(uint32_t)hi << 32) | (uint32_t)lo);
+}
+__device__ __forceinline__ BestX piece_get(const int32_t *p) {
+  int32_t x[11];
+#pragma unroll
+  for (int q = 0; q < 11; q++) x[q] = __ldcg(p + q);
+  BestX b{0, x[4], 0, join64(x[5], x[6]), join64(x[7], x[8]), join64(x[9], x[10])};
+  b.v = (i128)(((u128)(uint64_t)join64(x[2], x[3]) << 64) | (uint64_t)join64(x[0], x[1]));
+  return b;
+}
+
+// One thread's best of the listed slots q0, q0 + step, ... below q1 of a hub's
+// table, emptied as they are read.
+template <bool WIDE>
+__device__ __forceinline__ BestX hub_best(const Args &A, const GTable &G, int q0, int step, int q1, int32_t d,
+                                          int64_t m2, int64_t Ki) {
+  BestX b{0, -1, 0, 0, 0, 0};
+  for (; q0 < q1; q0 += step * HUGE_UNROLL) {
+    int32_t sl[HUGE_UNROLL], cc[HUGE_UNROLL];  // (loads before the stores that empty the slots)
+    int64_t kv[HUGE_UNROLL], sc[HUGE_UNROLL];
+#pragma unroll
+    for (int u = 0; u < HUGE_UNROLL; u++) {
+      int q = q0 + u * step;
+      sl[u] = q < q1 ? G.list[q] : -1;
+    }
+#pragma unroll
+    for (int u = 0; u < HUGE_UNROLL; u++) {
+      cc[u] = -1;
+      kv[u] = 0;
+      if (sl[u] >= 0) gt_read<WIDE>(G, sl[u], cc[u], kv[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < HUGE_UNROLL; u++)
+      if (sl[u] >= 0) gt_empty<WIDE>(G, sl[u]);
+#pragma unroll
+    for (int u = 0; u < HUGE_UNROLL; u++) sc[u] = cc[u] >= 0 && cc[u] != d ? A.S[cc[u]] : 0;
+#pragma unroll
+    for (int u = 0; u < HUGE_UNROLL; u++) {
+      if (cc[u] < 0) continue;
+      if (cc[u] == d) { b.kd += kv[u]; continue; }
+      i128 v = ld_gain<WIDE>(m2, kv[u], Ki, sc[u]);
+      if (ld_better(v, cc[u], b.v, b.c)) { b.v = v; b.c = cc[u]; b.kc = kv[u]; b.sc = sc[u]; }
+    }
+  }
+  return b;
+}
+
+struct Hub {
+  int32_t i, occ, d, dg, szd;
+  int64_t m2, Ki, Sd, base;
+  GTable G;
+};
 template <int KIND>
-__global__ void __launch_bounds__(HUGE_THREADS) k_huge_decide(Args A, const int64_t *tab_off) {
-  __shared__ int moved_s;
-  int64_t count = *A.count;
-  int64_t visits = 0, arcs = 0, moves = 0;
-  i128 dq = 0;
-  for (int64_t k = blockIdx.x; k < count; k += gridDim.x) {
-    int64_t i = A.list[k];
-    int64_t base = A.off[i], dg = A.deg[i];
-    int32_t *keys = A.gkeys + tab_off[k], *list = A.glist + tab_off[k];
-    int64_t *vals = A.gvals + tab_off[k];
-    int32_t occ = A.gocc[k];
-    int32_t d = A.C[i];
-    int64_t m2 = m2_of(A, i), Ki = A.K[i];
-    Best b{0, -1, 0, 0};
-    for (int32_t t = threadIdx.x; t < occ; t += blockDim.x) {
-      int32_t s = list[t];
-      int32_t c = keys[s];
-      int64_t kv = vals[s];
-      if (c == d) { b.kd += kv; continue; }
-      i128 v = (i128)m2 * kv - (i128)Ki * A.S[c];
-      if (ld_better(v, c, b.v, b.c)) { b.v = v; b.c = c; b.kc = kv; }
+__device__ __forceinline__ Hub hub_load(const Args &A, const int64_t *tab_off, int64_t k) {
+  Hub H;
+  H.i = A.list[k];
+  H.G = hub_table(A, tab_off, k);
+  H.occ = *H.G.occ;
+  H.d = A.C[H.i];
+  H.Ki = A.K[H.i];
+  H.m2 = m2_of(A, H.i);
+  H.dg = A.deg[H.i];
+  H.base = A.off[H.i];
+  H.Sd = A.S[H.d];
+  H.szd = KIND == KIND_MOVE ? A.size[H.d] : 0;
+  return H;
+}
+
+// The decision of hub H, by one thread: whether it moved.  The neighbours of a
+// moved hub are marked by its caller, or, above MARK_INLINE arcs in the
+// snapshot schedule, by the kernel that applies the moves.
+constexpr int MARK_INLINE = 2048;
+template <int KIND>
+__device__ __forceinline__ bool hub_decide(const Args &A, const Hub &H, BestX b, Tally &tl) {
+  // the winner's size matters only to the singleton rule (size_d == 1)
+  if (KIND == KIND_MOVE && !A.async_mode && b.c > H.d && H.szd == 1) b.szc = A.size[b.c];
+  i128 g = decide_x<KIND>(A, H.i, H.d, H.Ki, H.Sd, H.szd, H.m2, b);
+  bool mv = g > 0;
+  if (KIND == KIND_MOVE && !A.async_mode && mv) {
+    record_mover(A, H.i, b.c, g);
+    if (H.dg > MARK_INLINE) A.big_movers[atomicAdd(&A.cnt->big_movers, 1)] = H.i;
+  }
+  tl.visits++; tl.arcs += H.dg; tl.moves += mv; tl.dq += g;
+  return mv && (A.async_mode || H.dg <= MARK_INLINE);
+}
+
+template <int KIND, bool WIDE>
+__global__ void __launch_bounds__(HUGE_THREADS, 4) k_huge_decide(Args A, const int64_t *tab_off, BigTables big) {
+  __shared__ BestX sb[HUGE_THREADS / 32];
+  __shared__ int flag_s;
+  const int lane = threadIdx.x & 31;
+  const int64_t count = *A.count, nbig = *big.count, npc = nbig ? big.pieces[nbig] : 0;
+  Tally tl;
+  for (int64_t t = blockIdx.x; t < npc; t += gridDim.x) {  // block-uniform
+    int64_t at = ld_chunk_item(big.pieces, nbig, t), k = big.items[at], p = t - big.pieces[at];
+    Hub H = hub_load<KIND>(A, tab_off, k);
+    const int pieces = (H.occ + BIG_PIECE - 1) / BIG_PIECE;
+    int q0 = (int)p * BIG_PIECE, q1 = q0 + BIG_PIECE < H.occ ? q0 + BIG_PIECE : H.occ;
+    BestX b = block_bestx<WIDE>(
+        hub_best<WIDE>(A, H.G, q0 + (int)threadIdx.x, HUGE_THREADS, q1, H.d, H.m2, H.Ki), sb);
+    if (pieces > 1) {  // block-uniform
+      int32_t *part = H.G.list + H.occ;
+      if (threadIdx.x == 0) {
+        piece_put(part + p * PIECE_WORDS, b);
+        __threadfence();
+        flag_s = atomicAdd(&big.ticket[k], 1) == pieces - 1;
+        __threadfence();
+      }
+      __syncthreads();
+      if (!flag_s) continue;
+      b = BestX{0, -1, 0, 0, 0, 0};
+      for (int q = threadIdx.x; q < pieces; q += HUGE_THREADS) bestx_merge(b, piece_get(part + q * PIECE_WORDS));
+      b = block_bestx<WIDE>(b, sb);
     }
-    b = block_best(b);
-    for (int32_t t = threadIdx.x; t < occ; t += blockDim.x) {  // leave the table clean
-      int32_t s = list[t];
-      keys[s] = LD_EMPTY_KEY;
-      vals[s] = 0;
-    }
-    if (threadIdx.x == 0) {
-      i128 g = decide_leader<KIND>(A, i, b);
-      moved_s = g > 0;
-      visits++; arcs += dg; moves += g > 0; dq += g;
-    }
+    if (threadIdx.x == 0) flag_s = hub_decide<KIND>(A, H, b, tl);
     __syncthreads();
-    if (KIND == KIND_MOVE && moved_s) mark_neighbours(A, i, base, dg, threadIdx.x, blockDim.x);
+    if (KIND == KIND_MOVE && flag_s) mark_neighbours(A, H.i, H.base, H.dg, threadIdx.x, HUGE_THREADS);
     __syncthreads();
   }
-  if (threadIdx.x == 0) add_counters(A.cnt, KIND, visits, arcs, moves, dq);
+  for (int64_t k = ld_gtid() >> 5; k < count; k += ld_gstride() >> 5) {  // warp-uniform
+    if (A.gocc[k] > BIG_KEYS) continue;  // read in pieces
+    Hub H = hub_load<KIND>(A, tab_off, k);
+    BestX b = warp_bestx<WIDE>(hub_best<WIDE>(A, H.G, lane, 32, H.occ, H.d, H.m2, H.Ki));
+    int mark = 0;
+    if (lane == 0) mark = hub_decide<KIND>(A, H, b, tl);
+    mark = __shfl_sync(LD_FULL, mark, 0);
+    if (KIND == KIND_MOVE && mark) mark_neighbours(A, H.i, H.base, H.dg, lane, 32);
+  }
+  flush_tally<KIND>(A, tl);
 }
 
 // ---------------------------------------------------------------- collection
@@ -937,35 +912,44 @@ __global__ void k_collect(int64_t n, uint32_t *unproc, int cls, int classes_mask
   }
 }
 
-// Deferred moves of a sub-sweep (deterministic mode).
-// Batched handles also sum the gains and moves per graph (gid non-null).
-__global__ void k_apply_moves(const int32_t *movers, const int32_t *target, const DevCounters *cnt_c, int32_t *C,
-                              int64_t *S, const int64_t *K, int32_t *size, const int32_t *gid, const int64_t *mgain,
-                              unsigned long long *dqg, int64_t *movesg) {
-  int64_t m = cnt_c->movers;
+// Deferred moves of a sub-sweep (deterministic mode), and the neighbours of
+// the moved hubs above MARK_INLINE arcs, each hub cut into MARK_PARTS for as
+// many warps.  Batched handles also sum the gains and moves per graph (gid
+// non-null).
+constexpr int MARK_PARTS = 32;
+__global__ void k_apply_moves(Args A, unsigned long long *dqg, int64_t *movesg) {
+  const int32_t *gid = A.gid;
+  int64_t m = A.cnt->movers;
   for (int64_t t0 = (ld_gtid() & ~31ll); t0 < m; t0 += ld_gstride()) {  // warp-uniform trip count
     int64_t t = t0 + (threadIdx.x & 31);
     bool has = t < m;
     int32_t i = 0, gi = 0;
     i128 gain = 0;
     if (has) {
-      i = movers[t];
-      int32_t c = target[t];
-      int32_t d = C[i];
-      C[i] = c;
-      atomicAdd((unsigned long long *)&S[d], (unsigned long long)(-K[i]));
-      atomicAdd((unsigned long long *)&S[c], (unsigned long long)K[i]);
-      atomicSub(&size[d], 1);
-      atomicAdd(&size[c], 1);
+      i = A.movers[t];
+      int32_t c = A.mtarget[t];
+      int32_t d = A.C[i];
+      int64_t k = A.K[i];
+      A.C[i] = c;
+      atomicAdd((unsigned long long *)&A.S[d], (unsigned long long)(-k));
+      atomicAdd((unsigned long long *)&A.S[c], (unsigned long long)k);
+      atomicSub(&A.size[d], 1);
+      atomicAdd(&A.size[c], 1);
       if (gid) {
         gi = gid[i];
-        gain = (i128)(((u128)(uint64_t)mgain[2 * t + 1] << 64) | (u128)(uint64_t)mgain[2 * t]);
+        gain = (i128)(((u128)(uint64_t)A.mgain[2 * t + 1] << 64) | (u128)(uint64_t)A.mgain[2 * t]);
       }
     }
     if (gid) {
       ld_graph_add_i128(dqg, has, gi, gain);
       ld_graph_add_i64(movesg, has, gi, 1);
     }
+  }
+  int64_t parts = (int64_t)A.cnt->big_movers * MARK_PARTS;
+  for (int64_t t = ld_gtid() >> 5; t < parts; t += ld_gstride() >> 5) {  // warp-uniform
+    int32_t i = A.big_movers[t / MARK_PARTS];
+    int64_t dg = A.deg[i], len = (dg + MARK_PARTS - 1) / MARK_PARTS, a = (t % MARK_PARTS) * len;
+    if (a < dg) mark_neighbours(A, i, A.off[i] + a, dg - a < len ? dg - a : len, threadIdx.x & 31, 32);
   }
 }
 
@@ -1094,6 +1078,7 @@ Args make_args(leiden_handle *h, const LevelGraph &g) {
   A.unproc = h->unproc;
   A.movers = h->movers;
   A.mtarget = h->mtarget;
+  A.big_movers = h->ibuf2;
   A.cnt = h->dcnt;
   A.m2 = h->m2;
   if (g.gid) {
@@ -1109,17 +1094,22 @@ Args make_args(leiden_handle *h, const LevelGraph &g) {
 }
 
 // The block-bin kernels ask for the largest shared-memory carveout, so that
-// seven 29 KB stages fit on an SM (set once per device of the process).
+// seven stages fit on an SM (set once per device of the process).
+template <typename W, int KIND>
+void block_carveout_of() {
+  int co = cudaSharedmemCarveoutMaxShared;
+  cudaFuncSetAttribute(k_decide_block<W, KIND, false>, cudaFuncAttributePreferredSharedMemoryCarveout, co);
+  cudaFuncSetAttribute(k_decide_block<W, KIND, true>, cudaFuncAttributePreferredSharedMemoryCarveout, co);
+}
 void block_kernel_carveout() {
   static std::atomic<uint64_t> done{0};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) { cudaGetLastError(); return; }
   if (done.load(std::memory_order_relaxed) & (1ull << dev)) return;
-  int co = cudaSharedmemCarveoutMaxShared;
-  cudaFuncSetAttribute(k_decide_block<int32_t, KIND_MOVE>, cudaFuncAttributePreferredSharedMemoryCarveout, co);
-  cudaFuncSetAttribute(k_decide_block<int64_t, KIND_MOVE>, cudaFuncAttributePreferredSharedMemoryCarveout, co);
-  cudaFuncSetAttribute(k_decide_block<int32_t, KIND_REFINE>, cudaFuncAttributePreferredSharedMemoryCarveout, co);
-  cudaFuncSetAttribute(k_decide_block<int64_t, KIND_REFINE>, cudaFuncAttributePreferredSharedMemoryCarveout, co);
+  block_carveout_of<int32_t, KIND_MOVE>();
+  block_carveout_of<int64_t, KIND_MOVE>();
+  block_carveout_of<int32_t, KIND_REFINE>();
+  block_carveout_of<int64_t, KIND_REFINE>();
   cudaGetLastError();
   done.fetch_or(1ull << dev, std::memory_order_relaxed);
 }
@@ -1130,8 +1120,8 @@ void block_kernel_carveout() {
 // the handle's side streams beside the warp bin, joined before the caller
 // launches anything else: each of these kernels is bound by the latency of
 // its gathers and leaves most of the GPU idle in its tail.
-template <int KIND>
-void launch_bins(leiden_handle *h, const LevelGraph &g, Args A) {
+template <typename W, int KIND, bool WIDE>
+void launch_bins_of(leiden_handle *h, const LevelGraph &g, Args A) {
   cudaStream_t s = h->stream;
   int sms = h->sm_count;
   bool need_block = g.maxdeg > h->tune.warp_max, need_hub = g.maxdeg > h->tune.block_max;
@@ -1151,44 +1141,44 @@ void launch_bins(leiden_handle *h, const LevelGraph &g, Args A) {
     if (need_block) { sblock = h->side[0]; cudaStreamWaitEvent(sblock, h->fork_ev, 0); }
     if (need_hub) { shub = h->side[1]; cudaStreamWaitEvent(shub, h->fork_ev, 0); }
   }
-  A.list_tiny = h->bins + (int64_t)BIN_TINY * g.n;
-  A.count_tiny = &h->dcnt->bin_count[BIN_TINY];
-  for (int b = 0; b < NBINS; b++) {
+  auto bin = [&](int b) {
     A.list = h->bins + (int64_t)b * g.n;
     A.count = &h->dcnt->bin_count[b];
-    if (b == BIN_TINY) continue;  // with the warp bin
-    if (b == BIN_HUGE && g.maxdeg <= h->tune.block_max) continue;
-    if (b == BIN_BLOCK && g.maxdeg <= h->tune.warp_max) continue;
-    if (b == BIN_WARP) {
-      int grid = sms * h->tune.warp_blocks_per_sm;  // default 4: one wave at four resident blocks per SM
-      if (KIND == KIND_MOVE) kt_begin(h, KT_WARP);
-      if (g.w64) ld_note_launch(), k_decide_warp<int64_t, KIND><<<grid, WARPS_PER_BLOCK * 32, 0, s>>>(A);
-      else ld_note_launch(), k_decide_warp<int32_t, KIND><<<grid, WARPS_PER_BLOCK * 32, 0, s>>>(A);
-      if (KIND == KIND_MOVE) kt_end(h);
-    } else if (b == BIN_BLOCK) {
-      // default 7 blocks per SM: the shared stage (29 KB) and 71 registers
-      // for 128 threads admit 7, with the carveout set to favour shared memory
-      block_kernel_carveout();
-      int grid = sms * h->tune.block_blocks_per_sm;
-      if (KIND == KIND_MOVE) kt_begin(h, KT_BLOCK, sblock);
-      if (g.w64) ld_note_launch(), k_decide_block<int64_t, KIND><<<grid, BLOCK_THREADS, 0, sblock>>>(A);
-      else ld_note_launch(), k_decide_block<int32_t, KIND><<<grid, BLOCK_THREADS, 0, sblock>>>(A);
-      if (KIND == KIND_MOVE) kt_end(h, sblock);
-    } else {
-      A.gkeys = hs_keys(h);
-      A.gvals = hs_vals(h);
-      A.glist = hs_list(h);
-      A.gocc = h->hocc;
-      int64_t *tab_off = h->lbuf2, *ch_off = h->lbuf3;
-      launch_table_plan(A.list, A.count, g.deg, nullptr, g.n, tab_off, ch_off, shub);  // keys: communities of the level
-      ld_note_launch(), k_huge_zero_occ<<<sms, 256, 0, shub>>>(A.count, A.gocc);
-      if (KIND == KIND_MOVE) kt_begin(h, KT_HUGE_SCAN, shub);
-      int hg = sms * h->tune.hub_blocks_per_sm;
-      if (g.w64) ld_note_launch(), k_huge_scan<int64_t, KIND><<<hg, 256, 0, shub>>>(A, tab_off, ch_off);
-      else ld_note_launch(), k_huge_scan<int32_t, KIND><<<hg, 256, 0, shub>>>(A, tab_off, ch_off);
-      if (KIND == KIND_MOVE) kt_end(h, shub);
-      ld_note_launch(), k_huge_decide<KIND><<<sms * 8, HUGE_THREADS, 0, shub>>>(A, tab_off);
-    }
+  };
+  {
+    A.list_tiny = h->bins + (int64_t)BIN_TINY * g.n;
+    A.count_tiny = &h->dcnt->bin_count[BIN_TINY];
+    bin(BIN_WARP);
+    int grid = sms * h->tune.warp_blocks_per_sm;  // default 4: one wave at four resident blocks per SM
+    if (KIND == KIND_MOVE) kt_begin(h, KT_WARP);
+    ld_note_launch(), k_decide_warp<W, KIND, WIDE><<<grid, WARPS_PER_BLOCK * 32, 0, s>>>(A);
+    if (KIND == KIND_MOVE) kt_end(h);
+  }
+  if (need_block) {
+    // default 7 blocks per SM, with the carveout set to favour shared memory
+    block_kernel_carveout();
+    bin(BIN_BLOCK);
+    int grid = sms * h->tune.block_blocks_per_sm;
+    if (KIND == KIND_MOVE) kt_begin(h, KT_BLOCK, sblock);
+    ld_note_launch(), k_decide_block<W, KIND, WIDE><<<grid, BLOCK_THREADS, 0, sblock>>>(A);
+    if (KIND == KIND_MOVE) kt_end(h, sblock);
+  }
+  if (need_hub) {
+    bin(BIN_HUGE);
+    A.gkeys = hs_keys(h);
+    A.gvals = hs_vals(h);
+    A.glist = hs_list(h);
+    A.gocc = h->hocc;
+    int64_t *tab_off = h->lbuf2, *ch_off = h->lbuf3;
+    // keys: communities of the level
+    launch_table_plan(A.list, A.count, g.deg, nullptr, g.n, tab_off, ch_off, shub, A.gocc);
+    if (KIND == KIND_MOVE) kt_begin(h, KT_HUGE_SCAN, shub);
+    int hg = sms * h->tune.hub_blocks_per_sm;
+    ld_note_launch(), k_huge_scan<W, KIND, WIDE><<<hg, 256, 0, shub>>>(A, tab_off, ch_off);
+    if (KIND == KIND_MOVE) kt_end(h, shub);
+    BigTables big{h->ibuf1, &h->dcnt->hub_big, h->lbuf1, h->ibuf0};
+    launch_piece_plan(A.count, A.gocc, big, shub);
+    ld_note_launch(), k_huge_decide<KIND, WIDE><<<sms * 8, HUGE_THREADS, 0, shub>>>(A, tab_off, big);
   }
   if (fork) {
     for (int k = 0; k < 2; k++) {
@@ -1197,6 +1187,13 @@ void launch_bins(leiden_handle *h, const LevelGraph &g, Args A) {
       cudaStreamWaitEvent(s, h->join_ev[k], 0);
     }
   }
+}
+
+template <int KIND>
+void launch_bins(leiden_handle *h, const LevelGraph &g, const Args &A) {
+  bool wide = wide_sums(h);
+  if (g.w64) wide ? launch_bins_of<int64_t, KIND, true>(h, g, A) : launch_bins_of<int64_t, KIND, false>(h, g, A);
+  else wide ? launch_bins_of<int32_t, KIND, true>(h, g, A) : launch_bins_of<int32_t, KIND, false>(h, g, A);
 }
 
 }  // namespace
@@ -1275,7 +1272,7 @@ void count_sizes(leiden_handle *h, const int32_t *C, int64_t n, int32_t *size) {
 
 void lm_subsweep(leiden_handle *h, const LevelGraph &g, int cls, const uint8_t *in_range, int dynamic) {
   cudaStream_t s = h->stream;
-  cudaMemsetAsync(&h->dcnt->bin_count[0], 0, sizeof(int32_t) * 4 + sizeof(int32_t), s);  // bins + movers
+  cudaMemsetAsync(&h->dcnt->bin_count[0], 0, sizeof(int32_t) * 6, s);  // bins, movers, big movers
   ld_note_launch(), k_collect<<<grid_for((g.n + 31) / 32, 256), 256, 0, s>>>(
       g.n, h->unproc, cls, lm_classes(h) - 1, in_range, g.deg, h->bins, h->dcnt, g.gid, h->gc.lm_on, h->d_loff,
       h->tune);
@@ -1284,8 +1281,7 @@ void lm_subsweep(leiden_handle *h, const LevelGraph &g, int cls, const uint8_t *
   A.dynamic = dynamic;
   launch_bins<KIND_MOVE>(h, g, A);
   if (h->p.deterministic)
-    ld_note_launch(), k_apply_moves<<<h->sm_count * 4, 256, 0, s>>>(h->movers, h->mtarget, h->dcnt, h->Cp, h->Sp, h->Kp,
-                                                                    h->csize, g.gid, h->mgain, h->gc.dq, h->gc.moves);
+    ld_note_launch(), k_apply_moves<<<h->sm_count * 4, 256, 0, s>>>(A, h->gc.dq, h->gc.moves);
 }
 
 void refine_reset(leiden_handle *h, const LevelGraph &g) {

@@ -647,12 +647,12 @@ __global__ void __launch_bounds__(256) k_agg_block(AggArgs A) {
   }
 }
 
-// A table of at least ncomm slots is indexed by the key directly (dense);
-// a smaller one is an open-addressing hash table.
-__device__ __forceinline__ void agg_flush(WarpTable &T8, bool dense, int32_t *keys, int64_t *vals, int32_t *list,
-                                          int32_t *occ, int tmask) {
-  if (dense) wt_flush_dense(T8, keys, vals, list, occ);
-  else wt_flush(T8, keys, vals, list, occ, tmask);
+// The global table of the k-th listed community.  A table of at least ncomm
+// slots is indexed by the key directly (dense); a smaller one is an
+// open-addressing hash table.
+__device__ __forceinline__ GTable agg_table(const AggArgs &A, const int64_t *tab_off, int64_t k) {
+  int64_t o = tab_off[k], T = tab_off[k + 1] - o;
+  return GTable{A.gkeys + o, A.gvals + o, A.glist + o, &A.gocc[k], (int)(T - 1), T >= A.ncomm};
 }
 
 // Communities above BIN_BLOCK_MAX flat arcs: each has its own global table
@@ -670,10 +670,10 @@ __device__ __forceinline__ void agg_flush(WarpTable &T8, bool dense, int32_t *ke
 constexpr int AGG_SHORT = 16;  // at most this many arcs in range: a lane walks the member's row
 constexpr int AGG_SPAN = TABLE_CHUNK / 8;  // flat arcs of one warp in a chunk
 
-template <typename W>
-__device__ __forceinline__ void agg_take(const AggArgs &A, WarpTable &T8, bool dense, int32_t *keys, int64_t *vals,
-                                         int32_t *list, int32_t *occ, int tmask, int32_t self, const bool *valid,
-                                         const int32_t *j, const int64_t *wa, int64_t &ksum, int64_t &selfw) {
+template <bool WIDE>
+__device__ __forceinline__ void agg_take(const AggArgs &A, WarpTable<WIDE> &T8, const GTable &G, int32_t self,
+                                         const bool *valid, const int32_t *j, const int64_t *wa, int64_t &ksum,
+                                         int64_t &selfw) {
   int32_t cc[AGG_UNROLL];
 #pragma unroll
   for (int u = 0; u < AGG_UNROLL; u++) cc[u] = valid[u] ? A.C[j[u]] : 0;
@@ -682,26 +682,23 @@ __device__ __forceinline__ void agg_take(const AggArgs &A, WarpTable &T8, bool d
     bool own = valid[u] && cc[u] == self;
     ksum += wa[u];
     selfw += own ? wa[u] : 0;
-    if (T8.count > WT_LIMIT) agg_flush(T8, dense, keys, vals, list, occ, tmask);
-    wt_insert_lanes(T8, valid[u] && !own, cc[u], wa[u]);
+    if (T8.count > WT_LIMIT) wt_flush(T8, G);
+    if (valid[u] && !own) st_insert(T8, &T8.count, cc[u], wa[u]);
+    __syncwarp();
   }
 }
 
-template <typename W>
+template <typename W, bool WIDE>
 __global__ void __launch_bounds__(256, 4) k_agg_chunk_scan(AggArgs A, const int64_t *tab_off, const int64_t *ch_off) {
-  __shared__ WarpTable WT[8];  // per-warp sums by community
-  WarpTable &T8 = WT[threadIdx.x >> 5];
+  __shared__ WarpTable<WIDE> WT[8];  // per-warp sums by community
+  WarpTable<WIDE> &T8 = WT[threadIdx.x >> 5];
   wt_init(T8);
   int64_t count = *A.count;
   int64_t nch = ch_off[count];
   const W *w = (const W *)A.w;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (int64_t t = blockIdx.x; t < nch; t += gridDim.x) {
-    int64_t lo = 0, hi = count - 1;  // community k with ch_off[k] <= t < ch_off[k+1]
-    while (lo < hi) {
-      int64_t mid = (lo + hi + 1) >> 1;
-      if (ch_off[mid] <= t) lo = mid; else hi = mid - 1;
-    }
+    int64_t lo = ld_chunk_item(ch_off, count, t);
     int64_t c = A.list[lo];
     int64_t m0 = A.coff[c], m1 = A.coff[c + 1];
     int64_t fc = A.cflat[m0] + (t - ch_off[lo]) * TABLE_CHUNK, fe = A.cflat[m1];
@@ -709,12 +706,7 @@ __global__ void __launch_bounds__(256, 4) k_agg_chunk_scan(AggArgs A, const int6
     if (f1 > fc + TABLE_CHUNK) f1 = fc + TABLE_CHUNK;
     if (f1 > fe) f1 = fe;
     if (f0 >= f1) continue;  // warp-uniform: the chunk is short
-    int64_t T = tab_off[lo + 1] - tab_off[lo];
-    bool dense = T >= A.ncomm;  // every key (a community id) has its own slot
-    int tmask = (int)(T - 1);
-    int32_t *keys = A.gkeys + tab_off[lo], *list = A.glist + tab_off[lo];
-    int64_t *vals = A.gvals + tab_off[lo];
-    int32_t *occ = &A.gocc[lo];
+    GTable G = agg_table(A, tab_off, lo);
     // the member holding f0: the last a in [m0, m1) with cflat[a] <= f0,
     // narrowed 32-fold per step (cflat[a0] <= f0 holds throughout)
     int64_t a0 = m0, span = m1 - m0;
@@ -753,7 +745,7 @@ __global__ void __launch_bounds__(256, 4) k_agg_chunk_scan(AggArgs A, const int6
           j[u] = valid[u] ? mcol[jj + u] : 0;
           wa[u] = valid[u] ? (int64_t)mw[jj + u] : 0;
         }
-        agg_take<W>(A, T8, dense, keys, vals, list, occ, tmask, (int32_t)c, valid, j, wa, ksum, selfw);
+        agg_take<WIDE>(A, T8, G, (int32_t)c, valid, j, wa, ksum, selfw);
       }
       for (uint32_t med = __ballot_sync(LD_FULL, !shrt); med; med &= med - 1u) {  // warp-uniform
         int src = __ffs(med) - 1;
@@ -771,11 +763,11 @@ __global__ void __launch_bounds__(256, 4) k_agg_chunk_scan(AggArgs A, const int6
             j[u] = valid[u] ? pc[x] : 0;
             wa[u] = valid[u] ? (int64_t)pw[x] : 0;
           }
-          agg_take<W>(A, T8, dense, keys, vals, list, occ, tmask, (int32_t)c, valid, j, wa, ksum, selfw);
+          agg_take<WIDE>(A, T8, G, (int32_t)c, valid, j, wa, ksum, selfw);
         }
       }
     }
-    agg_flush(T8, dense, keys, vals, list, occ, tmask);
+    wt_flush(T8, G);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       ksum += __shfl_xor_sync(LD_FULL, ksum, o);
@@ -783,10 +775,7 @@ __global__ void __launch_bounds__(256, 4) k_agg_chunk_scan(AggArgs A, const int6
     }
     if (lane == 0) {
       if (ksum != 0) atomicAdd((unsigned long long *)&A.Kout[c], (unsigned long long)ksum);
-      if (selfw != 0) {
-        if (dense) ld_gtable_add_direct(keys, vals, list, occ, (int32_t)c, selfw);
-        else ld_gtable_insert(keys, vals, list, occ, tmask, (int32_t)c, selfw);
-      }
+      if (selfw != 0) gt_insert<WIDE>(G, (int32_t)c, selfw);
       // per flat arc: col, C of the neighbour and the weight
       atomicAdd((unsigned long long *)A.xk_bytes, (unsigned long long)((8 + sizeof(W)) * (f1 - f0)));
     }
@@ -798,6 +787,7 @@ __global__ void __launch_bounds__(256, 4) k_agg_chunk_scan(AggArgs A, const int6
 // k-th listed community (every community has at least one, which also
 // writes its degree).
 constexpr int EMIT_CHUNK = 2048;
+constexpr int EMIT_UNROLL = 4;
 
 __global__ void __launch_bounds__(1024) k_emit_plan(const int32_t *count_p, const int32_t *occ, int64_t *em_off) {
   __shared__ int64_t ws[32];
@@ -827,33 +817,36 @@ __global__ void __launch_bounds__(1024) k_emit_plan(const int32_t *count_p, cons
   if (threadIdx.x == 0) em_off[count] = carry;
 }
 
+template <bool WIDE>
 __global__ void __launch_bounds__(256) k_agg_list_emit(AggArgs A, const int64_t *tab_off, const int64_t *em_off) {
   int64_t count = *A.count;
   int64_t npc = em_off[count];
   for (int64_t t = blockIdx.x; t < npc; t += gridDim.x) {
-    int64_t k = 0, hi = count - 1;  // community k with em_off[k] <= t < em_off[k+1]
-    while (k < hi) {
-      int64_t mid = (k + hi + 1) >> 1;
-      if (em_off[mid] <= t) k = mid; else hi = mid - 1;
-    }
+    int64_t k = ld_chunk_item(em_off, count, t);
     int64_t c = A.list[k];
-    int32_t *keys = A.gkeys + tab_off[k], *list = A.glist + tab_off[k];
-    int64_t *vals = A.gvals + tab_off[k];
-    int64_t occ = A.gocc[k];
-    bool dense = tab_off[k + 1] - tab_off[k] >= A.ncomm;  // the list holds the keys themselves
-    int64_t q0 = (t - em_off[k]) * EMIT_CHUNK, q1 = q0 + EMIT_CHUNK < occ ? q0 + EMIT_CHUNK : occ;
+    GTable G = agg_table(A, tab_off, k);
+    int occ = *G.occ;
+    int q0 = (int)(t - em_off[k]) * EMIT_CHUNK, q1 = q0 + EMIT_CHUNK < occ ? q0 + EMIT_CHUNK : occ;
     int64_t base = A.yoff[c];
-    for (int64_t q = q0 + threadIdx.x; q < q1; q += blockDim.x) {
-      int32_t s = list[q];
-      int32_t key = dense ? s : keys[s];
-      keys[s] = LD_EMPTY_KEY;
-      A.ycol[base + q] = key;
-      A.yw[base + q] = vals[s];
-      vals[s] = 0;
+    for (int r = q0 + (int)threadIdx.x; r < q1; r += 256 * EMIT_UNROLL) {
+      int32_t sl[EMIT_UNROLL], key[EMIT_UNROLL];  // (loads before the stores that empty the slots)
+      int64_t w[EMIT_UNROLL];
+#pragma unroll
+      for (int u = 0; u < EMIT_UNROLL; u++) sl[u] = r + 256 * u < q1 ? G.list[r + 256 * u] : -1;
+#pragma unroll
+      for (int u = 0; u < EMIT_UNROLL; u++)
+        if (sl[u] >= 0) gt_read<WIDE>(G, sl[u], key[u], w[u]);
+#pragma unroll
+      for (int u = 0; u < EMIT_UNROLL; u++) {
+        if (sl[u] < 0) continue;
+        gt_empty<WIDE>(G, sl[u]);
+        A.ycol[base + r + 256 * u] = key[u];
+        A.yw[base + r + 256 * u] = w[u];
+      }
     }
     if (q0 == 0 && threadIdx.x == 0) {
-      A.ydeg[c] = (int32_t)occ;
-      atomicAdd((unsigned long long *)&A.tables[dense ? 1 : 0], 1ull);
+      A.ydeg[c] = occ;
+      atomicAdd((unsigned long long *)&A.tables[G.dense ? 1 : 0], 1ull);
     }
   }
 }
@@ -1113,12 +1106,14 @@ void aggregate(leiden_handle *h, const LevelGraph &g, int64_t ncomm, int out) {
     A.xk_bytes = &h->dcnt->xk_bytes[1];
     A.tables = h->dcnt->agg_tables;
     kt_begin(h, KT_AGG_CHUNK);
-    if (g.w64) ld_note_launch(), k_agg_chunk_scan<int64_t><<<sms * 16, 256, 0, s>>>(A, tab_off, ch_off);
-    else ld_note_launch(), k_agg_chunk_scan<int32_t><<<sms * 16, 256, 0, s>>>(A, tab_off, ch_off);
+    auto scan = wide_sums(h) ? (g.w64 ? k_agg_chunk_scan<int64_t, true> : k_agg_chunk_scan<int32_t, true>)
+                             : (g.w64 ? k_agg_chunk_scan<int64_t, false> : k_agg_chunk_scan<int32_t, false>);
+    ld_note_launch(), scan<<<sms * 16, 256, 0, s>>>(A, tab_off, ch_off);
     kt_end(h);
     int64_t *em_off = h->lbuf0;  // free again after the member fill
     ld_note_launch(), k_emit_plan<<<1, 1024, 0, s>>>(A.count, A.gocc, em_off);
-    ld_note_launch(), k_agg_list_emit<<<sms * 8, 256, 0, s>>>(A, tab_off, em_off);
+    auto emit = wide_sums(h) ? k_agg_list_emit<true> : k_agg_list_emit<false>;
+    ld_note_launch(), emit<<<sms * 8, 256, 0, s>>>(A, tab_off, em_off);
   }
 }
 

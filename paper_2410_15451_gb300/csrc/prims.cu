@@ -326,49 +326,91 @@ namespace {
 // sums, totals at index count).  An item's size is deg32[v] or
 // off64[v+1] - off64[v]; its table has pow2 >= 2*min(size, key_cap) slots
 // (key_cap bounds the distinct keys an item can have, e.g. the number of
-// communities) and it is cut into chunks of TABLE_CHUNK.
+// communities) and it is cut into chunks of TABLE_CHUNK.  occ (where given)
+// is zeroed for the listed items.
 __global__ void __launch_bounds__(1024) k_table_plan(const int32_t *list, const int32_t *count_p,
                                                       const int32_t *deg32, const int64_t *off64, int64_t key_cap,
-                                                      int64_t *tab_off, int64_t *ch_off) {
-  __shared__ int64_t ws[32][2];
-  __shared__ int64_t carry[2];
+                                                      int64_t *tab_off, int64_t *ch_off, int32_t *occ) {
+  __shared__ int64_t ws[2][32];
   int64_t count = *count_p;
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (threadIdx.x == 0) { carry[0] = 0; carry[1] = 0; }
-  __syncthreads();
-  for (int64_t base = 0; base < count; base += blockDim.x) {
+  int64_t carry[2] = {0, 0};
+  for (int64_t base = 0; base < count; base += blockDim.x) {  // block-uniform
     int64_t k = base + threadIdx.x;
-    int64_t t = 0, c = 0;
+    int64_t x[2] = {0, 0}, incl[2];
     if (k < count) {
       int32_t v = list[k];
       int64_t d = deg32 ? (int64_t)deg32[v] : off64[v + 1] - off64[v];
       int64_t keys = d < key_cap ? d : key_cap;
-      t = 1;
-      while (t < 2 * keys) t <<= 1;
-      c = d > 0 ? (d + TABLE_CHUNK - 1) / TABLE_CHUNK : 1;  // every item gets at least one chunk
+      x[0] = keys > 1 ? (int64_t)1 << (64 - __clzll(2 * keys - 1)) : 2 * keys + (keys < 1);
+      x[1] = d > 0 ? (d + TABLE_CHUNK - 1) / TABLE_CHUNK : 1;  // every item gets at least one chunk
+      if (occ) occ[k] = 0;
     }
-    int64_t it = t, ic = c;  // inclusive warp scans
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int64_t xt = __shfl_up_sync(LD_FULL, it, o), xc = __shfl_up_sync(LD_FULL, ic, o);
-      if (lane >= o) { it += xt; ic += xc; }
-    }
-    if (lane == 31) { ws[wid][0] = it; ws[wid][1] = ic; }
+    for (int q = 0; q < 2; q++) incl[q] = warp_incl_scan(x[q]);
+    if (lane == 31)
+#pragma unroll
+      for (int q = 0; q < 2; q++) ws[q][wid] = incl[q];
     __syncthreads();
-    if (threadIdx.x == 0) {
-      int64_t a = carry[0], b = carry[1];
-      for (int w = 0; w < (int)(blockDim.x >> 5); w++) {
-        int64_t x = ws[w][0], y = ws[w][1];
-        ws[w][0] = a; ws[w][1] = b;
-        a += x; b += y;
-      }
-      carry[0] = a; carry[1] = b;
+    int64_t before[2], total[2];
+#pragma unroll
+    for (int q = 0; q < 2; q++) {  // every warp scans the warps' sums itself
+      int64_t y = ws[q][lane], yi = warp_incl_scan(y);
+      before[q] = carry[q] + __shfl_sync(LD_FULL, yi - y, wid);
+      total[q] = __shfl_sync(LD_FULL, yi, 31);
     }
-    __syncthreads();
-    if (k < count) { tab_off[k] = ws[wid][0] + it - t; ch_off[k] = ws[wid][1] + ic - c; }
+    if (k < count) {
+      tab_off[k] = before[0] + incl[0] - x[0];
+      ch_off[k] = before[1] + incl[1] - x[1];
+    }
+#pragma unroll
+    for (int q = 0; q < 2; q++) carry[q] += total[q];
     __syncthreads();
   }
-  if (threadIdx.x == 0) { tab_off[count] = carry[0]; ch_off[count] = carry[1]; }
+  if (threadIdx.x == 0) {
+    tab_off[count] = carry[0];
+    ch_off[count] = carry[1];
+  }
+}
+
+// One block: the items whose tables hold more than BIG_KEYS keys, with the
+// offsets of their pieces of BIG_PIECE keys and their tickets zeroed.
+__global__ void __launch_bounds__(1024) k_piece_plan(const int32_t *count_p, const int32_t *occ, BigTables big) {
+  __shared__ int64_t ws[2][32];
+  int64_t count = *count_p;
+  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int64_t carry[2] = {0, 0};
+  for (int64_t base = 0; base < count; base += blockDim.x) {  // block-uniform
+    int64_t k = base + threadIdx.x;
+    int32_t o = k < count ? occ[k] : 0;
+    bool f = o > BIG_KEYS;
+    if (!__syncthreads_or(f)) continue;
+    int64_t x[2] = {f ? (o + BIG_PIECE - 1) / BIG_PIECE : 0, f ? 1 : 0}, incl[2];
+#pragma unroll
+    for (int q = 0; q < 2; q++) incl[q] = warp_incl_scan(x[q]);
+    if (lane == 31) { ws[0][wid] = incl[0]; ws[1][wid] = incl[1]; }
+    __syncthreads();
+    int64_t before[2], total[2];
+#pragma unroll
+    for (int q = 0; q < 2; q++) {
+      int64_t y = ws[q][lane], yi = warp_incl_scan(y);
+      before[q] = carry[q] + __shfl_sync(LD_FULL, yi - y, wid);
+      total[q] = __shfl_sync(LD_FULL, yi, 31);
+    }
+    if (f) {
+      int64_t at = before[1] + incl[1] - 1;
+      big.items[at] = (int32_t)k;
+      big.pieces[at] = before[0] + incl[0] - x[0];
+      big.ticket[k] = 0;
+    }
+    carry[0] += total[0];
+    carry[1] += total[1];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    big.pieces[carry[1]] = carry[0];
+    *big.count = (int32_t)carry[1];
+  }
 }
 
 __global__ void k_fill_i32(int32_t *p, int32_t v, int64_t n) {
@@ -396,8 +438,11 @@ void launch_fill_i64(int64_t *p, int64_t v, int64_t n, cudaStream_t s) {
   if (n > 0) ld_note_launch(), k_fill_i64<<<grid_for(n, 256), 256, 0, s>>>(p, v, n);
 }
 void launch_table_plan(const int32_t *list, const int32_t *count, const int32_t *deg32, const int64_t *off64,
-                       int64_t key_cap, int64_t *tab_off, int64_t *ch_off, cudaStream_t s) {
-  ld_note_launch(), k_table_plan<<<1, 1024, 0, s>>>(list, count, deg32, off64, key_cap, tab_off, ch_off);
+                       int64_t key_cap, int64_t *tab_off, int64_t *ch_off, cudaStream_t s, int32_t *occ) {
+  ld_note_launch(), k_table_plan<<<1, 1024, 0, s>>>(list, count, deg32, off64, key_cap, tab_off, ch_off, occ);
+}
+void launch_piece_plan(const int32_t *count, const int32_t *occ, const BigTables &big, cudaStream_t s) {
+  ld_note_launch(), k_piece_plan<<<1, 1024, 0, s>>>(count, occ, big);
 }
 
 void launch_iota_i32(int32_t *p, int64_t n, cudaStream_t s) {

@@ -82,3 +82,22 @@ def test_screening_expands_rows_of_every_length(name):
     assert np.array_equal(gpu.update(dels, ins, L.LEIDEN_DS), ref.update(dels, ins, oracle.DS))
     assert np.array_equal(gpu.affected(), ref.affected())
     assert np.array_equal(gpu.state()["K"], ref.state()["K"])
+
+
+HUB_SLOTS = [512, 513, 1025, 2048, 2049, 4097]  # distinct neighbour communities: warp, one piece, several pieces
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+def test_hub_tables_of_every_size(weighted):
+    """Hubs whose tables end at a warp's, a piece's and several pieces' limits,
+    with 32-bit sums (unit weights) and with 64-bit ones (2m above 2^32); hubs
+    that move mark their neighbours inline or in parts."""
+    g = stars([max(k, 1030) if k < 1030 else k for k in HUB_SLOTS] + HUB_SLOTS, weighted)
+    gpu = L.Leiden(g.n, g.off, g.col, g.w)
+    L.leiden_set_tuning(gpu.h, block_max=256)  # the hub path from 257 arcs on
+    ref = oracle.Oracle(g.n, g.off, g.col, g.w, schedule=oracle.SYNC)
+    assert np.array_equal(gpu.static(), ref.static())
+    assert gpu.trace() == ref.trace()
+    dels = [(2 + 3 * k, int(g.col[g.off[2 + 3 * k]]), 1) for k in range(len(HUB_SLOTS))]
+    assert np.array_equal(gpu.update(dels, [(0, 5, 1)], L.LEIDEN_ND), ref.update(dels, [(0, 5, 1)], oracle.ND))
+    assert gpu.trace() == ref.trace()
