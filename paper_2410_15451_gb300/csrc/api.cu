@@ -396,17 +396,11 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range)
     ph_bytes(h, LEIDEN_PHASE_SPLIT, 24 * (int64_t)h->hcnt->split_count + 8 * h->hcnt->split_arcs);
     ph_mark(h, LEIDEN_PHASE_AGGREGATE);
     ph_bytes(h, LEIDEN_PHASE_AGGREGATE, 4 * n);  // community count
-    if (B) {
+    if (B) {  // (one graph: counted by the renumbering, or by tracking in the last pass)
       CK(cudaMemsetAsync(h->gc.ncomm, 0, (size_t)G * sizeof(int32_t), s));
       count_communities(h, n, g.gid);
       sync_all(h);
       tr[2] = h->hcnt->list_count;
-    } else {
-      // only the trace needs the count: it is read with the next host sync
-      count_communities(h, n, g.gid);
-      if (lp < 10)
-        CK(cudaMemcpyAsync(&h->dcnt->pass_ncomm[lp], &h->dcnt->list_count, sizeof(int32_t),
-                           cudaMemcpyDeviceToDevice, s));
     }
     if (!B) {
       if (p.converge_any && (li <= 1 || !refined_any)) break;
@@ -436,7 +430,7 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range)
       }
       memcpy(hg.cont, cont.data(), (size_t)G);
       CK(cudaMemcpyAsync(h->gc.cont, hg.cont, (size_t)G, cudaMemcpyHostToDevice, s));
-      break_lookup(h);
+      break_lookup(h, n, g.gid, lp == 0);
       if (!any_cont) { looked_up = true; break; }
     }
     renumber_dense(h, n, g.gid);
@@ -449,6 +443,7 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range)
       if (B) CK(cudaMemcpyAsync(loff_h.data(), loff_next, (size_t)(G + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
       CK(cudaStreamSynchronize(s));
       ncomm = tot;
+      if (!B) tr[2] = ncomm;
     }
     lookup_dendrogram(h);
     // every aggregated level has at most the arcs of G^t (held since the
@@ -493,7 +488,7 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range)
   ph_bytes(h, LEIDEN_PHASE_TRACK, (B ? 0 : 12 * N) + 234 * N);  // final lookup; tracking's sweeps
   if (!B) lookup_dendrogram(h);
   else if (!looked_up) { h->err = "batched pass loop ended without a final lookup"; return LEIDEN_ERR_STATE; }
-  track_communities(h);
+  track_communities(h, h->Cp, g.n);
   ph_mark(h, PHASE_END);
   release_agg_buffers(h);
   sync_counters(h);
@@ -504,8 +499,7 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range)
     return LEIDEN_ERR_STATE;
   }
   h->trace[0] = passes;
-  if (!B)
-    for (int lp = 0; lp < passes && lp < 10; lp++) h->trace[2 + lp * 25 + 2] = h->hcnt->pass_ncomm[lp];
+  if (!B && passes <= 10) h->trace[2 + (passes - 1) * 25 + 2] = h->hcnt->list_count;
   st.passes = passes;
   st.lm_vertices = h->hcnt->processed;
   st.lm_arcs = h->hcnt->arcs;

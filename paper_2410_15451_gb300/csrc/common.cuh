@@ -44,12 +44,12 @@ struct DevCounters {
   int32_t big_count;              // splitting: long rows left to the block kernel
   int32_t large_count;            // batch apply: touched rows merged in chunks
   int32_t tr_occ;                 // tracking: filled slots of the pair table
+  int32_t tr_flagged;             // tracking: old communities without a majority candidate
   int32_t mid_count;              // batch apply: touched rows merged by one block each
   int32_t hub_big;                // local moving: listed hubs whose tables are read in pieces
   int64_t arena_used;             // next free arc slot of G^t (relocated rows go here)
   int64_t bcounts[8];             // batch apply: unique deletions, unique insertions, new arcs,
                                   //   touched rows, merge-buffer arcs
-  int32_t pass_ncomm[10];         // communities after refinement, per pass (trace)
   int64_t affected;               // |dV|: vertices flagged affected (counted into the frontier)
   int64_t split_arcs;             // splitting: arcs of the vertices listed for splitting
   int64_t deg_sum;                // degree sum of the level scanned by level_maxdeg (its arcs)

@@ -337,7 +337,9 @@ void renumber_dense(leiden_handle *h, int64_t n, const int32_t *gid);
 // Distinct ids of Cp -> dcnt->list_count (and gc.ncomm per graph when batched).
 void count_communities(leiden_handle *h, int64_t n, const int32_t *gid);
 void lookup_dendrogram(leiden_handle *h);  // batched: the continuing graphs only
-void break_lookup(leiden_handle *h);       // batched: final lookup of the stopping graphs
+// Batched: final lookup of the graphs that stop at this level (n vertices, graph
+// ids gid) and their communities' ids flagged in dE (cleared at the first level).
+void break_lookup(leiden_handle *h, int64_t n, const int32_t *gid, bool first);
 // Batched: graph ids of the next level's super-vertices and its graph ranges.
 void next_level_ids(leiden_handle *h, int64_t n, const int32_t *gid, int32_t *gid_next, int64_t *loff_next);
 void aggregate(leiden_handle *h, const LevelGraph &g, int64_t ncomm, int out_slot);
@@ -349,7 +351,7 @@ void pass_init(leiden_handle *h);
 void level_maxdeg(leiden_handle *h, const int32_t *deg, int64_t n);  // into dcnt->max_count
 
 // ------------------------------------------------------------ track.cu
-void track_communities(leiden_handle *h);  // Ctop vs C -> C, Sig, dSig
+void track_communities(leiden_handle *h, const int32_t *root, int64_t nroot);  // Ctop vs C -> C, Sig, dSig
 void modularity_terms(leiden_handle *h, const int32_t *C);  // into dcnt->sigma_intra / sq
 void recompute_weights(leiden_handle *h);  // K = row sums, m2 (device)
 void recompute_sigma(leiden_handle *h);    // Sigma from K and C

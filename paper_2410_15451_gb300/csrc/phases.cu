@@ -229,12 +229,18 @@ __global__ void k_lookup(int64_t N, const int32_t *Cp, int32_t *Ctop, const int3
 }
 // Final lookup of the graphs that stop at this pass, with the community id
 // moved from the level's range of the graph into its own vertex range (the
-// order within the graph, all that tracking uses, is kept).
+// order within the graph, all that tracking uses, is kept).  Their
+// communities are the level's roots (C'[c] == c).
 __global__ void k_break_lookup(int64_t N, const int32_t *Cp, int32_t *Ctop, const int32_t *gid0, const uint8_t *cont,
-                               const int64_t *loff, const int64_t *voff) {
+                               const int64_t *loff, const int64_t *voff, int64_t n, const int32_t *gid,
+                               uint8_t *used) {
   for (int64_t v = ld_gtid(); v < N; v += ld_gstride()) {
     int32_t g = gid0[v];
     if (loff[g + 1] > loff[g] && !cont[g]) Ctop[v] = (int32_t)(Cp[Ctop[v]] - loff[g] + voff[g]);
+    if (v < n) {
+      g = gid[v];
+      if (loff[g + 1] > loff[g] && !cont[g] && Cp[v] == (int32_t)v) used[v - loff[g] + voff[g]] = 1;
+    }
   }
 }
 // Graph of each super-vertex and the graphs' ranges at the next level.
@@ -1024,9 +1030,10 @@ void lookup_dendrogram(leiden_handle *h) {
   ld_note_launch(), k_lookup<<<grid_for(h->n, TB), TB, 0, h->stream>>>(h->n, h->Cp, h->Ctop, h->gid0, cont);
 }
 
-void break_lookup(leiden_handle *h) {
-  ld_note_launch(), k_break_lookup<<<grid_for(h->n, TB), TB, 0, h->stream>>>(h->n, h->Cp, h->Ctop, h->gid0, h->gc.cont,
-                                                                               h->d_loff, h->d_voff);
+void break_lookup(leiden_handle *h, int64_t n, const int32_t *gid, bool first) {
+  if (first) cudaMemsetAsync(h->dE, 0, (size_t)h->n, h->stream);
+  ld_note_launch(), k_break_lookup<<<grid_for(h->n, TB), TB, 0, h->stream>>>(
+      h->n, h->Cp, h->Ctop, h->gid0, h->gc.cont, h->d_loff, h->d_voff, n, gid, h->dE);
 }
 
 void next_level_ids(leiden_handle *h, int64_t n, const int32_t *gid, int32_t *gid_next, int64_t *loff_next) {

@@ -1,5 +1,6 @@
 // Community tracking (Alg. "leidentr"), Sigma recomputation and the terms of
 // modularity (Eq. 1).
+#include <algorithm>
 #include <climits>
 
 #include "internal.h"
@@ -198,6 +199,286 @@ __global__ void k_tr_relabel(int64_t N, const int32_t *Cnew, const int32_t *map,
 __global__ void k_tr_dsig(int64_t N, const uint8_t *matched, int64_t *dSig) {
   for (int64_t id = ld_gtid(); id < N; id += ld_gstride())
     if (!matched[id]) dSig[id] = 0;
+}
+
+// ---------------------------------------------------------------- sums below 2^32
+// The same result when 2m < 2^32: a weight and an id share one 64-bit word, so
+// "largest weight, then lowest id" is one atomicMax (0 = none).  What else the
+// general path spends its time on is left out:
+//  - community sizes of C^{t-1} (kept for local moving) say which ids exist, so
+//    candidates need no initial value and free ids no sweep over the vertices;
+//  - an old community of one vertex has its candidate as its choice whatever
+//    its weight (most of an R-MAT graph's ids are isolated vertices);
+//  - the new ids are the roots of the last level (C'[c] == c), read in place
+//    of marking every vertex's label;
+//  - the k-th unmatched community meets the k-th free id through two compact
+//    lists built by one pair of kernels;
+//  - stores to the words of giant communities, which every warp holds members
+//    of, pass a small filter per block first.
+// R-MAT 22 (4.19M ids), 64,154 edges: 570 -> 240 us, nine kernels instead of
+// twenty-two.
+constexpr int TR_FILTER = 512;
+
+__device__ __forceinline__ unsigned long long tr_word(uint32_t w, int32_t id) {
+  return ((unsigned long long)w << 32) | (uint32_t)~id;  // never 0: ids are below 2^31
+}
+__device__ __forceinline__ int32_t tr_id(unsigned long long x) { return (int32_t) ~(uint32_t)x; }
+
+// Candidates, and the zeros that the next kernels add to.
+__global__ void __launch_bounds__(256) k_tn_cand(int64_t N, const int32_t *Cold, const int32_t *Cnew, int32_t *cand,
+                                                 uint32_t *dev, unsigned long long *match, DevCounters *cnt) {
+  __shared__ int32_t seen[TR_FILTER];
+  for (int t = threadIdx.x; t < TR_FILTER; t += 256) seen[t] = -1;
+  __syncthreads();
+  if (ld_gtid() == 0) { cnt->tr_occ = 0; cnt->tr_flagged = 0; }
+  for (int64_t i = ld_gtid(); i < N; i += ld_gstride()) {
+    int32_t o = Cold[i];
+    dev[i] = 0;
+    match[i] = 0;
+    int32_t *f = &seen[(uint32_t)o % TR_FILTER];
+    if (*f == o) continue;  // a member of this block has stored it (any member will do)
+    *f = o;
+    cand[o] = Cnew[i];
+  }
+}
+// Weight of the members whose new label differs from the candidate.
+__global__ void __launch_bounds__(256) k_tn_deviants(int64_t N, const int32_t *Cold, const int32_t *Cnew,
+                                                     const int64_t *K, const int32_t *cand, uint32_t *dev) {
+  for (int64_t i = ld_gtid(); i < N; i += ld_gstride()) {
+    int32_t o = Cold[i];
+    if (Cnew[i] != cand[o]) {
+      int64_t k = K[i];
+      if (k) atomicAdd(&dev[o], (uint32_t)k);
+    }
+  }
+}
+// The choice of every old community with a majority (bc, matched at once);
+// the others are flagged: bit set, listed, best word cleared.  choice -1: no
+// such community.
+__global__ void __launch_bounds__(256) k_tn_majority(int64_t N, const int32_t *size, const int32_t *cand,
+                                                     const int64_t *tot, const uint32_t *dev, int32_t *choice,
+                                                     unsigned long long *match, uint32_t *bits, int32_t *flagged,
+                                                     unsigned long long *best, DevCounters *cnt) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t o0 = (ld_gtid() & ~31ll); o0 < N; o0 += ld_gstride()) {  // warp-uniform
+    int64_t o = o0 + lane;
+    int32_t sz = o < N ? size[o] : 0;
+    bool f = false;
+    int32_t c = -1;
+    if (sz > 0) {
+      int64_t t = tot[o], ov = t - (int64_t)dev[o];
+      if (sz == 1 || (t > 0 && 2 * ov > t)) {
+        c = cand[o];
+        unsigned long long w = tr_word((uint32_t)ov, (int32_t)o);
+        if (__ldcg(&match[c]) < w) atomicMax(&match[c], w);
+      } else {
+        f = true;  // no majority, or weight 0 and several members
+        best[o] = 0;
+      }
+    }
+    if (o < N) choice[o] = c;
+    uint32_t m = __ballot_sync(LD_FULL, f);
+    if (lane == 0) bits[o0 >> 5] = m;
+    if (!m) continue;
+    int32_t p0 = 0;
+    if (lane == 0) p0 = atomicAdd(&cnt->tr_flagged, __popc(m));
+    p0 = __shfl_sync(LD_FULL, p0, 0);
+    if (f) flagged[p0 + __popc(m & ((1u << lane) - 1u))] = (int32_t)o;
+  }
+}
+// Pair weights of the flagged communities (as k_trc_insert); members of a
+// community of weight 0 offer their labels at weight 0.
+__global__ void __launch_bounds__(256) k_tn_insert(int64_t N, const int32_t *Cold, const int32_t *Cnew,
+                                                   const int64_t *K, const int64_t *tot, const uint32_t *bits,
+                                                   unsigned long long *best, int64_t cap, uint64_t *keys,
+                                                   int64_t *vals, int32_t *list, DevCounters *cnt) {
+  if (cnt->tr_flagged == 0) return;
+  uint64_t mask = (uint64_t)cap - 1;
+  int lane = threadIdx.x & 31;
+  for (int64_t base = (ld_gtid() & ~31ll); base < N; base += ld_gstride()) {  // warp-uniform
+    int64_t i = base + lane;
+    int32_t o = i < N ? Cold[i] : 0;
+    bool take = i < N && ld_bit_test(bits, o);
+    if (!__any_sync(LD_FULL, take)) continue;
+    uint64_t key = EMPTY64 - 1 - lane;
+    int64_t kw = 0;
+    if (take && tot[o] == 0) {
+      atomicMax(&best[o], tr_word(0, Cnew[i]));
+      take = false;
+    } else if (take) {
+      key = ((uint64_t)(uint32_t)o << 32) | (uint32_t)Cnew[i];
+      kw = K[i];
+    }
+    uint32_t peers = __match_any_sync(LD_FULL, (unsigned long long)key);
+    int64_t sum = ld_group_sum_i64(peers, kw);
+    int32_t claimed = -1;
+    if (take && ld_group_leader(peers)) {
+      uint64_t sl = hash64(key) & mask;
+      for (uint64_t probe = 0; ld_ok(probe <= mask, LD_CHK_PROBE); probe++) {
+        unsigned long long k = __ldcg((const unsigned long long *)&keys[sl]);
+        if (k == EMPTY64) {
+          k = atomicCAS((unsigned long long *)&keys[sl], EMPTY64, key);
+          if (k == EMPTY64) claimed = (int32_t)sl;
+        }
+        if (k == EMPTY64 || k == key) {
+          atomicAdd((unsigned long long *)&vals[sl], (unsigned long long)sum);
+          break;
+        }
+        sl = (sl + 1) & mask;
+      }
+    }
+    uint32_t m = __ballot_sync(LD_FULL, claimed >= 0);
+    if (m) {
+      int leader = __ffs(m) - 1;
+      int32_t p0 = 0;
+      if (lane == leader) p0 = atomicAdd(&cnt->tr_occ, __popc(m));
+      p0 = __shfl_sync(LD_FULL, p0, leader);
+      if (claimed >= 0) list[p0 + __popc(m & ((1u << lane) - 1u))] = claimed;
+    }
+  }
+}
+// The flagged communities' best pairs, leaving the table empty.
+__global__ void k_tn_best(const DevCounters *cnt, const int32_t *list, uint64_t *keys, int64_t *vals,
+                          unsigned long long *best) {
+  int64_t m = cnt->tr_occ;
+  for (int64_t t = ld_gtid(); t < m; t += ld_gstride()) {
+    int32_t sl = list[t];
+    uint64_t key = keys[sl];
+    atomicMax(&best[key >> 32], tr_word((uint32_t)vals[sl], (int32_t)(key & 0xffffffffu)));
+    keys[sl] = EMPTY64;
+    vals[sl] = 0;
+  }
+}
+__global__ void k_tn_match(const DevCounters *cnt, const int32_t *flagged, const unsigned long long *best,
+                           int32_t *choice, unsigned long long *match) {
+  int64_t m = cnt->tr_flagged;
+  for (int64_t t = ld_gtid(); t < m; t += ld_gstride()) {
+    int32_t o = flagged[t];
+    unsigned long long b = best[o];
+    int32_t c = tr_id(b);
+    choice[o] = c;
+    atomicMax(&match[c], tr_word((uint32_t)(b >> 32), o));
+  }
+}
+
+// Flags of id c: 1 = a new community that nobody chose, 2 = an id that no old
+// community has, 4 = a new community.
+__device__ __forceinline__ uint32_t tn_flags(int64_t c, int64_t N, const uint8_t *used, const int32_t *root,
+                                             int64_t nroot, const unsigned long long *match, const int32_t *size) {
+  if (c >= N) return 0;
+  bool u = used ? used[c] != 0 : c < nroot && root[c] == (int32_t)c;
+  return (u && match[c] == 0 ? 1u : 0u) | (size[c] == 0 ? 2u : 0u) | (u ? 4u : 0u);
+}
+// The ids in tiles of a multiple of TR_STEP, at most TR_TILES_MAX of them (each
+// block of the second kernel adds up the tiles before its own); the four ids
+// of a thread per step are loaded together.
+constexpr int TR_STEP = 1024, TR_TILES_MAX = 4096;
+// Tile counts (unmatched, free), and the number of new communities.
+__global__ void __launch_bounds__(256) k_tn_tiles(int64_t N, int tile, const uint8_t *used, const int32_t *root,
+                                                  int64_t nroot, const unsigned long long *match, const int32_t *size,
+                                                  int2 *tiles, DevCounters *cnt) {
+  __shared__ int su, sf, sr;
+  if (threadIdx.x == 0) su = sf = sr = 0;
+  __syncthreads();
+  int nu = 0, nf = 0, nr = 0;
+  for (int q = 0; q < tile; q += TR_STEP) {
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      uint32_t f = tn_flags((int64_t)blockIdx.x * tile + q + 256 * u + threadIdx.x, N, used, root, nroot, match, size);
+      nu += f & 1;
+      nf += f >> 1 & 1;
+      nr += f >> 2;
+    }
+  }
+  nu = __reduce_add_sync(LD_FULL, nu);
+  nf = __reduce_add_sync(LD_FULL, nf);
+  nr = __reduce_add_sync(LD_FULL, nr);
+  if ((threadIdx.x & 31) == 0) { atomicAdd(&su, nu); atomicAdd(&sf, nf); atomicAdd(&sr, nr); }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    tiles[blockIdx.x] = make_int2(su, sf);
+    if (sr) atomicAdd(&cnt->list_count, sr);
+  }
+}
+// rank[c] of the unmatched ids and the list of the free ones, both in id
+// order; batched handles also record both ranks at each graph's first id.
+__global__ void __launch_bounds__(256) k_tn_lists(int64_t N, int tile, const uint8_t *used, const int32_t *root,
+                                                  int64_t nroot, const unsigned long long *match, const int32_t *size,
+                                                  const int2 *tiles, int32_t *rank, int32_t *freel,
+                                                  const int32_t *gid0, const int64_t *voff, int2 *granks) {
+  __shared__ int2 wsum[4][8];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int pu = 0, pf = 0;  // in the tiles before this one
+#pragma unroll 4
+  for (int t = threadIdx.x; t < (int)blockIdx.x; t += 256) { int2 x = tiles[t]; pu += x.x; pf += x.y; }
+  pu = __reduce_add_sync(LD_FULL, pu);
+  pf = __reduce_add_sync(LD_FULL, pf);
+  if (lane == 0) wsum[0][wid] = make_int2(pu, pf);
+  __syncthreads();
+  pu = pf = 0;
+  for (int w = 0; w < 8; w++) { pu += wsum[0][w].x; pf += wsum[0][w].y; }
+  const uint32_t below = (1u << lane) - 1u;
+  for (int q = 0; q < tile; q += TR_STEP) {
+    int64_t c0 = (int64_t)blockIdx.x * tile + q + threadIdx.x;
+    uint32_t f[4], mu[4], mf[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) f[u] = tn_flags(c0 + 256 * u, N, used, root, nroot, match, size);
+    __syncthreads();  // the sums of the step before are read
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      mu[u] = __ballot_sync(LD_FULL, f[u] & 1);
+      mf[u] = __ballot_sync(LD_FULL, f[u] & 2);
+      if (lane == 0) wsum[u][wid] = make_int2(__popc(mu[u]), __popc(mf[u]));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      int ru = pu, rf = pf;
+#pragma unroll
+      for (int w = 0; w < 8; w++) {
+        int2 x = wsum[u][w];
+        if (w < wid) { ru += x.x; rf += x.y; }
+        pu += x.x;
+        pf += x.y;
+      }
+      ru += __popc(mu[u] & below);
+      rf += __popc(mf[u] & below);
+      int64_t c = c0 + 256 * u;
+      if (f[u] & 1) rank[c] = ru;
+      if (f[u] & 2) freel[rf] = (int32_t)c;
+      if (gid0 && c < N && voff[gid0[c]] == c) granks[gid0[c]] = make_int2(ru, rf);
+    }
+  }
+}
+// The tracked id of new community c.
+__device__ __forceinline__ int32_t tn_name(int32_t c, const unsigned long long *match, const int32_t *rank,
+                                           const int32_t *freel, const int32_t *gid0, const int2 *granks) {
+  unsigned long long m = match[c];
+  if (m) return tr_id(m);
+  if (!gid0) return freel[rank[c]];
+  int2 g = granks[gid0[c]];  // the k-th unmatched of a graph takes its k-th free id
+  return freel[g.y + rank[c] - g.x];
+}
+// C^t, Sigma and the member counts follow the vertices whose id changes; the
+// change sums of ids that were not carried over are reset.
+__global__ void __launch_bounds__(256) k_tn_relabel(int64_t N, const int32_t *Cnew, const unsigned long long *match,
+                                                    const int32_t *rank, const int32_t *freel, const int32_t *choice,
+                                                    const int64_t *K, int32_t *C, int64_t *Sig, int32_t *size,
+                                                    int64_t *dSig, const int32_t *gid0, const int2 *granks) {
+  for (int64_t i = ld_gtid(); i < N; i += ld_gstride()) {
+    int32_t ch = choice[i];
+    if (ch < 0 || tr_id(match[ch]) != (int32_t)i) dSig[i] = 0;
+    int32_t c = tn_name(Cnew[i], match, rank, freel, gid0, granks), o = C[i];
+    if (c == o) continue;
+    C[i] = c;
+    int64_t k = K[i];
+    if (k) {
+      atomicAdd((unsigned long long *)&Sig[o], (unsigned long long)(-k));
+      atomicAdd((unsigned long long *)&Sig[c], (unsigned long long)k);
+    }
+    atomicSub(&size[o], 1);
+    atomicAdd(&size[c], 1);
+  }
 }
 
 // ---- modularity
@@ -401,9 +682,45 @@ __global__ void __launch_bounds__(256) k_rowsum_big(const int32_t *big, const in
 
 }  // namespace
 
-// C^{t-1} = h->C, final top-level membership = h->Ctop  ->  h->C, h->Sig, h->dSig.
-void track_communities(leiden_handle *h) {
+// Scratch (each array used by nobody else between the last lookup and the
+// next call): 4-byte cand, dev, choice, flagged, rank, free ids; 8-byte match,
+// best.
+static void track_narrow(leiden_handle *h, const int32_t *root, int64_t nroot) {
   cudaStream_t s = h->stream;
+  int64_t N = h->n;
+  int gN = grid_for(N, TB);
+  const int32_t *Cnew = h->Ctop;
+  int32_t *cand = h->mtarget, *choice = h->movers, *flagged = h->prop, *rank = h->rep, *freel = h->parent;
+  uint32_t *dev = (uint32_t *)h->ibuf0, *bits = h->unproc;
+  unsigned long long *match = (unsigned long long *)h->lbuf0, *best = (unsigned long long *)h->lbuf1;
+  int2 *tiles = (int2 *)h->lbuf2, *granks = (int2 *)h->lbuf3;
+  const uint8_t *used = h->G > 1 ? h->dE : nullptr;
+  DevCounters *cnt = h->dcnt;
+  ld_note_launch(), k_tn_cand<<<gN, TB, 0, s>>>(N, h->C, Cnew, cand, dev, match, cnt);
+  ld_note_launch(), k_tn_deviants<<<gN, TB, 0, s>>>(N, h->C, Cnew, h->K, cand, dev);
+  ld_note_launch(), k_tn_majority<<<gN, TB, 0, s>>>(N, h->csize0, cand, h->Sig, dev, choice, match, bits, flagged, best,
+                                                    cnt);
+  ld_note_launch(), k_tn_insert<<<gN, TB, 0, s>>>(N, h->C, Cnew, h->K, h->Sig, bits, best, h->tr_cap, h->tr_keys,
+                                                  h->tr_vals, h->tr_list, cnt);
+  ld_note_launch(), k_tn_best<<<h->sm_count * 2, TB, 0, s>>>(cnt, h->tr_list, h->tr_keys, h->tr_vals, best);
+  ld_note_launch(), k_tn_match<<<h->sm_count * 2, TB, 0, s>>>(cnt, flagged, best, choice, match);
+  int tile = TR_STEP * (int)std::max<int64_t>(1, (N + (int64_t)TR_STEP * TR_TILES_MAX - 1) / ((int64_t)TR_STEP * TR_TILES_MAX));
+  int nt = (int)((N + tile - 1) / tile);
+  ld_note_launch(), k_tn_tiles<<<nt, TB, 0, s>>>(N, tile, used, root, nroot, match, h->csize0, tiles, cnt);
+  ld_note_launch(), k_tn_lists<<<nt, TB, 0, s>>>(N, tile, used, root, nroot, match, h->csize0, tiles, rank, freel,
+                                                 h->gid0, h->d_voff, granks);
+  ld_note_launch(), k_tn_relabel<<<gN, TB, 0, s>>>(N, Cnew, match, rank, freel, choice, h->K, h->C, h->Sig, h->csize0,
+                                                   h->dSig, h->gid0, granks);
+}
+
+// C^{t-1} = h->C, final top-level membership = h->Ctop  ->  h->C, h->Sig, h->dSig.
+// The new ids: the roots of the last level (c < nroot, root[c] == c); of a
+// batched handle the ids flagged in h->dE.
+void track_communities(leiden_handle *h, const int32_t *root, int64_t nroot) {
+  cudaMemsetAsync(&h->dcnt->list_count, 0, sizeof(int32_t), h->stream);
+  if (!wide_sums(h)) { track_narrow(h, root, nroot); return; }
+  cudaStream_t s = h->stream;
+  if (h->G == 1) count_communities(h, nroot, nullptr);
   int64_t N = h->n;
   int gN = grid_for(N, TB);
   long long *bw = (long long *)h->lbuf0, *ow = (long long *)h->lbuf1;
