@@ -28,9 +28,9 @@ double i128_to_double(i128 x) {
 GraphCounters gc_layout(void *base, int G) {
   char *q = (char *)base;
   GraphCounters c;
-  c.dq = (unsigned long long *)q;  q += 16 * (size_t)G;
-  c.sq = (unsigned long long *)q;  q += 16 * (size_t)G;
+  c.dq = (unsigned long long *)q;  q += 16 * (size_t)G;  // dq and moves are cleared together
   c.moves = (int64_t *)q;          q += 8 * (size_t)G;
+  c.sq = (unsigned long long *)q;  q += 16 * (size_t)G;
   c.m2 = (int64_t *)q;             q += 8 * (size_t)G;
   c.sigma = (int64_t *)q;          q += 8 * (size_t)G;
   c.accepted = (int32_t *)q;       q += 4 * (size_t)G;
@@ -250,7 +250,7 @@ void sync_all(leiden_handle *h) {
 // graph keeps its own iteration count and stops iterating when its own dQ
 // reaches tau, keeps its own refinement rounds, and leaves the pass loop at
 // its own break (its final lookup is done then and it is not aggregated).
-leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range) {
+leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range, bool dense) {
   cudaStream_t s = h->stream;
   const leiden_params &p = h->p;
   int64_t N = h->n;
@@ -280,15 +280,16 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range)
   // must move per unit of its work (vertex of the level, arc scanned, move,
   // listed vertex), with the sizes of the arrays it reads and writes.
   ph_mark(h, LEIDEN_PHASE_MOVE);
-  ph_bytes(h, LEIDEN_PHASE_MOVE, 45 * N + N / 8);  // dV -> frontier bits; Ctop; copies of C', K', Sigma'
-  pass_init(h);
-  CK(cudaMemsetAsync(&h->dcnt->processed, 0, 14 * sizeof(int64_t), s));  // processed .. lmk_bytes
+  ph_bytes(h, LEIDEN_PHASE_MOVE, 37 * N + N / 8);  // dV -> frontier bits; copies of C', Sigma', sizes; smallest members
+  pass_init(h, dynamic != 0);
+  CK(cudaMemsetAsync(&h->dcnt->processed, 0, 13 * sizeof(int64_t), s));  // processed .. lmk_bytes
   int64_t m2 = h->m2;
   LevelGraph g = level0(h);
   double tau = p.tau;
   int slot = 0;
   int passes = 0;
   bool looked_up = false;  // batched: every graph had its final lookup
+  bool last_first = true;  // no aggregated level yet
   leiden_stats &st = h->stats;
   int64_t moves_total = 0;
   int64_t subsweep_words = 0;     // frontier words read by the collection kernels
@@ -315,17 +316,10 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range)
       CK(cudaMemcpyAsync(h->gc.lm_on, hg.lm_on, (size_t)G, cudaMemcpyHostToDevice, s));
     }
     if (lp > 0) ph_mark(h, LEIDEN_PHASE_MOVE);
-    ph_bytes(h, LEIDEN_PHASE_MOVE, (lp > 0 || !dynamic ? 4 : 8) * n);  // community sizes
-    lm_prepare(h, g, lp > 0 || !dynamic ? SIZES_ONES : SIZES_KEPT);
     int li = p.max_iterations;
     for (int it = 0; it < p.max_iterations; it++) {
-      CK(cudaMemsetAsync(&h->dcnt->dq[0], 0, 2 * sizeof(unsigned long long), s));
-      CK(cudaMemsetAsync(&h->dcnt->moves, 0, sizeof(int64_t), s));
-      if (B) {
-        CK(cudaMemsetAsync(h->gc.dq, 0, (size_t)G * 2 * sizeof(unsigned long long), s));
-        CK(cudaMemsetAsync(h->gc.moves, 0, (size_t)G * sizeof(int64_t), s));
-      }
-      for (int cls = 0; cls < lm_classes(h); cls++) lm_subsweep(h, g, cls, lp == 0 ? in_range : nullptr, dynamic);
+      if (B) CK(cudaMemsetAsync(h->gc.dq, 0, (size_t)G * 24, s));  // dq, moves
+      lm_iteration(h, g, lp == 0 ? in_range : nullptr, dynamic, dense || lp > 0);
       subsweep_words += (int64_t)lm_classes(h) * ((n + 31) / 32);
       sync_all(h);
       kt_resolve(h);
@@ -357,12 +351,10 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range)
     }
     tr[1] = li;
     ph_mark(h, LEIDEN_PHASE_SPLIT);
-    ph_bytes(h, LEIDEN_PHASE_SPLIT, 64 * n);  // subset renumbering (58 B per vertex), split flags (6 B)
-    subset_renumber(h, n);
-    split_communities(h, g);
+    ph_bytes(h, LEIDEN_PHASE_SPLIT, 31 * n);  // smallest members (8 B per vertex, 4 per id), new ids and flags (19 B)
+    renumber_and_split(h, g);
     ph_mark(h, LEIDEN_PHASE_REFINE);
     ph_bytes(h, LEIDEN_PHASE_REFINE, 29 * n);  // bounds C'_B, reset of the refined bounds
-    CK(cudaMemcpyAsync(h->CB, h->Cp, (size_t)n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
     if (B) CK(cudaMemsetAsync(h->gc.refined, 0, (size_t)G, s));
     refine_reset(h, g);
     int rounds = 0;
@@ -445,7 +437,8 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range)
       ncomm = tot;
       if (!B) tr[2] = ncomm;
     }
-    lookup_dendrogram(h);
+    lookup_dendrogram(h, lp == 0);
+    last_first = false;
     // every aggregated level has at most the arcs of G^t (held since the
     // call's start; re-taken only if the batch outgrew the bound)
     if (!acquire_agg_buffers(h, h->g_arcs)) { h->err = "aggregation buffers (stream-ordered pool)"; return LEIDEN_ERR_OOM; }
@@ -486,9 +479,10 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range)
   }
   ph_mark(h, LEIDEN_PHASE_TRACK);
   ph_bytes(h, LEIDEN_PHASE_TRACK, (B ? 0 : 12 * N) + 234 * N);  // final lookup; tracking's sweeps
-  if (!B) lookup_dendrogram(h);
-  else if (!looked_up) { h->err = "batched pass loop ended without a final lookup"; return LEIDEN_ERR_STATE; }
-  track_communities(h, h->Cp, g.n);
+  if (!B && !last_first) lookup_dendrogram(h, false);
+  if (B && !looked_up) { h->err = "batched pass loop ended without a final lookup"; return LEIDEN_ERR_STATE; }
+  // a call of one pass: the membership is C' itself
+  track_communities(h, !B && last_first ? h->Cp : h->Ctop, h->Cp, g.n);
   ph_mark(h, PHASE_END);
   release_agg_buffers(h);
   sync_counters(h);
@@ -602,7 +596,9 @@ leiden_status do_update(leiden_handle *h, const leiden_edge *d_del, int64_t n_de
   }
   h->g_maxdeg = h->hcnt->max_count;
   h->g_huge_slots = h->hcnt->huge_slots;
-  st = run_leiden(h, 1, mode == LEIDEN_DS ? h->dV : nullptr);
+  // a DF batch marks at most the two ends of each of its edges
+  bool dense = mode != LEIDEN_DF || 16 * (n_del + n_ins) > h->n;
+  st = run_leiden(h, 1, mode == LEIDEN_DS ? h->dV : nullptr, dense);
   if (st != LEIDEN_OK) {
     h->broken = true;
     release_agg_buffers(h);
@@ -754,7 +750,7 @@ leiden_status leiden_create(const leiden_params *params, int64_t n, const int64_
   for (auto pp : i32s) A(dalloc(h, pp, n + 1));
   int64_t **i64s[] = {&h->Kp, &h->Sp, &h->S2, &h->lbuf0, &h->lbuf1, &h->lbuf2, &h->lbuf3, &h->coff, &h->cflat};
   for (auto pp : i64s) A(dalloc(h, pp, n + 2));
-  uint8_t **u8s[] = {&h->dS, &h->dR, &h->dS2, &h->dR2, &h->dE, &h->dCf};
+  uint8_t **u8s[] = {&h->dS, &h->dR, &h->dR2, &h->dE, &h->dCf};
   for (auto pp : u8s) A(dalloc(h, pp, n + 1));
   A(dalloc(h, &h->unproc, n / 32 + 2));
   A(dalloc(h, &h->bins, (int64_t)NBINS * n));
@@ -899,7 +895,7 @@ int64_t leiden_footprint_bytes(const leiden_params *params, int64_t n, const int
   int64_t b = 0;
   b += 8 * (n + 1) + 8 * n + 8 * total;                              // G^t: off, deg, rcap, col, w
   b += 4 * n + 24 * n + n;                                            // C, K, Sigma, dSigma, dV
-  b += 56 * (n + 1) + 72 * (n + 2) + 6 * (n + 1);                     // per-pass work arrays
+  b += 56 * (n + 1) + 72 * (n + 2) + 5 * (n + 1);                     // per-pass work arrays
   b += 4 * (n / 32 + 2) + 16 * n + 4 * (n + 1) + 8 * n;               // frontier, bins, hocc, cand
   b += 2 * (8 * (n + 2) + 4 * (n + 1));                              // aggregated levels' offsets, degrees
   b += 16 * tc + 4 * n + (int64_t)scan_tmp_bytes(2 * n + 2);          // tracking, scans
@@ -971,7 +967,7 @@ leiden_status leiden_static(leiden_handle *h, int32_t *membership_out) {
   }
   h->g_maxdeg = h->hcnt->max_count;
   h->g_huge_slots = h->hcnt->huge_slots;
-  st = run_leiden(h, 0, nullptr);
+  st = run_leiden(h, 0, nullptr, true);
   if (st != LEIDEN_OK) {
     h->broken = true;
     release_agg_buffers(h);

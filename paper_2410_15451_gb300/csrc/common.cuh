@@ -15,22 +15,30 @@ typedef unsigned __int128 u128;
 // ---------------------------------------------------------------- counters
 // One block of device counters per handle, mirrored to pinned host memory at
 // the few host synchronisation points of a call.
+// Counters of one sub-sweep.  A local-moving iteration uses one set per class,
+// so that all are cleared together before it (SUB_RING classes at a time).
+struct SubCounters {
+  int32_t bin_count[4];           // vertices in each degree bin
+  int32_t movers;                 // deferred moves (SYNC)
+  int32_t big_movers;             // moved hubs whose neighbours are marked by a kernel of their own
+  int32_t pad[2];
+};
+constexpr int SUB_RING = 16;
+
 struct DevCounters {
   unsigned long long dq[2];       // sum of accepted gains g (int128, two's complement)
-  int32_t bin_count[4];           // vertices in each degree bin of the current sub-sweep
-  int32_t movers;                 // deferred moves of the current sub-sweep (SYNC)
-  int32_t big_movers;             // moved hubs whose neighbours are marked when the moves are applied
+  int64_t moves;                  // local-moving moves of the iteration
+  SubCounters sub[SUB_RING];      // (dq .. sub: cleared together)
+  SubCounters ref;                // bins of a refinement round or of aggregation
   int32_t accepted;               // refinement moves applied in this round
   int32_t cand_count[2];          // refinement candidate lists (ping-pong)
   int32_t error;                  // batch validation error (first offending arc + 1)
   int32_t overflow;               // a touched CSR row outgrew its capacity
   int32_t list_count;             // generic list length
   int32_t ncomm;                  // communities after dense renumbering
-  int32_t split_count;            // vertices in communities to split
   int32_t max_count;              // max degree (level), max community degree
   int64_t processed;              // local-moving vertex visits
   int64_t arcs;                   // local-moving arcs scanned
-  int64_t moves;                  // local-moving moves
   int64_t ref_processed;          // refinement vertex visits
   int64_t ref_arcs;               // refinement arcs scanned
   int64_t lmk_visits[3];          // local moving per timed kernel (warp range, block bin, hub scan):
@@ -41,7 +49,6 @@ struct DevCounters {
   unsigned long long sq[2];       // modularity: sum of Sigma_c^2 (int128)
   int64_t batch_dw;               // batch: change of 2m
   int64_t huge_slots;             // table slots the vertices above the block bin need
-  int32_t big_count;              // splitting: long rows left to the block kernel
   int32_t large_count;            // batch apply: touched rows merged in chunks
   int32_t tr_occ;                 // tracking: filled slots of the pair table
   int32_t tr_flagged;             // tracking: old communities without a majority candidate
@@ -51,7 +58,9 @@ struct DevCounters {
   int64_t bcounts[8];             // batch apply: unique deletions, unique insertions, new arcs,
                                   //   touched rows, merge-buffer arcs
   int64_t affected;               // |dV|: vertices flagged affected (counted into the frontier)
-  int64_t split_arcs;             // splitting: arcs of the vertices listed for splitting
+  int64_t split_arcs;             // splitting: arcs of the vertices listed for splitting,
+  int32_t split_count;            //   these vertices,
+  int32_t big_count;              //   and long rows (also of the row kernels) left to a chunked one
   int64_t deg_sum;                // degree sum of the level scanned by level_maxdeg (its arcs)
   int64_t xk_bytes[3];            // algorithmic bytes of the other timed kernels (split sampling,
                                   //   giant-community aggregation scan, block merge of touched rows)
@@ -400,6 +409,50 @@ __device__ __forceinline__ void wt_flush(WarpTable<WIDE> &T, const GTable &G) {
   __syncwarp();
   if (lane == 0) T.count = 0;
   __syncwarp();
+}
+
+// ---------------------------------------------------------------- block appends
+// A block of 256 threads appends its items to up to CATS lists at once, one
+// atomic per list and step: one atomic per warp on a list's length costs more
+// than the sweep itself (4.19M vertices: 131k of them on one word).  An item
+// is a set of categories (bit q: list q); each thread has APPEND_UNROLL items
+// per step.  All threads call it; at[u][q] is the item's place in list q.
+constexpr int APPEND_UNROLL = 4;
+constexpr int APPEND_STEP = 256 * APPEND_UNROLL;
+template <int CATS>
+struct BlockAppend {
+  int32_t off[CATS][APPEND_UNROLL * 8];
+};
+template <int CATS>
+__device__ __forceinline__ void block_append(BlockAppend<CATS> &B, const uint32_t *cats, int32_t *const *lengths,
+                                             int32_t (*at)[CATS]) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const uint32_t below = (1u << lane) - 1u;
+  __syncthreads();  // the places of the step before are read
+#pragma unroll
+  for (int u = 0; u < APPEND_UNROLL; u++)
+#pragma unroll
+    for (int q = 0; q < CATS; q++) {
+      uint32_t m = __ballot_sync(LD_FULL, cats[u] >> q & 1);
+      at[u][q] = __popc(m & below);
+      if (lane == 0) B.off[q][u * 8 + wid] = __popc(m);
+    }
+  __syncthreads();
+  for (int q = wid; q < CATS; q += 8) {  // a warp per list: 32 counts
+    int32_t v = B.off[q][lane], incl = v, base = 0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      int32_t y = __shfl_up_sync(LD_FULL, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31 && incl) base = atomicAdd(lengths[q], incl);
+    B.off[q][lane] = __shfl_sync(LD_FULL, base, 31) + incl - v;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < APPEND_UNROLL; u++)
+#pragma unroll
+    for (int q = 0; q < CATS; q++) at[u][q] += B.off[q][u * 8 + wid];
 }
 
 // Per-graph sums of a batched handle: every lane of the warp calls these;

@@ -118,9 +118,10 @@ struct leiden_handle {
   int32_t *Cp = nullptr, *CB = nullptr, *Ctop = nullptr, *csize = nullptr, *rep = nullptr;
   int32_t *csize0 = nullptr;  // [n] member counts of C^t (kept by tracking for the next call)
   int32_t *prop = nullptr, *parent = nullptr, *ibuf0 = nullptr, *ibuf1 = nullptr, *ibuf2 = nullptr;
+  const int64_t *Kc = nullptr;  // K of the current level: K at level 0, then Kp
   int64_t *Kp = nullptr, *Sp = nullptr, *S2 = nullptr, *lbuf0 = nullptr, *lbuf1 = nullptr;
   int64_t *lbuf2 = nullptr, *lbuf3 = nullptr;
-  uint8_t *dS = nullptr, *dR = nullptr, *dS2 = nullptr, *dR2 = nullptr, *dE = nullptr, *dCf = nullptr;
+  uint8_t *dS = nullptr, *dR = nullptr, *dR2 = nullptr, *dE = nullptr, *dCf = nullptr;
   uint32_t *unproc = nullptr;  // bitmap, words = n/32 + 2
   int32_t *bins = nullptr;     // NBINS * n
   int32_t *movers = nullptr;   // [n]
@@ -313,15 +314,13 @@ inline int lm_classes(const leiden_handle *h) {
 inline bool wide_sums(const leiden_handle *h) { return h->m2 >= ((int64_t)1 << 32); }
 
 // ------------------------------------------------------------ move.cu
-// One local-moving sub-sweep of class `cls` (0 .. classes-1).
-void lm_subsweep(leiden_handle *h, const LevelGraph &g, int cls, const uint8_t *in_range, int dynamic);
+// One local-moving iteration: a sub-sweep per class.  The frontier, C', Sigma',
+// sizes and dq, moves (cleared here) are on the device.  dense: more than about
+// an eighth of the vertices may be in the frontier (how it is collected).
+void lm_iteration(leiden_handle *h, const LevelGraph &g, const uint8_t *in_range, int dynamic, bool dense);
 // Refinement: reset, then one round (SYNC) or one sweep (async) of moves.
 void refine_reset(leiden_handle *h, const LevelGraph &g);
 void refine_round(leiden_handle *h, const LevelGraph &g, int slot);
-// Community sizes of C' for the singleton rule: all ones (C' the identity),
-// the sizes kept by the last tracking (C' = C^{t-1}), or counted.
-enum { SIZES_ONES = 0, SIZES_KEPT = 1, SIZES_COUNT = 2 };
-void lm_prepare(leiden_handle *h, const LevelGraph &g, int sizes_from);
 void count_sizes(leiden_handle *h, const int32_t *C, int64_t n, int32_t *size);
 bool ensure_hslots(leiden_handle *h, int64_t slots);     // false: allocation failed
 int32_t *hs_keys(leiden_handle *h);  // global table scratch: keys, values, slot lists
@@ -329,14 +328,17 @@ int64_t *hs_vals(leiden_handle *h);
 int32_t *hs_list(leiden_handle *h);
 
 // ------------------------------------------------------------ phases.cu
-void subset_renumber(leiden_handle *h, int64_t n);
-void split_communities(leiden_handle *h, const LevelGraph &g);
+// Subset renumbering of Cp (ids become smallest members; dR2 = dR by the new
+// ids) and splitting of the flagged communities.
+void renumber_and_split(leiden_handle *h, const LevelGraph &g);
 // Ranks in lbuf0, count in lbuf0[n]; batched (gid non-null): only the
 // graphs flagged in gc.cont, the others mapped to the spare id lbuf0[n].
 void renumber_dense(leiden_handle *h, int64_t n, const int32_t *gid);
 // Distinct ids of Cp -> dcnt->list_count (and gc.ncomm per graph when batched).
 void count_communities(leiden_handle *h, int64_t n, const int32_t *gid);
-void lookup_dendrogram(leiden_handle *h);  // batched: the continuing graphs only
+// Batched: the continuing graphs only.  first: Ctop is still the identity (and
+// not written).
+void lookup_dendrogram(leiden_handle *h, bool first);
 // Batched: final lookup of the graphs that stop at this level (n vertices, graph
 // ids gid) and their communities' ids flagged in dE (cleared at the first level).
 void break_lookup(leiden_handle *h, int64_t n, const int32_t *gid, bool first);
@@ -344,14 +346,13 @@ void break_lookup(leiden_handle *h, int64_t n, const int32_t *gid, bool first);
 void next_level_ids(leiden_handle *h, int64_t n, const int32_t *gid, int32_t *gid_next, int64_t *loff_next);
 void aggregate(leiden_handle *h, const LevelGraph &g, int64_t ncomm, int out_slot);
 void reset_next_pass(leiden_handle *h, int64_t ncomm, int out_slot);
-void mark_all_unprocessed(leiden_handle *h, int64_t n);
-// Pass-loop start: frontier from dV (counted into affected), Ctop = identity,
-// C' = C, K' = K, Sigma' = Sigma.
-void pass_init(leiden_handle *h);
+// Pass-loop start: frontier from dV (counted into affected), C' = C, K' is K,
+// Sigma' = Sigma, sizes (kept ones, or all 1), smallest members cleared.
+void pass_init(leiden_handle *h, bool sizes_kept);
 void level_maxdeg(leiden_handle *h, const int32_t *deg, int64_t n);  // into dcnt->max_count
 
 // ------------------------------------------------------------ track.cu
-void track_communities(leiden_handle *h, const int32_t *root, int64_t nroot);  // Ctop vs C -> C, Sig, dSig
+void track_communities(leiden_handle *h, const int32_t *Cnew, const int32_t *root, int64_t nroot);
 void modularity_terms(leiden_handle *h, const int32_t *C);  // into dcnt->sigma_intra / sq
 void recompute_weights(leiden_handle *h);  // K = row sums, m2 (device)
 void recompute_sigma(leiden_handle *h);    // Sigma from K and C

@@ -14,6 +14,7 @@
 // move as soon as it is found.
 #include <algorithm>
 #include <atomic>
+#include <cstddef>
 
 #include "internal.h"
 
@@ -58,6 +59,7 @@ struct Args {
   int32_t *accg;
   uint8_t *refg;
   DevCounters *cnt;
+  SubCounters *sub;      // of this sub-sweep
   int dynamic;
   int async_mode;
   int classes_mask;
@@ -224,7 +226,7 @@ __device__ __forceinline__ void record_movers(const Args &A, bool mv, int32_t i,
   if (!m) return;
   int lane = threadIdx.x & 31;
   int32_t p0 = 0;
-  if (lane == __ffs(m) - 1) p0 = atomicAdd(&A.cnt->movers, __popc(m));
+  if (lane == __ffs(m) - 1) p0 = atomicAdd(&A.sub->movers, __popc(m));
   p0 = __shfl_sync(LD_FULL, p0, __ffs(m) - 1);
   if (mv) {
     int32_t slot = p0 + __popc(m & ((1u << lane) - 1u));
@@ -236,7 +238,7 @@ __device__ __forceinline__ void record_movers(const Args &A, bool mv, int32_t i,
 
 // One thread's deferred move.
 __device__ __forceinline__ void record_mover(const Args &A, int32_t i, int32_t c, i128 g) {
-  int32_t slot = atomicAdd(&A.cnt->movers, 1);
+  int32_t slot = atomicAdd(&A.sub->movers, 1);
   A.movers[slot] = i;
   A.mtarget[slot] = c;
   if (A.mgain) { A.mgain[2 * slot] = (int64_t)(u128)g; A.mgain[2 * slot + 1] = (int64_t)((u128)g >> 64); }
@@ -792,7 +794,7 @@ __device__ __forceinline__ Hub hub_load(const Args &A, const int64_t *tab_off, i
 
 // The decision of hub H, by one thread: whether it moved.  The neighbours of a
 // moved hub are marked by its caller, or, above MARK_INLINE arcs in the
-// snapshot schedule, by the kernel that applies the moves.
+// snapshot schedule, by a kernel of their own.
 constexpr int MARK_INLINE = 2048;
 template <int KIND>
 __device__ __forceinline__ bool hub_decide(const Args &A, const Hub &H, BestX b, Tally &tl) {
@@ -802,7 +804,7 @@ __device__ __forceinline__ bool hub_decide(const Args &A, const Hub &H, BestX b,
   bool mv = g > 0;
   if (KIND == KIND_MOVE && !A.async_mode && mv) {
     record_mover(A, H.i, b.c, g);
-    if (H.dg > MARK_INLINE) A.big_movers[atomicAdd(&A.cnt->big_movers, 1)] = H.i;
+    if (H.dg > MARK_INLINE) A.big_movers[atomicAdd(&A.sub->big_movers, 1)] = H.i;
   }
   tl.visits++; tl.arcs += H.dg; tl.moves += mv; tl.dq += g;
   return mv && (A.async_mode || H.dg <= MARK_INLINE);
@@ -854,72 +856,112 @@ __global__ void __launch_bounds__(HUGE_THREADS, 4) k_huge_decide(Args A, const i
 }
 
 // ---------------------------------------------------------------- collection
+// The bin of a degree.
+__device__ __forceinline__ int bin_of(int dg, const leiden_tuning &tn) {
+  return dg <= tn.tiny_max ? BIN_TINY : dg <= tn.warp_max ? BIN_WARP : dg <= tn.block_max ? BIN_BLOCK : BIN_HUGE;
+}
+
+struct CollectArgs {
+  int cls;
+  int32_t *bins;
+  SubCounters *sub;
+  const int64_t *loff;
+  leiden_tuning tn;
+};
+
+// The bin of frontier vertex v in this sub-sweep: a bin, NBINS (taken, but not
+// listed: out of range, or without arcs, whose taking is its visit), or -1 (of
+// another class, or of a batched graph whose iterations ended; the class of
+// such a vertex is taken on its id within its graph).
+__device__ __forceinline__ int collect_bin(const Args &A, const CollectArgs &Q, int64_t v) {
+  int64_t vl = A.gid ? v - Q.loff[A.gid[v]] : v;
+  if (ld_class_of(vl, A.classes_mask) != Q.cls || (A.gid && !A.lm_on[A.gid[v]])) return -1;
+  if (A.in_range && !A.in_range[v]) return NBINS;
+  int dg = A.deg[v];
+  return dg == 0 ? NBINS : bin_of(dg, Q.tn);
+}
+
 // Take the unprocessed vertices of class `cls` (clearing their bits) and
-// append the in-range ones to the degree bins.
-__global__ void k_collect(int64_t n, uint32_t *unproc, int cls, int classes_mask, const uint8_t *in_range,
-                          const int32_t *deg, int32_t *bins, DevCounters *cnt, const int32_t *gid,
-                          const uint8_t *lm_on, const int64_t *loff, leiden_tuning tn) {
-  // Each lane reads one bitmap word and sorts its set bits into per-bin
-  // masks; a warp scan over the lanes' counts then places every vertex, so
-  // a warp appends the vertices of its 32 words in id order with one atomic
-  // per bin, however sparse the frontier is.  The bits taken are cleared
-  // with one write per word (each word belongs to one lane here).
+// append the in-range ones to the degree bins.  Dense frontiers (all vertices,
+// or more than an eighth of them, see lm_iteration): a block takes 32 bitmap
+// words at a time, a lane per bit, so that the degrees are loaded side by
+// side, and appends with one atomic per bin.  Sparse ones: a warp takes 32
+// words, a lane per word, and a scan over the lanes' counts places every
+// vertex with one atomic per bin and warp.  Us per launch, sparse and dense
+// form: R-MAT 22 DF, 64,154 edges (1 bit in 40) 11.6 and 22.4; R-MAT 20 ND 12.5
+// and 10.4; a rolled back batch of 0.1 of its edges 12.3 and 5.7 (a lane
+// walking a full word waits for 32 degrees one after the other).
+__device__ __forceinline__ void collect_sparse(const Args &A, const CollectArgs &Q) {
   int lane = threadIdx.x & 31;
-  int64_t nwords = (n + 31) >> 5;
+  int64_t n = A.n, nwords = (n + 31) >> 5;
   int64_t warp = ld_gtid() >> 5, nwarps = ld_gstride() >> 5;
   for (int64_t w0 = warp * 32; w0 < nwords; w0 += nwarps * 32) {  // warp-uniform
     int64_t wi = w0 + lane;
-    uint32_t word = wi < nwords ? unproc[wi] : 0u, rest = word, taken = 0u;
+    uint32_t word = wi < nwords ? A.unproc[wi] : 0u, taken = 0u;
     uint32_t bm[NBINS];
 #pragma unroll
     for (int b = 0; b < NBINS; b++) bm[b] = 0u;
-    while (rest) {
+    for (uint32_t rest = word; rest; rest &= rest - 1u) {
       int bit = __ffs(rest) - 1;
-      rest &= rest - 1u;
-      int64_t v = (wi << 5) + bit;
-      if (v >= n) break;
-      // batched handles: the class of a vertex is taken on its id within
-      // its graph, and graphs whose iterations ended are skipped
-      int64_t vl = gid ? v - loff[gid[v]] : v;
-      if (ld_class_of(vl, classes_mask) != cls || (gid && !lm_on[gid[v]])) continue;
-      taken |= 1u << bit;
-      if (in_range && !in_range[v]) continue;
-      // a vertex without arcs has no candidate community: taking it is its visit
-      int dg = deg[v];
-      if (dg == 0) continue;
-      int bin = dg <= tn.tiny_max ? BIN_TINY : dg <= tn.warp_max ? BIN_WARP : dg <= tn.block_max ? BIN_BLOCK : BIN_HUGE;
+      int bin = collect_bin(A, Q, (wi << 5) + bit);
+      if (bin >= 0) taken |= 1u << bit;
 #pragma unroll
       for (int b = 0; b < NBINS; b++)
         if (bin == b) bm[b] |= 1u << bit;
     }
 #pragma unroll
     for (int b = 0; b < NBINS; b++) {
-      int k = __popc(bm[b]), incl = k;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(LD_FULL, incl, o);
-        if (lane >= o) incl += y;
-      }
+      int k = __popc(bm[b]), incl = ld_warp_incl_i32(k);
       int total = __shfl_sync(LD_FULL, incl, 31);
       if (total == 0) continue;  // warp-uniform
       int32_t pos0 = 0;
-      if (lane == 31) pos0 = atomicAdd(&cnt->bin_count[b], total);
+      if (lane == 31) pos0 = atomicAdd(&Q.sub->bin_count[b], total);
       pos0 = __shfl_sync(LD_FULL, pos0, 31) + incl - k;
-      int32_t *dst = bins + (int64_t)b * n + pos0;
+      int32_t *dst = Q.bins + (int64_t)b * n + pos0;
       for (uint32_t m = bm[b]; m; m &= m - 1u) *dst++ = (int32_t)((wi << 5) + __ffs(m) - 1);
     }
-    if (taken) unproc[wi] = word & ~taken;
+    if (taken) A.unproc[wi] = word & ~taken;
+  }
+}
+__device__ __forceinline__ void collect_dense(const Args &A, const CollectArgs &Q) {
+  __shared__ BlockAppend<NBINS> B;
+  int32_t *const lengths[NBINS] = {&Q.sub->bin_count[0], &Q.sub->bin_count[1], &Q.sub->bin_count[2],
+                                   &Q.sub->bin_count[3]};
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t n = A.n, nwords = (n + 31) >> 5;
+  for (int64_t w0 = (int64_t)blockIdx.x * 32; w0 < nwords; w0 += (int64_t)gridDim.x * 32) {  // block-uniform
+    uint32_t word[APPEND_UNROLL], cats[APPEND_UNROLL];
+#pragma unroll
+    for (int u = 0; u < APPEND_UNROLL; u++) {
+      int64_t wi = w0 + 8 * u + wid;
+      word[u] = wi < nwords ? A.unproc[wi] : 0u;
+    }
+    bool some = false;
+#pragma unroll
+    for (int u = 0; u < APPEND_UNROLL; u++) {
+      int64_t wi = w0 + 8 * u + wid;
+      int bin = word[u] >> lane & 1u ? collect_bin(A, Q, (wi << 5) + lane) : -1;
+      uint32_t taken = __ballot_sync(LD_FULL, bin >= 0);
+      if (lane == 0 && taken) A.unproc[wi] = word[u] & ~taken;
+      cats[u] = bin >= 0 && bin < NBINS ? 1u << bin : 0u;
+      some = some || cats[u];
+    }
+    if (!__syncthreads_or(some)) continue;
+    int32_t at[APPEND_UNROLL][NBINS];
+    block_append<NBINS>(B, cats, lengths, at);
+#pragma unroll
+    for (int u = 0; u < APPEND_UNROLL; u++)
+#pragma unroll
+      for (int b = 0; b < NBINS; b++)
+        if (cats[u] >> b & 1) Q.bins[(int64_t)b * n + at[u][b]] = (int32_t)(((w0 + 8 * u + wid) << 5) + lane);
   }
 }
 
-// Deferred moves of a sub-sweep (deterministic mode), and the neighbours of
-// the moved hubs above MARK_INLINE arcs, each hub cut into MARK_PARTS for as
-// many warps.  Batched handles also sum the gains and moves per graph (gid
-// non-null).
-constexpr int MARK_PARTS = 32;
-__global__ void k_apply_moves(Args A, unsigned long long *dqg, int64_t *movesg) {
+// Deferred moves of a sub-sweep (deterministic mode).  Batched handles also
+// sum the gains and moves per graph (gid non-null).
+__device__ __forceinline__ void apply_moves(const Args &A, unsigned long long *dqg, int64_t *movesg) {
   const int32_t *gid = A.gid;
-  int64_t m = A.cnt->movers;
+  int64_t m = A.sub->movers;
   for (int64_t t0 = (ld_gtid() & ~31ll); t0 < m; t0 += ld_gstride()) {  // warp-uniform trip count
     int64_t t = t0 + (threadIdx.x & 31);
     bool has = t < m;
@@ -945,7 +987,24 @@ __global__ void k_apply_moves(Args A, unsigned long long *dqg, int64_t *movesg) 
       ld_graph_add_i64(movesg, has, gi, 1);
     }
   }
-  int64_t parts = (int64_t)A.cnt->big_movers * MARK_PARTS;
+}
+
+// Between two sub-sweeps: the moves of one are applied and the vertices of the
+// next are collected (they touch different arrays).  `apply`: there was one
+// before; Q.cls < 0: there is none after.
+template <bool DENSE>
+__global__ void __launch_bounds__(256) k_apply_collect(Args A, bool apply, unsigned long long *dqg, int64_t *movesg, CollectArgs Q) {
+  if (apply) apply_moves(A, dqg, movesg);
+  if (Q.cls < 0) return;
+  if (DENSE) collect_dense(A, Q);
+  else collect_sparse(A, Q);
+}
+
+// The neighbours of the moved hubs above MARK_INLINE arcs, each hub cut into
+// MARK_PARTS for as many warps (before the next vertices are collected).
+constexpr int MARK_PARTS = 32;
+__global__ void k_mark_hubs(Args A) {
+  int64_t parts = (int64_t)A.sub->big_movers * MARK_PARTS;
   for (int64_t t = ld_gtid() >> 5; t < parts; t += ld_gstride() >> 5) {  // warp-uniform
     int32_t i = A.big_movers[t / MARK_PARTS];
     int64_t dg = A.deg[i], len = (dg + MARK_PARTS - 1) / MARK_PARTS, a = (t % MARK_PARTS) * len;
@@ -966,61 +1025,73 @@ __global__ void k_sizes(const int32_t *C, int64_t n, int32_t *size) {
 }
 
 // ---- refinement
-// Reset the vertices of refined bounds to singletons and list them.
-__global__ void k_refine_reset(int64_t n, const int32_t *CB, const uint8_t *dR, int32_t *C, int64_t *S,
-                               const int64_t *K, int32_t *prop, int32_t *cand, DevCounters *cnt, const int32_t *gid,
-                               uint8_t *refg) {
-  int lane = threadIdx.x & 31;
-  for (int64_t base = (ld_gtid() & ~31ll); base < n; base += ld_gstride()) {
-    int64_t i = base + lane;
-    bool r = i < n && dR[CB[i]];
-    if (i < n) prop[i] = r ? 0 : -1;
-    if (r) { C[i] = (int32_t)i; S[i] = K[i]; }
-    if (r && gid) refg[gid[i]] = 1;  // the graph has a vertex in a refined bound
-    uint32_t m = __ballot_sync(LD_FULL, r);
-    if (!m) continue;
-    int32_t p0 = 0;
-    if (lane == 0) p0 = atomicAdd(&cnt->cand_count[0], __popc(m));
-    p0 = __shfl_sync(LD_FULL, p0, 0);
-    if (r) cand[p0 + __popc(m & ((1u << lane) - 1u))] = (int32_t)i;
+// The bounds C'_B = C', and the vertices of refined bounds reset to singletons
+// and listed.
+__global__ void __launch_bounds__(256) k_refine_reset(int64_t n, int32_t *CB, const uint8_t *dR, int32_t *C, int64_t *S,
+                                                      const int64_t *K, int32_t *prop, int32_t *cand, DevCounters *cnt,
+                                                      const int32_t *gid, uint8_t *refg) {
+  __shared__ BlockAppend<1> B;
+  int32_t *const lengths[1] = {&cnt->cand_count[0]};
+  for (int64_t b0 = (int64_t)blockIdx.x * APPEND_STEP; b0 < n; b0 += (int64_t)gridDim.x * APPEND_STEP) {
+    uint32_t cats[APPEND_UNROLL];
+    int32_t at[APPEND_UNROLL][1];
+#pragma unroll
+    for (int u = 0; u < APPEND_UNROLL; u++) {
+      int64_t i = b0 + 256 * u + threadIdx.x;
+      cats[u] = 0;
+      if (i >= n) continue;
+      int32_t c = C[i];
+      bool r = dR[c];
+      CB[i] = c;
+      prop[i] = r ? 0 : -1;
+      if (r) { C[i] = (int32_t)i; S[i] = K[i]; }
+      if (r && gid) refg[gid[i]] = 1;  // the graph has a vertex in a refined bound
+      cats[u] = r;
+    }
+    block_append<1>(B, cats, lengths, at);
+#pragma unroll
+    for (int u = 0; u < APPEND_UNROLL; u++)
+      if (cats[u]) cand[at[u][0]] = (int32_t)(b0 + 256 * u + threadIdx.x);
   }
 }
 
 // Keep the candidates that are still alone in their community and bin them
 // by degree; reset their proposals.
-__global__ void k_refine_collect(const int32_t *cand_in, const int32_t *count_in, int32_t *cand_out,
-                                 int32_t *count_out, int64_t n, const int32_t *C, const int64_t *S, const int64_t *K,
-                                 const int32_t *deg, int32_t *prop, int32_t *bins, DevCounters *cnt, leiden_tuning tn) {
-  int lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(256) k_refine_collect(const int32_t *cand_in, const int32_t *count_in,
+                                                        int32_t *cand_out, int32_t *count_out, int64_t n,
+                                                        const int32_t *C, const int64_t *S, const int64_t *K,
+                                                        const int32_t *deg, int32_t *prop, int32_t *bins,
+                                                        SubCounters *sub, leiden_tuning tn) {
+  __shared__ BlockAppend<NBINS + 1> B;
+  int32_t *const lengths[NBINS + 1] = {&sub->bin_count[0], &sub->bin_count[1], &sub->bin_count[2], &sub->bin_count[3],
+                                       count_out};
   int64_t m = *count_in;
-  for (int64_t base = (ld_gtid() & ~31ll); base < m; base += ld_gstride()) {
-    int64_t t = base + lane;
-    int32_t i = t < m ? cand_in[t] : -1;
-    bool keep = false;
-    if (i >= 0) {
-      prop[i] = -1;
-      keep = S[C[i]] == K[i];
-    }
-    int bin = -1;
-    if (keep) {
-      int dg = deg[i];  // without arcs: no proposal (prop stays -1)
-      bin = dg == 0 ? -1 : dg <= tn.tiny_max ? BIN_TINY : dg <= tn.warp_max ? BIN_WARP : dg <= tn.block_max ? BIN_BLOCK : BIN_HUGE;
-    }
-    uint32_t km = __ballot_sync(LD_FULL, keep);
-    if (km) {
-      int32_t p0 = 0;
-      if (lane == __ffs(km) - 1) p0 = atomicAdd(count_out, __popc(km));
-      p0 = __shfl_sync(LD_FULL, p0, __ffs(km) - 1);
-      if (keep) cand_out[p0 + __popc(km & ((1u << lane) - 1u))] = i;
+  for (int64_t b0 = (int64_t)blockIdx.x * APPEND_STEP; b0 < m; b0 += (int64_t)gridDim.x * APPEND_STEP) {
+    uint32_t cats[APPEND_UNROLL];
+    int32_t at[APPEND_UNROLL][NBINS + 1], v[APPEND_UNROLL];
+#pragma unroll
+    for (int u = 0; u < APPEND_UNROLL; u++) {
+      int64_t t = b0 + 256 * u + threadIdx.x;
+      cats[u] = 0;
+      v[u] = t < m ? cand_in[t] : -1;
     }
 #pragma unroll
-    for (int b = 0; b < NBINS; b++) {
-      uint32_t mm = __ballot_sync(LD_FULL, bin == b);
-      if (!mm) continue;
-      int32_t q0 = 0;
-      if (lane == __ffs(mm) - 1) q0 = atomicAdd(&cnt->bin_count[b], __popc(mm));
-      q0 = __shfl_sync(LD_FULL, q0, __ffs(mm) - 1);
-      if (bin == b) bins[(int64_t)b * n + q0 + __popc(mm & ((1u << lane) - 1u))] = i;
+    for (int u = 0; u < APPEND_UNROLL; u++) {
+      int32_t i = v[u];
+      if (i < 0) continue;
+      prop[i] = -1;
+      if (S[C[i]] != K[i]) continue;
+      int dg = deg[i];  // without arcs: no proposal (prop stays -1)
+      cats[u] = (1u << NBINS) | (dg ? 1u << bin_of(dg, tn) : 0u);
+    }
+    block_append<NBINS + 1>(B, cats, lengths, at);
+#pragma unroll
+    for (int u = 0; u < APPEND_UNROLL; u++) {
+      if (!cats[u]) continue;
+      cand_out[at[u][NBINS]] = v[u];
+#pragma unroll
+      for (int b = 0; b < NBINS; b++)
+        if (cats[u] >> b & 1) bins[(int64_t)b * n + at[u][b]] = v[u];
     }
   }
 }
@@ -1070,7 +1141,7 @@ Args make_args(leiden_handle *h, const LevelGraph &g) {
   A.w = g.w;
   A.C = h->Cp;
   A.S = h->Sp;
-  A.K = h->Kp;
+  A.K = h->Kc;
   A.size = h->csize;
   A.CB = h->CB;
   A.prop = h->prop;
@@ -1080,11 +1151,13 @@ Args make_args(leiden_handle *h, const LevelGraph &g) {
   A.mtarget = h->mtarget;
   A.big_movers = h->ibuf2;
   A.cnt = h->dcnt;
+  A.sub = &h->dcnt->ref;
   A.m2 = h->m2;
   if (g.gid) {
     A.gid = g.gid;
     A.m2g = h->gc.m2;
     A.mgain = h->mgain;
+    A.lm_on = h->gc.lm_on;
     A.accg = h->gc.accepted;
     A.refg = h->gc.refined;
   }
@@ -1143,11 +1216,11 @@ void launch_bins_of(leiden_handle *h, const LevelGraph &g, Args A) {
   }
   auto bin = [&](int b) {
     A.list = h->bins + (int64_t)b * g.n;
-    A.count = &h->dcnt->bin_count[b];
+    A.count = &A.sub->bin_count[b];
   };
   {
     A.list_tiny = h->bins + (int64_t)BIN_TINY * g.n;
-    A.count_tiny = &h->dcnt->bin_count[BIN_TINY];
+    A.count_tiny = &A.sub->bin_count[BIN_TINY];
     bin(BIN_WARP);
     int grid = sms * h->tune.warp_blocks_per_sm;  // default 4: one wave at four resident blocks per SM
     if (KIND == KIND_MOVE) kt_begin(h, KT_WARP);
@@ -1254,41 +1327,54 @@ int32_t *hs_keys(leiden_handle *h) { return (int32_t *)h->hscratch; }
 int64_t *hs_vals(leiden_handle *h) { return (int64_t *)((char *)h->hscratch + (size_t)h->hslots * 4); }
 int32_t *hs_list(leiden_handle *h) { return (int32_t *)((char *)h->hscratch + (size_t)h->hslots * 12); }
 
-void lm_prepare(leiden_handle *h, const LevelGraph &g, int sizes_from) {
-  if (sizes_from == SIZES_ONES) {  // C' is the identity: every community is one vertex
-    launch_fill_i32(h->csize, 1, g.n, h->stream);
-  } else if (sizes_from == SIZES_KEPT) {  // C' = C^{t-1}: sizes kept by the last tracking
-    cudaMemcpyAsync(h->csize, h->csize0, (size_t)g.n * sizeof(int32_t), cudaMemcpyDeviceToDevice, h->stream);
-  } else {
-    cudaMemsetAsync(h->csize, 0, (size_t)g.n * sizeof(int32_t), h->stream);
-    ld_note_launch(), k_sizes<<<grid_for(g.n, 256), 256, 0, h->stream>>>(h->Cp, g.n, h->csize);
-  }
-}
-
 void count_sizes(leiden_handle *h, const int32_t *C, int64_t n, int32_t *size) {
   cudaMemsetAsync(size, 0, (size_t)n * sizeof(int32_t), h->stream);
   ld_note_launch(), k_sizes<<<grid_for(n, 256), 256, 0, h->stream>>>(C, n, size);
 }
 
-void lm_subsweep(leiden_handle *h, const LevelGraph &g, int cls, const uint8_t *in_range, int dynamic) {
+void lm_iteration(leiden_handle *h, const LevelGraph &g, const uint8_t *in_range, int dynamic, bool dense) {
   cudaStream_t s = h->stream;
-  cudaMemsetAsync(&h->dcnt->bin_count[0], 0, sizeof(int32_t) * 6, s);  // bins, movers, big movers
-  ld_note_launch(), k_collect<<<grid_for((g.n + 31) / 32, 256), 256, 0, s>>>(
-      g.n, h->unproc, cls, lm_classes(h) - 1, in_range, g.deg, h->bins, h->dcnt, g.gid, h->gc.lm_on, h->d_loff,
-      h->tune);
+  const int classes = lm_classes(h);
+  const bool deferred = h->p.deterministic;
   Args A = make_args(h, g);
   A.in_range = in_range;
   A.dynamic = dynamic;
-  launch_bins<KIND_MOVE>(h, g, A);
-  if (h->p.deterministic)
-    ld_note_launch(), k_apply_moves<<<h->sm_count * 4, 256, 0, s>>>(A, h->gc.dq, h->gc.moves);
+  CollectArgs Q{0, h->bins, nullptr, h->d_loff, h->tune};
+  auto kernel = dense ? k_apply_collect<true> : k_apply_collect<false>;
+  const int grid = grid_for((g.n + 31) / 32, dense ? 32 : 256);  // bitmap words per block
+  bool pending = false;  // the moves of the class before wait to be applied
+  cudaMemsetAsync(h->dcnt->dq, 0, offsetof(DevCounters, ref), s);
+  for (int cls = 0; cls < classes; cls++) {
+    Q.cls = cls;
+    Q.sub = &h->dcnt->sub[cls % SUB_RING];
+    if (cls && cls % SUB_RING == 0) {  // the sets are used again
+      if (pending) {
+        CollectArgs none = Q;
+        none.cls = -1;
+        ld_note_launch(), kernel<<<grid, 256, 0, s>>>(A, true, h->gc.dq, h->gc.moves, none);
+        pending = false;
+      }
+      cudaMemsetAsync(h->dcnt->sub, 0, sizeof(h->dcnt->sub), s);
+    }
+    ld_note_launch(), kernel<<<grid, 256, 0, s>>>(A, pending, h->gc.dq, h->gc.moves, Q);
+    A.sub = Q.sub;
+    launch_bins<KIND_MOVE>(h, g, A);
+    if (deferred && g.maxdeg > h->tune.block_max && g.maxdeg > MARK_INLINE)
+      ld_note_launch(), k_mark_hubs<<<h->sm_count * 4, 256, 0, s>>>(A);
+    pending = deferred;
+  }
+  if (pending) {
+    Q.cls = -1;
+    ld_note_launch(), kernel<<<h->sm_count * 4, 256, 0, s>>>(A, true, h->gc.dq, h->gc.moves, Q);
+  }
 }
 
 void refine_reset(leiden_handle *h, const LevelGraph &g) {
   cudaStream_t s = h->stream;
   cudaMemsetAsync(&h->dcnt->cand_count[0], 0, sizeof(int32_t), s);
-  ld_note_launch(), k_refine_reset<<<grid_for(g.n, 256), 256, 0, s>>>(g.n, h->CB, h->dR, h->Cp, h->Sp, h->Kp, h->prop, h->cand,
-                                                    h->dcnt, g.gid, h->gc.refined);
+  ld_note_launch(), k_refine_reset<<<grid_for(g.n, APPEND_STEP), 256, 0, s>>>(g.n, h->CB, h->dR2, h->Cp, h->Sp, h->Kc,
+                                                                              h->prop, h->cand, h->dcnt, g.gid,
+                                                                              h->gc.refined);
 }
 
 // One round on the candidates of list `slot` (cand + slot*n, count
@@ -1297,14 +1383,15 @@ void refine_round(leiden_handle *h, const LevelGraph &g, int slot) {
   cudaStream_t s = h->stream;
   int32_t *in = h->cand + (int64_t)slot * g.n, *out = h->cand + (int64_t)(1 - slot) * g.n;
   int32_t *cin = &h->dcnt->cand_count[slot], *cout = &h->dcnt->cand_count[1 - slot];
-  cudaMemsetAsync(&h->dcnt->bin_count[0], 0, sizeof(int32_t) * 4, s);
+  static_assert(offsetof(DevCounters, accepted) == offsetof(DevCounters, ref) + sizeof(SubCounters), "cleared together");
+  cudaMemsetAsync(&h->dcnt->ref, 0, sizeof(SubCounters) + sizeof(int32_t), s);  // bins, accepted
   cudaMemsetAsync(cout, 0, sizeof(int32_t), s);
-  cudaMemsetAsync(&h->dcnt->accepted, 0, sizeof(int32_t), s);
-  ld_note_launch(), k_refine_collect<<<grid_for(g.n, 256), 256, 0, s>>>(in, cin, out, cout, g.n, h->Cp, h->Sp, h->Kp, g.deg, h->prop,
-                                                      h->bins, h->dcnt, h->tune);
+  ld_note_launch(), k_refine_collect<<<grid_for(g.n, APPEND_STEP), 256, 0, s>>>(in, cin, out, cout, g.n, h->Cp, h->Sp,
+                                                                                h->Kc, g.deg, h->prop, h->bins,
+                                                                                &h->dcnt->ref, h->tune);
   Args A = make_args(h, g);
   launch_bins<KIND_REFINE>(h, g, A);
-  ld_note_launch(), k_refine_accept<<<h->sm_count * 4, 256, 0, s>>>(out, cout, h->prop, h->Cp, h->Sp, h->Kp, h->dcnt,
+  ld_note_launch(), k_refine_accept<<<h->sm_count * 4, 256, 0, s>>>(out, cout, h->prop, h->Cp, h->Sp, h->Kc, h->dcnt,
                                                                      g.gid, h->gc.accepted);
 }
 

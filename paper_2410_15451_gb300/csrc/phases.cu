@@ -4,6 +4,7 @@
 // "leidenag").
 #include <algorithm>
 #include <climits>
+#include <cstddef>
 
 #include "internal.h"
 
@@ -12,54 +13,57 @@ namespace {
 constexpr int TB = 256;
 
 // ---------------------------------------------------------------- Alg. leidensr
-__global__ void k_sr_init(int64_t n, int32_t *rep, int64_t *S2, uint8_t *dS2, uint8_t *dR2) {
-  for (int64_t c = ld_gtid(); c < n; c += ld_gstride()) { rep[c] = INT_MAX; S2[c] = 0; dS2[c] = 0; dR2[c] = 0; }
-}
-// rep[c] = smallest member; a vertex only competes while it is below the
-// value already there (a plain read first spares most atomics).
+// rep[c] = smallest member (cleared at the start of the level); a vertex only
+// competes while it is below the value already there (a plain read first
+// spares most atomics).
 __global__ void k_sr_min(int64_t n, const int32_t *C, int32_t *rep) {
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) {
     int32_t c = C[i];
     if ((int32_t)i < rep[c]) atomicMin(&rep[c], (int32_t)i);
   }
 }
-__global__ void k_sr_rekey(int64_t n, const int32_t *rep, const int64_t *S, const uint8_t *dS, const uint8_t *dR,
-                           int64_t *S2, uint8_t *dS2, uint8_t *dR2) {
-  for (int64_t c = ld_gtid(); c < n; c += ld_gstride()) {
-    int32_t r = rep[c];
-    if (r == INT_MAX) continue;
-    S2[r] = S[c]; dS2[r] = dS[c]; dR2[r] = dR[c];
-  }
-}
-__global__ void k_sr_remap(int64_t n, const int32_t *rep, int32_t *C) {
-  for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) C[i] = rep[C[i]];
-}
-
-// ---------------------------------------------------------------- Alg. leidensp
-// Components of the flagged communities by lock-free union-find: a root is
-// only ever hooked under a smaller root, so every component ends with its
-// smallest vertex as root -- the label a BFS from the lowest vertex gives.
-__global__ void k_split_init(int64_t n, const int32_t *C, const uint8_t *dS, const uint8_t *dR, const int32_t *deg,
-                             int32_t *parent, int32_t *list, DevCounters *cnt, int split_all) {
-  int lane = threadIdx.x & 31;
+// C' in smallest members; the refinement flag moves with the id (the smallest
+// member writes it; Sigma' is not carried over, because only singletons of
+// refined bounds are read after this point and their Sigma' is set by the
+// reset); and the vertices of the communities to split are listed, each its
+// own component (Alg. leidensp): components by lock-free union-find, where a
+// root is only ever hooked under a smaller root, so every component ends with
+// its smallest vertex as root -- the label a BFS from the lowest vertex gives.
+// One sweep in place of four with one atomic per warp on the list's length
+// (R-MAT 22: 190 -> 59 us with the search for the smallest members).
+__global__ void __launch_bounds__(256) k_remap_list(int64_t n, const int32_t *rep, const uint8_t *dS,
+                                                    const uint8_t *dR, const int32_t *deg, int32_t *C, uint8_t *dR2,
+                                                    int32_t *parent, int32_t *list, DevCounters *cnt, int split_all) {
+  __shared__ BlockAppend<1> B;
+  int32_t *const lengths[1] = {&cnt->split_count};
   int64_t arcs = 0;  // arcs of the listed vertices (work counter)
-  for (int64_t base = (ld_gtid() & ~31ll); base < n; base += ld_gstride()) {
-    int64_t i = base + lane;
-    bool f = false;
-    if (i < n) {
-      int32_t c = C[i];
-      f = (split_all || dS[c]) && !dR[c];
-      if (f) { parent[i] = (int32_t)i; arcs += deg[i]; }
+  for (int64_t b0 = (int64_t)blockIdx.x * APPEND_STEP; b0 < n; b0 += (int64_t)gridDim.x * APPEND_STEP) {
+    uint32_t cats[APPEND_UNROLL];
+    int32_t at[APPEND_UNROLL][1], c[APPEND_UNROLL], r[APPEND_UNROLL];
+#pragma unroll
+    for (int u = 0; u < APPEND_UNROLL; u++) {
+      int64_t i = b0 + 256 * u + threadIdx.x;
+      c[u] = i < n ? C[i] : -1;
     }
-    uint32_t m = __ballot_sync(LD_FULL, f);
-    if (!m) continue;
-    int32_t p0 = 0;
-    if (lane == 0) p0 = atomicAdd(&cnt->split_count, __popc(m));
-    p0 = __shfl_sync(LD_FULL, p0, 0);
-    if (f) list[p0 + __popc(m & ((1u << lane) - 1u))] = (int32_t)i;
+#pragma unroll
+    for (int u = 0; u < APPEND_UNROLL; u++) {
+      int64_t i = b0 + 256 * u + threadIdx.x;
+      cats[u] = 0;
+      if (c[u] < 0) continue;
+      r[u] = rep[c[u]];
+      uint8_t ref = dR[c[u]];
+      cats[u] = (split_all || dS[c[u]]) && !ref;
+      C[i] = r[u];
+      dR2[i] = r[u] == (int32_t)i ? ref : 0;
+      if (cats[u]) { parent[i] = (int32_t)i; arcs += deg[i]; }
+    }
+    block_append<1>(B, cats, lengths, at);
+#pragma unroll
+    for (int u = 0; u < APPEND_UNROLL; u++)
+      if (cats[u]) list[at[u][0]] = (int32_t)(b0 + 256 * u + threadIdx.x);
   }
   arcs = ld_warp_sum_i64(arcs);
-  if (lane == 0 && arcs) atomicAdd((unsigned long long *)&cnt->split_arcs, (unsigned long long)arcs);
+  if ((threadIdx.x & 31) == 0 && arcs) atomicAdd((unsigned long long *)&cnt->split_arcs, (unsigned long long)arcs);
 }
 
 __device__ __forceinline__ int32_t uf_find(int32_t *parent, int32_t x) {
@@ -223,9 +227,11 @@ __global__ void k_rank(int64_t n, const int64_t *rank, int32_t *C, const int32_t
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride())
     C[i] = (int32_t)((!gid || cont[gid[i]]) ? rank[C[i]] : rank[n]);
 }
-__global__ void k_lookup(int64_t N, const int32_t *Cp, int32_t *Ctop, const int32_t *gid0, const uint8_t *cont) {
+// (first: Ctop is the identity, which is not written out)
+__global__ void k_lookup(int64_t N, const int32_t *Cp, int32_t *Ctop, const int32_t *gid0, const uint8_t *cont,
+                         bool first) {
   for (int64_t v = ld_gtid(); v < N; v += ld_gstride())
-    if (!gid0 || cont[gid0[v]]) Ctop[v] = Cp[Ctop[v]];
+    if (!gid0 || cont[gid0[v]]) Ctop[v] = Cp[first ? v : Ctop[v]];
 }
 // Final lookup of the graphs that stop at this pass, with the community id
 // moved from the level's range of the graph into its own vertex range (the
@@ -233,10 +239,10 @@ __global__ void k_lookup(int64_t N, const int32_t *Cp, int32_t *Ctop, const int3
 // communities are the level's roots (C'[c] == c).
 __global__ void k_break_lookup(int64_t N, const int32_t *Cp, int32_t *Ctop, const int32_t *gid0, const uint8_t *cont,
                                const int64_t *loff, const int64_t *voff, int64_t n, const int32_t *gid,
-                               uint8_t *used) {
+                               uint8_t *used, bool first) {
   for (int64_t v = ld_gtid(); v < N; v += ld_gstride()) {
     int32_t g = gid0[v];
-    if (loff[g + 1] > loff[g] && !cont[g]) Ctop[v] = (int32_t)(Cp[Ctop[v]] - loff[g] + voff[g]);
+    if (loff[g + 1] > loff[g] && !cont[g]) Ctop[v] = (int32_t)(Cp[first ? v : Ctop[v]] - loff[g] + voff[g]);
     if (v < n) {
       g = gid[v];
       if (loff[g + 1] > loff[g] && !cont[g] && Cp[v] == (int32_t)v) used[v - loff[g] + voff[g]] = 1;
@@ -881,7 +887,7 @@ __global__ void k_agg_bin(int64_t ncomm, const int64_t *yoff, const int64_t *cof
       uint32_t m = __ballot_sync(LD_FULL, bin == b);
       if (!m) continue;
       int32_t p0 = 0;
-      if (lane == __ffs(m) - 1) p0 = atomicAdd(&cnt->bin_count[b], __popc(m));
+      if (lane == __ffs(m) - 1) p0 = atomicAdd(&cnt->ref.bin_count[b], __popc(m));
       p0 = __shfl_sync(LD_FULL, p0, __ffs(m) - 1);
       if (bin == b) bins[(int64_t)b * ncomm + p0 + __popc(m & ((1u << lane) - 1u))] = (int32_t)c;
     }
@@ -889,26 +895,25 @@ __global__ void k_agg_bin(int64_t ncomm, const int64_t *yoff, const int64_t *cof
 }
 
 // ---------------------------------------------------------------- pass reset
+// The state of the next level, every super-vertex on its own and unprocessed.
 __global__ void k_next_pass(int64_t nc, const int64_t *Kout, int64_t *Kp, int64_t *Sp, int32_t *Cp, uint8_t *dR,
-                            uint8_t *dS) {
+                            uint8_t *dS, int32_t *size, int32_t *rep, uint32_t *bm) {
   for (int64_t c = ld_gtid(); c < nc; c += ld_gstride()) {
     Kp[c] = Kout[c]; Sp[c] = Kout[c]; Cp[c] = (int32_t)c; dR[c] = 1; dS[c] = 0;
-  }
-}
-__global__ void k_bits_all(int64_t n, uint32_t *bm) {
-  int64_t words = (n + 31) >> 5;
-  for (int64_t w = ld_gtid(); w < words; w += ld_gstride()) {
-    int64_t rem = n - (w << 5);
-    bm[w] = rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u);
+    size[c] = 1;
+    rep[c] = INT_MAX;
+    if ((c & 31) == 0) bm[c >> 5] = nc - c >= 32 ? 0xffffffffu : (1u << (nc - c)) - 1u;
   }
 }
 // Start of the pass loop in one sweep: the affected flags become the
-// frontier bitmap (and are counted), Ctop = identity, C' = C, K' = K,
-// Sigma' = Sigma.  Four vertices per thread with 16-byte loads and stores
-// (the arrays start 256-byte aligned); eight lanes make one bitmap word.
-// A tail of n % 32 vertices is done one per lane by the first warp.
-__global__ void k_pass_init(int64_t n, const uint8_t *dV, uint32_t *bm, int32_t *Ctop, const int32_t *C, int32_t *Cp,
-                            const int64_t *K, int64_t *Kp, const int64_t *Sig, int64_t *Sp, DevCounters *cnt) {
+// frontier bitmap (and are counted), C' = C, Sigma' = Sigma, sizes from the
+// kept ones (null: all 1), smallest members cleared.  Four vertices per
+// thread with 16-byte loads and stores (the arrays start 256-byte aligned);
+// eight lanes make one bitmap word.  A tail of n % 32 vertices is done one per
+// lane by the first warp.
+__global__ void k_pass_init(int64_t n, const uint8_t *dV, uint32_t *bm, const int32_t *C, int32_t *Cp,
+                            const int64_t *Sig, int64_t *Sp, const int32_t *size0, int32_t *size, int32_t *rep,
+                            DevCounters *cnt) {
   int lane = threadIdx.x & 31;
   int64_t set = 0;
   int64_t nq = (n >> 5) << 3;  // quads of whole 32-vertex words
@@ -916,15 +921,13 @@ __global__ void k_pass_init(int64_t n, const uint8_t *dV, uint32_t *bm, int32_t 
     int64_t q = q0 + lane;
     uint32_t nib = 0;
     if (q < nq) {
-      int64_t v = q << 2;
       uint32_t f = ((const uint32_t *)dV)[q];
       nib = (f & 0xffu ? 1u : 0u) | (f & 0xff00u ? 2u : 0u) | (f & 0xff0000u ? 4u : 0u) | (f & 0xff000000u ? 8u : 0u);
-      ((int4 *)Ctop)[q] = make_int4((int)v, (int)v + 1, (int)v + 2, (int)v + 3);
       ((int4 *)Cp)[q] = ((const int4 *)C)[q];
-      ((longlong2 *)Kp)[2 * q] = ((const longlong2 *)K)[2 * q];
-      ((longlong2 *)Kp)[2 * q + 1] = ((const longlong2 *)K)[2 * q + 1];
       ((longlong2 *)Sp)[2 * q] = ((const longlong2 *)Sig)[2 * q];
       ((longlong2 *)Sp)[2 * q + 1] = ((const longlong2 *)Sig)[2 * q + 1];
+      ((int4 *)size)[q] = size0 ? ((const int4 *)size0)[q] : make_int4(1, 1, 1, 1);
+      ((int4 *)rep)[q] = make_int4(INT_MAX, INT_MAX, INT_MAX, INT_MAX);
     }
     uint32_t word = nib << ((lane & 7) * 4);  // lanes 8k..8k+7 hold word q/8
 #pragma unroll
@@ -939,10 +942,10 @@ __global__ void k_pass_init(int64_t n, const uint8_t *dV, uint32_t *bm, int32_t 
     bool in = v < n;
     uint32_t m = __ballot_sync(LD_FULL, in && dV[v]);
     if (in) {
-      Ctop[v] = (int32_t)v;
       Cp[v] = C[v];
-      Kp[v] = K[v];
       Sp[v] = Sig[v];
+      size[v] = size0 ? size0[v] : 1;
+      rep[v] = INT_MAX;
     }
     if (lane == 0 && (nq << 2) < n) {
       bm[nq >> 3] = m;
@@ -981,32 +984,24 @@ __global__ void k_maxdeg(int64_t n, const int32_t *deg, DevCounters *cnt, int bl
 
 }  // namespace
 
-void subset_renumber(leiden_handle *h, int64_t n) {
+void renumber_and_split(leiden_handle *h, const LevelGraph &g) {
   cudaStream_t s = h->stream;
-  int g = grid_for(n, TB);
-  ld_note_launch(), k_sr_init<<<g, TB, 0, s>>>(n, h->rep, h->S2, h->dS2, h->dR2);
-  ld_note_launch(), k_sr_min<<<g, TB, 0, s>>>(n, h->Cp, h->rep);
-  ld_note_launch(), k_sr_rekey<<<g, TB, 0, s>>>(n, h->rep, h->Sp, h->dS, h->dR, h->S2, h->dS2, h->dR2);
-  ld_note_launch(), k_sr_remap<<<g, TB, 0, s>>>(n, h->rep, h->Cp);
-  std::swap(h->Sp, h->S2);
-  std::swap(h->dS, h->dS2);
-  std::swap(h->dR, h->dR2);
-}
-
-void split_communities(leiden_handle *h, const LevelGraph &g) {
-  cudaStream_t s = h->stream;
-  cudaMemsetAsync(&h->dcnt->split_count, 0, sizeof(int32_t), s);
-  cudaMemsetAsync(&h->dcnt->split_arcs, 0, sizeof(int64_t), s);
+  static_assert(offsetof(DevCounters, split_arcs) + sizeof(int64_t) == offsetof(DevCounters, split_count) &&
+                    offsetof(DevCounters, split_count) + sizeof(int32_t) == offsetof(DevCounters, big_count),
+                "cleared together");
+  cudaMemsetAsync(&h->dcnt->split_arcs, 0, sizeof(int64_t) + 2 * sizeof(int32_t), s);
   int32_t *list = h->ibuf1;
-  ld_note_launch(), k_split_init<<<grid_for(g.n, TB), TB, 0, s>>>(g.n, h->Cp, h->dS, h->dR, g.deg, h->parent, list,
-                                                                  h->dcnt, h->p.split_all);
+  ld_note_launch(), k_sr_min<<<grid_for(g.n, TB), TB, 0, s>>>(g.n, h->Cp, h->rep);
+  ld_note_launch(), k_remap_list<<<grid_for(g.n, APPEND_STEP), 256, 0, s>>>(g.n, h->rep, h->dS, h->dR, g.deg, h->Cp,
+                                                                            h->dR2, h->parent, list, h->dcnt,
+                                                                            h->p.split_all);
   kt_begin(h, KT_SPLIT_SAMPLE);
   ld_note_launch(), k_split_sample<<<h->sm_count * 16, TB, 0, s>>>(list, h->dcnt, g.off, g.deg, g.col, h->Cp, h->parent);
   kt_end(h);
   ld_note_launch(), k_split_flatten<<<h->sm_count * 8, TB, 0, s>>>(list, h->dcnt, h->parent);
-  cudaMemsetAsync(&h->dcnt->big_count, 0, sizeof(int32_t), s);
   ld_note_launch(), k_split_link_rest<<<h->sm_count * 8, TB, 0, s>>>(list, h->dcnt, g.off, g.deg, g.col, h->Cp, h->parent, h->ibuf2);
-  ld_note_launch(), k_split_link_big<<<h->sm_count, 1024, 0, s>>>(h->ibuf2, h->dcnt, g.off, g.deg, g.col, h->Cp, h->parent);
+  if (g.maxdeg > SPLIT_BIG)
+    ld_note_launch(), k_split_link_big<<<h->sm_count, 1024, 0, s>>>(h->ibuf2, h->dcnt, g.off, g.deg, g.col, h->Cp, h->parent);
   ld_note_launch(), k_split_compress<<<h->sm_count * 8, TB, 0, s>>>(list, h->dcnt, h->parent, h->Cp);
 }
 
@@ -1025,15 +1020,15 @@ void renumber_dense(leiden_handle *h, int64_t n, const int32_t *gid) {
   ld_note_launch(), k_rank<<<grid_for(n, TB), TB, 0, s>>>(n, h->lbuf0, h->Cp, gid, cont);
 }
 
-void lookup_dendrogram(leiden_handle *h) {
+void lookup_dendrogram(leiden_handle *h, bool first) {
   const uint8_t *cont = h->gid0 ? h->gc.cont : nullptr;
-  ld_note_launch(), k_lookup<<<grid_for(h->n, TB), TB, 0, h->stream>>>(h->n, h->Cp, h->Ctop, h->gid0, cont);
+  ld_note_launch(), k_lookup<<<grid_for(h->n, TB), TB, 0, h->stream>>>(h->n, h->Cp, h->Ctop, h->gid0, cont, first);
 }
 
 void break_lookup(leiden_handle *h, int64_t n, const int32_t *gid, bool first) {
   if (first) cudaMemsetAsync(h->dE, 0, (size_t)h->n, h->stream);
   ld_note_launch(), k_break_lookup<<<grid_for(h->n, TB), TB, 0, h->stream>>>(
-      h->n, h->Cp, h->Ctop, h->gid0, h->gc.cont, h->d_loff, h->d_voff, n, gid, h->dE);
+      h->n, h->Cp, h->Ctop, h->gid0, h->gc.cont, h->d_loff, h->d_voff, n, gid, h->dE, first);
 }
 
 void next_level_ids(leiden_handle *h, int64_t n, const int32_t *gid, int32_t *gid_next, int64_t *loff_next) {
@@ -1061,7 +1056,7 @@ void aggregate(leiden_handle *h, const LevelGraph &g, int64_t ncomm, int out) {
   cudaMemsetAsync(&h->dcnt->max_count, 0, sizeof(int32_t), s);
   cudaMemsetAsync(&h->dcnt->huge_slots, 0, sizeof(int64_t), s);
   ld_note_launch(), k_yoff<<<grid_for(ncomm + 1, TB), TB, 0, s>>>(ncomm, h->coff, h->cflat, h->y_off[out], h->dcnt);
-  cudaMemsetAsync(&h->dcnt->bin_count[0], 0, sizeof(int32_t) * 4, s);
+  cudaMemsetAsync(&h->dcnt->ref, 0, sizeof(SubCounters), s);
   ld_note_launch(), k_agg_bin<<<grid_for(ncomm, TB), TB, 0, s>>>(ncomm, h->y_off[out], h->coff, h->bins, h->dcnt);
   cudaMemcpyAsync(&h->hcnt->max_count, &h->dcnt->max_count, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
   cudaMemcpyAsync(&h->hcnt->huge_slots, &h->dcnt->huge_slots, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
@@ -1084,16 +1079,16 @@ void aggregate(leiden_handle *h, const LevelGraph &g, int64_t ncomm, int out) {
   A.Kout = h->S2;
   int sms = h->sm_count;
   A.list = h->bins + (int64_t)BIN_TINY * ncomm;
-  A.count = &h->dcnt->bin_count[BIN_TINY];
+  A.count = &h->dcnt->ref.bin_count[BIN_TINY];
   if (g.w64) ld_note_launch(), k_agg_tiny<int64_t><<<sms * 8, 256, 0, s>>>(A);
   else ld_note_launch(), k_agg_tiny<int32_t><<<sms * 8, 256, 0, s>>>(A);
   A.list = h->bins;
-  A.count = &h->dcnt->bin_count[BIN_WARP];
+  A.count = &h->dcnt->ref.bin_count[BIN_WARP];
   if (g.w64) ld_note_launch(), k_agg_warp<int64_t><<<sms * 8, AGG_WARPS * 32, 0, s>>>(A);
   else ld_note_launch(), k_agg_warp<int32_t><<<sms * 8, AGG_WARPS * 32, 0, s>>>(A);
   if (maxc > BIN_WARP_MAX) {
     A.list = h->bins + ncomm;
-    A.count = &h->dcnt->bin_count[BIN_BLOCK];
+    A.count = &h->dcnt->ref.bin_count[BIN_BLOCK];
     if (g.w64) ld_note_launch(), k_agg_block<int64_t><<<sms * 4, 256, 0, s>>>(A);
     else ld_note_launch(), k_agg_block<int32_t><<<sms * 4, 256, 0, s>>>(A);
   }
@@ -1101,7 +1096,7 @@ void aggregate(leiden_handle *h, const LevelGraph &g, int64_t ncomm, int out) {
     // a table per listed community at once: at most huge_slots slots
     if (!ensure_hslots(h, h->hcnt->huge_slots)) { h->fatal = LEIDEN_ERR_OOM; h->err = "global table scratch"; return; }
     A.list = h->bins + 2 * ncomm;
-    A.count = &h->dcnt->bin_count[BIN_HUGE];
+    A.count = &h->dcnt->ref.bin_count[BIN_HUGE];
     A.gkeys = hs_keys(h);
     A.gvals = hs_vals(h);
     A.glist = hs_list(h);
@@ -1126,19 +1121,16 @@ void aggregate(leiden_handle *h, const LevelGraph &g, int64_t ncomm, int out) {
 
 void reset_next_pass(leiden_handle *h, int64_t ncomm, int out) {
   (void)out;
-  cudaStream_t s = h->stream;
-  ld_note_launch(), k_next_pass<<<grid_for(ncomm, TB), TB, 0, s>>>(ncomm, h->S2, h->Kp, h->Sp, h->Cp, h->dR, h->dS);
-  mark_all_unprocessed(h, ncomm);
+  ld_note_launch(), k_next_pass<<<grid_for(ncomm, TB), TB, 0, h->stream>>>(ncomm, h->S2, h->Kp, h->Sp, h->Cp, h->dR,
+                                                                           h->dS, h->csize, h->rep, h->unproc);
+  h->Kc = h->Kp;
 }
 
-void mark_all_unprocessed(leiden_handle *h, int64_t n) {
-  ld_note_launch(), k_bits_all<<<grid_for((n + 31) / 32, TB), TB, 0, h->stream>>>(n, h->unproc);
-}
-
-void pass_init(leiden_handle *h) {
+void pass_init(leiden_handle *h, bool sizes_kept) {
   cudaMemsetAsync(&h->dcnt->affected, 0, sizeof(int64_t), h->stream);
-  ld_note_launch(), k_pass_init<<<grid_for(h->n, TB), TB, 0, h->stream>>>(h->n, h->dV, h->unproc, h->Ctop, h->C, h->Cp,
-                                                                          h->K, h->Kp, h->Sig, h->Sp, h->dcnt);
+  ld_note_launch(), k_pass_init<<<grid_for(h->n, TB), TB, 0, h->stream>>>(
+      h->n, h->dV, h->unproc, h->C, h->Cp, h->Sig, h->Sp, sizes_kept ? h->csize0 : nullptr, h->csize, h->rep, h->dcnt);
+  h->Kc = h->K;
 }
 
 void level_maxdeg(leiden_handle *h, const int32_t *deg, int64_t n) {

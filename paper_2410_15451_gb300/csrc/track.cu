@@ -685,11 +685,10 @@ __global__ void __launch_bounds__(256) k_rowsum_big(const int32_t *big, const in
 // Scratch (each array used by nobody else between the last lookup and the
 // next call): 4-byte cand, dev, choice, flagged, rank, free ids; 8-byte match,
 // best.
-static void track_narrow(leiden_handle *h, const int32_t *root, int64_t nroot) {
+static void track_narrow(leiden_handle *h, const int32_t *Cnew, const int32_t *root, int64_t nroot) {
   cudaStream_t s = h->stream;
   int64_t N = h->n;
   int gN = grid_for(N, TB);
-  const int32_t *Cnew = h->Ctop;
   int32_t *cand = h->mtarget, *choice = h->movers, *flagged = h->prop, *rank = h->rep, *freel = h->parent;
   uint32_t *dev = (uint32_t *)h->ibuf0, *bits = h->unproc;
   unsigned long long *match = (unsigned long long *)h->lbuf0, *best = (unsigned long long *)h->lbuf1;
@@ -713,12 +712,12 @@ static void track_narrow(leiden_handle *h, const int32_t *root, int64_t nroot) {
                                                    h->dSig, h->gid0, granks);
 }
 
-// C^{t-1} = h->C, final top-level membership = h->Ctop  ->  h->C, h->Sig, h->dSig.
+// C^{t-1} = h->C, final top-level membership = Cnew  ->  h->C, h->Sig, h->dSig.
 // The new ids: the roots of the last level (c < nroot, root[c] == c); of a
 // batched handle the ids flagged in h->dE.
-void track_communities(leiden_handle *h, const int32_t *root, int64_t nroot) {
+void track_communities(leiden_handle *h, const int32_t *Cnew, const int32_t *root, int64_t nroot) {
   cudaMemsetAsync(&h->dcnt->list_count, 0, sizeof(int32_t), h->stream);
-  if (!wide_sums(h)) { track_narrow(h, root, nroot); return; }
+  if (!wide_sums(h)) { track_narrow(h, Cnew, root, nroot); return; }
   cudaStream_t s = h->stream;
   if (h->G == 1) count_communities(h, nroot, nullptr);
   int64_t N = h->n;
@@ -729,17 +728,17 @@ void track_communities(leiden_handle *h, const int32_t *root, int64_t nroot) {
   int64_t *dev = h->Sp;
   ld_note_launch(), k_tr_init<<<gN, TB, 0, s>>>(N, bw, bc, ow, ob, cand, used, dev);
   cudaMemsetAsync(&h->dcnt->tr_occ, 0, sizeof(int32_t), s);
-  ld_note_launch(), k_trc_cand<<<gN, TB, 0, s>>>(N, h->C, h->Ctop, cand);
-  ld_note_launch(), k_trc_deviants<<<gN, TB, 0, s>>>(N, h->C, h->Ctop, h->K, cand, dev);
+  ld_note_launch(), k_trc_cand<<<gN, TB, 0, s>>>(N, h->C, Cnew, cand);
+  ld_note_launch(), k_trc_deviants<<<gN, TB, 0, s>>>(N, h->C, Cnew, h->K, cand, dev);
   ld_note_launch(), k_trc_majority<<<gN, TB, 0, s>>>(N, cand, h->Sig, dev, bw, bc, flag);
   int32_t *occ = &h->dcnt->tr_occ;
-  ld_note_launch(), k_trc_insert<<<gN, TB, 0, s>>>(N, h->C, h->Ctop, h->K, flag, bc, h->tr_cap, h->tr_keys, h->tr_vals,
+  ld_note_launch(), k_trc_insert<<<gN, TB, 0, s>>>(N, h->C, Cnew, h->K, flag, bc, h->tr_cap, h->tr_keys, h->tr_vals,
                                                    h->tr_list, occ);
   ld_note_launch(), k_trc_best_w<<<h->sm_count * 8, TB, 0, s>>>(occ, h->tr_list, h->tr_keys, h->tr_vals, bw);
   ld_note_launch(), k_trc_best_c<<<h->sm_count * 8, TB, 0, s>>>(occ, h->tr_list, h->tr_keys, h->tr_vals, bw, bc);
   ld_note_launch(), k_tr_best_old_w<<<gN, TB, 0, s>>>(N, bc, bw, ow);
   ld_note_launch(), k_tr_best_old_b<<<gN, TB, 0, s>>>(N, bc, bw, ow, ob);
-  ld_note_launch(), k_tr_new_used<<<gN, TB, 0, s>>>(N, h->Ctop, used);
+  ld_note_launch(), k_tr_new_used<<<gN, TB, 0, s>>>(N, Cnew, used);
   int32_t *unmatched = h->rep, *freef = h->prop;
   ld_note_launch(), k_tr_flags<<<gN, TB, 0, s>>>(N, used, ob, bc, unmatched, freef);
   int64_t *urank = h->lbuf2, *frank = h->lbuf3;
@@ -750,7 +749,7 @@ void track_communities(leiden_handle *h, const int32_t *root, int64_t nroot) {
   uint8_t *matched = h->dE;
   cudaMemsetAsync(matched, 0, (size_t)N, s);
   ld_note_launch(), k_tr_map<<<gN, TB, 0, s>>>(N, used, ob, urank, frank, flist, map, matched, h->gid0, h->d_voff);
-  ld_note_launch(), k_tr_relabel<<<gN, TB, 0, s>>>(N, h->Ctop, map, h->K, h->C, h->Sig, h->csize0);
+  ld_note_launch(), k_tr_relabel<<<gN, TB, 0, s>>>(N, Cnew, map, h->K, h->C, h->Sig, h->csize0);
   ld_note_launch(), k_tr_dsig<<<gN, TB, 0, s>>>(N, matched, h->dSig);
 }
 
