@@ -1,6 +1,7 @@
 // C ABI of the GB300 dynamic Leiden library and the pass loop of Alg.
 // "leiden" (Appendix A.4) that drives the kernels.
 #include <algorithm>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <numeric>
@@ -147,8 +148,8 @@ void kt_end(leiden_handle *h, cudaStream_t s) {
 void kt_reset(leiden_handle *h) {
   h->kt_used = 0;
   for (int k = 0; k < KT_KERNELS; k++) { h->kt_ms[k] = 0; h->kt_launches[k] = 0; }
-  cudaMemsetAsync(h->dcnt->xk_bytes, 0, sizeof(h->dcnt->xk_bytes), h->stream);
-  cudaMemsetAsync(h->dcnt->agg_tables, 0, sizeof(h->dcnt->agg_tables), h->stream);
+  // the call's counters
+  cudaMemsetAsync(&h->dcnt->error, 0, offsetof(DevCounters, m2) - offsetof(DevCounters, error), h->stream);
 }
 
 void kt_resolve(leiden_handle *h) {
@@ -282,7 +283,6 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range,
   ph_mark(h, LEIDEN_PHASE_MOVE);
   ph_bytes(h, LEIDEN_PHASE_MOVE, 37 * N + N / 8);  // dV -> frontier bits; copies of C', Sigma', sizes; smallest members
   pass_init(h, dynamic != 0);
-  CK(cudaMemsetAsync(&h->dcnt->processed, 0, 13 * sizeof(int64_t), s));  // processed .. lmk_bytes
   int64_t m2 = h->m2;
   LevelGraph g = level0(h);
   double tau = p.tau;
@@ -327,6 +327,8 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range,
       CKF();
       i128 dq = read_i128(h->hcnt->dq);
       int64_t mv = h->hcnt->moves;
+      if (B && lp == 0 && it == 0)
+        for (int gi = 0; gi < G; gi++) h->m2g[gi] = hg.m2[gi];
       if (it < 20) tr[5 + it] = mv;
       moves_total += mv;
       st.lm_iterations++;
@@ -581,21 +583,7 @@ leiden_status do_update(leiden_handle *h, const leiden_edge *d_del, int64_t n_de
     release_agg_buffers(h);
     return st;
   }
-  ph_bytes(h, LEIDEN_PHASE_BATCH, 4 * h->n);  // degrees scanned for the bins
-  level_maxdeg(h, h->g_deg, h->n);
-  sync_all(h);
-  if (cudaError_t e = cudaGetLastError()) {
-    h->err = std::string("after the batch: ") + cudaGetErrorString(e);
-    h->broken = true;
-    return LEIDEN_ERR_CUDA;
-  }
-  h->m2 = h->hcnt->m2;
-  if (h->G > 1) {
-    GraphCounters hg = gc_layout(h->gc_host, h->G);
-    for (int gi = 0; gi < h->G; gi++) h->m2g[gi] = hg.m2[gi];
-  }
-  h->g_maxdeg = h->hcnt->max_count;
-  h->g_huge_slots = h->hcnt->huge_slots;
+  h->m2 += h->batch_dw;
   // a DF batch marks at most the two ends of each of its edges
   bool dense = mode != LEIDEN_DF || 16 * (n_del + n_ins) > h->n;
   st = run_leiden(h, 1, mode == LEIDEN_DS ? h->dV : nullptr, dense);
@@ -744,13 +732,18 @@ leiden_status leiden_create(const leiden_params *params, int64_t n, const int64_
   A(dalloc(h, &h->K, n));
   A(dalloc(h, &h->Sig, n));
   A(dalloc(h, &h->dSig, n));
-  A(dalloc(h, &h->dV, n));
+  {
+    int64_t na = (n + 256) & ~(int64_t)255;
+    A(dalloc(h, &h->dV, 3 * na));
+    h->dS = h->dV ? h->dV + na : nullptr;
+    h->dR = h->dV ? h->dV + 2 * na : nullptr;
+  }
   int32_t **i32s[] = {&h->Cp, &h->CB, &h->Ctop, &h->csize, &h->csize0, &h->rep, &h->prop, &h->parent,
                       &h->ibuf0, &h->ibuf1, &h->ibuf2, &h->movers, &h->mtarget, &h->cverts};
   for (auto pp : i32s) A(dalloc(h, pp, n + 1));
   int64_t **i64s[] = {&h->Kp, &h->Sp, &h->S2, &h->lbuf0, &h->lbuf1, &h->lbuf2, &h->lbuf3, &h->coff, &h->cflat};
   for (auto pp : i64s) A(dalloc(h, pp, n + 2));
-  uint8_t **u8s[] = {&h->dS, &h->dR, &h->dR2, &h->dE, &h->dCf};
+  uint8_t **u8s[] = {&h->dR2, &h->dE, &h->dCf};
   for (auto pp : u8s) A(dalloc(h, pp, n + 1));
   A(dalloc(h, &h->unproc, n / 32 + 2));
   A(dalloc(h, &h->bins, (int64_t)NBINS * n));
@@ -894,8 +887,8 @@ int64_t leiden_footprint_bytes(const leiden_params *params, int64_t n, const int
   int64_t hs = (level0_huge_slots(deg) + 1023) & ~(int64_t)1023;
   int64_t b = 0;
   b += 8 * (n + 1) + 8 * n + 8 * total;                              // G^t: off, deg, rcap, col, w
-  b += 4 * n + 24 * n + n;                                            // C, K, Sigma, dSigma, dV
-  b += 56 * (n + 1) + 72 * (n + 2) + 5 * (n + 1);                     // per-pass work arrays
+  b += 4 * n + 24 * n + 3 * (n + 256);                                // C, K, Sigma, dSigma, dV, dS, dR
+  b += 56 * (n + 1) + 72 * (n + 2) + 3 * (n + 1);                     // per-pass work arrays
   b += 4 * (n / 32 + 2) + 16 * n + 4 * (n + 1) + 8 * n;               // frontier, bins, hocc, cand
   b += 2 * (8 * (n + 2) + 4 * (n + 1));                              // aggregated levels' offsets, degrees
   b += 16 * tc + 4 * n + (int64_t)scan_tmp_bytes(2 * n + 2);          // tracking, scans

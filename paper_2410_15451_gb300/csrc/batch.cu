@@ -30,6 +30,13 @@ __device__ __forceinline__ int64_t lower_bound_u64(const uint64_t *a, int64_t n,
   return lo;
 }
 
+// Ids in range, no self-loop, a positive weight to insert, and (batched handles)
+// both ends in one graph.
+__device__ __forceinline__ bool valid_edge(const leiden_edge &x, bool del, int64_t n, const int32_t *gid0) {
+  if (x.u < 0 || x.u >= n || x.v < 0 || x.v >= n || x.u == x.v || (!del && x.w <= 0)) return false;
+  return !gid0 || gid0[x.u] == gid0[x.v];
+}
+
 // Mirror each undirected edge into two arcs keyed (src << vb) | dst and
 // validate it.  error := 1 on any violation.  Deletions and insertions go
 // into one array for one sort: the 2*n_del deletion arcs first (weight 0),
@@ -41,9 +48,7 @@ __global__ void k_expand(const leiden_edge *del, int64_t n_del, const leiden_edg
   for (int64_t e = ld_gtid(); e < n_del + n_ins; e += ld_gstride()) {
     bool is_del = e < n_del;
     leiden_edge x = is_del ? del[e] : ins[e - n_del];
-    bool bad = x.u < 0 || x.u >= n || x.v < 0 || x.v >= n || x.u == x.v || (!is_del && x.w <= 0);
-    if (!bad && gid0 && gid0[x.u] != gid0[x.v]) bad = true;  // batched: an edge between two graphs
-    if (bad) {
+    if (!valid_edge(x, is_del, n, gid0)) {
       atomicExch(&cnt->error, 1);
       x.u = 0; x.v = 1 % (int32_t)(n > 1 ? n : 1); x.w = 1;
     }
@@ -57,13 +62,13 @@ __global__ void k_expand(const leiden_edge *del, int64_t n_del, const leiden_edg
   }
 }
 
-// Clear the insertion tag of the sorted insertion arcs.
-__global__ void k_untag(uint64_t *key, int64_t n, uint64_t mask) {
-  for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) key[i] &= mask;
-}
-
-__global__ void k_head_flags(const uint64_t *key, int64_t n, int32_t *flag) {
-  for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) flag[i] = (i == 0 || key[i] != key[i - 1]) ? 1 : 0;
+// Heads of the runs of equal keys over both parts of the sorted batch (the
+// insertion tag keeps them apart); IW zeroed for the sums.
+__global__ void k_head_flags(const uint64_t *key, int64_t n, int32_t *flag, int64_t *zero, int64_t nzero) {
+  for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) {
+    flag[i] = (i == 0 || key[i] != key[i - 1]) ? 1 : 0;
+    if (i < nzero) zero[i] = 0;
+  }
 }
 
 // Unique keys (and summed payload) into out_key/out_w at the scanned positions.
@@ -76,50 +81,92 @@ __global__ void k_unique(const uint64_t *key, const int64_t *w, int64_t n, const
   }
 }
 
-// Deletions must name existing arcs; record the stored weight.
-__global__ void k_check_deletions(const uint64_t *dkey, const int64_t *nd_p, int vb, const int64_t *off,
-                                  const int32_t *deg, const int32_t *col, const int32_t *w, int64_t *dw,
-                                  DevCounters *cnt) {
-  uint64_t mask = (1ull << vb) - 1;
-  int64_t nd = *nd_p;
-  for (int64_t i = ld_gtid(); i < nd; i += ld_gstride()) {
-    int32_t u = (int32_t)(dkey[i] >> vb), v = (int32_t)(dkey[i] & mask);
-    const int32_t *row = col + off[u];
-    int64_t p = lower_bound_i32(row, deg[u], v);
-    if (p < deg[u] && row[p] == v) dw[i] = w[off[u] + p];
-    else { dw[i] = 0; atomicExch(&cnt->error, 2); }
+// The same for the batch: deletions collapse (-> dkey), insertions lose their
+// tag and add up (-> ikey, iw); counts [0] and [1].
+__global__ void k_unique_batch(const uint64_t *key, const int64_t *w, int64_t nda, int64_t nia, const int32_t *flag,
+                               const int64_t *pos, uint64_t mask, uint64_t *dkey, uint64_t *ikey, int64_t *iw,
+                               int64_t *counts) {
+  const int64_t nd = pos[nda];
+  if (ld_gtid() == 0) {
+    counts[0] = nd;
+    counts[1] = pos[nda + nia] - nd;
   }
-}
-
-// Insertions: existing arc (not deleted in this batch) -> state 1, position;
-// otherwise state 0 (a new arc).
-__global__ void k_classify_insertions(const uint64_t *ikey, const int64_t *ni_p, const uint64_t *dkey,
-                                      const int64_t *nd_p, int vb, const int64_t *off, const int32_t *deg,
-                                      const int32_t *col, int32_t *state, int64_t *ipos) {
-  uint64_t mask = (1ull << vb) - 1;
-  int64_t ni = *ni_p, nd = *nd_p;
-  for (int64_t i = ld_gtid(); i < ni; i += ld_gstride()) {
-    int32_t u = (int32_t)(ikey[i] >> vb), v = (int32_t)(ikey[i] & mask);
-    const int32_t *row = col + off[u];
-    int64_t p = lower_bound_i32(row, deg[u], v);
-    bool found = p < deg[u] && row[p] == v;
-    if (found) {
-      int64_t q = lower_bound_u64(dkey, nd, ikey[i]);
-      if (q < nd && dkey[q] == ikey[i]) found = false;  // deleted, then inserted again
+  for (int64_t i = ld_gtid(); i < nda + nia; i += ld_gstride()) {
+    int64_t p = pos[i] + flag[i] - 1;
+    if (i < nda) {
+      if (flag[i]) dkey[p] = key[i];
+    } else {
+      if (flag[i]) ikey[p - nd] = key[i] & mask;
+      atomicAdd((unsigned long long *)&iw[p - nd], (unsigned long long)w[i]);
     }
-    state[i] = found ? 1 : 0;
-    ipos[i] = found ? off[u] + p : -1;
   }
 }
 
-// Flags of the new arcs over the bound nb >= ni (zero past ni).
-__global__ void k_new_flags(const int32_t *state, const int64_t *ni_p, int64_t nb, int32_t *flag) {
-  int64_t ni = *ni_p;
-  for (int64_t i = ld_gtid(); i < nb; i += ld_gstride()) flag[i] = i < ni && state[i] == 0 ? 1 : 0;
+// What both batch paths need of the graph and of the handle's parameters.
+struct BatchGraph {
+  int64_t n;
+  const int64_t *off;
+  const int32_t *deg, *rcap, *col, *w, *gid0;
+  int64_t colcap;
+  double slack;
+  int min_slack, block_max, vb;
+};
+
+// A deletion must name an existing arc: its stored weight (0 and error 2 if not).
+__device__ __forceinline__ int64_t deleted_weight(const BatchGraph &G, uint64_t key, DevCounters *cnt) {
+  int32_t u = (int32_t)(key >> G.vb), v = (int32_t)(key & ((1ull << G.vb) - 1));
+  const int32_t *row = G.col + G.off[u];
+  int64_t p = lower_bound_i32(row, G.deg[u], v);
+  if (p < G.deg[u] && row[p] == v) return G.w[G.off[u] + p];
+  atomicExch(&cnt->error, 2);
+  return 0;
+}
+// The arc an insertion adds to, or -1: a new arc (also when the batch deletes
+// the existing one; dkey: its nd sorted deletions).
+__device__ __forceinline__ int64_t existing_arc(const BatchGraph &G, uint64_t key, const uint64_t *dkey, int64_t nd) {
+  int32_t u = (int32_t)(key >> G.vb), v = (int32_t)(key & ((1ull << G.vb) - 1));
+  const int32_t *row = G.col + G.off[u];
+  int64_t p = lower_bound_i32(row, G.deg[u], v);
+  if (p >= G.deg[u] || row[p] != v) return -1;
+  int64_t q = lower_bound_u64(dkey, nd, key);
+  return q < nd && dkey[q] == key ? -1 : G.off[u] + p;
+}
+
+// Deletions checked (stored weights -> dw), insertions classified: state 1 and
+// position of an existing arc, state 0 for a new one, flagged (over the bound
+// nia >= ni, zero past ni).  The change of 2m is summed.
+__global__ void __launch_bounds__(256) k_check_batch(BatchGraph G, const uint64_t *dkey, const uint64_t *ikey,
+                                                     const int64_t *iw, const int64_t *counts, int64_t nda, int64_t nia,
+                                                     int64_t *dw, int32_t *state, int64_t *ipos, int32_t *flag,
+                                                     DevCounters *cnt) {
+  __shared__ unsigned long long sum;
+  if (threadIdx.x == 0) sum = 0;
+  __syncthreads();
+  const int64_t nd = counts[0], ni = counts[1];
+  int64_t acc = 0;
+  for (int64_t i = ld_gtid(); i < nda + nia; i += ld_gstride()) {
+    if (i < nda) {
+      if (i < nd) acc -= dw[i] = deleted_weight(G, dkey[i], cnt);
+      continue;
+    }
+    int64_t k = i - nda;
+    flag[k] = 0;
+    if (k >= ni) continue;
+    int64_t p = existing_arc(G, ikey[k], dkey, nd);
+    state[k] = p >= 0;
+    ipos[k] = p;
+    flag[k] = p < 0;
+    acc += iw[k];
+  }
+  acc = ld_warp_sum_i64(acc);
+  if ((threadIdx.x & 31) == 0 && acc) atomicAdd(&sum, (unsigned long long)acc);
+  __syncthreads();
+  if (threadIdx.x == 0 && sum) atomicAdd((unsigned long long *)&cnt->batch_dw, sum);
 }
 
 __global__ void k_compact_new(const uint64_t *ikey, const int64_t *iw, int64_t ni, const int32_t *flag,
-                              const int64_t *pos, uint64_t *okey, int64_t *ow) {
+                              const int64_t *pos, uint64_t *okey, int64_t *ow, int64_t *count) {
+  if (ld_gtid() == 0) *count = pos[ni];
   for (int64_t i = ld_gtid(); i < ni; i += ld_gstride())
     if (flag[i]) { okey[pos[i]] = ikey[i]; ow[pos[i]] = iw[i]; }
 }
@@ -143,48 +190,263 @@ __global__ void k_touched_rows(const uint64_t *dkey, const int64_t *nd_p, const 
   }
 }
 
-// Leaves the row bitmap clear for the next call (every set bit belongs to a
-// listed row).
-__global__ void k_clear_row_bits(const int32_t *rows, const int64_t *nrows_p, uint32_t *bits) {
-  int64_t nrows = *nrows_p;
-  for (int64_t r = ld_gtid(); r < nrows; r += ld_gstride()) bits[rows[r] >> 5] = 0;
+// Table slots a hub of d arcs needs (0 below the hub path).
+__device__ __forceinline__ int64_t hub_slots(int64_t d, int block_max) {
+  return d > block_max ? (int64_t)1 << (64 - __clzll(2 * d - 1)) : 0;
 }
 
-// New length of each touched row and its segments in the two arc lists.
-// A row that outgrows its capacity moves to the spill arena at the end of
-// the arc arrays with fresh slack (dst, newcap); if the arena is full the
-// whole CSR is rebuilt instead (overflow flag).  Lengths are written up to
-// the bound nb >= nrows (zero past nrows) so that their scan needs no host
-// count.  A batch already found invalid takes no arena space.
-__global__ void k_row_plan(const int32_t *rows, const int64_t *nrows_p, int64_t nb, int vb, const uint64_t *dkey,
-                           const int64_t *nd_p, const uint64_t *nkey, const int64_t *nn_p, const int64_t *off,
-                           const int32_t *deg, const int32_t *rcap, int32_t *dlo, int32_t *dhi, int32_t *ilo,
-                           int32_t *ihi, int64_t *len, int64_t *dst, int32_t *newcap, double slack, int min_slack,
-                           int64_t colcap, int32_t *olddeg, int32_t *large, int32_t *mid, DevCounters *cnt) {
-  int64_t nrows = *nrows_p, nd = *nd_p, nn = *nn_p;
-  bool invalid = cnt->error != 0;
+// Where the plan of a touched row goes.
+struct RowPlan {
+  int32_t *dlo, *dhi, *ilo, *ihi;
+  int64_t *len, *dst;
+  int32_t *newcap, *olddeg, *large, *mid;
+};
+
+// Plan of touched row r = vertex u: its segments in the two arc lists, its new
+// length, its class, and a new place at the end of the arc arrays with fresh
+// slack if it outgrows its capacity (if the arena is full the whole CSR is
+// rebuilt instead: overflow).  A batch already found invalid takes no arena
+// space.  Returns the new length; slots: the change of the hub tables' size.
+__device__ __forceinline__ int64_t plan_row(const BatchGraph &G, const RowPlan &P, int64_t r, uint64_t u,
+                                            const uint64_t *dkey, int64_t nd, const uint64_t *nkey, int64_t nn,
+                                            bool invalid, DevCounters *cnt, int64_t &slots) {
+  int64_t a = lower_bound_u64(dkey, nd, u << G.vb), b = lower_bound_u64(dkey, nd, (u + 1) << G.vb);
+  int64_t c = lower_bound_u64(nkey, nn, u << G.vb), d = lower_bound_u64(nkey, nn, (u + 1) << G.vb);
+  P.dlo[r] = (int32_t)a; P.dhi[r] = (int32_t)b; P.ilo[r] = (int32_t)c; P.ihi[r] = (int32_t)d;
+  int32_t dg = G.deg[u];
+  int64_t L = (int64_t)dg - (b - a) + (d - c), dst = G.off[u];
+  int32_t newcap = 0;
+  P.len[r] = L;
+  P.olddeg[r] = dg;
+  if (L > MERGE_MID) P.large[atomicAdd(&cnt->large_count, 1)] = (int32_t)r;
+  else if (L > MERGE_SMALL) P.mid[atomicAdd(&cnt->mid_count, 1)] = (int32_t)r;
+  if (L > G.rcap[u] && !invalid) {
+    int64_t extra = (int64_t)((double)L * G.slack);
+    if (extra < G.min_slack) extra = G.min_slack;
+    int64_t cap = L + extra;
+    dst = (int64_t)atomicAdd((unsigned long long *)&cnt->arena_used, (unsigned long long)cap);
+    if (dst + cap > G.colcap) atomicExch(&cnt->overflow, 1);
+    newcap = (int32_t)cap;
+  }
+  P.dst[r] = dst;
+  P.newcap[r] = newcap;
+  slots += hub_slots(L, G.block_max) - hub_slots(dg, G.block_max);
+  return L;
+}
+
+// Plans of the touched rows; lengths are written up to the bound nb >= nrows
+// (zero past nrows) so that their scan needs no host count.  Leaves the row
+// bitmap clear for the next call (every set bit belongs to a listed row).
+__global__ void __launch_bounds__(256) k_row_plan(BatchGraph G, RowPlan P, const int32_t *rows, const int64_t *nrows_p,
+                                                  int64_t nb, const uint64_t *dkey, const int64_t *nd_p,
+                                                  const uint64_t *nkey, const int64_t *nn_p, uint32_t *bits,
+                                                  int64_t *total, DevCounters *cnt) {
+  __shared__ unsigned long long sum_s, slots_s;
+  __shared__ int max_s;
+  if (threadIdx.x == 0) { sum_s = 0; slots_s = 0; max_s = 0; }
+  __syncthreads();
+  const int64_t nrows = *nrows_p, nd = *nd_p, nn = *nn_p;
+  const bool invalid = cnt->error != 0;
+  int64_t sum = 0, slots = 0;
+  int mx = 0;
   for (int64_t r = ld_gtid(); r < nb; r += ld_gstride()) {
-    if (r >= nrows) { len[r] = 0; continue; }
-    uint64_t u = (uint64_t)rows[r];
-    int64_t a = lower_bound_u64(dkey, nd, u << vb), b = lower_bound_u64(dkey, nd, (u + 1) << vb);
-    int64_t c = lower_bound_u64(nkey, nn, u << vb), d = lower_bound_u64(nkey, nn, (u + 1) << vb);
-    dlo[r] = (int32_t)a; dhi[r] = (int32_t)b; ilo[r] = (int32_t)c; ihi[r] = (int32_t)d;
-    int64_t L = (int64_t)deg[u] - (b - a) + (d - c);
-    len[r] = L;
-    olddeg[r] = deg[u];
-    if (L > MERGE_MID) large[atomicAdd(&cnt->large_count, 1)] = (int32_t)r;
-    else if (L > MERGE_SMALL) mid[atomicAdd(&cnt->mid_count, 1)] = (int32_t)r;
-    dst[r] = off[u];
-    newcap[r] = 0;
-    if (L > rcap[u] && !invalid) {
-      int64_t extra = (int64_t)((double)L * slack);
-      if (extra < min_slack) extra = min_slack;
-      int64_t cap = L + extra;
-      int64_t p = (int64_t)atomicAdd((unsigned long long *)&cnt->arena_used, (unsigned long long)cap);
-      if (p + cap > colcap) atomicExch(&cnt->overflow, 1);
-      dst[r] = p;
-      newcap[r] = (int32_t)cap;
+    if (r >= nrows) { P.len[r] = 0; continue; }
+    int32_t u = rows[r];
+    bits[u >> 5] = 0;
+    int64_t L = plan_row(G, P, r, (uint64_t)u, dkey, nd, nkey, nn, invalid, cnt, slots);
+    sum += L;
+    mx = max(mx, (int)L);
+  }
+  sum = ld_warp_sum_i64(sum);
+  slots = ld_warp_sum_i64(slots);
+  mx = __reduce_max_sync(LD_FULL, mx);
+  if ((threadIdx.x & 31) == 0) {
+    if (sum) atomicAdd(&sum_s, (unsigned long long)sum);
+    if (slots) atomicAdd(&slots_s, (unsigned long long)slots);
+    if (mx) atomicMax(&max_s, mx);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (sum_s) atomicAdd((unsigned long long *)total, sum_s);
+    if (slots_s) atomicAdd((unsigned long long *)&cnt->slot_change, slots_s);
+    if (max_s) atomicMax(&cnt->max_row, max_s);
+  }
+}
+
+// ---------------------------------------------------------------- small batches
+// A batch of at most SMALL_ARCS arcs is expanded, sorted, deduplicated, checked
+// and planned by one block in shared memory: the steps are a chain, and at
+// this size each of them costs a launch more than its work (23 launches and
+// clears of the path above; 100 edges on 10k vertices: 433 -> 302 us a call,
+// the kernel itself 22 us).
+constexpr int SMALL_ARCS = 2048;
+
+// Exclusive sums of the threads' values over a block of 1024, the total in *total.
+__device__ __forceinline__ int64_t block_excl_1024(int64_t v, int64_t *ws, int64_t *total) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int64_t incl = ld_warp_incl_i64(v);
+  __syncthreads();
+  if (lane == 31) ws[wid] = incl;
+  __syncthreads();
+  int64_t y = ws[lane], yi = ld_warp_incl_i64(y);
+  *total = __shfl_sync(LD_FULL, yi, 31);
+  return __shfl_sync(LD_FULL, yi - y, wid) + incl - v;
+}
+
+struct SmallOut {
+  uint64_t *dkey, *ikey, *nkey;
+  int64_t *dw, *iw, *nw, *ipos, *tmp_off;
+  int32_t *state, *rows;
+};
+
+__global__ void __launch_bounds__(1024) k_small_batch(BatchGraph G, RowPlan P, SmallOut O, const leiden_edge *del,
+                                                      int n_del, const leiden_edge *ins, int n_ins, DevCounters *cnt) {
+  __shared__ uint64_t sk[SMALL_ARCS];     // arcs by key, then the unique ones: deletions, insertions
+  __shared__ int64_t sw[SMALL_ARCS];      // summed weights of the unique arcs, then the new arcs' keys
+  __shared__ int32_t si[SMALL_ARCS];      // input positions, then the touched rows
+  __shared__ int64_t ws[32];
+  __shared__ int nrows_s, max_s;
+  const int tid = threadIdx.x, nda = 2 * n_del, na = 2 * (n_del + n_ins), vb = G.vb;
+  const uint64_t mask = (1ull << (2 * vb)) - 1, tag = 1ull << (2 * vb);
+  if (tid == 0) { nrows_s = 0; max_s = 0; }
+  int N2 = 2;
+  while (N2 < na) N2 <<= 1;
+  for (int t = tid; t < N2; t += 1024) {
+    uint64_t key = ~0ull;  // padding sorts last (its positions are larger)
+    if (t < na) {
+      int e = t >> 1;
+      bool d = e < n_del;
+      leiden_edge x = d ? del[e] : ins[e - n_del];
+      if (!valid_edge(x, d, G.n, G.gid0)) {
+        atomicExch(&cnt->error, 1);
+        x.u = 0; x.v = 1 % (int32_t)(G.n > 1 ? G.n : 1);
+      }
+      key = (t & 1 ? ((uint64_t)x.v << vb) | (uint64_t)x.u : ((uint64_t)x.u << vb) | (uint64_t)x.v) | (d ? 0ull : tag);
     }
+    sk[t] = key;
+    si[t] = t;
+  }
+  __syncthreads();
+  for (int k = 2; k <= N2; k <<= 1)  // bitonic network
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      for (int t = tid; t < N2; t += 1024) {
+        int u = t ^ j;
+        if (u <= t) continue;
+        uint64_t a = sk[t], b = sk[u];
+        if ((a > b) == ((t & k) == 0) && a != b) {
+          int32_t x = si[t];
+          sk[t] = b; sk[u] = a; si[t] = si[u]; si[u] = x;
+        }
+      }
+      __syncthreads();
+    }
+  // unique arcs: thread t holds the sorted ones 2t and 2t + 1
+  uint64_t key[2];
+  int64_t w[2];
+  bool head[2];
+#pragma unroll
+  for (int q = 0; q < 2; q++) {
+    int t = 2 * tid + q;
+    head[q] = t < na && (t == 0 || sk[t] != sk[t - 1]);
+    key[q] = t < na ? sk[t] : 0;
+    int e = t < na ? si[t] >> 1 : 0;
+    w[q] = t < na && e >= n_del ? ins[e - n_del].w : 0;
+  }
+  int64_t nu, nd, total;
+  int64_t pos = block_excl_1024((int)head[0] + (int)head[1], ws, &nu);
+  block_excl_1024((int)(head[0] && key[0] < tag) + (int)(head[1] && key[1] < tag), ws, &nd);
+  for (int t = tid; t < SMALL_ARCS; t += 1024) sw[t] = 0;
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 2; q++) {
+    pos += head[q];
+    if (2 * tid + q < na) {
+      if (head[q]) sk[pos - 1] = key[q] & mask;
+      if (w[q]) atomicAdd((unsigned long long *)&sw[pos - 1], (unsigned long long)w[q]);
+    }
+  }
+  __syncthreads();
+  // deletions checked, insertions classified (unique arcs 2t and 2t + 1)
+  const int64_t ni = nu - nd;
+  int64_t dsum = 0;
+  bool fresh[2] = {false, false};
+#pragma unroll
+  for (int q = 0; q < 2; q++) {
+    int t = 2 * tid + q;
+    if (t >= nu) continue;
+    key[q] = sk[t];
+    w[q] = sw[t];
+    if (t < nd) {
+      int64_t x = deleted_weight(G, key[q], cnt);
+      O.dkey[t] = key[q];
+      O.dw[t] = x;
+      dsum -= x;
+    } else {
+      int64_t p = existing_arc(G, key[q], sk, nd);
+      O.ikey[t - nd] = key[q];
+      O.iw[t - nd] = w[q];
+      O.state[t - nd] = p >= 0;
+      O.ipos[t - nd] = p;
+      fresh[q] = p < 0;
+      dsum += w[q];
+    }
+  }
+  int64_t nn, at = block_excl_1024((int)fresh[0] + (int)fresh[1], ws, &nn);  // (its barriers: sw has been read)
+  uint64_t *nk = (uint64_t *)sw;
+#pragma unroll
+  for (int q = 0; q < 2; q++)
+    if (fresh[q]) {
+      nk[at] = key[q];
+      O.nkey[at] = key[q];
+      O.nw[at] = w[q];
+      at++;
+    }
+  block_excl_1024(dsum, ws, &total);
+  if (tid == 0) cnt->batch_dw = total;
+  __syncthreads();
+  // touched rows: the heads of the sources' runs, a new arc's only if no deletion has its source
+  for (int t = tid; t < nd + nn; t += 1024) {
+    const uint64_t *L = t < nd ? sk : nk;
+    int64_t k = t < nd ? t : t - nd;
+    uint64_t u = L[k] >> vb;
+    if (k > 0 && (L[k - 1] >> vb) == u) continue;
+    if (t >= nd) {
+      int64_t q = lower_bound_u64(sk, nd, u << vb);
+      if (q < nd && (sk[q] >> vb) == u) continue;
+    }
+    si[atomicAdd(&nrows_s, 1)] = (int32_t)u;
+  }
+  __syncthreads();
+  const int nrows = nrows_s;
+  const bool invalid = *(volatile int32_t *)&cnt->error != 0;
+  int64_t len[2] = {0, 0}, slots = 0;
+#pragma unroll
+  for (int q = 0; q < 2; q++) {
+    int r = 2 * tid + q;
+    if (r >= nrows) continue;
+    O.rows[r] = si[r];
+    len[q] = plan_row(G, P, r, (uint64_t)si[r], sk, nd, nk, nn, invalid, cnt, slots);
+  }
+  int64_t off = block_excl_1024(len[0] + len[1], ws, &total), st;
+#pragma unroll
+  for (int q = 0; q < 2; q++) {
+    int r = 2 * tid + q;
+    if (r < nrows) O.tmp_off[r] = off;
+    off += len[q];
+    if (r == nrows - 1) O.tmp_off[nrows] = off;
+  }
+  block_excl_1024(slots, ws, &st);
+  int mx = __reduce_max_sync(LD_FULL, (int)max(len[0], len[1]));
+  if ((tid & 31) == 0) atomicMax(&max_s, mx);
+  __syncthreads();
+  if (tid == 0) {
+    cnt->bcounts[0] = nd;
+    cnt->bcounts[1] = ni;
+    cnt->bcounts[2] = nn;
+    cnt->bcounts[3] = nrows;
+    cnt->bcounts[4] = total;
+    cnt->slot_change = st;
+    cnt->max_row = max_s;
   }
 }
 
@@ -455,18 +717,6 @@ __global__ void k_rowsrc(const int32_t *rows, const int64_t *nrows_p, int32_t *r
 }
 
 // ----- marking (uses C^{t-1}, and K^{t-1}, Sigma^{t-1}, 2m^{t-1} for DS)
-__global__ void k_mark_df(const uint64_t *dkey, int64_t nd, const uint64_t *ikey, int64_t ni, int vb,
-                          const int32_t *C, uint8_t *dV) {
-  uint64_t mask = (1ull << vb) - 1;
-  for (int64_t i = ld_gtid(); i < nd + ni; i += ld_gstride()) {
-    bool del = i < nd;
-    uint64_t k = del ? dkey[i] : ikey[i - nd];
-    int32_t u = (int32_t)(k >> vb), v = (int32_t)(k & mask);
-    bool same = C[u] == C[v];
-    if (del ? same : !same) dV[u] = 1;
-  }
-}
-
 __global__ void k_mark_ds_del(const uint64_t *dkey, int64_t nd, int vb, const int32_t *C, uint8_t *dV, uint8_t *dE,
                               uint8_t *dCf) {
   uint64_t mask = (1ull << vb) - 1;
@@ -568,40 +818,80 @@ __global__ void k_ds_expand_communities(const uint8_t *dCf, const int32_t *C, in
     if (dCf[C[i]]) dV[i] = 1;
 }
 
-// Alg. update (updateWeights, updateChanges) on both arc lists.
-__global__ void k_update_weights(const uint64_t *dkey, const int64_t *dw, int64_t nd, const uint64_t *ikey,
-                                 const int64_t *iw, int64_t ni, int vb, const int32_t *C, int64_t *K, int64_t *Sig,
-                                 int64_t *dSig, DevCounters *cnt, const int32_t *gid0, int64_t *m2g) {
-  int64_t acc = 0;
+// Alg. update (updateWeights, updateChanges) on both arc lists, with the DF
+// marking (dV non-null; it reads C^{t-1} only).  The arcs of giant communities
+// meet on a few words of Sigma and Delta Sigma: a block first adds them up in a
+// small shared table (an arc whose slot another community holds adds
+// directly), the lanes of the warp's first community in one add
+// (R-MAT 20, 1.6M edges: 361 -> 138 us).
+constexpr int UPD_SLOTS = 256;
+__global__ void __launch_bounds__(256) k_update_weights(const uint64_t *dkey, const int64_t *dw, int64_t nd,
+                                                        const uint64_t *ikey, const int64_t *iw, int64_t ni, int vb,
+                                                        const int32_t *C, int64_t *K, int64_t *Sig, int64_t *dSig,
+                                                        DevCounters *cnt, const int32_t *gid0, int64_t *m2g,
+                                                        uint8_t *dV) {
+  __shared__ int32_t hk[UPD_SLOTS];
+  __shared__ unsigned long long hs[UPD_SLOTS], hw[UPD_SLOTS];
+  for (int t = threadIdx.x; t < UPD_SLOTS; t += 256) { hk[t] = -1; hs[t] = 0; hw[t] = 0; }
+  __syncthreads();
+  if (ld_gtid() == 0) cnt->m2 += cnt->batch_dw;
+  const int lane = threadIdx.x & 31;
+  const uint64_t mask = (1ull << vb) - 1;
+  auto add = [&](int32_t c, int64_t s, int64_t w) {
+    int t = (int)(ld_hash32((uint32_t)c) & (UPD_SLOTS - 1));
+    int32_t k = hk[t];
+    if (k == -1) {
+      k = atomicCAS(&hk[t], -1, c);
+      if (k == -1) k = c;
+    }
+    if (k == c) {
+      atomicAdd(&hs[t], (unsigned long long)s);
+      atomicAdd(&hw[t], (unsigned long long)w);
+    } else {
+      atomicAdd((unsigned long long *)&Sig[c], (unsigned long long)s);
+      atomicAdd((unsigned long long *)&dSig[c], (unsigned long long)w);
+    }
+  };
   for (int64_t i0 = (ld_gtid() & ~31ll); i0 < nd + ni; i0 += ld_gstride()) {  // warp-uniform trip count
-    int64_t i = i0 + (threadIdx.x & 31);
+    int64_t i = i0 + lane;
     bool has = i < nd + ni;
-    int64_t s = 0;
-    int32_t u = 0;
+    int64_t s = 0, w = 0;
+    int32_t u = 0, c = -1;
     if (has) {
       bool del = i < nd;
       uint64_t k = del ? dkey[i] : ikey[i - nd];
-      int64_t w = del ? dw[i] : iw[i - nd];
+      w = del ? dw[i] : iw[i - nd];
       u = (int32_t)(k >> vb);
-      int32_t c = C[u];
+      c = C[u];
       s = del ? -w : w;
       atomicAdd((unsigned long long *)&K[u], (unsigned long long)s);
-      atomicAdd((unsigned long long *)&Sig[c], (unsigned long long)s);
-      atomicAdd((unsigned long long *)&dSig[c], (unsigned long long)w);
-      acc += s;
+      if (dV && del == (c == C[(int32_t)(k & mask)])) dV[u] = 1;
+    }
+    int32_t c0 = __shfl_sync(LD_FULL, c, 0);
+    bool first = c == c0;
+    if (__popc(__ballot_sync(LD_FULL, first)) > 4) {  // warp-uniform
+      int64_t ss = ld_warp_sum_i64(first ? s : 0), sw = ld_warp_sum_i64(first ? w : 0);
+      if (lane == 0) add(c0, ss, sw);
+      if (has && !first) add(c, s, w);
+    } else if (has) {
+      add(c, s, w);
     }
     // batched: 2m per graph (a signed sum; the helper adds two's-complement values)
     if (gid0) ld_graph_add_i64(m2g, has, has ? gid0[u] : 0, s);
   }
-  acc = ld_warp_sum_i64(acc);
-  if ((threadIdx.x & 31) == 0 && acc) atomicAdd((unsigned long long *)&cnt->m2, (unsigned long long)acc);
+  __syncthreads();
+  for (int t = threadIdx.x; t < UPD_SLOTS; t += 256)
+    if (hk[t] >= 0) {
+      if (hs[t]) atomicAdd((unsigned long long *)&Sig[hk[t]], hs[t]);
+      if (hw[t]) atomicAdd((unsigned long long *)&dSig[hk[t]], hw[t]);
+    }
 }
 
 // Alg. leidenmk: dS for same-community deletions; dR for same-community
 // arcs of either list with dSigma/Sigma > tau_re.
 __global__ void k_mark_communities(const uint64_t *dkey, int64_t nd, const uint64_t *ikey, int64_t ni, int vb,
                                    const int32_t *C, const int64_t *Sig, const int64_t *dSig, double tau_re,
-                                   uint8_t *dS, uint8_t *dR) {
+                                   uint8_t *dS, uint8_t *dR, DevCounters *cnt) {
   uint64_t mask = (1ull << vb) - 1;
   for (int64_t i = ld_gtid(); i < nd + ni; i += ld_gstride()) {
     bool del = i < nd;
@@ -610,11 +900,15 @@ __global__ void k_mark_communities(const uint64_t *dkey, int64_t nd, const uint6
     int32_t c = C[u];
     if (c != C[v]) continue;
     if (del) dS[c] = 1;
-    if ((double)dSig[c] / (double)Sig[c] > tau_re) dR[c] = 1;
+    if ((double)dSig[c] / (double)Sig[c] > tau_re) {
+      dR[c] = 1;
+      cnt->refine_marks = 1;  // (any value but 0: is there one?)
+    }
   }
 }
 __global__ void k_reset_changes(const uint64_t *dkey, int64_t nd, const uint64_t *ikey, int64_t ni, int vb,
-                                const int32_t *C, const uint8_t *dR, int64_t *dSig) {
+                                const int32_t *C, const uint8_t *dR, int64_t *dSig, const DevCounters *cnt) {
+  if (cnt->refine_marks == 0) return;
   for (int64_t i = ld_gtid(); i < nd + ni; i += ld_gstride()) {
     uint64_t k = i < nd ? dkey[i] : ikey[i - nd];
     int32_t c = C[(int32_t)(k >> vb)];
@@ -663,11 +957,11 @@ cudaError_t ensure_batch(leiden_handle *h, int64_t edges) {
                    (void **)&nb.row_tmp_off, (void **)&nb.row_dst, (void **)&nb.row_newcap, (void **)&nb.row_olddeg,
                    (void **)&nb.row_large, (void **)&nb.row_mid, (void **)&nb.ds_key, (void **)&nb.ds_key_alt,
                    (void **)&nb.ds_w, (void **)&nb.ds_w_alt, (void **)&nb.ds_ukey, (void **)&nb.ds_uw};
-  // dkey, dkey_alt, iw and iw_alt hold the deletion and insertion arcs of
-  // one sort together (2 * arcs); ikey, ikey_alt and iw_alt's unique part
+  // dkey, dkey_alt, iw, iw_alt, flag and pos hold the deletion and insertion
+  // arcs of one sort together (2 * arcs); ikey, ikey_alt and iw_alt's unique part
   // at most one kind
   size_t bytes[] = {16 * (size_t)arcs, 16 * (size_t)arcs, 8 * (size_t)arcs, 8 * (size_t)arcs, 16 * (size_t)arcs,
-                    16 * (size_t)arcs, 8 * (size_t)arcs, 4 * (size_t)(arcs + 1), 8 * (size_t)(arcs + 1),
+                    16 * (size_t)arcs, 8 * (size_t)arcs, 4 * (size_t)(2 * arcs + 1), 8 * (size_t)(2 * arcs + 1),
                     4 * (size_t)arcs, 8 * (size_t)arcs, 4 * (size_t)rows, 4 * (size_t)rows, 4 * (size_t)rows,
                     4 * (size_t)rows, 4 * (size_t)rows, 8 * (size_t)(rows + 1), 8 * (size_t)(rows + 1),
                     8 * (size_t)(rows + 1), 4 * (size_t)(rows + 1), 4 * (size_t)(rows + 1), 4 * (size_t)(rows + 1),
@@ -796,68 +1090,48 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
   DevCounters *cnt = h->dcnt;
   if (ensure_batch(h, std::max(n_del, n_ins)) != cudaSuccess) return fail(h, LEIDEN_ERR_OOM, "batch buffers");
   int64_t nda = 2 * n_del, nia = 2 * n_ins;
-  if (ensure_scan_tmp(h, std::max(sort_tmp_bytes(nda + nia), scan_tmp_bytes(n + 1))) != cudaSuccess)
+  if (ensure_scan_tmp(h, std::max(sort_tmp_bytes(nda + nia), scan_tmp_bytes(std::max(n, nda + nia) + 1))) != cudaSuccess)
     return fail(h, LEIDEN_ERR_OOM, "scan tmp");
-  cudaMemsetAsync(&cnt->error, 0, sizeof(int32_t), s);
-  cudaMemsetAsync(&cnt->overflow, 0, sizeof(int32_t), s);
-  cudaMemsetAsync(&cnt->large_count, 0, sizeof(int32_t), s);
-  cudaMemsetAsync(&cnt->mid_count, 0, sizeof(int32_t), s);
-  // one sort of both: the deletion arcs sorted in dkey[0, nda), the
-  // insertion arcs and their weights in dkey, iw [nda, nda + nia)
-  if (n_del + n_ins > 0)
-    ld_note_launch(), k_expand<<<grid_for(n_del + n_ins, TB), TB, 0, s>>>(d_del, n_del, d_ins, n_ins, n, vb, b.dkey,
-                                                                          b.iw, cnt, h->gid0);
-  radix_sort_u64(b.dkey, b.dkey_alt, b.iw, b.iw_alt, nda + nia, 2 * vb + 1, h->scan_tmp, s);
-  uint64_t *SD = b.dkey, *SI = b.dkey + nda;
-  int64_t *SIW = b.iw + nda;
-  if (nia > 0) ld_note_launch(), k_untag<<<grid_for(nia, TB), TB, 0, s>>>(SI, nia, (1ull << (2 * vb)) - 1);
-  // deduplicate: deletions collapse (-> DK), insertions add up (-> IK, IW).
-  // The counts stay on the device until the one host read below: launches
-  // are sized by the bounds nda, nia and read the counts themselves.
-  int64_t *counts = b.counts;  // [0] nd, [1] ni, [2] new arcs, [3] touched rows, [4] merge-buffer arcs
-  cudaMemsetAsync(counts, 0, 8 * sizeof(int64_t), s);
+  // [0] nd, [1] ni, [2] new arcs, [3] touched rows, [4] merge-buffer arcs (cleared
+  // with the call's counters): they stay on the device until the one host read
+  // below; launches are sized by the bounds nda, nia
+  int64_t *counts = b.counts;
   uint64_t *DK = b.dkey_alt, *IK = b.ikey_alt;
   int64_t *IW = b.iw_alt, *DW = b.dw;
-  if (nda > 0) {
-    ld_note_launch(), k_head_flags<<<grid_for(nda, TB), TB, 0, s>>>(SD, nda, b.flag);
-    exclusive_scan_i32_to_i64(b.flag, b.pos, nda, h->scan_tmp, s);
-    ld_note_launch(), k_unique<<<grid_for(nda, TB), TB, 0, s>>>(SD, nullptr, nda, b.flag, b.pos, DK, nullptr);
-    cudaMemcpyAsync(counts + 0, b.pos + nda, sizeof(int64_t), cudaMemcpyDeviceToDevice, s);
-  }
-  if (nia > 0) {
-    ld_note_launch(), k_head_flags<<<grid_for(nia, TB), TB, 0, s>>>(SI, nia, b.flag);
-    exclusive_scan_i32_to_i64(b.flag, b.pos, nia, h->scan_tmp, s);
-    cudaMemsetAsync(IW, 0, (size_t)nia * sizeof(int64_t), s);
-    ld_note_launch(), k_unique<<<grid_for(nia, TB), TB, 0, s>>>(SI, SIW, nia, b.flag, b.pos, IK, IW);
-    cudaMemcpyAsync(counts + 1, b.pos + nia, sizeof(int64_t), cudaMemcpyDeviceToDevice, s);
-  }
-  // deletions must exist (stored weight -> DW); insertions: existing or new
-  if (nda > 0)
-    ld_note_launch(), k_check_deletions<<<grid_for(nda, TB), TB, 0, s>>>(DK, counts + 0, vb, h->g_off, h->g_deg,
-                                                                         h->g_col, h->g_w, DW, cnt);
   uint64_t *NK = b.ikey;  // new insertions, compacted in sorted order
   int64_t *NW = b.iw;      // (the sorted raw arcs there are consumed by then)
-  if (nia > 0) {
-    ld_note_launch(), k_classify_insertions<<<grid_for(nia, TB), TB, 0, s>>>(IK, counts + 1, DK, counts + 0, vb,
-                                                                             h->g_off, h->g_deg, h->g_col,
-                                                                             b.ins_state, b.ins_pos);
-    ld_note_launch(), k_new_flags<<<grid_for(nia, TB), TB, 0, s>>>(b.ins_state, counts + 1, nia, b.flag);
-    exclusive_scan_i32_to_i64(b.flag, b.pos, nia, h->scan_tmp, s);
-    ld_note_launch(), k_compact_new<<<grid_for(nia, TB), TB, 0, s>>>(IK, IW, nia, b.flag, b.pos, NK, NW);
-    cudaMemcpyAsync(counts + 2, b.pos + nia, sizeof(int64_t), cudaMemcpyDeviceToDevice, s);
-  }
-  // rows whose structure changes: sources of deletions and of new arcs
-  int64_t nb = std::min<int64_t>(n, nda + nia);  // bound on the touched rows
-  if (nb > 0) {
+  BatchGraph G{n, h->g_off, h->g_deg, h->g_rcap, h->g_col, h->g_w, h->gid0, h->g_cap, h->p.slack, h->p.min_slack,
+               h->tune.block_max, vb};
+  RowPlan P{b.row_dlo, b.row_dhi, b.row_ilo, b.row_ihi, b.row_len, b.row_dst, b.row_newcap, b.row_olddeg, b.row_large,
+            b.row_mid};
+  if (nda + nia == 0) {
+  } else if (nda + nia <= SMALL_ARCS) {
+    SmallOut O{DK, IK, NK, DW, IW, NW, b.ins_pos, b.row_tmp_off, b.ins_state, b.rows};
+    ld_note_launch(), k_small_batch<<<1, 1024, 0, s>>>(G, P, O, d_del, (int)n_del, d_ins, (int)n_ins, cnt);
+  } else {
+    // one sort of both: the deletion arcs sorted in dkey[0, nda), the
+    // insertion arcs and their weights in dkey, iw [nda, nda + nia)
+    ld_note_launch(), k_expand<<<grid_for(n_del + n_ins, TB), TB, 0, s>>>(d_del, n_del, d_ins, n_ins, n, vb, b.dkey,
+                                                                          b.iw, cnt, h->gid0);
+    radix_sort_u64(b.dkey, b.dkey_alt, b.iw, b.iw_alt, nda + nia, 2 * vb + 1, h->scan_tmp, s);
+    ld_note_launch(), k_head_flags<<<grid_for(nda + nia, TB), TB, 0, s>>>(b.dkey, nda + nia, b.flag, IW, nia);
+    exclusive_scan_i32_to_i64(b.flag, b.pos, nda + nia, h->scan_tmp, s);
+    ld_note_launch(), k_unique_batch<<<grid_for(nda + nia, TB), TB, 0, s>>>(
+        b.dkey, b.iw, nda, nia, b.flag, b.pos, (1ull << (2 * vb)) - 1, DK, IK, IW, counts);
+    // deletions must exist (stored weight -> DW); insertions: existing or new
+    ld_note_launch(), k_check_batch<<<grid_for(nda + nia, TB), TB, 0, s>>>(G, DK, IK, IW, counts, nda, nia, DW,
+                                                                           b.ins_state, b.ins_pos, b.flag, cnt);
+    if (nia > 0) {
+      exclusive_scan_i32_to_i64(b.flag, b.pos, nia, h->scan_tmp, s);
+      ld_note_launch(), k_compact_new<<<grid_for(nia, TB), TB, 0, s>>>(IK, IW, nia, b.flag, b.pos, NK, NW, counts + 2);
+    }
+    // rows whose structure changes: sources of deletions and of new arcs
+    int64_t nb = std::min<int64_t>(n, nda + nia);  // bound on the touched rows
     ld_note_launch(), k_touched_rows<<<grid_for(nda + nia, TB), TB, 0, s>>>(DK, counts + 0, NK, counts + 2, vb,
                                                                             b.row_bits, b.rows, counts + 3);
-    ld_note_launch(), k_clear_row_bits<<<grid_for(nb, TB), TB, 0, s>>>(b.rows, counts + 3, b.row_bits);
-    ld_note_launch(), k_row_plan<<<grid_for(nb, TB), TB, 0, s>>>(
-        b.rows, counts + 3, nb, vb, DK, counts + 0, NK, counts + 2, h->g_off, h->g_deg, h->g_rcap, b.row_dlo,
-        b.row_dhi, b.row_ilo, b.row_ihi, b.row_len, b.row_dst, b.row_newcap, h->p.slack, h->p.min_slack, h->g_cap,
-        b.row_olddeg, b.row_large, b.row_mid, cnt);
+    ld_note_launch(), k_row_plan<<<grid_for(nb, TB), TB, 0, s>>>(G, P, b.rows, counts + 3, nb, DK, counts + 0, NK,
+                                                                 counts + 2, b.row_bits, counts + 4, cnt);
     exclusive_scan_i64(b.row_len, b.row_tmp_off, nb, h->scan_tmp, s);
-    cudaMemcpyAsync(counts + 4, b.row_tmp_off + nb, sizeof(int64_t), cudaMemcpyDeviceToDevice, s);
   }
   // the one host read before the graph changes: counts, validation, overflow
   cudaMemcpyAsync(h->hcnt, h->dcnt, sizeof(DevCounters), cudaMemcpyDeviceToHost, s);
@@ -870,7 +1144,7 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
   bool overflow = nrows > 0 && h->hcnt->overflow != 0;
   if (ensure_tmp_rows(h, tmp_total) != cudaSuccess) return fail(h, LEIDEN_ERR_OOM, "merge buffer");
   // ---- apply: from here on the handle changes
-  if (ni > 0) ld_note_launch(), k_add_existing<<<grid_for(ni, TB), TB, 0, s>>>(b.ins_pos, b.ins_state, IW, ni, h->g_w);
+  if (ni > nn) ld_note_launch(), k_add_existing<<<grid_for(ni, TB), TB, 0, s>>>(b.ins_pos, b.ins_state, IW, ni, h->g_w);
   if (nrows > 0) {
     if (!overflow) {
       MergeArgs M{b.rows, counts + 3, vb, DK, NK, NW, b.row_dlo, b.row_dhi, b.row_ilo, b.row_ihi, b.row_len,
@@ -879,30 +1153,37 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
       // the three row classes write disjoint rows and merge-buffer ranges:
       // short rows on the handle's stream, mid rows and long rows on its
       // side streams, joined before the marking below
-      bool fork = h->tune.overlap && side_streams(h);
+      const bool some_mid = h->hcnt->mid_count > 0, some_long = h->hcnt->large_count > 0,
+                 some_small = nrows > (int64_t)h->hcnt->mid_count + h->hcnt->large_count;
+      bool fork = (some_mid || some_long) && h->tune.overlap && side_streams(h);
       cudaStream_t smid = s, slong = s;
       if (fork) {
         cudaEventRecord(h->fork_ev, s);
         smid = h->side[0];
         slong = h->side[1];
-        cudaStreamWaitEvent(smid, h->fork_ev, 0);
-        cudaStreamWaitEvent(slong, h->fork_ev, 0);
+        if (some_mid) cudaStreamWaitEvent(smid, h->fork_ev, 0);
+        if (some_long) cudaStreamWaitEvent(slong, h->fork_ev, 0);
       }
-      ld_note_launch(), k_merge_small<<<grid_for((nrows + MERGE_WARPS - 1) / MERGE_WARPS, 1, h->sm_count * 16), MERGE_WARPS * 32, 0,
+      if (some_small) ld_note_launch(), k_merge_small<<<grid_for((nrows + MERGE_WARPS - 1) / MERGE_WARPS, 1, h->sm_count * 16), MERGE_WARPS * 32, 0,
                       s>>>(M);
-      kt_begin(h, KT_MERGE_MID, smid);
-      ld_note_launch(), k_merge_mid<<<h->sm_count * 7, 256, 0, smid>>>(M, b.row_mid, &cnt->mid_count,  // 32 KB: 7 per SM
-                                                                      &cnt->xk_bytes[2]);
-      kt_end(h, smid);
-      // long rows: chunks over the old row, then chunks over the new row
-      int32_t *large = b.row_large;
-      const int32_t *nlarge = &cnt->large_count;
-      launch_table_plan(large, nlarge, b.row_olddeg, nullptr, INT64_MAX, h->lbuf0, h->lbuf1, slong);
-      ld_note_launch(), k_merge_chunks_write<<<h->sm_count * 16, 256, 0, slong>>>(M, large, nlarge, h->lbuf1);
-      launch_table_plan(large, nlarge, nullptr, b.row_tmp_off, INT64_MAX, h->lbuf2, h->lbuf3, slong);
-      ld_note_launch(), k_merge_chunks_copy<<<h->sm_count * 16, 256, 0, slong>>>(M, large, nlarge, h->lbuf3);
+      if (some_mid) {
+        kt_begin(h, KT_MERGE_MID, smid);
+        ld_note_launch(), k_merge_mid<<<h->sm_count * 7, 256, 0, smid>>>(M, b.row_mid, &cnt->mid_count,  // 32 KB: 7 per SM
+                                                                        &cnt->xk_bytes[2]);
+        kt_end(h, smid);
+      }
+      if (some_long) {
+        // long rows: chunks over the old row, then chunks over the new row
+        int32_t *large = b.row_large;
+        const int32_t *nlarge = &cnt->large_count;
+        launch_table_plan(large, nlarge, b.row_olddeg, nullptr, INT64_MAX, h->lbuf0, h->lbuf1, slong);
+        ld_note_launch(), k_merge_chunks_write<<<h->sm_count * 16, 256, 0, slong>>>(M, large, nlarge, h->lbuf1);
+        launch_table_plan(large, nlarge, nullptr, b.row_tmp_off, INT64_MAX, h->lbuf2, h->lbuf3, slong);
+        ld_note_launch(), k_merge_chunks_copy<<<h->sm_count * 16, 256, 0, slong>>>(M, large, nlarge, h->lbuf3);
+      }
       if (fork) {
         for (int k = 0; k < 2; k++) {
+          if (!(k == 0 ? some_mid : some_long)) continue;
           cudaEventRecord(h->join_ev[k], h->side[k]);
           cudaStreamWaitEvent(s, h->join_ev[k], 0);
         }
@@ -921,15 +1202,17 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
   }
   h->g_arcs = h->g_arcs - nd + nn;
   h->stats.batch_arcs = nd + ni;
-  // ---- affected vertices (C^{t-1}; DS also K^{t-1}, Sigma^{t-1}, 2m^{t-1})
+  h->batch_dw = h->hcnt->batch_dw;
+  h->g_maxdeg = std::max(h->g_maxdeg, h->hcnt->max_row);  // (a bound: the longest row may have shrunk)
+  h->g_huge_slots += h->hcnt->slot_change;
+  // ---- affected vertices (C^{t-1}; DS also K^{t-1}, Sigma^{t-1}, 2m^{t-1}; DF
+  // with the weights below), dS and dR (the three flag arrays are neighbours)
   uint8_t *dV = h->dV;
-  if (mode == LEIDEN_ND) {
-    cudaMemsetAsync(dV, 1, (size_t)n, s);
-  } else {
-    cudaMemsetAsync(dV, 0, (size_t)n, s);
-    if (mode == LEIDEN_DF) {
-      if (nd + ni > 0) ld_note_launch(), k_mark_df<<<grid_for(nd + ni, TB), TB, 0, s>>>(DK, nd, IK, ni, vb, h->C, dV);
-    } else {
+  size_t flags = (size_t)(h->dR - h->dV) + (size_t)n;
+  cudaMemsetAsync(dV, 0, flags, s);
+  if (mode == LEIDEN_ND) cudaMemsetAsync(dV, 1, (size_t)n, s);
+  if (mode == LEIDEN_DS) {
+    {
       cudaMemsetAsync(h->dE, 0, (size_t)n, s);
       cudaMemsetAsync(h->dCf, 0, (size_t)n, s);
       if (nd > 0) ld_note_launch(), k_mark_ds_del<<<grid_for(nd, TB), TB, 0, s>>>(DK, nd, vb, h->C, dV, h->dE, h->dCf);
@@ -937,7 +1220,7 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
         // H of each insertion source: (src, C[dst]) pairs, sorted, runs summed
         ld_note_launch(), k_ds_keys<<<grid_for(ni, TB), TB, 0, s>>>(IK, IW, ni, vb, h->C, b.ds_key, b.ds_w);
         radix_sort_u64(b.ds_key, b.ds_key_alt, b.ds_w, b.ds_w_alt, ni, 64, h->scan_tmp, s);
-        ld_note_launch(), k_head_flags<<<grid_for(ni, TB), TB, 0, s>>>(b.ds_key, ni, b.flag);
+        ld_note_launch(), k_head_flags<<<grid_for(ni, TB), TB, 0, s>>>(b.ds_key, ni, b.flag, nullptr, 0);
         exclusive_scan_i32_to_i64(b.flag, b.pos, ni, h->scan_tmp, s);
         cudaMemsetAsync(b.ds_uw, 0, (size_t)ni * sizeof(int64_t), s);
         ld_note_launch(), k_unique<<<grid_for(ni, TB), TB, 0, s>>>(b.ds_key, b.ds_w, ni, b.flag, b.pos, b.ds_ukey, b.ds_uw);
@@ -954,14 +1237,13 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
     }
   }
   // ---- Alg. update, then Alg. leidenmk (dS, dR; reset dSigma of refined)
-  cudaMemsetAsync(h->dS, 0, (size_t)n, s);
-  cudaMemsetAsync(h->dR, 0, (size_t)n, s);
   if (nd + ni > 0) {
     ld_note_launch(), k_update_weights<<<grid_for(nd + ni, TB), TB, 0, s>>>(DK, DW, nd, IK, IW, ni, vb, h->C, h->K, h->Sig, h->dSig,
-                                                           cnt, h->gid0, h->gc.m2);
+                                                           cnt, h->gid0, h->gc.m2,
+                                                           mode == LEIDEN_DF ? dV : nullptr);
     ld_note_launch(), k_mark_communities<<<grid_for(nd + ni, TB), TB, 0, s>>>(DK, nd, IK, ni, vb, h->C, h->Sig, h->dSig,
-                                                             h->p.tau_refine, h->dS, h->dR);
-    ld_note_launch(), k_reset_changes<<<grid_for(nd + ni, TB), TB, 0, s>>>(DK, nd, IK, ni, vb, h->C, h->dR, h->dSig);
+                                                             h->p.tau_refine, h->dS, h->dR, cnt);
+    ld_note_launch(), k_reset_changes<<<grid_for(nd + ni, TB), TB, 0, s>>>(DK, nd, IK, ni, vb, h->C, h->dR, h->dSig, cnt);
   }
   // Algorithmic bytes of the batch phase: the edge triples read (12 B per
   // edge); per raw arc its expansion and sort (48 B: key and weight written,

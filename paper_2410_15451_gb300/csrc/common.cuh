@@ -26,17 +26,25 @@ struct SubCounters {
 constexpr int SUB_RING = 16;
 
 struct DevCounters {
+  // a local-moving iteration: dq .. sub are cleared together
   unsigned long long dq[2];       // sum of accepted gains g (int128, two's complement)
   int64_t moves;                  // local-moving moves of the iteration
-  SubCounters sub[SUB_RING];      // (dq .. sub: cleared together)
+  SubCounters sub[SUB_RING];
   SubCounters ref;                // bins of a refinement round or of aggregation
   int32_t accepted;               // refinement moves applied in this round
   int32_t cand_count[2];          // refinement candidate lists (ping-pong)
-  int32_t error;                  // batch validation error (first offending arc + 1)
-  int32_t overflow;               // a touched CSR row outgrew its capacity
+  // error .. refine_marks: cleared together at the start of a call
+  int32_t error;                  // batch validation error
+  int32_t overflow;               // a touched CSR row outgrew its capacity and the spill arena
   int32_t list_count;             // generic list length
-  int32_t ncomm;                  // communities after dense renumbering
   int32_t max_count;              // max degree (level), max community degree
+  int32_t large_count;            // batch apply: touched rows merged in chunks
+  int32_t mid_count;              // batch apply: touched rows merged by one block each
+  int32_t tr_occ;                 // tracking: filled slots of the pair table
+  int32_t tr_flagged;             // tracking: old communities without a majority candidate
+  int32_t hub_big;                // local moving: listed hubs whose tables are read in pieces
+  int32_t max_row;                // batch apply: longest touched row
+  int32_t pad;
   int64_t processed;              // local-moving vertex visits
   int64_t arcs;                   // local-moving arcs scanned
   int64_t ref_processed;          // refinement vertex visits
@@ -44,17 +52,11 @@ struct DevCounters {
   int64_t lmk_visits[3];          // local moving per timed kernel (warp range, block bin, hub scan):
   int64_t lmk_arcs[3];            //   vertex visits, arcs scanned and algorithmic bytes
   int64_t lmk_bytes[3];
-  int64_t m2;                     // 2m (sum of arc weights), device copy
   int64_t sigma_intra;            // modularity: intra-community arc weight
   unsigned long long sq[2];       // modularity: sum of Sigma_c^2 (int128)
   int64_t batch_dw;               // batch: change of 2m
+  int64_t slot_change;            // batch: change of huge_slots by the touched rows
   int64_t huge_slots;             // table slots the vertices above the block bin need
-  int32_t large_count;            // batch apply: touched rows merged in chunks
-  int32_t tr_occ;                 // tracking: filled slots of the pair table
-  int32_t tr_flagged;             // tracking: old communities without a majority candidate
-  int32_t mid_count;              // batch apply: touched rows merged by one block each
-  int32_t hub_big;                // local moving: listed hubs whose tables are read in pieces
-  int64_t arena_used;             // next free arc slot of G^t (relocated rows go here)
   int64_t bcounts[8];             // batch apply: unique deletions, unique insertions, new arcs,
                                   //   touched rows, merge-buffer arcs
   int64_t affected;               // |dV|: vertices flagged affected (counted into the frontier)
@@ -66,6 +68,10 @@ struct DevCounters {
                                   //   giant-community aggregation scan, block merge of touched rows)
   int64_t agg_tables[2];          // aggregation's per-community global tables: [0] hashed, [1] indexed
                                   //   by the key (the table has a slot per community)
+  int64_t refine_marks;           // batch: communities marked for refinement (counted per arc)
+  // kept between calls
+  int64_t m2;                     // 2m (sum of arc weights), device copy
+  int64_t arena_used;             // next free arc slot of G^t (relocated rows go here)
 };
 
 // ---------------------------------------------------------------- checked build

@@ -103,11 +103,12 @@ struct leiden_handle {
   int32_t g_maxdeg = 0;
   int64_t g_huge_slots = 0;
   int64_t m2 = 0;            // 2m = sum of arc weights
+  int64_t batch_dw = 0;      // change of 2m by the batch being applied
 
   // auxiliary state {C, K, Sigma, Delta Sigma}
   int32_t *C = nullptr;
   int64_t *K = nullptr, *Sig = nullptr, *dSig = nullptr;
-  uint8_t *dV = nullptr;
+  uint8_t *dV = nullptr;     // dV, dS, dR: one allocation, cleared together
   bool has_static = false;
   // A call that failed after it began to change the handle's state (a
   // failed allocation or CUDA error mid-call) leaves it broken: every later

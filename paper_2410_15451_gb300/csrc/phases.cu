@@ -1127,7 +1127,6 @@ void reset_next_pass(leiden_handle *h, int64_t ncomm, int out) {
 }
 
 void pass_init(leiden_handle *h, bool sizes_kept) {
-  cudaMemsetAsync(&h->dcnt->affected, 0, sizeof(int64_t), h->stream);
   ld_note_launch(), k_pass_init<<<grid_for(h->n, TB), TB, 0, h->stream>>>(
       h->n, h->dV, h->unproc, h->C, h->Cp, h->Sig, h->Sp, sizes_kept ? h->csize0 : nullptr, h->csize, h->rep, h->dcnt);
   h->Kc = h->K;

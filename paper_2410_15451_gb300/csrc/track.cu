@@ -716,7 +716,6 @@ static void track_narrow(leiden_handle *h, const int32_t *Cnew, const int32_t *r
 // The new ids: the roots of the last level (c < nroot, root[c] == c); of a
 // batched handle the ids flagged in h->dE.
 void track_communities(leiden_handle *h, const int32_t *Cnew, const int32_t *root, int64_t nroot) {
-  cudaMemsetAsync(&h->dcnt->list_count, 0, sizeof(int32_t), h->stream);
   if (!wide_sums(h)) { track_narrow(h, Cnew, root, nroot); return; }
   cudaStream_t s = h->stream;
   if (h->G == 1) count_communities(h, nroot, nullptr);

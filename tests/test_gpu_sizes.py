@@ -62,3 +62,56 @@ def test_ids_at_tile_edges(n, mode):
         assert np.array_equal(gpu.update(d, i, mode[0]), ref.update(d, i, mode[1]))
         cur = synth.apply_batch_numpy(cur, d, i)
         same(gpu, ref)
+
+
+@pytest.mark.parametrize("n_del,n_ins", [(0, 1), (1, 0), (0, 1024), (1, 1023), (512, 512), (1, 1024), (700, 325), (0, 0)])
+def test_batches_at_the_one_block_limit(n_del, n_ins):
+    """2 * (deletions + insertions) arcs up to 2048 are planned by one block, more
+    by the sort's passes: repeated edges, insertions of existing edges, deleted
+    edges inserted again and rows that outgrow their slack on both sides."""
+    g = synth.planted_partition(3000, 30, 12.0, 0.2, 5)
+    src = np.repeat(np.arange(g.n), np.diff(g.off))
+    up = np.flatnonzero(src < g.col)
+    rng = np.random.default_rng(n_del * 4099 + n_ins)
+    for mode in MODES:
+        gpu = L.Leiden(g.n, g.off, g.col, g.w, slack=0.0, min_slack=1)
+        ref = oracle.Oracle(g.n, g.off, g.col, g.w, schedule=oracle.SYNC)
+        gpu.static(), ref.static()
+        e = rng.choice(up, n_del, replace=n_del > 600)
+        d = np.stack([src[e], g.col[e], np.ones(n_del, np.int64)], 1).astype(np.int32)
+        u = rng.integers(0, g.n, n_ins)
+        v = (u + rng.integers(1, g.n, n_ins)) % g.n
+        i = np.stack([u, v, rng.integers(1, 5, n_ins)], 1).astype(np.int32)
+        k = n_ins // 8
+        again = rng.choice(up, k)  # existing edges, some of them deleted above
+        i[:k, 0], i[:k, 1] = src[again], g.col[again]
+        if n_del and k:
+            i[0, :2] = d[0, 1], d[0, 0]
+        i[k:2 * k, 0] = 7  # one row gets an eighth of the insertions
+        i[:, 1] = np.where(i[:, 0] == i[:, 1], (i[:, 1] + 1) % g.n, i[:, 1])
+        assert np.array_equal(gpu.update(d, i, mode[0]), ref.update(d, i, mode[1]))
+        same(gpu, ref)
+
+
+@pytest.mark.parametrize("size", [3, 1500])
+def test_invalid_batches_leave_the_graph(size):
+    """On both sides of the one-block limit: a bad edge among good ones."""
+    g = synth.planted_partition(2000, 20, 10.0, 0.2, 62)
+    gpu = L.Leiden(g.n, g.off, g.col, g.w)
+    gpu.static()
+    before = gpu.state()
+    dels, ins = synth.random_batch(g, size, seed=4)
+    absent = next(v for v in range(1, g.n) if v not in g.col[g.off[0]:g.off[1]])
+    for d, i in [(np.vstack([dels, [[0, absent, 1]]]), ins), (dels, np.vstack([ins, [[3, 3, 1]]])),
+                 (dels, np.vstack([ins, [[1, 2, 0]]])), (dels, np.vstack([ins, [[1, g.n, 1]]])),
+                 (dels, np.vstack([ins, [[-1, 2, 1]]]))]:
+        with pytest.raises(L.LeidenError) as e:
+            gpu.update(d, i, L.LEIDEN_DF)
+        assert e.value.status == L.LEIDEN_ERR_BATCH
+        after = gpu.state()
+        assert all(np.array_equal(before[k], after[k]) for k in ("C", "K", "Sigma", "dSigma"))
+        assert np.array_equal(gpu.graph()[1], g.col)
+    ref = oracle.Oracle(g.n, g.off, g.col, g.w, schedule=oracle.SYNC)
+    ref.static()
+    assert np.array_equal(gpu.update(dels, ins, L.LEIDEN_DF), ref.update(dels, ins, oracle.DF))
+    same(gpu, ref)
