@@ -242,6 +242,44 @@ void sync_all(leiden_handle *h) {
   cudaStreamSynchronize(h->stream);
 }
 
+// Pinned host staging of at least `bytes` (grows geometrically); false if it
+// cannot be had, and the caller copies from pageable memory instead.
+bool ensure_pinned(leiden_handle *h, size_t bytes) {
+  if (bytes <= h->pin_bytes) return true;
+  size_t want = std::max(bytes, 2 * h->pin_bytes);
+  if (h->pin) {
+    cudaStreamSynchronize(h->stream);
+    cudaFreeHost(h->pin);
+    h->pin = nullptr;
+    h->pin_bytes = 0;
+  }
+  if (cudaMallocHost(&h->pin, want) != cudaSuccess) {
+    cudaGetLastError();
+    h->pin = nullptr;
+    return false;
+  }
+  h->pin_bytes = want;
+  return true;
+}
+
+// Where a call's membership goes (host or device pointer, or null).
+struct Output {
+  int32_t *ptr = nullptr;
+  bool device = false;
+  bool staged = false;  // in the pinned buffer, to be copied to ptr after the sync
+};
+
+// The copy of C^t, enqueued before the call's last sync so that the one wait
+// covers it: through the pinned buffer at full link speed, then one host copy.
+leiden_status enqueue_output(leiden_handle *h, Output &o) {
+  if (!o.ptr) return LEIDEN_OK;
+  size_t bytes = (size_t)h->n * sizeof(int32_t);
+  o.staged = !o.device && ensure_pinned(h, bytes);
+  CK(cudaMemcpyAsync(o.staged ? h->pin : (void *)o.ptr, h->C, bytes,
+                     o.device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
+  return LEIDEN_OK;
+}
+
 // Alg. leiden: passes of local moving, subset renumbering, splitting,
 // refinement, then renumbering, lookup and aggregation; finally lookup and
 // tracking.  Expects: Cp = C^{t-1} copy source in h->C, Kp/Sp from h->K,
@@ -251,7 +289,7 @@ void sync_all(leiden_handle *h) {
 // graph keeps its own iteration count and stops iterating when its own dQ
 // reaches tau, keeps its own refinement rounds, and leaves the pass loop at
 // its own break (its final lookup is done then and it is not aggregated).
-leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range, bool dense) {
+leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range, bool dense, Output out) {
   cudaStream_t s = h->stream;
   const leiden_params &p = h->p;
   int64_t N = h->n;
@@ -290,6 +328,7 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range,
   int passes = 0;
   bool looked_up = false;  // batched: every graph had its final lookup
   bool last_first = true;  // no aggregated level yet
+  bool split_unread = false;  // the split's counters come with the next sync
   leiden_stats &st = h->stats;
   int64_t moves_total = 0;
   int64_t subsweep_words = 0;     // frontier words read by the collection kernels
@@ -356,9 +395,15 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range,
     ph_bytes(h, LEIDEN_PHASE_SPLIT, 31 * n);  // smallest members (8 B per vertex, 4 per id), new ids and flags (19 B)
     renumber_and_split(h, g);
     ph_mark(h, LEIDEN_PHASE_REFINE);
-    ph_bytes(h, LEIDEN_PHASE_REFINE, 29 * n);  // bounds C'_B, reset of the refined bounds
-    if (B) CK(cudaMemsetAsync(h->gc.refined, 0, (size_t)G, s));
-    refine_reset(h, g);
+    // a batch that marked no community for refinement (read with the last
+    // iteration's counters) has nothing to reset or propose in the first pass:
+    // one round without candidates, by definition
+    const bool refine = lp > 0 || !dynamic || h->hcnt->refine_marks != 0;
+    ph_bytes(h, LEIDEN_PHASE_REFINE, refine ? 29 * n : 8);  // bounds C'_B, reset of the refined bounds; or the mark
+    if (refine) {
+      if (B) CK(cudaMemsetAsync(h->gc.refined, 0, (size_t)G, s));
+      refine_reset(h, g);
+    }
     int rounds = 0;
     int refined_any = 0;
     // Both modes repeat rounds until no move applies: in the in-place mode a
@@ -366,7 +411,7 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range,
     // A graph of a batch counts the rounds up to its first round without a
     // move (its state does not change after that).
     int max_rounds = p.max_iterations;
-    for (int r = 0; r < max_rounds; r++) {
+    for (int r = 0; refine && r < max_rounds; r++) {
       if (B) CK(cudaMemsetAsync(h->gc.accepted, 0, (size_t)G * sizeof(int32_t), s));
       refine_round(h, g, r & 1);
       rounds++;
@@ -384,10 +429,17 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range,
       }
       if (h->hcnt->accepted == 0) break;
     }
+    if (!refine) {
+      rounds = 1;
+      if (B)
+        for (int gi = 0; gi < G; gi++)
+          if (!refdone[gi]) rounds_g[gi] = 1;
+    }
     tr[3] = refined_any;
     tr[4] = rounds;
     // listed vertices (parent, list, compress: 24 B) and their arcs (col, C: 8 B)
-    ph_bytes(h, LEIDEN_PHASE_SPLIT, 24 * (int64_t)h->hcnt->split_count + 8 * h->hcnt->split_arcs);
+    if (refine) ph_bytes(h, LEIDEN_PHASE_SPLIT, 24 * (int64_t)h->hcnt->split_count + 8 * h->hcnt->split_arcs);
+    split_unread = !refine;
     ph_mark(h, LEIDEN_PHASE_AGGREGATE);
     ph_bytes(h, LEIDEN_PHASE_AGGREGATE, 4 * n);  // community count
     if (B) {  // (one graph: counted by the renumbering, or by tracking in the last pass)
@@ -450,6 +502,8 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range,
     sync_counters(h);
     CK(cudaGetLastError());
     CKF();
+    if (split_unread) ph_bytes(h, LEIDEN_PHASE_SPLIT, 24 * (int64_t)h->hcnt->split_count + 8 * h->hcnt->split_arcs);
+    split_unread = false;
     {
       // dense renumbering (36 B per vertex), lookup (12 B per vertex of G),
       // community-vertex lists (56 B per vertex), per community offsets,
@@ -487,9 +541,13 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range,
   track_communities(h, !B && last_first ? h->Cp : h->Ctop, h->Cp, g.n);
   ph_mark(h, PHASE_END);
   release_agg_buffers(h);
-  sync_counters(h);
+  if (leiden_status e = enqueue_output(h, out)) return e;
+  cudaMemcpyAsync(h->hcnt, h->dcnt, sizeof(DevCounters), cudaMemcpyDeviceToHost, s);
+  CK(cudaStreamSynchronize(s));
   CK(cudaGetLastError());
+  if (out.staged) memcpy(out.ptr, h->pin, (size_t)N * sizeof(int32_t));
   ph_resolve(h);
+  if (split_unread) ph_bytes(h, LEIDEN_PHASE_SPLIT, 24 * (int64_t)h->hcnt->split_count + 8 * h->hcnt->split_arcs);
   if (unsigned int code = check_word_move() | check_word_phases() | check_word_track()) {
     h->err = "a device-side check of the checked build failed (code " + std::to_string(code) + ")";
     return LEIDEN_ERR_STATE;
@@ -530,43 +588,8 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range,
   return LEIDEN_OK;
 }
 
-// Pinned host staging of at least `bytes` (grows geometrically); false if it
-// cannot be had, and the caller copies from pageable memory instead.
-bool ensure_pinned(leiden_handle *h, size_t bytes) {
-  if (bytes <= h->pin_bytes) return true;
-  size_t want = std::max(bytes, 2 * h->pin_bytes);
-  if (h->pin) {
-    cudaStreamSynchronize(h->stream);
-    cudaFreeHost(h->pin);
-    h->pin = nullptr;
-    h->pin_bytes = 0;
-  }
-  if (cudaMallocHost(&h->pin, want) != cudaSuccess) {
-    cudaGetLastError();
-    h->pin = nullptr;
-    return false;
-  }
-  h->pin_bytes = want;
-  return true;
-}
-
-leiden_status finish_call(leiden_handle *h, int32_t *out, bool device_out) {
-  cudaStream_t s = h->stream;
-  size_t bytes = (size_t)h->n * sizeof(int32_t);
-  if (out && !device_out && ensure_pinned(h, bytes)) {
-    // device -> pinned at full link speed, then one host copy
-    CK(cudaMemcpyAsync(h->pin, h->C, bytes, cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    memcpy(out, h->pin, bytes);
-    return LEIDEN_OK;
-  }
-  if (out) CK(cudaMemcpyAsync(out, h->C, bytes, device_out ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  return LEIDEN_OK;
-}
-
 leiden_status do_update(leiden_handle *h, const leiden_edge *d_del, int64_t n_del, const leiden_edge *d_ins,
-                        int64_t n_ins, leiden_mode mode) {
+                        int64_t n_ins, leiden_mode mode, Output out) {
   h->stats = leiden_stats{};
   h->ph_used = 0;
   kt_reset(h);
@@ -586,7 +609,7 @@ leiden_status do_update(leiden_handle *h, const leiden_edge *d_del, int64_t n_de
   h->m2 += h->batch_dw;
   // a DF batch marks at most the two ends of each of its edges
   bool dense = mode != LEIDEN_DF || 16 * (n_del + n_ins) > h->n;
-  st = run_leiden(h, 1, mode == LEIDEN_DS ? h->dV : nullptr, dense);
+  st = run_leiden(h, 1, mode == LEIDEN_DS ? h->dV : nullptr, dense, out);
   if (st != LEIDEN_OK) {
     h->broken = true;
     release_agg_buffers(h);
@@ -960,14 +983,14 @@ leiden_status leiden_static(leiden_handle *h, int32_t *membership_out) {
   }
   h->g_maxdeg = h->hcnt->max_count;
   h->g_huge_slots = h->hcnt->huge_slots;
-  st = run_leiden(h, 0, nullptr, true);
+  st = run_leiden(h, 0, nullptr, true, Output{membership_out});
   if (st != LEIDEN_OK) {
     h->broken = true;
     release_agg_buffers(h);
     return st;
   }
   h->has_static = true;
-  return finish_call(h, membership_out, false);
+  return LEIDEN_OK;
 }
 
 leiden_status leiden_update(leiden_handle *h, const leiden_edge *del, int64_t n_del, const leiden_edge *ins,
@@ -979,33 +1002,32 @@ leiden_status leiden_update(leiden_handle *h, const leiden_edge *del, int64_t n_
     h->err = "invalid batch arguments";
     return LEIDEN_ERR_ARG;
   }
-  // stage the host batch in device memory (upload buffers grow on demand)
-  int64_t need = std::max<int64_t>(std::max(n_del, n_ins), 1);
+  // stage the host batch in device memory, deletions then insertions (the
+  // upload buffer grows on demand, geometrically: a freed one stalls the device)
+  int64_t need = std::max<int64_t>(n_del + n_ins, 1);
   if (need > h->up_cap) {
-    need = std::max<int64_t>(need, 2 * h->up_cap);  // geometric growth (fewer device-wide frees)
+    need = std::max<int64_t>(need, 2 * h->up_cap);
     for (auto &q : h->owned)
-      if (q && (q == h->up_del || q == h->up_ins)) { cudaFree(q); q = nullptr; }
-    h->up_del = h->up_ins = nullptr;
+      if (q && q == h->up) { cudaFree(q); q = nullptr; }
+    h->up = nullptr;
     h->up_cap = 0;
-    CK(dalloc(h, &h->up_del, need));
-    CK(dalloc(h, &h->up_ins, need));
+    CK(dalloc(h, &h->up, need));
     h->up_cap = need;
   }
-  leiden_edge *dd = h->up_del, *di = h->up_ins;
+  leiden_edge *dd = h->up, *di = h->up + n_del;
   size_t bd = (size_t)n_del * sizeof(leiden_edge), bi = (size_t)n_ins * sizeof(leiden_edge);
   CK(cudaStreamSynchronize(h->stream));  // the pinned buffer may still feed an earlier copy
   if (ensure_pinned(h, bd + bi)) {
-    // host -> pinned, then one asynchronous copy each at full link speed
+    // host -> pinned, then one asynchronous copy at full link speed
     char *pp = (char *)h->pin;
-    if (n_del) { memcpy(pp, del, bd); CK(cudaMemcpyAsync(dd, pp, bd, cudaMemcpyHostToDevice, h->stream)); }
-    if (n_ins) { memcpy(pp + bd, ins, bi); CK(cudaMemcpyAsync(di, pp + bd, bi, cudaMemcpyHostToDevice, h->stream)); }
+    if (n_del) memcpy(pp, del, bd);
+    if (n_ins) memcpy(pp + bd, ins, bi);
+    if (bd + bi) CK(cudaMemcpyAsync(dd, pp, bd + bi, cudaMemcpyHostToDevice, h->stream));
   } else {
     if (n_del) CK(cudaMemcpyAsync(dd, del, bd, cudaMemcpyHostToDevice, h->stream));
     if (n_ins) CK(cudaMemcpyAsync(di, ins, bi, cudaMemcpyHostToDevice, h->stream));
   }
-  st = do_update(h, dd, n_del, di, n_ins, mode);
-  if (st != LEIDEN_OK) return st;
-  return finish_call(h, membership_out, false);
+  return do_update(h, dd, n_del, di, n_ins, mode, Output{membership_out});
 }
 
 leiden_status leiden_update_device(leiden_handle *h, const leiden_edge *del, int64_t n_del, const leiden_edge *ins,
@@ -1017,9 +1039,7 @@ leiden_status leiden_update_device(leiden_handle *h, const leiden_edge *del, int
     h->err = "invalid batch arguments";
     return LEIDEN_ERR_ARG;
   }
-  st = do_update(h, del, n_del, ins, n_ins, mode);
-  if (st != LEIDEN_OK) return st;
-  return finish_call(h, membership_out, true);
+  return do_update(h, del, n_del, ins, n_ins, mode, Output{membership_out, true});
 }
 
 leiden_status leiden_modularity(leiden_handle *h, const int32_t *membership, double *q_out) {

@@ -183,7 +183,7 @@ struct leiden_handle {
   std::vector<int64_t> gtrace;        // host per-graph traces, G x (2 + 10*25)
 
   BatchBuffers b;
-  leiden_edge *up_del = nullptr, *up_ins = nullptr;  // staging of host batches
+  leiden_edge *up = nullptr;  // staging of host batches: deletions, then insertions
   int64_t up_cap = 0;
   void *pin = nullptr;      // pinned host staging: batches in, membership out
   size_t pin_bytes = 0;
