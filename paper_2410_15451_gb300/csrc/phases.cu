@@ -378,18 +378,6 @@ __global__ void k_yoff(int64_t ncomm, const int64_t *coff, const int64_t *cflat,
   }
 }
 
-__device__ __forceinline__ void agg_insert(int32_t *keys, int64_t *vals, int tmask, int32_t c, int64_t w) {
-  uint32_t s = ld_hash32((uint32_t)c) & (uint32_t)tmask;
-  for (uint32_t probe = 0; ld_ok(probe <= (uint32_t)tmask, LD_CHK_PROBE); probe++) {
-    int32_t k = atomicCAS(&keys[s], LD_EMPTY_KEY, c);
-    if (k == LD_EMPTY_KEY || k == c) {
-      atomicAdd((unsigned long long *)&vals[s], (unsigned long long)w);
-      return;
-    }
-    s = (s + 1) & (uint32_t)tmask;
-  }
-}
-
 struct AggArgs {
   int64_t ncomm;
   const int64_t *off;
@@ -434,50 +422,26 @@ __device__ __forceinline__ int agg_member_of(const int64_t *ms, int nb, int64_t 
   return lo;
 }
 
-template <int GROUP>
-// Emit the table as the super-row of c and leave every slot empty again.
-__device__ __forceinline__ void agg_emit(const AggArgs &A, int64_t c, int t0, int stride, int32_t *keys,
-                                         int64_t *vals, int T, int32_t *rowcount, int64_t *rowsum) {
-  int64_t base = A.yoff[c];
-  for (int s = t0; s < T; s += stride) {
-    int32_t k = keys[s];
-    if (k == LD_EMPTY_KEY) continue;
-    int64_t v = vals[s];
-    keys[s] = LD_EMPTY_KEY;
-    vals[s] = 0;
-    int32_t p = atomicAdd(rowcount, 1);
-    A.ycol[base + p] = k;
-    A.yw[base + p] = v;
-    atomicAdd((unsigned long long *)rowsum, (unsigned long long)v);
-  }
-}
-
 constexpr int AGG_WARPS = 8;
-constexpr int AGG_WARP_TABLE = 256;
-constexpr int AGG_BLOCK_TABLE = 2048;
 
 // Communities of at most BIN_WARP_MAX flat arcs, a warp each: the warp
 // holds 32 members at a time in registers (lane i the i-th), and a lane
-// finds the member of its flat arc with five shuffles.
-template <typename W>
+// finds the member of its flat arc with five shuffles.  The table lists its
+// filled slots, so the super-row is the list (no table to clear or scan, no
+// counter to place an entry: R-MAT 21, static: 1065 -> 534 us), and K is
+// the sum of the arcs read.
+template <typename W, bool WIDE>
 __global__ void __launch_bounds__(AGG_WARPS * 32) k_agg_warp(AggArgs A) {
-  __shared__ int32_t skeys[AGG_WARPS][AGG_WARP_TABLE];
-  __shared__ int64_t svals[AGG_WARPS][AGG_WARP_TABLE];
-  __shared__ int32_t scount[AGG_WARPS];
-  __shared__ int64_t ssum[AGG_WARPS];
+  __shared__ WarpTable<WIDE> WT[AGG_WARPS];
   const W *w = (const W *)A.w;
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  WarpTable<WIDE> &T = WT[wid];
+  wt_init(T);
   int64_t count = *A.count;
   for (int64_t t = (int64_t)blockIdx.x * AGG_WARPS + wid; t < count; t += (int64_t)gridDim.x * AGG_WARPS) {
     int64_t c = A.list[t];
-    int64_t dg = A.yoff[c + 1] - A.yoff[c];
-    int T = 32;
-    while (T < 2 * dg) T <<= 1;
-    for (int s = lane; s < T; s += 32) { skeys[wid][s] = LD_EMPTY_KEY; svals[wid][s] = 0; }
-    if (lane == 0) { scount[wid] = 0; ssum[wid] = 0; }
-    __syncwarp();
     int64_t m0 = A.coff[c], m1 = A.coff[c + 1];
-    int64_t selfw = 0;  // arcs inside the community: summed in registers, added once
+    int64_t selfw = 0, ksum = 0;  // arcs inside the community: summed in registers, added once
     for (int64_t ab = m0; ab < m1; ab += 32) {  // warp-uniform
       int nb = m1 - ab < 32 ? (int)(m1 - ab) : 32;
       int64_t s = 0, r = 0;
@@ -510,18 +474,34 @@ __global__ void __launch_bounds__(AGG_WARPS * 32) k_agg_warp(AggArgs A) {
         for (int u = 0; u < AGG_UNROLL; u++) cj[u] = valid[u] ? A.C[j[u]] : -1;
 #pragma unroll
         for (int u = 0; u < AGG_UNROLL; u++) {
+          ksum += wa[u];
           if (cj[u] == (int32_t)c) selfw += wa[u];
-          else if (valid[u]) agg_insert(skeys[wid], svals[wid], T - 1, cj[u], wa[u]);
+          else if (valid[u]) st_insert(T, &T.count, cj[u], wa[u]);
         }
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) selfw += __shfl_xor_sync(LD_FULL, selfw, o);
-    if (lane == 0 && selfw) agg_insert(skeys[wid], svals[wid], T - 1, (int32_t)c, selfw);
+    ksum = ld_warp_sum_i64(ksum);
+    selfw = ld_warp_sum_i64(selfw);
     __syncwarp();
-    agg_emit<32>(A, c, lane, 32, skeys[wid], svals[wid], T, &scount[wid], &ssum[wid]);
+    const int n = T.count;
+    const int64_t base = A.yoff[c];
+    for (int q = lane; q < n; q += 32) {
+      int32_t key;
+      int64_t v;
+      st_take(T, q, key, v);
+      A.ycol[base + q] = key;
+      A.yw[base + q] = v;
+    }
     __syncwarp();
-    if (lane == 0) { A.ydeg[c] = scount[wid]; A.Kout[c] = ssum[wid]; }
+    if (lane == 0) {
+      if (selfw) {
+        A.ycol[base + n] = (int32_t)c;
+        A.yw[base + n] = selfw;
+      }
+      A.ydeg[c] = n + (selfw != 0);
+      A.Kout[c] = ksum;
+      T.count = 0;
+    }
     __syncwarp();
   }
 }
@@ -591,29 +571,26 @@ __global__ void __launch_bounds__(256) k_agg_tiny(AggArgs A) {
 }
 
 // Communities of BIN_WARP_MAX+1..BIN_BLOCK_MAX flat arcs, a block each, with
-// the members staged AGG_MB at a time in shared memory.
-template <typename W>
+// the members staged AGG_MB at a time in shared memory and a listed table as
+// above (R-MAT 21, static, level 0: 2748 -> 722 us).
+template <typename W, bool WIDE>
 __global__ void __launch_bounds__(256) k_agg_block(AggArgs A) {
-  __shared__ int32_t keys[AGG_BLOCK_TABLE];
-  __shared__ int64_t vals[AGG_BLOCK_TABLE];
+  __shared__ STable<WIDE, STAGE_SLOTS, STAGE_FILL, uint16_t> T;
+  __shared__ int32_t filled;
+  __shared__ unsigned long long self_s, sum_s;
   __shared__ int64_t ms[AGG_MB + 1];
   __shared__ int64_t mr[AGG_MB];
-  __shared__ int32_t rc;
-  __shared__ int64_t rs;
   const W *w = (const W *)A.w;
   int64_t count = *A.count;
+  st_clear(T, threadIdx.x, 256, STAGE_SLOTS);
+  if (threadIdx.x == 0) { filled = 0; self_s = 0; sum_s = 0; }
   for (int64_t t = blockIdx.x; t < count; t += gridDim.x) {
     int64_t c = A.list[t];
-    int64_t dg = A.yoff[c + 1] - A.yoff[c];
-    int T = 32;
-    while (T < 2 * dg) T <<= 1;
-    for (int s = threadIdx.x; s < T; s += blockDim.x) { keys[s] = LD_EMPTY_KEY; vals[s] = 0; }
-    if (threadIdx.x == 0) { rc = 0; rs = 0; }
     int64_t m0 = A.coff[c], m1 = A.coff[c + 1];
-    int64_t selfw = 0;  // arcs inside the community: summed in registers, added once per warp
+    int64_t selfw = 0, ksum = 0;  // arcs inside the community: summed in registers, added once per warp
     for (int64_t ab = m0; ab < m1; ab += AGG_MB) {  // block-uniform
       int nb = m1 - ab < AGG_MB ? (int)(m1 - ab) : AGG_MB;
-      __syncthreads();  // the table is cleared and the previous batch has been read
+      __syncthreads();  // the previous batch has been read
       if ((int)threadIdx.x < nb) {
         int64_t s = A.cflat[ab + threadIdx.x];
         ms[threadIdx.x] = s;
@@ -643,18 +620,41 @@ __global__ void __launch_bounds__(256) k_agg_block(AggArgs A) {
         for (int u = 0; u < AGG_UNROLL; u++) cj[u] = valid[u] ? A.C[j[u]] : -1;
 #pragma unroll
         for (int u = 0; u < AGG_UNROLL; u++) {
+          ksum += wa[u];
           if (cj[u] == (int32_t)c) selfw += wa[u];
-          else if (valid[u]) agg_insert(keys, vals, T - 1, cj[u], wa[u]);
+          else if (valid[u]) st_insert(T, &filled, cj[u], wa[u]);
         }
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) selfw += __shfl_xor_sync(LD_FULL, selfw, o);
-    if ((threadIdx.x & 31) == 0 && selfw) agg_insert(keys, vals, T - 1, (int32_t)c, selfw);
+    ksum = ld_warp_sum_i64(ksum);
+    selfw = ld_warp_sum_i64(selfw);
+    if ((threadIdx.x & 31) == 0) {
+      if (ksum) atomicAdd(&sum_s, (unsigned long long)ksum);
+      if (selfw) atomicAdd(&self_s, (unsigned long long)selfw);
+    }
     __syncthreads();
-    agg_emit<256>(A, c, threadIdx.x, blockDim.x, keys, vals, T, &rc, &rs);
+    const int n = filled;
+    const int64_t base = A.yoff[c];
+    for (int q = threadIdx.x; q < n; q += 256) {
+      int32_t key;
+      int64_t v;
+      st_take(T, q, key, v);
+      A.ycol[base + q] = key;
+      A.yw[base + q] = v;
+    }
     __syncthreads();
-    if (threadIdx.x == 0) { A.ydeg[c] = rc; A.Kout[c] = rs; }
+    if (threadIdx.x == 0) {
+      int64_t sw = (int64_t)self_s;
+      if (sw) {
+        A.ycol[base + n] = (int32_t)c;
+        A.yw[base + n] = sw;
+      }
+      A.ydeg[c] = n + (sw != 0);
+      A.Kout[c] = (int64_t)sum_s;
+      filled = 0;
+      self_s = 0;
+      sum_s = 0;
+    }
     __syncthreads();
   }
 }
@@ -1084,13 +1084,16 @@ void aggregate(leiden_handle *h, const LevelGraph &g, int64_t ncomm, int out) {
   else ld_note_launch(), k_agg_tiny<int32_t><<<sms * 8, 256, 0, s>>>(A);
   A.list = h->bins;
   A.count = &h->dcnt->ref.bin_count[BIN_WARP];
-  if (g.w64) ld_note_launch(), k_agg_warp<int64_t><<<sms * 8, AGG_WARPS * 32, 0, s>>>(A);
-  else ld_note_launch(), k_agg_warp<int32_t><<<sms * 8, AGG_WARPS * 32, 0, s>>>(A);
+  const bool wide = wide_sums(h);
+  auto agg_warp = wide ? (g.w64 ? k_agg_warp<int64_t, true> : k_agg_warp<int32_t, true>)
+                       : (g.w64 ? k_agg_warp<int64_t, false> : k_agg_warp<int32_t, false>);
+  ld_note_launch(), agg_warp<<<sms * 8, AGG_WARPS * 32, 0, s>>>(A);
   if (maxc > BIN_WARP_MAX) {
     A.list = h->bins + ncomm;
     A.count = &h->dcnt->ref.bin_count[BIN_BLOCK];
-    if (g.w64) ld_note_launch(), k_agg_block<int64_t><<<sms * 4, 256, 0, s>>>(A);
-    else ld_note_launch(), k_agg_block<int32_t><<<sms * 4, 256, 0, s>>>(A);
+    auto agg_block = wide ? (g.w64 ? k_agg_block<int64_t, true> : k_agg_block<int32_t, true>)
+                          : (g.w64 ? k_agg_block<int64_t, false> : k_agg_block<int32_t, false>);
+    ld_note_launch(), agg_block<<<sms * 8, 256, 0, s>>>(A);
   }
   if (maxc > BIN_BLOCK_MAX) {
     // a table per listed community at once: at most huge_slots slots
@@ -1108,13 +1111,13 @@ void aggregate(leiden_handle *h, const LevelGraph &g, int64_t ncomm, int out) {
     A.xk_bytes = &h->dcnt->xk_bytes[1];
     A.tables = h->dcnt->agg_tables;
     kt_begin(h, KT_AGG_CHUNK);
-    auto scan = wide_sums(h) ? (g.w64 ? k_agg_chunk_scan<int64_t, true> : k_agg_chunk_scan<int32_t, true>)
+    auto scan = wide ? (g.w64 ? k_agg_chunk_scan<int64_t, true> : k_agg_chunk_scan<int32_t, true>)
                              : (g.w64 ? k_agg_chunk_scan<int64_t, false> : k_agg_chunk_scan<int32_t, false>);
     ld_note_launch(), scan<<<sms * 16, 256, 0, s>>>(A, tab_off, ch_off);
     kt_end(h);
     int64_t *em_off = h->lbuf0;  // free again after the member fill
     ld_note_launch(), k_emit_plan<<<1, 1024, 0, s>>>(A.count, A.gocc, em_off);
-    auto emit = wide_sums(h) ? k_agg_list_emit<true> : k_agg_list_emit<false>;
+    auto emit = wide ? k_agg_list_emit<true> : k_agg_list_emit<false>;
     ld_note_launch(), emit<<<sms * 8, 256, 0, s>>>(A, tab_off, em_off);
   }
 }
