@@ -125,7 +125,7 @@ typedef struct {
    * degree; per arc read 8 B: col, C of the neighbour), [1] the chunked scan
    * of communities above 1024 member arcs in aggregation (per arc: col, C of
    * the neighbour and the weight), [2] the block merge of touched rows of
-   * 257..4096 arcs (per arc: the old row read and the new row written,
+   * 1025..4096 arcs (per arc: the old row read and the new row written,
    * 16 B; per batch arc 16 B). */
   int64_t xk_launches[3];
   int64_t xk_bytes[3];

@@ -9,9 +9,13 @@
 namespace {
 
 constexpr int TB = 256;
-constexpr int MERGE_SMALL = 256;  // touched rows up to this new length merge in one warp (8 KB of
-                                  // shared staging per block keeps many rows in flight)
-constexpr int MERGE_MID = 4096;   // up to this length: one block, staged in shared memory, in place
+// Touched rows by new length: a warp with 2 KB of shared staging, a warp with
+// 8 KB, a block with 32 KB, and above that chunks over all SMs.  A row is a chain
+// of dependent loads (its plan, its place, the row), so what counts is how many
+// are in flight: 64, 28 and 7 per SM.
+constexpr int MERGE_SMALL = 256;
+constexpr int MERGE_WARP = 1024;
+constexpr int MERGE_MID = 4096;
 
 __device__ __forceinline__ int64_t lower_bound_i32(const int32_t *a, int64_t n, int32_t x) {
   int64_t lo = 0, hi = n;
@@ -199,7 +203,7 @@ __device__ __forceinline__ int64_t hub_slots(int64_t d, int block_max) {
 struct RowPlan {
   int32_t *dlo, *dhi, *ilo, *ihi;
   int64_t *len, *dst;
-  int32_t *newcap, *olddeg, *large, *mid;
+  int32_t *newcap, *olddeg, *large, *mid, *warp;
 };
 
 // Plan of touched row r = vertex u: its segments in the two arc lists, its new
@@ -219,7 +223,8 @@ __device__ __forceinline__ int64_t plan_row(const BatchGraph &G, const RowPlan &
   P.len[r] = L;
   P.olddeg[r] = dg;
   if (L > MERGE_MID) P.large[atomicAdd(&cnt->large_count, 1)] = (int32_t)r;
-  else if (L > MERGE_SMALL) P.mid[atomicAdd(&cnt->mid_count, 1)] = (int32_t)r;
+  else if (L > MERGE_WARP) P.mid[atomicAdd(&cnt->mid_count, 1)] = (int32_t)r;
+  else if (L > MERGE_SMALL) P.warp[atomicAdd(&cnt->warp_count, 1)] = (int32_t)r;
   if (L > G.rcap[u] && !invalid) {
     int64_t extra = (int64_t)((double)L * G.slack);
     if (extra < G.min_slack) extra = G.min_slack;
@@ -498,10 +503,9 @@ __global__ void k_merge_rows(const int32_t *rows, const int64_t *nrows_p, int vb
 
 // In-place merge of the touched rows that fit their capacity (no overflow).
 // Output position of an old element x at p: p - |D < x| + |I < x|; of the
-// k-th new arc y: k + |row < y| - |D < y|.  Rows of at most MERGE_SMALL
-// arcs are merged by one warp through shared memory, longer rows by one
-// block through the global merge buffer; each writes back after all its
-// reads are done, so the old row is never overwritten while still read.
+// k-th new arc y: k + |row < y| - |D < y|.  Everything before the first change
+// stays where it is (unless the row is relocated); the rest is staged in
+// shared memory and written back after all of the row's reads.
 constexpr int MERGE_WARPS = 4;
 
 struct MergeArgs {
@@ -528,7 +532,9 @@ __device__ __forceinline__ void finish_row(const MergeArgs &A, int64_t r, int32_
   }
 }
 
-// D, I: the row's deletion keys and new-arc keys (global or staged copies).
+// Rows of at most MERGE_SMALL arcs, a warp each, moved whole: the search for the
+// first change and the registers of the longer rows' form below cost more than
+// the row (R-MAT 22: 60 us, with that form 92).
 __device__ __forceinline__ void merge_row_into(const MergeArgs &A, int64_t r, int t0, int stride, int32_t *ocol,
                                                int32_t *ow, const uint64_t *D, const uint64_t *I) {
   uint64_t mask = (1ull << A.vb) - 1;
@@ -577,8 +583,118 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32) k_merge_small(MergeArgs A) {
   }
 }
 
-// Rows of MERGE_SMALL..MERGE_MID arcs: one block each, staged in shared
-// memory and written back after all of the row's reads.
+// Most rows get a handful of arcs: up to MERGE_FEW of either kind are held one
+// per lane and counted with shuffles, more are searched.
+constexpr int MERGE_FEW = 8;
+constexpr int MERGE_UNROLL = 4;
+
+// Row r merged by `threads` threads (whole warps; t0: the thread's index) into
+// the stage from its first changed position on (0 for a row that moves).
+// Returns its vertex; first: that position.
+__device__ __forceinline__ int32_t merge_tail(const MergeArgs &A, int64_t r, int t0, int threads, int32_t *scol,
+                                              int32_t *sw, int &first) {
+  const int lane = threadIdx.x & 31;
+  const uint64_t mask = (1ull << A.vb) - 1;
+  const int32_t u = A.rows[r];
+  const int64_t b = A.off[u];
+  const int dg = A.deg[u], nD = A.dhi[r] - A.dlo[r], nI = A.ihi[r] - A.ilo[r];
+  const int32_t *row = A.col + b, *roww = A.w + b;
+  const uint64_t *D = A.dkey + A.dlo[r], *I = A.nkey + A.ilo[r];
+  const int64_t *IW = A.nw + A.ilo[r];
+  const uint64_t ubase = (uint64_t)u << A.vb;
+  const bool few = nD <= MERGE_FEW && nI <= MERGE_FEW, one = threads == 32;
+  const int32_t dv = lane < nD ? (int32_t)(D[lane] & mask) : 0, iv = lane < nI ? (int32_t)(I[lane] & mask) : 0;
+  const int64_t iw = lane < nI ? IW[lane] : 0;
+  int below = 0;  // (few, one warp) row elements below this lane's new arc
+  first = 0;
+  if (!A.newcap[r]) {
+    int32_t x = __shfl_sync(LD_FULL, nD ? dv : iv, 0);
+    if (nD && nI) x = min(x, __shfl_sync(LD_FULL, iv, 0));
+    first = (int)lower_bound_i32(row, dg, x);
+    below = first;
+  }
+  for (int p0 = first + (t0 & ~31); p0 < dg; p0 += threads * MERGE_UNROLL) {  // warp-uniform
+    int32_t x[MERGE_UNROLL], xw[MERGE_UNROLL];
+#pragma unroll
+    for (int q = 0; q < MERGE_UNROLL; q++) {
+      int p = p0 + q * threads + lane;
+      x[q] = p < dg ? row[p] : INT32_MAX;
+      xw[q] = p < dg ? roww[p] : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < MERGE_UNROLL; q++) {
+      if (p0 + q * threads >= dg) break;  // warp-uniform
+      int p = p0 + q * threads + lane;
+      int dless = 0, iless = 0;
+      bool gone = false;
+      if (few) {
+        for (int k = 0; k < nD; k++) {
+          int32_t y = __shfl_sync(LD_FULL, dv, k);
+          dless += y < x[q];
+          gone = gone || y == x[q];
+        }
+        for (int k = 0; k < nI; k++) {
+          int32_t y = __shfl_sync(LD_FULL, iv, k);
+          iless += y < x[q];
+          int c = __popc(__ballot_sync(LD_FULL, x[q] < y));
+          if (lane == k) below += c;
+        }
+      } else if (p < dg) {
+        const uint64_t key = ubase | (uint64_t)x[q];
+        dless = (int)lower_bound_u64(D, nD, key);
+        gone = dless < nD && D[dless] == key;
+        iless = (int)lower_bound_u64(I, nI, key);
+      }
+      if (p < dg && !gone) {
+        int o = p - dless + iless - first;
+        scol[o] = x[q];
+        sw[o] = xw[q];
+      }
+    }
+  }
+  if (few && one) {
+    int dless = 0;
+    for (int k = 0; k < nD; k++) dless += __shfl_sync(LD_FULL, dv, k) < iv;
+    if (lane < nI) {
+      int o = lane + below - dless - first;
+      scol[o] = iv;
+      sw[o] = (int32_t)iw;
+    }
+    return u;
+  }
+  for (int k = t0; k < nI; k += threads) {
+    int32_t y = (int32_t)(I[k] & mask);
+    int o = k + (int)lower_bound_i32(row, dg, y) - (int)lower_bound_u64(D, nD, ubase | (uint64_t)y) - first;
+    scol[o] = y;
+    sw[o] = (int32_t)IW[k];
+  }
+  return u;
+}
+
+// Rows of MERGE_SMALL+1..MERGE_WARP arcs, a warp each.  With a block each (and a
+// search of both arc lists per element), these and the block's rows took 277 us
+// (R-MAT 22, 64,154 edges); now 55 and 88.
+__global__ void __launch_bounds__(MERGE_WARPS * 32) k_merge_warp(MergeArgs A, const int32_t *list,
+                                                                 const int32_t *count_p) {
+  __shared__ int32_t scol[MERGE_WARPS][MERGE_WARP];
+  __shared__ int32_t sw[MERGE_WARPS][MERGE_WARP];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t count = *count_p;
+  for (int64_t k = (int64_t)blockIdx.x * MERGE_WARPS + wid; k < count; k += (int64_t)gridDim.x * MERGE_WARPS) {
+    const int64_t r = list[k];
+    const int64_t L = A.len[r];
+    int first;
+    const int32_t u = merge_tail(A, r, lane, 32, scol[wid], sw[wid], first);
+    __syncwarp();
+    const int64_t o = A.dst[r] + first;
+    const int n = (int)L - first;
+    for (int x = lane; x < n; x += 32) { A.col[o + x] = scol[wid][x]; A.w[o + x] = sw[wid][x]; }
+    if (lane == 0) finish_row(A, r, u, L);
+    __syncwarp();
+  }
+}
+
+// Rows of MERGE_WARP+1..MERGE_MID arcs: one block each.
 __global__ void __launch_bounds__(256) k_merge_mid(MergeArgs A, const int32_t *mid, const int32_t *count_p,
                                                    int64_t *xk_bytes) {
   __shared__ int32_t scol[MERGE_MID];
@@ -588,12 +704,14 @@ __global__ void __launch_bounds__(256) k_merge_mid(MergeArgs A, const int32_t *m
   for (int64_t k = blockIdx.x; k < count; k += gridDim.x) {
     int64_t r = mid[k];
     int64_t L = A.len[r];
-    int32_t u = A.rows[r];
-    if (threadIdx.x == 0) bytes += 8 * ((int64_t)A.deg[u] + L) + 16 * (A.dhi[r] - A.dlo[r] + A.ihi[r] - A.ilo[r]);
-    merge_row_into(A, r, threadIdx.x, blockDim.x, scol, sw, A.dkey + A.dlo[r], A.nkey + A.ilo[r]);
+    if (threadIdx.x == 0)
+      bytes += 8 * ((int64_t)A.deg[A.rows[r]] + L) + 16 * (A.dhi[r] - A.dlo[r] + A.ihi[r] - A.ilo[r]);
+    int first;
+    const int32_t u = merge_tail(A, r, threadIdx.x, 256, scol, sw, first);
     __syncthreads();
-    int64_t o = A.dst[r];
-    for (int64_t x = threadIdx.x; x < L; x += blockDim.x) { A.col[o + x] = scol[x]; A.w[o + x] = sw[x]; }
+    const int64_t o = A.dst[r] + first;
+    const int n = (int)L - first;
+    for (int x = threadIdx.x; x < n; x += 256) { A.col[o + x] = scol[x]; A.w[o + x] = sw[x]; }
     if (threadIdx.x == 0) finish_row(A, r, u, L);
     __syncthreads();
   }
@@ -609,11 +727,7 @@ __global__ void __launch_bounds__(256) k_merge_chunks_write(MergeArgs A, const i
   int64_t nch = ch_off[count];
   uint64_t mask = (1ull << A.vb) - 1;
   for (int64_t t = blockIdx.x; t < nch; t += gridDim.x) {
-    int64_t lo = 0, hi = count - 1;
-    while (lo < hi) {
-      int64_t mid = (lo + hi + 1) >> 1;
-      if (ch_off[mid] <= t) lo = mid; else hi = mid - 1;
-    }
+    int64_t lo = ld_chunk_item(ch_off, count, t);
     int64_t r = large[lo];
     int32_t u = A.rows[r];
     const int32_t *row = A.col + A.off[u];
@@ -658,11 +772,7 @@ __global__ void __launch_bounds__(256) k_merge_chunks_copy(MergeArgs A, const in
   int64_t count = *count_p;
   int64_t nch = ch_off[count];
   for (int64_t t = blockIdx.x; t < nch; t += gridDim.x) {
-    int64_t lo = 0, hi = count - 1;
-    while (lo < hi) {
-      int64_t mid = (lo + hi + 1) >> 1;
-      if (ch_off[mid] <= t) lo = mid; else hi = mid - 1;
-    }
+    int64_t lo = ld_chunk_item(ch_off, count, t);
     int64_t r = large[lo];
     int64_t L = A.len[r];
     int64_t c = t - ch_off[lo];
@@ -955,7 +1065,7 @@ cudaError_t ensure_batch(leiden_handle *h, int64_t edges) {
                    (void **)&nb.ins_state, (void **)&nb.ins_pos, (void **)&nb.rows, (void **)&nb.row_dlo,
                    (void **)&nb.row_dhi, (void **)&nb.row_ilo, (void **)&nb.row_ihi, (void **)&nb.row_len,
                    (void **)&nb.row_tmp_off, (void **)&nb.row_dst, (void **)&nb.row_newcap, (void **)&nb.row_olddeg,
-                   (void **)&nb.row_large, (void **)&nb.row_mid, (void **)&nb.ds_key, (void **)&nb.ds_key_alt,
+                   (void **)&nb.row_large, (void **)&nb.row_mid, (void **)&nb.row_warp, (void **)&nb.ds_key, (void **)&nb.ds_key_alt,
                    (void **)&nb.ds_w, (void **)&nb.ds_w_alt, (void **)&nb.ds_ukey, (void **)&nb.ds_uw};
   // dkey, dkey_alt, iw, iw_alt, flag and pos hold the deletion and insertion
   // arcs of one sort together (2 * arcs); ikey, ikey_alt and iw_alt's unique part
@@ -965,7 +1075,7 @@ cudaError_t ensure_batch(leiden_handle *h, int64_t edges) {
                     4 * (size_t)arcs, 8 * (size_t)arcs, 4 * (size_t)rows, 4 * (size_t)rows, 4 * (size_t)rows,
                     4 * (size_t)rows, 4 * (size_t)rows, 8 * (size_t)(rows + 1), 8 * (size_t)(rows + 1),
                     8 * (size_t)(rows + 1), 4 * (size_t)(rows + 1), 4 * (size_t)(rows + 1), 4 * (size_t)(rows + 1),
-                    4 * (size_t)(rows + 1), 8 * (size_t)arcs, 8 * (size_t)arcs, 8 * (size_t)arcs, 8 * (size_t)arcs,
+                    4 * (size_t)(rows + 1), 4 * (size_t)(rows + 1), 8 * (size_t)arcs, 8 * (size_t)arcs, 8 * (size_t)arcs, 8 * (size_t)arcs,
                     8 * (size_t)arcs, 8 * (size_t)arcs};
   constexpr int NB = sizeof(slot) / sizeof(slot[0]);
   static_assert(NB == sizeof(bytes) / sizeof(bytes[0]), "one size per batch buffer");
@@ -1103,7 +1213,7 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
   BatchGraph G{n, h->g_off, h->g_deg, h->g_rcap, h->g_col, h->g_w, h->gid0, h->g_cap, h->p.slack, h->p.min_slack,
                h->tune.block_max, vb};
   RowPlan P{b.row_dlo, b.row_dhi, b.row_ilo, b.row_ihi, b.row_len, b.row_dst, b.row_newcap, b.row_olddeg, b.row_large,
-            b.row_mid};
+            b.row_mid, b.row_warp};
   if (nda + nia == 0) {
   } else if (nda + nia <= SMALL_ARCS) {
     SmallOut O{DK, IK, NK, DW, IW, NW, b.ins_pos, b.row_tmp_off, b.ins_state, b.rows};
@@ -1154,7 +1264,8 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
       // short rows on the handle's stream, mid rows and long rows on its
       // side streams, joined before the marking below
       const bool some_mid = h->hcnt->mid_count > 0, some_long = h->hcnt->large_count > 0,
-                 some_small = nrows > (int64_t)h->hcnt->mid_count + h->hcnt->large_count;
+                 some_warp = h->hcnt->warp_count > 0,
+                 some_small = nrows > (int64_t)h->hcnt->mid_count + h->hcnt->large_count + h->hcnt->warp_count;
       bool fork = (some_mid || some_long) && h->tune.overlap && side_streams(h);
       cudaStream_t smid = s, slong = s;
       if (fork) {
@@ -1164,8 +1275,13 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
         if (some_mid) cudaStreamWaitEvent(smid, h->fork_ev, 0);
         if (some_long) cudaStreamWaitEvent(slong, h->fork_ev, 0);
       }
-      if (some_small) ld_note_launch(), k_merge_small<<<grid_for((nrows + MERGE_WARPS - 1) / MERGE_WARPS, 1, h->sm_count * 16), MERGE_WARPS * 32, 0,
-                      s>>>(M);
+      if (some_warp)
+        ld_note_launch(), k_merge_warp<<<
+            grid_for((h->hcnt->warp_count + MERGE_WARPS - 1) / MERGE_WARPS, 1, h->sm_count * 7), MERGE_WARPS * 32, 0, s>>>(
+            M, b.row_warp, &cnt->warp_count);
+      if (some_small)
+        ld_note_launch(), k_merge_small<<<grid_for((nrows + MERGE_WARPS - 1) / MERGE_WARPS, 1, h->sm_count * 16),
+                                          MERGE_WARPS * 32, 0, s>>>(M);
       if (some_mid) {
         kt_begin(h, KT_MERGE_MID, smid);
         ld_note_launch(), k_merge_mid<<<h->sm_count * 7, 256, 0, smid>>>(M, b.row_mid, &cnt->mid_count,  // 32 KB: 7 per SM

@@ -70,6 +70,7 @@ struct BatchBuffers {
   int32_t *row_olddeg = nullptr;                         // degree of the row before the batch
   int32_t *row_large = nullptr;                          // touched rows merged in chunks
   int32_t *row_mid = nullptr;                            // touched rows merged by one block each
+  int32_t *row_warp = nullptr;                           // touched rows merged by one warp with a large stage
   uint64_t *ds_key = nullptr, *ds_key_alt = nullptr, *ds_ukey = nullptr;  // DS (src, C[dst]) pairs
   int64_t *ds_w = nullptr, *ds_w_alt = nullptr, *ds_uw = nullptr;
   int64_t *counts = nullptr;                             // device counts of the batch pipeline (in DevCounters)

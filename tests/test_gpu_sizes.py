@@ -115,3 +115,39 @@ def test_invalid_batches_leave_the_graph(size):
     ref.static()
     assert np.array_equal(gpu.update(dels, ins, L.LEIDEN_DF), ref.update(dels, ins, oracle.DF))
     same(gpu, ref)
+
+
+@pytest.mark.parametrize("arcs_each", [1, 8, 9, 40])
+def test_rows_merged_at_every_class_limit(arcs_each):
+    """Rows that end at a merge class's limit (256, 1024, 4096 arcs), with few and
+    many batch arcs each, changed at the front, in the middle and at the end, in
+    place and relocated."""
+    lengths = [250, 256, 257, 1000, 1024, 1025, 4090, 4096, 4097, 5000]
+    n = 6000
+    hubs = {10 + 500 * k: m for k, m in enumerate(lengths)}
+    edges = set()
+    for h, m in hubs.items():
+        others = [v for v in range(n) if v not in hubs][:m]
+        edges |= {(min(h, v), max(h, v)) for v in others}
+    from tests.helpers import csr_from_edges
+
+    off, col, w = csr_from_edges(n, sorted(edges))
+    rng = np.random.default_rng(arcs_each)
+    for slack in (dict(slack=0.25, min_slack=64), dict(slack=0.0, min_slack=0)):
+        gpu = L.Leiden(n, off, col, w.astype(np.int32), **slack)
+        ref = oracle.Oracle(n, off, col, w.astype(np.int32), schedule=oracle.SYNC)
+        gpu.static(), ref.static()
+        d, i = [], []
+        for h, m in hubs.items():
+            row = col[off[h]:off[h + 1]]
+            gone = [int(row[0]), int(row[-1])] + rng.choice(row, arcs_each).tolist()
+            d += [(h, v, 1) for v in gone[:arcs_each]]
+            there = set(row.tolist())
+            absent = [v for v in range(n - 1, 0, -1) if v not in hubs and v not in there][:arcs_each]
+            i += [(h, v, 2) for v in absent] + [(h, gone[0], 3)]  # one comes back with another weight
+        for mode in MODES[2:]:
+            assert np.array_equal(gpu.update(d, i, mode[0]), ref.update(d, i, mode[1]))
+            same(gpu, ref)
+            i2 = [(u, v, x) for u, v, x in i]
+            assert np.array_equal(gpu.update(i2, [], mode[0]), ref.update(i2, [], mode[1]))  # all taken out again
+            same(gpu, ref)
