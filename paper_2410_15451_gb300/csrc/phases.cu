@@ -145,6 +145,57 @@ __global__ void k_split_sample(const int32_t *list, DevCounters *cnt, const int6
   if (lane == 0 && bytes) atomicAdd((unsigned long long *)&cnt->xk_bytes[0], (unsigned long long)bytes);
 }
 
+// The same links in two steps, for graphs above SPLIT_APART vertices: a thread
+// per vertex finds its two neighbours, four arcs at a time; then the links of
+// every eighth listed vertex, a flattening, and the links of the others, which
+// by then mostly find in two loads that their ends agree.  In the form above
+// the lanes of a warp wait for each other's chains of lookups; this one pays
+// two more sweeps and more failed hooks.  Sampling and linking together:
+// R-MAT 22 (2.4M listed) 376 us above, 334 here; R-MAT 20 (650k) 70 and 101, the
+// web-like graph (777k vertices) 101 and 143.
+constexpr int64_t SPLIT_APART = (int64_t)1 << 21;
+constexpr int SPLIT_WINDOW = 4;   // arcs loaded at once
+__global__ void __launch_bounds__(256) k_split_find(const int32_t *list, DevCounters *cnt, const int64_t *off,
+                                                    const int32_t *deg, const int32_t *col, const int32_t *C,
+                                                    int2 *hit) {
+  int64_t m = cnt->split_count;
+  int64_t bytes = 0;  // algorithmic bytes: per vertex 20, per arc read 8
+  for (int64_t t = ld_gtid(); t < m; t += ld_gstride()) {
+    int32_t i = list[t], c = C[i];
+    int64_t b = off[i];
+    int d = deg[i] < SPLIT_SAMPLE_SCAN ? deg[i] : SPLIT_SAMPLE_SCAN, a = 0;
+    int2 h = make_int2(-1, -1);
+    while (a < d && h.y < 0) {
+      int32_t j[SPLIT_WINDOW], cj[SPLIT_WINDOW];
+#pragma unroll
+      for (int u = 0; u < SPLIT_WINDOW; u++) j[u] = a + u < d ? col[b + a + u] : i;
+#pragma unroll
+      for (int u = 0; u < SPLIT_WINDOW; u++) cj[u] = j[u] != i ? C[j[u]] : -1;
+#pragma unroll
+      for (int u = 0; u < SPLIT_WINDOW; u++)
+        if (cj[u] == c) {
+          if (h.x < 0) h.x = j[u];
+          else if (h.y < 0) h.y = j[u];
+        }
+      a += SPLIT_WINDOW;
+    }
+    hit[t] = h;
+    bytes += 20 + 8 * (a < d ? a : d);
+  }
+  bytes = ld_warp_sum_i64(bytes);
+  if ((threadIdx.x & 31) == 0 && bytes) atomicAdd((unsigned long long *)&cnt->xk_bytes[0], (unsigned long long)bytes);
+}
+__global__ void __launch_bounds__(256) k_split_link(const int32_t *list, const DevCounters *cnt, int32_t *parent,
+                                                    const int2 *hit, bool rest) {
+  int64_t m = cnt->split_count, k = rest ? (m >> 3) * 7 + (m & 7 ? (m & 7) - 1 : 0) : (m + 7) >> 3;
+  for (int64_t q = ld_gtid(); q < k; q += ld_gstride()) {
+    int64_t t = rest ? q + q / 7 + 1 : q << 3;  // the q-th t with t % 8 != 0, or == 0
+    int2 h = hit[t];
+    if (h.x >= 0) uf_unite(parent, list[t], h.x);
+    if (h.y >= 0) uf_unite(parent, list[t], h.y);
+  }
+}
+
 __global__ void k_split_flatten(const int32_t *list, const DevCounters *cnt, int32_t *parent) {
   int64_t m = cnt->split_count;
   for (int64_t t = ld_gtid(); t < m; t += ld_gstride()) {
@@ -996,7 +1047,16 @@ void renumber_and_split(leiden_handle *h, const LevelGraph &g) {
                                                                             h->dR2, h->parent, list, h->dcnt,
                                                                             h->p.split_all);
   kt_begin(h, KT_SPLIT_SAMPLE);
-  ld_note_launch(), k_split_sample<<<h->sm_count * 16, TB, 0, s>>>(list, h->dcnt, g.off, g.deg, g.col, h->Cp, h->parent);
+  if (g.n <= SPLIT_APART) {
+    ld_note_launch(), k_split_sample<<<h->sm_count * 16, TB, 0, s>>>(list, h->dcnt, g.off, g.deg, g.col, h->Cp,
+                                                                     h->parent);
+  } else {
+    int2 *hit = (int2 *)h->lbuf0;
+    ld_note_launch(), k_split_find<<<h->sm_count * 8, 256, 0, s>>>(list, h->dcnt, g.off, g.deg, g.col, h->Cp, hit);
+    ld_note_launch(), k_split_link<<<h->sm_count * 4, 256, 0, s>>>(list, h->dcnt, h->parent, hit, false);
+    ld_note_launch(), k_split_flatten<<<h->sm_count * 8, TB, 0, s>>>(list, h->dcnt, h->parent);
+    ld_note_launch(), k_split_link<<<h->sm_count * 8, 256, 0, s>>>(list, h->dcnt, h->parent, hit, true);
+  }
   kt_end(h);
   ld_note_launch(), k_split_flatten<<<h->sm_count * 8, TB, 0, s>>>(list, h->dcnt, h->parent);
   ld_note_launch(), k_split_link_rest<<<h->sm_count * 8, TB, 0, s>>>(list, h->dcnt, g.off, g.deg, g.col, h->Cp, h->parent, h->ibuf2);
