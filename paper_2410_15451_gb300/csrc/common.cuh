@@ -593,6 +593,16 @@ __device__ __forceinline__ int64_t ld_chunk_item(const int64_t *ch_off, int64_t 
   return lo;
 }
 
+// ---------------------------------------------------------------- programmatic launches
+// A kernel launched by launch_after (internal.h) may start while the kernel
+// before it on the stream still runs; it calls this before it touches memory:
+// the wait ends when that kernel has completed and its writes are visible.  It
+// first lets the kernel after itself start (and wait) in turn.
+__device__ __forceinline__ void ld_after_previous() {
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
+}
+
 // Grid-stride helpers.
 __device__ __forceinline__ int64_t ld_gtid() { return (int64_t)blockIdx.x * blockDim.x + threadIdx.x; }
 __device__ __forceinline__ int64_t ld_gstride() { return (int64_t)gridDim.x * blockDim.x; }

@@ -263,6 +263,23 @@ unsigned int check_word_phases();
 unsigned int check_word_track();
 unsigned int check_selftest(cudaStream_t s);
 
+// Launch of a kernel that begins with ld_after_previous(): its blocks are
+// scheduled while the kernel before it on the stream drains, which hides most of
+// the launch latency in chains of short kernels.
+template <typename... P, typename... A>
+inline void launch_after(void (*kernel)(P...), int grid, int block, cudaStream_t s, const A &...args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // ------------------------------------------------------------ prims.cu
 // Exclusive scan of n values; out[n] receives the total.  `tmp` must hold
 // scan_tmp_bytes(n) bytes.  in == out is allowed.

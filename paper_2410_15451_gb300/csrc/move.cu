@@ -460,9 +460,11 @@ __device__ __forceinline__ void warp_step(const Args &A, int32_t i, int lane, Wa
 template <typename W, int KIND, bool WIDE>
 __global__ void __launch_bounds__(WARPS_PER_BLOCK * 32, 4) k_decide_warp(Args A) {
   __shared__ WarpTable<WIDE> WT[WARPS_PER_BLOCK];
+  ld_after_previous();
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int64_t ntiny = *A.count_tiny, nwarp = *A.count;
   int64_t ngroups = (ntiny + 3) / 4, total = ngroups + nwarp;
+  if ((int64_t)blockIdx.x * WARPS_PER_BLOCK >= total) return;
   int64_t gw = (int64_t)blockIdx.x * WARPS_PER_BLOCK + wid, nw = (int64_t)gridDim.x * WARPS_PER_BLOCK;
   wt_init(WT[wid]);
   Tally tl;
@@ -502,12 +504,13 @@ __global__ void __launch_bounds__(BLOCK_THREADS) k_decide_block(Args A) {
   __shared__ BlockStage<WIDE> S;
   __shared__ BestX sb[BLOCK_THREADS / 32];
   __shared__ int moved_s;
+  const int64_t count = *A.count;
+  if (blockIdx.x >= count) return;
   st_clear(S, threadIdx.x, BLOCK_THREADS, STAGE_SLOTS);
   if (threadIdx.x < 2) S.count[threadIdx.x] = 0;
   __syncthreads();
   const W *w = (const W *)A.w;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  int64_t count = *A.count;
   int64_t visits = 0, arcs = 0, moves = 0;
   i128 dq = 0;
   int par = 0;
@@ -641,10 +644,11 @@ __global__ void __launch_bounds__(256) k_huge_scan(Args A, const int64_t *tab_of
   // own community and one more are summed in registers, as in the other bins.
   __shared__ WarpTable<WIDE> WT[8];
   WarpTable<WIDE> &T8 = WT[threadIdx.x >> 5];
-  wt_init(T8);
   const int lane = threadIdx.x & 31;
   int64_t count = *A.count;
   int64_t nch = ch_off[count];
+  if (blockIdx.x >= nch) return;
+  wt_init(T8);
   for (int64_t t = blockIdx.x; t < nch; t += gridDim.x) {
     int64_t lo = ld_chunk_item(ch_off, count, t);
     int64_t i = A.list[lo];
@@ -994,6 +998,7 @@ __device__ __forceinline__ void apply_moves(const Args &A, unsigned long long *d
 // before; Q.cls < 0: there is none after.
 template <bool DENSE>
 __global__ void __launch_bounds__(256) k_apply_collect(Args A, bool apply, unsigned long long *dqg, int64_t *movesg, CollectArgs Q) {
+  ld_after_previous();
   if (apply) apply_moves(A, dqg, movesg);
   if (Q.cls < 0) return;
   if (DENSE) collect_dense(A, Q);
@@ -1062,6 +1067,7 @@ __global__ void __launch_bounds__(256) k_refine_collect(const int32_t *cand_in, 
                                                         const int32_t *C, const int64_t *S, const int64_t *K,
                                                         const int32_t *deg, int32_t *prop, int32_t *bins,
                                                         SubCounters *sub, leiden_tuning tn) {
+  ld_after_previous();
   __shared__ BlockAppend<NBINS + 1> B;
   int32_t *const lengths[NBINS + 1] = {&sub->bin_count[0], &sub->bin_count[1], &sub->bin_count[2], &sub->bin_count[3],
                                        count_out};
@@ -1105,6 +1111,7 @@ __device__ __forceinline__ bool holds(const int32_t *prop, int32_t v) {
 }
 __global__ void k_refine_accept(const int32_t *cand, const int32_t *count, const int32_t *prop, int32_t *C, int64_t *S,
                                 const int64_t *K, DevCounters *cnt, const int32_t *gid, int32_t *accg) {
+  ld_after_previous();
   int64_t m = *count;
   int32_t acc = 0;
   for (int64_t t0 = (ld_gtid() & ~31ll); t0 < m; t0 += ld_gstride()) {  // warp-uniform trip count
@@ -1222,9 +1229,10 @@ void launch_bins_of(leiden_handle *h, const LevelGraph &g, Args A) {
     A.list_tiny = h->bins + (int64_t)BIN_TINY * g.n;
     A.count_tiny = &A.sub->bin_count[BIN_TINY];
     bin(BIN_WARP);
-    int grid = sms * h->tune.warp_blocks_per_sm;  // default 4: one wave at four resident blocks per SM
+    // default 4: one wave at four resident blocks per SM (a level of few vertices needs less)
+    int grid = grid_for(g.n, WARPS_PER_BLOCK, sms * h->tune.warp_blocks_per_sm);
     if (KIND == KIND_MOVE) kt_begin(h, KT_WARP);
-    ld_note_launch(), k_decide_warp<W, KIND, WIDE><<<grid, WARPS_PER_BLOCK * 32, 0, s>>>(A);
+    ld_note_launch(), launch_after(k_decide_warp<W, KIND, WIDE>, grid, WARPS_PER_BLOCK * 32, s, A);
     if (KIND == KIND_MOVE) kt_end(h);
   }
   if (need_block) {
@@ -1351,12 +1359,12 @@ void lm_iteration(leiden_handle *h, const LevelGraph &g, const uint8_t *in_range
       if (pending) {
         CollectArgs none = Q;
         none.cls = -1;
-        ld_note_launch(), kernel<<<grid, 256, 0, s>>>(A, true, h->gc.dq, h->gc.moves, none);
+        ld_note_launch(), launch_after(kernel, grid, 256, s, A, true, h->gc.dq, h->gc.moves, none);
         pending = false;
       }
       cudaMemsetAsync(h->dcnt->sub, 0, sizeof(h->dcnt->sub), s);
     }
-    ld_note_launch(), kernel<<<grid, 256, 0, s>>>(A, pending, h->gc.dq, h->gc.moves, Q);
+    ld_note_launch(), launch_after(kernel, grid, 256, s, A, pending, h->gc.dq, h->gc.moves, Q);
     A.sub = Q.sub;
     launch_bins<KIND_MOVE>(h, g, A);
     if (deferred && g.maxdeg > h->tune.block_max && g.maxdeg > MARK_INLINE)
@@ -1365,7 +1373,7 @@ void lm_iteration(leiden_handle *h, const LevelGraph &g, const uint8_t *in_range
   }
   if (pending) {
     Q.cls = -1;
-    ld_note_launch(), kernel<<<h->sm_count * 4, 256, 0, s>>>(A, true, h->gc.dq, h->gc.moves, Q);
+    ld_note_launch(), launch_after(kernel, std::min(grid, h->sm_count * 4), 256, s, A, true, h->gc.dq, h->gc.moves, Q);
   }
 }
 
@@ -1386,13 +1394,12 @@ void refine_round(leiden_handle *h, const LevelGraph &g, int slot) {
   static_assert(offsetof(DevCounters, accepted) == offsetof(DevCounters, ref) + sizeof(SubCounters), "cleared together");
   cudaMemsetAsync(&h->dcnt->ref, 0, sizeof(SubCounters) + sizeof(int32_t), s);  // bins, accepted
   cudaMemsetAsync(cout, 0, sizeof(int32_t), s);
-  ld_note_launch(), k_refine_collect<<<grid_for(g.n, APPEND_STEP), 256, 0, s>>>(in, cin, out, cout, g.n, h->Cp, h->Sp,
-                                                                                h->Kc, g.deg, h->prop, h->bins,
-                                                                                &h->dcnt->ref, h->tune);
+  ld_note_launch(), launch_after(k_refine_collect, grid_for(g.n, APPEND_STEP), 256, s, in, cin, out, cout, g.n, h->Cp,
+                                 h->Sp, h->Kc, g.deg, h->prop, h->bins, &h->dcnt->ref, h->tune);
   Args A = make_args(h, g);
   launch_bins<KIND_REFINE>(h, g, A);
-  ld_note_launch(), k_refine_accept<<<h->sm_count * 4, 256, 0, s>>>(out, cout, h->prop, h->Cp, h->Sp, h->Kc, h->dcnt,
-                                                                     g.gid, h->gc.accepted);
+  ld_note_launch(), launch_after(k_refine_accept, grid_for(g.n, 256, h->sm_count * 4), 256, s, out, cout, h->prop, h->Cp,
+                                 h->Sp, h->Kc, h->dcnt, g.gid, h->gc.accepted);
 }
 
 LD_CHECK_WORD_READER(check_word_move)

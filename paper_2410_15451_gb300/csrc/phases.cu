@@ -17,6 +17,7 @@ constexpr int TB = 256;
 // competes while it is below the value already there (a plain read first
 // spares most atomics).
 __global__ void k_sr_min(int64_t n, const int32_t *C, int32_t *rep) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) {
     int32_t c = C[i];
     if ((int32_t)i < rep[c]) atomicMin(&rep[c], (int32_t)i);
@@ -34,6 +35,7 @@ __global__ void k_sr_min(int64_t n, const int32_t *C, int32_t *rep) {
 __global__ void __launch_bounds__(256) k_remap_list(int64_t n, const int32_t *rep, const uint8_t *dS,
                                                     const uint8_t *dR, const int32_t *deg, int32_t *C, uint8_t *dR2,
                                                     int32_t *parent, int32_t *list, DevCounters *cnt, int split_all) {
+  ld_after_previous();
   __shared__ BlockAppend<1> B;
   int32_t *const lengths[1] = {&cnt->split_count};
   int64_t arcs = 0;  // arcs of the listed vertices (work counter)
@@ -99,6 +101,7 @@ constexpr int SPLIT_LANES = 4;  // lanes per vertex; each reads two arcs of a wi
 // holding the first SPLIT_SAMPLES same-community neighbours link.
 __global__ void k_split_sample(const int32_t *list, DevCounters *cnt, const int64_t *off, const int32_t *deg,
                                const int32_t *col, const int32_t *C, int32_t *parent) {
+  ld_after_previous();
   int64_t m = cnt->split_count;
   int lane = threadIdx.x & 31, grp = lane / SPLIT_LANES, sub = lane % SPLIT_LANES;
   constexpr int GROUPS = 32 / SPLIT_LANES;
@@ -197,6 +200,7 @@ __global__ void __launch_bounds__(256) k_split_link(const int32_t *list, const D
 }
 
 __global__ void k_split_flatten(const int32_t *list, const DevCounters *cnt, int32_t *parent) {
+  ld_after_previous();
   int64_t m = cnt->split_count;
   for (int64_t t = ld_gtid(); t < m; t += ld_gstride()) {
     int32_t i = list[t];
@@ -212,6 +216,7 @@ __global__ void k_split_flatten(const int32_t *list, const DevCounters *cnt, int
 constexpr int SPLIT_BIG = 2048;  // longer rows go to the block kernel
 __global__ void k_split_link_rest(const int32_t *list, DevCounters *cnt, const int64_t *off, const int32_t *deg,
                                   const int32_t *col, const int32_t *C, int32_t *parent, int32_t *big) {
+  ld_after_previous();
   int lane = threadIdx.x & 31;
   int64_t m = cnt->split_count;
   // 32 listed vertices per warp: the root lookups run a lane each, then the
@@ -259,6 +264,7 @@ __global__ void __launch_bounds__(1024) k_split_link_big(const int32_t *big, con
 }
 
 __global__ void k_split_compress(const int32_t *list, const DevCounters *cnt, int32_t *parent, int32_t *C) {
+  ld_after_previous();
   int64_t m = cnt->split_count;
   for (int64_t t = ld_gtid(); t < m; t += ld_gstride()) {
     int32_t i = list[t];
@@ -1042,27 +1048,27 @@ void renumber_and_split(leiden_handle *h, const LevelGraph &g) {
                 "cleared together");
   cudaMemsetAsync(&h->dcnt->split_arcs, 0, sizeof(int64_t) + 2 * sizeof(int32_t), s);
   int32_t *list = h->ibuf1;
-  ld_note_launch(), k_sr_min<<<grid_for(g.n, TB), TB, 0, s>>>(g.n, h->Cp, h->rep);
-  ld_note_launch(), k_remap_list<<<grid_for(g.n, APPEND_STEP), 256, 0, s>>>(g.n, h->rep, h->dS, h->dR, g.deg, h->Cp,
+  ld_note_launch(), launch_after(k_sr_min, grid_for(g.n, TB), TB, s, g.n, h->Cp, h->rep);
+  ld_note_launch(), launch_after(k_remap_list, grid_for(g.n, APPEND_STEP), 256, s, g.n, h->rep, h->dS, h->dR, g.deg, h->Cp,
                                                                             h->dR2, h->parent, list, h->dcnt,
                                                                             h->p.split_all);
   kt_begin(h, KT_SPLIT_SAMPLE);
   if (g.n <= SPLIT_APART) {
-    ld_note_launch(), k_split_sample<<<h->sm_count * 16, TB, 0, s>>>(list, h->dcnt, g.off, g.deg, g.col, h->Cp,
+    ld_note_launch(), launch_after(k_split_sample, h->sm_count * 16, TB, s, list, h->dcnt, g.off, g.deg, g.col, h->Cp,
                                                                      h->parent);
   } else {
     int2 *hit = (int2 *)h->lbuf0;
     ld_note_launch(), k_split_find<<<h->sm_count * 8, 256, 0, s>>>(list, h->dcnt, g.off, g.deg, g.col, h->Cp, hit);
     ld_note_launch(), k_split_link<<<h->sm_count * 4, 256, 0, s>>>(list, h->dcnt, h->parent, hit, false);
-    ld_note_launch(), k_split_flatten<<<h->sm_count * 8, TB, 0, s>>>(list, h->dcnt, h->parent);
+    ld_note_launch(), launch_after(k_split_flatten, h->sm_count * 8, TB, s, list, h->dcnt, h->parent);
     ld_note_launch(), k_split_link<<<h->sm_count * 8, 256, 0, s>>>(list, h->dcnt, h->parent, hit, true);
   }
   kt_end(h);
-  ld_note_launch(), k_split_flatten<<<h->sm_count * 8, TB, 0, s>>>(list, h->dcnt, h->parent);
-  ld_note_launch(), k_split_link_rest<<<h->sm_count * 8, TB, 0, s>>>(list, h->dcnt, g.off, g.deg, g.col, h->Cp, h->parent, h->ibuf2);
+  ld_note_launch(), launch_after(k_split_flatten, h->sm_count * 8, TB, s, list, h->dcnt, h->parent);
+  ld_note_launch(), launch_after(k_split_link_rest, h->sm_count * 8, TB, s, list, h->dcnt, g.off, g.deg, g.col, h->Cp, h->parent, h->ibuf2);
   if (g.maxdeg > SPLIT_BIG)
     ld_note_launch(), k_split_link_big<<<h->sm_count, 1024, 0, s>>>(h->ibuf2, h->dcnt, g.off, g.deg, g.col, h->Cp, h->parent);
-  ld_note_launch(), k_split_compress<<<h->sm_count * 8, TB, 0, s>>>(list, h->dcnt, h->parent, h->Cp);
+  ld_note_launch(), launch_after(k_split_compress, h->sm_count * 8, TB, s, list, h->dcnt, h->parent, h->Cp);
 }
 
 void count_communities(leiden_handle *h, int64_t n, const int32_t *gid) {

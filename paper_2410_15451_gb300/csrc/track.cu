@@ -230,6 +230,7 @@ __device__ __forceinline__ int32_t tr_id(unsigned long long x) { return (int32_t
 // carry their own id (isolated ones, mostly) do not pass through it.
 __global__ void __launch_bounds__(256) k_tn_cand(int64_t N, const int32_t *Cold, const int32_t *Cnew, int32_t *cand,
                                                  uint32_t *dev, unsigned long long *match, DevCounters *cnt) {
+  ld_after_previous();
   __shared__ int32_t seen[TR_FILTER];
   for (int t = threadIdx.x; t < TR_FILTER; t += 256) seen[t] = -1;
   __syncthreads();
@@ -261,6 +262,7 @@ __global__ void __launch_bounds__(256) k_tn_cand(int64_t N, const int32_t *Cold,
 // Weight of the members whose new label differs from the candidate.
 __global__ void __launch_bounds__(256) k_tn_deviants(int64_t N, const int32_t *Cold, const int32_t *Cnew,
                                                      const int64_t *K, const int32_t *cand, uint32_t *dev) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < N; i += ld_gstride()) {
     int32_t o = Cold[i];
     if (Cnew[i] != cand[o]) {
@@ -276,6 +278,7 @@ __global__ void __launch_bounds__(256) k_tn_majority(int64_t N, const int32_t *s
                                                      const int64_t *tot, const uint32_t *dev, int32_t *choice,
                                                      unsigned long long *match, uint32_t *bits, int32_t *flagged,
                                                      unsigned long long *best, DevCounters *cnt) {
+  ld_after_previous();
   const int lane = threadIdx.x & 31;
   for (int64_t o0 = (ld_gtid() & ~31ll); o0 < N; o0 += ld_gstride()) {  // warp-uniform
     int64_t o = o0 + lane;
@@ -309,6 +312,7 @@ __global__ void __launch_bounds__(256) k_tn_insert(int64_t N, const int32_t *Col
                                                    const int64_t *K, const int64_t *tot, const uint32_t *bits,
                                                    unsigned long long *best, int64_t cap, uint64_t *keys,
                                                    int64_t *vals, int32_t *list, DevCounters *cnt) {
+  ld_after_previous();
   if (cnt->tr_flagged == 0) return;
   uint64_t mask = (uint64_t)cap - 1;
   int lane = threadIdx.x & 31;
@@ -357,6 +361,7 @@ __global__ void __launch_bounds__(256) k_tn_insert(int64_t N, const int32_t *Col
 // The flagged communities' best pairs, leaving the table empty.
 __global__ void k_tn_best(const DevCounters *cnt, const int32_t *list, uint64_t *keys, int64_t *vals,
                           unsigned long long *best) {
+  ld_after_previous();
   int64_t m = cnt->tr_occ;
   for (int64_t t = ld_gtid(); t < m; t += ld_gstride()) {
     int32_t sl = list[t];
@@ -368,6 +373,7 @@ __global__ void k_tn_best(const DevCounters *cnt, const int32_t *list, uint64_t 
 }
 __global__ void k_tn_match(const DevCounters *cnt, const int32_t *flagged, const unsigned long long *best,
                            int32_t *choice, unsigned long long *match) {
+  ld_after_previous();
   int64_t m = cnt->tr_flagged;
   for (int64_t t = ld_gtid(); t < m; t += ld_gstride()) {
     int32_t o = flagged[t];
@@ -394,6 +400,7 @@ constexpr int TR_STEP = 1024, TR_TILES_MAX = 4096;
 __global__ void __launch_bounds__(256) k_tn_tiles(int64_t N, int tile, const uint8_t *used, const int32_t *root,
                                                   int64_t nroot, const unsigned long long *match, const int32_t *size,
                                                   int2 *tiles, DevCounters *cnt) {
+  ld_after_previous();
   __shared__ int su, sf, sr;
   if (threadIdx.x == 0) su = sf = sr = 0;
   __syncthreads();
@@ -423,6 +430,7 @@ __global__ void __launch_bounds__(256) k_tn_lists(int64_t N, int tile, const uin
                                                   int64_t nroot, const unsigned long long *match, const int32_t *size,
                                                   const int2 *tiles, int32_t *rank, int32_t *freel,
                                                   const int32_t *gid0, const int64_t *voff, int2 *granks) {
+  ld_after_previous();
   __shared__ int2 wsum[4][8];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int pu = 0, pf = 0;  // in the tiles before this one
@@ -482,6 +490,7 @@ __global__ void __launch_bounds__(256) k_tn_relabel(int64_t N, const int32_t *Cn
                                                     const int32_t *rank, const int32_t *freel, const int32_t *choice,
                                                     const int64_t *K, int32_t *C, int64_t *Sig, int32_t *size,
                                                     int64_t *dSig, const int32_t *gid0, const int2 *granks) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < N; i += ld_gstride()) {
     int32_t ch = choice[i];
     if (ch < 0 || tr_id(match[ch]) != (int32_t)i) dSig[i] = 0;
@@ -712,20 +721,20 @@ static void track_narrow(leiden_handle *h, const int32_t *Cnew, const int32_t *r
   int2 *tiles = (int2 *)h->lbuf2, *granks = (int2 *)h->lbuf3;
   const uint8_t *used = h->G > 1 ? h->dE : nullptr;
   DevCounters *cnt = h->dcnt;
-  ld_note_launch(), k_tn_cand<<<grid_for(N, TB, h->sm_count * 4), TB, 0, s>>>(N, h->C, Cnew, cand, dev, match, cnt);
-  ld_note_launch(), k_tn_deviants<<<gN, TB, 0, s>>>(N, h->C, Cnew, h->K, cand, dev);
-  ld_note_launch(), k_tn_majority<<<gN, TB, 0, s>>>(N, h->csize0, cand, h->Sig, dev, choice, match, bits, flagged, best,
+  ld_note_launch(), launch_after(k_tn_cand, grid_for(N, TB, h->sm_count * 4), TB, s, N, h->C, Cnew, cand, dev, match, cnt);
+  ld_note_launch(), launch_after(k_tn_deviants, gN, TB, s, N, h->C, Cnew, h->K, cand, dev);
+  ld_note_launch(), launch_after(k_tn_majority, gN, TB, s, N, h->csize0, cand, h->Sig, dev, choice, match, bits, flagged, best,
                                                     cnt);
-  ld_note_launch(), k_tn_insert<<<gN, TB, 0, s>>>(N, h->C, Cnew, h->K, h->Sig, bits, best, h->tr_cap, h->tr_keys,
+  ld_note_launch(), launch_after(k_tn_insert, gN, TB, s, N, h->C, Cnew, h->K, h->Sig, bits, best, h->tr_cap, h->tr_keys,
                                                   h->tr_vals, h->tr_list, cnt);
-  ld_note_launch(), k_tn_best<<<h->sm_count * 2, TB, 0, s>>>(cnt, h->tr_list, h->tr_keys, h->tr_vals, best);
-  ld_note_launch(), k_tn_match<<<h->sm_count * 2, TB, 0, s>>>(cnt, flagged, best, choice, match);
+  ld_note_launch(), launch_after(k_tn_best, h->sm_count * 2, TB, s, cnt, h->tr_list, h->tr_keys, h->tr_vals, best);
+  ld_note_launch(), launch_after(k_tn_match, h->sm_count * 2, TB, s, cnt, flagged, best, choice, match);
   int tile = TR_STEP * (int)std::max<int64_t>(1, (N + (int64_t)TR_STEP * TR_TILES_MAX - 1) / ((int64_t)TR_STEP * TR_TILES_MAX));
   int nt = (int)((N + tile - 1) / tile);
-  ld_note_launch(), k_tn_tiles<<<nt, TB, 0, s>>>(N, tile, used, root, nroot, match, h->csize0, tiles, cnt);
-  ld_note_launch(), k_tn_lists<<<nt, TB, 0, s>>>(N, tile, used, root, nroot, match, h->csize0, tiles, rank, freel,
+  ld_note_launch(), launch_after(k_tn_tiles, nt, TB, s, N, tile, used, root, nroot, match, h->csize0, tiles, cnt);
+  ld_note_launch(), launch_after(k_tn_lists, nt, TB, s, N, tile, used, root, nroot, match, h->csize0, tiles, rank, freel,
                                                  h->gid0, h->d_voff, granks);
-  ld_note_launch(), k_tn_relabel<<<gN, TB, 0, s>>>(N, Cnew, match, rank, freel, choice, h->K, h->C, h->Sig, h->csize0,
+  ld_note_launch(), launch_after(k_tn_relabel, gN, TB, s, N, Cnew, match, rank, freel, choice, h->K, h->C, h->Sig, h->csize0,
                                                    h->dSig, h->gid0, granks);
 }
 
