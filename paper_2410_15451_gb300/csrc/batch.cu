@@ -48,6 +48,7 @@ __device__ __forceinline__ bool valid_edge(const leiden_edge &x, bool del, int64
 // deletions come first and each part is sorted by its keys.
 __global__ void k_expand(const leiden_edge *del, int64_t n_del, const leiden_edge *ins, int64_t n_ins,
                          int64_t n, int vb, uint64_t *key, int64_t *w, DevCounters *cnt, const int32_t *gid0) {
+  ld_after_previous();
   const uint64_t ins_bit = 1ull << (2 * vb);
   for (int64_t e = ld_gtid(); e < n_del + n_ins; e += ld_gstride()) {
     bool is_del = e < n_del;
@@ -69,6 +70,7 @@ __global__ void k_expand(const leiden_edge *del, int64_t n_del, const leiden_edg
 // Heads of the runs of equal keys over both parts of the sorted batch (the
 // insertion tag keeps them apart); IW zeroed for the sums.
 __global__ void k_head_flags(const uint64_t *key, int64_t n, int32_t *flag, int64_t *zero, int64_t nzero) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) {
     flag[i] = (i == 0 || key[i] != key[i - 1]) ? 1 : 0;
     if (i < nzero) zero[i] = 0;
@@ -78,6 +80,7 @@ __global__ void k_head_flags(const uint64_t *key, int64_t n, int32_t *flag, int6
 // Unique keys (and summed payload) into out_key/out_w at the scanned positions.
 __global__ void k_unique(const uint64_t *key, const int64_t *w, int64_t n, const int32_t *flag, const int64_t *pos,
                          uint64_t *out_key, int64_t *out_w) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) {
     int64_t p = pos[i] + flag[i] - 1;
     if (flag[i]) out_key[p] = key[i];
@@ -90,6 +93,7 @@ __global__ void k_unique(const uint64_t *key, const int64_t *w, int64_t n, const
 __global__ void k_unique_batch(const uint64_t *key, const int64_t *w, int64_t nda, int64_t nia, const int32_t *flag,
                                const int64_t *pos, uint64_t mask, uint64_t *dkey, uint64_t *ikey, int64_t *iw,
                                int64_t *counts) {
+  ld_after_previous();
   const int64_t nd = pos[nda];
   if (ld_gtid() == 0) {
     counts[0] = nd;
@@ -143,6 +147,7 @@ __global__ void __launch_bounds__(256) k_check_batch(BatchGraph G, const uint64_
                                                      const int64_t *iw, const int64_t *counts, int64_t nda, int64_t nia,
                                                      int64_t *dw, int32_t *state, int64_t *ipos, int32_t *flag,
                                                      DevCounters *cnt) {
+  ld_after_previous();
   __shared__ unsigned long long sum;
   if (threadIdx.x == 0) sum = 0;
   __syncthreads();
@@ -170,6 +175,7 @@ __global__ void __launch_bounds__(256) k_check_batch(BatchGraph G, const uint64_
 
 __global__ void k_compact_new(const uint64_t *ikey, const int64_t *iw, int64_t ni, const int32_t *flag,
                               const int64_t *pos, uint64_t *okey, int64_t *ow, int64_t *count) {
+  ld_after_previous();
   if (ld_gtid() == 0) *count = pos[ni];
   for (int64_t i = ld_gtid(); i < ni; i += ld_gstride())
     if (flag[i]) { okey[pos[i]] = ikey[i]; ow[pos[i]] = iw[i]; }
@@ -181,6 +187,7 @@ __global__ void k_compact_new(const uint64_t *ikey, const int64_t *iw, int64_t n
 // appends the row.  Work is O(batch), not O(n).
 __global__ void k_touched_rows(const uint64_t *dkey, const int64_t *nd_p, const uint64_t *nkey, const int64_t *nn_p,
                                int vb, uint32_t *bits, int32_t *rows, int64_t *nrows) {
+  ld_after_previous();
   int64_t nd = *nd_p, nn = *nn_p;
   for (int64_t t = ld_gtid(); t < nd + nn; t += ld_gstride()) {
     bool del = t < nd;
@@ -246,6 +253,7 @@ __global__ void __launch_bounds__(256) k_row_plan(BatchGraph G, RowPlan P, const
                                                   int64_t nb, const uint64_t *dkey, const int64_t *nd_p,
                                                   const uint64_t *nkey, const int64_t *nn_p, uint32_t *bits,
                                                   int64_t *total, DevCounters *cnt) {
+  ld_after_previous();
   __shared__ unsigned long long sum_s, slots_s;
   __shared__ int max_s;
   if (threadIdx.x == 0) { sum_s = 0; slots_s = 0; max_s = 0; }
@@ -306,6 +314,7 @@ struct SmallOut {
 
 __global__ void __launch_bounds__(1024) k_small_batch(BatchGraph G, RowPlan P, SmallOut O, const leiden_edge *del,
                                                       int n_del, const leiden_edge *ins, int n_ins, DevCounters *cnt) {
+  ld_after_previous();
   __shared__ uint64_t sk[SMALL_ARCS];     // arcs by key, then the unique ones: deletions, insertions
   __shared__ int64_t sw[SMALL_ARCS];      // summed weights of the unique arcs, then the new arcs' keys
   __shared__ int32_t si[SMALL_ARCS];      // input positions, then the touched rows
@@ -456,6 +465,7 @@ __global__ void __launch_bounds__(1024) k_small_batch(BatchGraph G, RowPlan P, S
 }
 
 __global__ void k_add_existing(const int64_t *ipos, const int32_t *state, const int64_t *iw, int64_t ni, int32_t *w) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < ni; i += ld_gstride())
     if (state[i]) w[ipos[i]] += (int32_t)iw[i];
 }
@@ -465,6 +475,7 @@ __global__ void k_merge_rows(const int32_t *rows, const int64_t *nrows_p, int vb
                              const uint64_t *nkey, const int64_t *nw, const int32_t *dlo, const int32_t *dhi,
                              const int32_t *ilo, const int32_t *ihi, const int64_t *tmp_off, const int64_t *off,
                              const int32_t *deg, const int32_t *col, const int32_t *w, int32_t *tcol, int32_t *tw) {
+  ld_after_previous();
   int64_t nrows = *nrows_p;
   int lane = threadIdx.x & 31;
   int64_t warp = ld_gtid() >> 5, nwarps = ld_gstride() >> 5;
@@ -566,6 +577,7 @@ __device__ __forceinline__ void merge_row_into(const MergeArgs &A, int64_t r, in
 }
 
 __global__ void __launch_bounds__(MERGE_WARPS * 32) k_merge_small(MergeArgs A) {
+  ld_after_previous();
   __shared__ int32_t scol[MERGE_WARPS][MERGE_SMALL];
   __shared__ int32_t sw[MERGE_WARPS][MERGE_SMALL];
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -676,6 +688,7 @@ __device__ __forceinline__ int32_t merge_tail(const MergeArgs &A, int64_t r, int
 // (R-MAT 22, 64,154 edges); now 55 and 88.
 __global__ void __launch_bounds__(MERGE_WARPS * 32) k_merge_warp(MergeArgs A, const int32_t *list,
                                                                  const int32_t *count_p) {
+  ld_after_previous();
   __shared__ int32_t scol[MERGE_WARPS][MERGE_WARP];
   __shared__ int32_t sw[MERGE_WARPS][MERGE_WARP];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -697,6 +710,7 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32) k_merge_warp(MergeArgs A, co
 // Rows of MERGE_WARP+1..MERGE_MID arcs: one block each.
 __global__ void __launch_bounds__(256) k_merge_mid(MergeArgs A, const int32_t *mid, const int32_t *count_p,
                                                    int64_t *xk_bytes) {
+  ld_after_previous();
   __shared__ int32_t scol[MERGE_MID];
   __shared__ int32_t sw[MERGE_MID];
   int64_t count = *count_p;
@@ -723,6 +737,7 @@ __global__ void __launch_bounds__(256) k_merge_mid(MergeArgs A, const int32_t *m
 // first chunk of a row also places its new arcs.
 __global__ void __launch_bounds__(256) k_merge_chunks_write(MergeArgs A, const int32_t *large,
                                                             const int32_t *count_p, const int64_t *ch_off) {
+  ld_after_previous();
   int64_t count = *count_p;
   int64_t nch = ch_off[count];
   uint64_t mask = (1ull << A.vb) - 1;
@@ -769,6 +784,7 @@ __global__ void __launch_bounds__(256) k_merge_chunks_write(MergeArgs A, const i
 // the new degree and any relocation.
 __global__ void __launch_bounds__(256) k_merge_chunks_copy(MergeArgs A, const int32_t *large,
                                                            const int32_t *count_p, const int64_t *ch_off) {
+  ld_after_previous();
   int64_t count = *count_p;
   int64_t nch = ch_off[count];
   for (int64_t t = blockIdx.x; t < nch; t += gridDim.x) {
@@ -788,12 +804,15 @@ __global__ void __launch_bounds__(256) k_merge_chunks_copy(MergeArgs A, const in
 
 // ----- rebuild with fresh slack (when a row outgrows its capacity)
 __global__ void k_row_lengths(const int32_t *deg, int64_t n, int64_t *len) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) len[i] = deg[i];
 }
 __global__ void k_touched_lengths(const int32_t *rows, const int64_t *nrows_p, const int64_t *rlen, int64_t *len) {
+  ld_after_previous();
   for (int64_t r = ld_gtid(); r < *nrows_p; r += ld_gstride()) len[rows[r]] = rlen[r];
 }
 __global__ void k_capacity(const int64_t *len, int64_t n, double slack, int min_slack, int64_t *cap) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) {
     int64_t L = len[i];
     int64_t extra = (int64_t)((double)L * slack);
@@ -806,6 +825,7 @@ __global__ void k_copy_rows_rebuild(int64_t n, const int64_t *old_off, const int
                                     const int32_t *old_w, const int32_t *rowsrc, const int64_t *tmp_off,
                                     const int64_t *rlen, const int32_t *tcol, const int32_t *tw,
                                     const int64_t *new_off, int32_t *new_deg, int32_t *new_col, int32_t *new_w) {
+  ld_after_previous();
   int lane = threadIdx.x & 31;
   int64_t warp = ld_gtid() >> 5, nwarps = ld_gstride() >> 5;
   for (int64_t u = warp; u < n; u += nwarps) {
@@ -820,15 +840,18 @@ __global__ void k_copy_rows_rebuild(int64_t n, const int64_t *old_off, const int
   }
 }
 __global__ void k_set_rcap(const int64_t *cap, int64_t n, int32_t *rcap) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) rcap[i] = (int32_t)cap[i];
 }
 __global__ void k_rowsrc(const int32_t *rows, const int64_t *nrows_p, int32_t *rowsrc) {
+  ld_after_previous();
   for (int64_t r = ld_gtid(); r < *nrows_p; r += ld_gstride()) rowsrc[rows[r]] = (int32_t)r;
 }
 
 // ----- marking (uses C^{t-1}, and K^{t-1}, Sigma^{t-1}, 2m^{t-1} for DS)
 __global__ void k_mark_ds_del(const uint64_t *dkey, int64_t nd, int vb, const int32_t *C, uint8_t *dV, uint8_t *dE,
                               uint8_t *dCf) {
+  ld_after_previous();
   uint64_t mask = (1ull << vb) - 1;
   for (int64_t i = ld_gtid(); i < nd; i += ld_gstride()) {
     int32_t u = (int32_t)(dkey[i] >> vb), v = (int32_t)(dkey[i] & mask);
@@ -840,6 +863,7 @@ __global__ void k_mark_ds_del(const uint64_t *dkey, int64_t nd, int vb, const in
 // arcs get the key ~0 and sort last.
 __global__ void k_ds_keys(const uint64_t *ikey, const int64_t *iw, int64_t ni, int vb, const int32_t *C,
                           uint64_t *okey, int64_t *ow) {
+  ld_after_previous();
   uint64_t mask = (1ull << vb) - 1;
   for (int64_t i = ld_gtid(); i < ni; i += ld_gstride()) {
     int32_t u = (int32_t)(ikey[i] >> vb), v = (int32_t)(ikey[i] & mask);
@@ -853,6 +877,7 @@ __global__ void k_ds_keys(const uint64_t *ikey, const int64_t *iw, int64_t ni, i
 __global__ void k_ds_best(const uint64_t *pkey, const int64_t *pw, const int64_t *np_p, int vb, const int64_t *K,
                           const int64_t *Sig, const DevCounters *cnt, uint8_t *dV, uint8_t *dE, uint8_t *dCf,
                           const int32_t *gid0, const int64_t *m2g) {
+  ld_after_previous();
   int64_t np = *np_p;
   uint64_t mask = (1ull << vb) - 1;
   for (int64_t i = ld_gtid(); i < np; i += ld_gstride()) {
@@ -879,6 +904,7 @@ __global__ void k_ds_best(const uint64_t *pkey, const int64_t *pw, const int64_t
 __global__ void __launch_bounds__(256) k_ds_expand_neighbours(const uint8_t *dE, int64_t n, const int64_t *off,
                                                               const int32_t *deg, const int32_t *col, uint8_t *dV,
                                                               int32_t *big, DevCounters *cnt) {
+  ld_after_previous();
   const int lane = threadIdx.x & 31;
   int64_t warp = ld_gtid() >> 5, nw = ld_gstride() >> 5;
   for (int64_t r = warp * 32; r < n; r += nw * 32) {  // warp-uniform
@@ -911,6 +937,7 @@ __global__ void __launch_bounds__(256) k_ds_expand_neighbours(const uint8_t *dE,
 __global__ void __launch_bounds__(256) k_ds_expand_big(const int32_t *big, const int64_t *ch_off, const int64_t *off,
                                                        const int32_t *deg, const int32_t *col, uint8_t *dV,
                                                        const DevCounters *cnt) {
+  ld_after_previous();
   const int64_t count = cnt->big_count;
   if (count == 0) return;
   const int64_t nch = ch_off[count];
@@ -924,6 +951,7 @@ __global__ void __launch_bounds__(256) k_ds_expand_big(const int32_t *big, const
   }
 }
 __global__ void k_ds_expand_communities(const uint8_t *dCf, const int32_t *C, int64_t n, uint8_t *dV) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride())
     if (dCf[C[i]]) dV[i] = 1;
 }
@@ -940,6 +968,7 @@ __global__ void __launch_bounds__(256) k_update_weights(const uint64_t *dkey, co
                                                         const int32_t *C, int64_t *K, int64_t *Sig, int64_t *dSig,
                                                         DevCounters *cnt, const int32_t *gid0, int64_t *m2g,
                                                         uint8_t *dV) {
+  ld_after_previous();
   __shared__ int32_t hk[UPD_SLOTS];
   __shared__ unsigned long long hs[UPD_SLOTS], hw[UPD_SLOTS];
   for (int t = threadIdx.x; t < UPD_SLOTS; t += 256) { hk[t] = -1; hs[t] = 0; hw[t] = 0; }
@@ -1002,6 +1031,7 @@ __global__ void __launch_bounds__(256) k_update_weights(const uint64_t *dkey, co
 __global__ void k_mark_communities(const uint64_t *dkey, int64_t nd, const uint64_t *ikey, int64_t ni, int vb,
                                    const int32_t *C, const int64_t *Sig, const int64_t *dSig, double tau_re,
                                    uint8_t *dS, uint8_t *dR, DevCounters *cnt) {
+  ld_after_previous();
   uint64_t mask = (1ull << vb) - 1;
   for (int64_t i = ld_gtid(); i < nd + ni; i += ld_gstride()) {
     bool del = i < nd;
@@ -1018,6 +1048,7 @@ __global__ void k_mark_communities(const uint64_t *dkey, int64_t nd, const uint6
 }
 __global__ void k_reset_changes(const uint64_t *dkey, int64_t nd, const uint64_t *ikey, int64_t ni, int vb,
                                 const int32_t *C, const uint8_t *dR, int64_t *dSig, const DevCounters *cnt) {
+  ld_after_previous();
   if (cnt->refine_marks == 0) return;
   for (int64_t i = ld_gtid(); i < nd + ni; i += ld_gstride()) {
     uint64_t k = i < nd ? dkey[i] : ikey[i - nd];
@@ -1155,9 +1186,9 @@ static leiden_status rebuild_graph(leiden_handle *h, int64_t nrows_host, const i
   int64_t n = h->n;
   BatchBuffers &b = h->b;
   int64_t *len = h->lbuf0, *cap = h->lbuf1;
-  ld_note_launch(), k_row_lengths<<<grid_for(n, TB), TB, 0, s>>>(h->g_deg, n, len);
-  ld_note_launch(), k_touched_lengths<<<grid_for(nrows_host, TB), TB, 0, s>>>(b.rows, nrows_dev, b.row_len, len);
-  ld_note_launch(), k_capacity<<<grid_for(n, TB), TB, 0, s>>>(len, n, h->p.slack, h->p.min_slack, cap);
+  ld_note_launch(), launch_after(k_row_lengths, grid_for(n, TB), TB, s, h->g_deg, n, len);
+  ld_note_launch(), launch_after(k_touched_lengths, grid_for(nrows_host, TB), TB, s, b.rows, nrows_dev, b.row_len, len);
+  ld_note_launch(), launch_after(k_capacity, grid_for(n, TB), TB, s, len, n, h->p.slack, h->p.min_slack, cap);
   int64_t *new_off = nullptr;
   if (grow(h, &new_off, n + 1) != cudaSuccess) return fail(h, LEIDEN_ERR_OOM, "rebuild: offsets");
   if (ensure_scan_tmp(h, scan_tmp_bytes(n + 1)) != cudaSuccess) return fail(h, LEIDEN_ERR_OOM, "scan tmp");
@@ -1170,14 +1201,14 @@ static leiden_status rebuild_graph(leiden_handle *h, int64_t nrows_host, const i
   if (grow(h, &new_col, total) != cudaSuccess || grow(h, &new_w, total) != cudaSuccess ||
       grow(h, &new_deg, n) != cudaSuccess)
     return fail(h, LEIDEN_ERR_OOM, "rebuild: arcs");
-  ld_note_launch(), k_set_rcap<<<grid_for(n, TB), TB, 0, s>>>(cap, n, h->g_rcap);
+  ld_note_launch(), launch_after(k_set_rcap, grid_for(n, TB), TB, s, cap, n, h->g_rcap);
   cudaMemcpyAsync(&h->dcnt->arena_used, &used, sizeof(int64_t), cudaMemcpyHostToDevice, s);
   int32_t *rowsrc = h->ibuf2;
   launch_fill_i32(rowsrc, -1, n, s);
-  ld_note_launch(), k_rowsrc<<<grid_for(nrows_host, TB), TB, 0, s>>>(b.rows, nrows_dev, rowsrc);
-  ld_note_launch(), k_copy_rows_rebuild<<<grid_for(n * 32, TB), TB, 0, s>>>(n, h->g_off, h->g_deg, h->g_col, h->g_w, rowsrc,
-                                                          b.row_tmp_off, b.row_len, b.tmp_col, b.tmp_w, new_off,
-                                                          new_deg, new_col, new_w);
+  ld_note_launch(), launch_after(k_rowsrc, grid_for(nrows_host, TB), TB, s, b.rows, nrows_dev, rowsrc);
+  ld_note_launch(), launch_after(k_copy_rows_rebuild, grid_for(n * 32, TB), TB, s, n, h->g_off, h->g_deg, h->g_col,
+                                 h->g_w, rowsrc, b.row_tmp_off, b.row_len, b.tmp_col, b.tmp_w, new_off, new_deg,
+                                 new_col, new_w);
   cudaStreamSynchronize(s);
   release(h, h->g_off);
   release(h, h->g_col);
@@ -1217,30 +1248,31 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
   if (nda + nia == 0) {
   } else if (nda + nia <= SMALL_ARCS) {
     SmallOut O{DK, IK, NK, DW, IW, NW, b.ins_pos, b.row_tmp_off, b.ins_state, b.rows};
-    ld_note_launch(), k_small_batch<<<1, 1024, 0, s>>>(G, P, O, d_del, (int)n_del, d_ins, (int)n_ins, cnt);
+    ld_note_launch(), launch_after(k_small_batch, 1, 1024, s, G, P, O, d_del, (int)n_del, d_ins, (int)n_ins, cnt);
   } else {
     // one sort of both: the deletion arcs sorted in dkey[0, nda), the
     // insertion arcs and their weights in dkey, iw [nda, nda + nia)
-    ld_note_launch(), k_expand<<<grid_for(n_del + n_ins, TB), TB, 0, s>>>(d_del, n_del, d_ins, n_ins, n, vb, b.dkey,
-                                                                          b.iw, cnt, h->gid0);
+    ld_note_launch(), launch_after(k_expand, grid_for(n_del + n_ins, TB), TB, s, d_del, n_del, d_ins, n_ins, n, vb,
+                                   b.dkey, b.iw, cnt, h->gid0);
     radix_sort_u64(b.dkey, b.dkey_alt, b.iw, b.iw_alt, nda + nia, 2 * vb + 1, h->scan_tmp, s);
-    ld_note_launch(), k_head_flags<<<grid_for(nda + nia, TB), TB, 0, s>>>(b.dkey, nda + nia, b.flag, IW, nia);
+    ld_note_launch(), launch_after(k_head_flags, grid_for(nda + nia, TB), TB, s, b.dkey, nda + nia, b.flag, IW, nia);
     exclusive_scan_i32_to_i64(b.flag, b.pos, nda + nia, h->scan_tmp, s);
-    ld_note_launch(), k_unique_batch<<<grid_for(nda + nia, TB), TB, 0, s>>>(
-        b.dkey, b.iw, nda, nia, b.flag, b.pos, (1ull << (2 * vb)) - 1, DK, IK, IW, counts);
+    ld_note_launch(), launch_after(k_unique_batch, grid_for(nda + nia, TB), TB, s, b.dkey, b.iw, nda, nia, b.flag,
+                                   b.pos, (1ull << (2 * vb)) - 1, DK, IK, IW, counts);
     // deletions must exist (stored weight -> DW); insertions: existing or new
-    ld_note_launch(), k_check_batch<<<grid_for(nda + nia, TB), TB, 0, s>>>(G, DK, IK, IW, counts, nda, nia, DW,
-                                                                           b.ins_state, b.ins_pos, b.flag, cnt);
+    ld_note_launch(), launch_after(k_check_batch, grid_for(nda + nia, TB), TB, s, G, DK, IK, IW, counts, nda, nia, DW,
+                                   b.ins_state, b.ins_pos, b.flag, cnt);
     if (nia > 0) {
       exclusive_scan_i32_to_i64(b.flag, b.pos, nia, h->scan_tmp, s);
-      ld_note_launch(), k_compact_new<<<grid_for(nia, TB), TB, 0, s>>>(IK, IW, nia, b.flag, b.pos, NK, NW, counts + 2);
+      ld_note_launch(), launch_after(k_compact_new, grid_for(nia, TB), TB, s, IK, IW, nia, b.flag, b.pos, NK, NW,
+                                     counts + 2);
     }
     // rows whose structure changes: sources of deletions and of new arcs
     int64_t nb = std::min<int64_t>(n, nda + nia);  // bound on the touched rows
-    ld_note_launch(), k_touched_rows<<<grid_for(nda + nia, TB), TB, 0, s>>>(DK, counts + 0, NK, counts + 2, vb,
-                                                                            b.row_bits, b.rows, counts + 3);
-    ld_note_launch(), k_row_plan<<<grid_for(nb, TB), TB, 0, s>>>(G, P, b.rows, counts + 3, nb, DK, counts + 0, NK,
-                                                                 counts + 2, b.row_bits, counts + 4, cnt);
+    ld_note_launch(), launch_after(k_touched_rows, grid_for(nda + nia, TB), TB, s, DK, counts + 0, NK, counts + 2, vb,
+                                   b.row_bits, b.rows, counts + 3);
+    ld_note_launch(), launch_after(k_row_plan, grid_for(nb, TB), TB, s, G, P, b.rows, counts + 3, nb, DK, counts + 0,
+                                   NK, counts + 2, b.row_bits, counts + 4, cnt);
     exclusive_scan_i64(b.row_len, b.row_tmp_off, nb, h->scan_tmp, s);
   }
   // the one host read before the graph changes: counts, validation, overflow
@@ -1254,7 +1286,8 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
   bool overflow = nrows > 0 && h->hcnt->overflow != 0;
   if (ensure_tmp_rows(h, tmp_total) != cudaSuccess) return fail(h, LEIDEN_ERR_OOM, "merge buffer");
   // ---- apply: from here on the handle changes
-  if (ni > nn) ld_note_launch(), k_add_existing<<<grid_for(ni, TB), TB, 0, s>>>(b.ins_pos, b.ins_state, IW, ni, h->g_w);
+  if (ni > nn) ld_note_launch(), launch_after(k_add_existing, grid_for(ni, TB), TB, s, b.ins_pos, b.ins_state, IW, ni,
+                                              h->g_w);
   if (nrows > 0) {
     if (!overflow) {
       MergeArgs M{b.rows, counts + 3, vb, DK, NK, NW, b.row_dlo, b.row_dhi, b.row_ilo, b.row_ihi, b.row_len,
@@ -1276,15 +1309,16 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
         if (some_long) cudaStreamWaitEvent(slong, h->fork_ev, 0);
       }
       if (some_warp)
-        ld_note_launch(), k_merge_warp<<<
-            grid_for((h->hcnt->warp_count + MERGE_WARPS - 1) / MERGE_WARPS, 1, h->sm_count * 7), MERGE_WARPS * 32, 0, s>>>(
-            M, b.row_warp, &cnt->warp_count);
+        ld_note_launch(), launch_after(k_merge_warp,
+                                       grid_for((h->hcnt->warp_count + MERGE_WARPS - 1) / MERGE_WARPS, 1, h->sm_count * 7),
+                                       MERGE_WARPS * 32, s, M, b.row_warp, &cnt->warp_count);
       if (some_small)
-        ld_note_launch(), k_merge_small<<<grid_for((nrows + MERGE_WARPS - 1) / MERGE_WARPS, 1, h->sm_count * 16),
-                                          MERGE_WARPS * 32, 0, s>>>(M);
+        ld_note_launch(), launch_after(k_merge_small,
+                                       grid_for((nrows + MERGE_WARPS - 1) / MERGE_WARPS, 1, h->sm_count * 16),
+                                       MERGE_WARPS * 32, s, M);
       if (some_mid) {
         kt_begin(h, KT_MERGE_MID, smid);
-        ld_note_launch(), k_merge_mid<<<h->sm_count * 7, 256, 0, smid>>>(M, b.row_mid, &cnt->mid_count,  // 32 KB: 7 per SM
+        ld_note_launch(), launch_after(k_merge_mid, h->sm_count * 7, 256, smid, M, b.row_mid, &cnt->mid_count,  // 32 KB: 7 per SM
                                                                         &cnt->xk_bytes[2]);
         kt_end(h, smid);
       }
@@ -1293,9 +1327,9 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
         int32_t *large = b.row_large;
         const int32_t *nlarge = &cnt->large_count;
         launch_table_plan(large, nlarge, b.row_olddeg, nullptr, INT64_MAX, h->lbuf0, h->lbuf1, slong);
-        ld_note_launch(), k_merge_chunks_write<<<h->sm_count * 16, 256, 0, slong>>>(M, large, nlarge, h->lbuf1);
+        ld_note_launch(), launch_after(k_merge_chunks_write, h->sm_count * 16, 256, slong, M, large, nlarge, h->lbuf1);
         launch_table_plan(large, nlarge, nullptr, b.row_tmp_off, INT64_MAX, h->lbuf2, h->lbuf3, slong);
-        ld_note_launch(), k_merge_chunks_copy<<<h->sm_count * 16, 256, 0, slong>>>(M, large, nlarge, h->lbuf3);
+        ld_note_launch(), launch_after(k_merge_chunks_copy, h->sm_count * 16, 256, slong, M, large, nlarge, h->lbuf3);
       }
       if (fork) {
         for (int k = 0; k < 2; k++) {
@@ -1305,9 +1339,9 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
         }
       }
     } else {
-      ld_note_launch(), k_merge_rows<<<grid_for(nrows * 32, TB), TB, 0, s>>>(b.rows, counts + 3, vb, DK, NK, NW, b.row_dlo,
-                                                           b.row_dhi, b.row_ilo, b.row_ihi, b.row_tmp_off, h->g_off,
-                                                           h->g_deg, h->g_col, h->g_w, b.tmp_col, b.tmp_w);
+      ld_note_launch(), launch_after(k_merge_rows, grid_for(nrows * 32, TB), TB, s, b.rows, counts + 3, vb, DK, NK, NW,
+                                     b.row_dlo, b.row_dhi, b.row_ilo, b.row_ihi, b.row_tmp_off, h->g_off, h->g_deg,
+                                     h->g_col, h->g_w, b.tmp_col, b.tmp_w);
       leiden_status st = rebuild_graph(h, nrows, counts + 3);
       h->stats.rebuilds++;
       if (st != LEIDEN_OK) {
@@ -1331,35 +1365,37 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
     {
       cudaMemsetAsync(h->dE, 0, (size_t)n, s);
       cudaMemsetAsync(h->dCf, 0, (size_t)n, s);
-      if (nd > 0) ld_note_launch(), k_mark_ds_del<<<grid_for(nd, TB), TB, 0, s>>>(DK, nd, vb, h->C, dV, h->dE, h->dCf);
+      if (nd > 0) ld_note_launch(), launch_after(k_mark_ds_del, grid_for(nd, TB), TB, s, DK, nd, vb, h->C, dV, h->dE,
+                                                 h->dCf);
       if (ni > 0) {
         // H of each insertion source: (src, C[dst]) pairs, sorted, runs summed
-        ld_note_launch(), k_ds_keys<<<grid_for(ni, TB), TB, 0, s>>>(IK, IW, ni, vb, h->C, b.ds_key, b.ds_w);
+        ld_note_launch(), launch_after(k_ds_keys, grid_for(ni, TB), TB, s, IK, IW, ni, vb, h->C, b.ds_key, b.ds_w);
         radix_sort_u64(b.ds_key, b.ds_key_alt, b.ds_w, b.ds_w_alt, ni, 64, h->scan_tmp, s);
-        ld_note_launch(), k_head_flags<<<grid_for(ni, TB), TB, 0, s>>>(b.ds_key, ni, b.flag, nullptr, 0);
+        ld_note_launch(), launch_after(k_head_flags, grid_for(ni, TB), TB, s, b.ds_key, ni, b.flag, nullptr, 0);
         exclusive_scan_i32_to_i64(b.flag, b.pos, ni, h->scan_tmp, s);
         cudaMemsetAsync(b.ds_uw, 0, (size_t)ni * sizeof(int64_t), s);
-        ld_note_launch(), k_unique<<<grid_for(ni, TB), TB, 0, s>>>(b.ds_key, b.ds_w, ni, b.flag, b.pos, b.ds_ukey, b.ds_uw);
-        ld_note_launch(), k_ds_best<<<grid_for(ni, TB), TB, 0, s>>>(b.ds_ukey, b.ds_uw, b.pos + ni, vb, h->K, h->Sig, cnt, dV, h->dE,
-                                                  h->dCf, h->gid0, h->gc.m2);
+        ld_note_launch(), launch_after(k_unique, grid_for(ni, TB), TB, s, b.ds_key, b.ds_w, ni, b.flag, b.pos,
+                                       b.ds_ukey, b.ds_uw);
+        ld_note_launch(), launch_after(k_ds_best, grid_for(ni, TB), TB, s, b.ds_ukey, b.ds_uw, b.pos + ni, vb, h->K,
+                                       h->Sig, cnt, dV, h->dE, h->dCf, h->gid0, h->gc.m2);
       }
       cudaMemsetAsync(&cnt->big_count, 0, sizeof(int32_t), s);
-      ld_note_launch(), k_ds_expand_neighbours<<<grid_for(n, TB), TB, 0, s>>>(h->dE, n, h->g_off, h->g_deg, h->g_col,
-                                                                              dV, h->ibuf0, cnt);
+      ld_note_launch(), launch_after(k_ds_expand_neighbours, grid_for(n, TB), TB, s, h->dE, n, h->g_off, h->g_deg,
+                                     h->g_col, dV, h->ibuf0, cnt);
       launch_table_plan(h->ibuf0, &cnt->big_count, h->g_deg, nullptr, 1, h->lbuf0, h->lbuf1, s);
-      ld_note_launch(), k_ds_expand_big<<<h->sm_count * 8, TB, 0, s>>>(h->ibuf0, h->lbuf1, h->g_off, h->g_deg,
-                                                                       h->g_col, dV, cnt);
-      ld_note_launch(), k_ds_expand_communities<<<grid_for(n, TB), TB, 0, s>>>(h->dCf, h->C, n, dV);
+      ld_note_launch(), launch_after(k_ds_expand_big, h->sm_count * 8, TB, s, h->ibuf0, h->lbuf1, h->g_off, h->g_deg,
+                                     h->g_col, dV, cnt);
+      ld_note_launch(), launch_after(k_ds_expand_communities, grid_for(n, TB), TB, s, h->dCf, h->C, n, dV);
     }
   }
   // ---- Alg. update, then Alg. leidenmk (dS, dR; reset dSigma of refined)
   if (nd + ni > 0) {
-    ld_note_launch(), k_update_weights<<<grid_for(nd + ni, TB), TB, 0, s>>>(DK, DW, nd, IK, IW, ni, vb, h->C, h->K, h->Sig, h->dSig,
-                                                           cnt, h->gid0, h->gc.m2,
-                                                           mode == LEIDEN_DF ? dV : nullptr);
-    ld_note_launch(), k_mark_communities<<<grid_for(nd + ni, TB), TB, 0, s>>>(DK, nd, IK, ni, vb, h->C, h->Sig, h->dSig,
-                                                             h->p.tau_refine, h->dS, h->dR, cnt);
-    ld_note_launch(), k_reset_changes<<<grid_for(nd + ni, TB), TB, 0, s>>>(DK, nd, IK, ni, vb, h->C, h->dR, h->dSig, cnt);
+    ld_note_launch(), launch_after(k_update_weights, grid_for(nd + ni, TB), TB, s, DK, DW, nd, IK, IW, ni, vb, h->C,
+                                   h->K, h->Sig, h->dSig, cnt, h->gid0, h->gc.m2, mode == LEIDEN_DF ? dV : nullptr);
+    ld_note_launch(), launch_after(k_mark_communities, grid_for(nd + ni, TB), TB, s, DK, nd, IK, ni, vb, h->C, h->Sig,
+                                   h->dSig, h->p.tau_refine, h->dS, h->dR, cnt);
+    ld_note_launch(), launch_after(k_reset_changes, grid_for(nd + ni, TB), TB, s, DK, nd, IK, ni, vb, h->C, h->dR,
+                                   h->dSig, cnt);
   }
   // Algorithmic bytes of the batch phase: the edge triples read (12 B per
   // edge); per raw arc its expansion and sort (48 B: key and weight written,

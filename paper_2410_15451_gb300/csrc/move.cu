@@ -459,6 +459,7 @@ __device__ __forceinline__ void warp_step(const Args &A, int32_t i, int lane, Wa
 // vertices, the rest one warp-bin vertex each.
 template <typename W, int KIND, bool WIDE>
 __global__ void __launch_bounds__(WARPS_PER_BLOCK * 32, 4) k_decide_warp(Args A) {
+  ld_after_previous();
   __shared__ WarpTable<WIDE> WT[WARPS_PER_BLOCK];
   ld_after_previous();
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -501,6 +502,7 @@ struct BlockStage : STable<WIDE, STAGE_SLOTS, STAGE_FILL, uint16_t> {
 
 template <typename W, int KIND, bool WIDE>
 __global__ void __launch_bounds__(BLOCK_THREADS) k_decide_block(Args A) {
+  ld_after_previous();
   __shared__ BlockStage<WIDE> S;
   __shared__ BestX sb[BLOCK_THREADS / 32];
   __shared__ int moved_s;
@@ -638,6 +640,7 @@ __device__ __forceinline__ GTable hub_table(const Args &A, const int64_t *tab_of
 
 template <typename W, int KIND, bool WIDE>
 __global__ void __launch_bounds__(256) k_huge_scan(Args A, const int64_t *tab_off, const int64_t *ch_off) {
+  ld_after_previous();
   // Each warp sums its arcs per community in a private shared table first
   // (the neighbours of a hub fall into few communities), then each distinct
   // community updates the vertex's global table once per flush.  The hub's
@@ -816,6 +819,7 @@ __device__ __forceinline__ bool hub_decide(const Args &A, const Hub &H, BestX b,
 
 template <int KIND, bool WIDE>
 __global__ void __launch_bounds__(HUGE_THREADS, 4) k_huge_decide(Args A, const int64_t *tab_off, BigTables big) {
+  ld_after_previous();
   __shared__ BestX sb[HUGE_THREADS / 32];
   __shared__ int flag_s;
   const int lane = threadIdx.x & 31;
@@ -997,7 +1001,8 @@ __device__ __forceinline__ void apply_moves(const Args &A, unsigned long long *d
 // next are collected (they touch different arrays).  `apply`: there was one
 // before; Q.cls < 0: there is none after.
 template <bool DENSE>
-__global__ void __launch_bounds__(256) k_apply_collect(Args A, bool apply, unsigned long long *dqg, int64_t *movesg, CollectArgs Q) {
+__global__ void __launch_bounds__(256)
+    k_apply_collect(Args A, bool apply, unsigned long long *dqg, int64_t *movesg, CollectArgs Q) {
   ld_after_previous();
   if (apply) apply_moves(A, dqg, movesg);
   if (Q.cls < 0) return;
@@ -1009,6 +1014,7 @@ __global__ void __launch_bounds__(256) k_apply_collect(Args A, bool apply, unsig
 // MARK_PARTS for as many warps (before the next vertices are collected).
 constexpr int MARK_PARTS = 32;
 __global__ void k_mark_hubs(Args A) {
+  ld_after_previous();
   int64_t parts = (int64_t)A.sub->big_movers * MARK_PARTS;
   for (int64_t t = ld_gtid() >> 5; t < parts; t += ld_gstride() >> 5) {  // warp-uniform
     int32_t i = A.big_movers[t / MARK_PARTS];
@@ -1020,6 +1026,7 @@ __global__ void k_mark_hubs(Args A) {
 // Community sizes; lanes with the same community add once (giant
 // communities would otherwise serialise on one counter).
 __global__ void k_sizes(const int32_t *C, int64_t n, int32_t *size) {
+  ld_after_previous();
   int lane = threadIdx.x & 31;
   for (int64_t base = (ld_gtid() & ~31ll); base < n; base += ld_gstride()) {
     int64_t i = base + lane;
@@ -1035,6 +1042,7 @@ __global__ void k_sizes(const int32_t *C, int64_t n, int32_t *size) {
 __global__ void __launch_bounds__(256) k_refine_reset(int64_t n, int32_t *CB, const uint8_t *dR, int32_t *C, int64_t *S,
                                                       const int64_t *K, int32_t *prop, int32_t *cand, DevCounters *cnt,
                                                       const int32_t *gid, uint8_t *refg) {
+  ld_after_previous();
   __shared__ BlockAppend<1> B;
   int32_t *const lengths[1] = {&cnt->cand_count[0]};
   for (int64_t b0 = (int64_t)blockIdx.x * APPEND_STEP; b0 < n; b0 += (int64_t)gridDim.x * APPEND_STEP) {
@@ -1241,7 +1249,7 @@ void launch_bins_of(leiden_handle *h, const LevelGraph &g, Args A) {
     bin(BIN_BLOCK);
     int grid = sms * h->tune.block_blocks_per_sm;
     if (KIND == KIND_MOVE) kt_begin(h, KT_BLOCK, sblock);
-    ld_note_launch(), k_decide_block<W, KIND, WIDE><<<grid, BLOCK_THREADS, 0, sblock>>>(A);
+    ld_note_launch(), launch_after(k_decide_block<W, KIND, WIDE>, grid, BLOCK_THREADS, sblock, A);
     if (KIND == KIND_MOVE) kt_end(h, sblock);
   }
   if (need_hub) {
@@ -1255,11 +1263,11 @@ void launch_bins_of(leiden_handle *h, const LevelGraph &g, Args A) {
     launch_table_plan(A.list, A.count, g.deg, nullptr, g.n, tab_off, ch_off, shub, A.gocc);
     if (KIND == KIND_MOVE) kt_begin(h, KT_HUGE_SCAN, shub);
     int hg = sms * h->tune.hub_blocks_per_sm;
-    ld_note_launch(), k_huge_scan<W, KIND, WIDE><<<hg, 256, 0, shub>>>(A, tab_off, ch_off);
+    ld_note_launch(), launch_after(k_huge_scan<W, KIND, WIDE>, hg, 256, shub, A, tab_off, ch_off);
     if (KIND == KIND_MOVE) kt_end(h, shub);
     BigTables big{h->ibuf1, &h->dcnt->hub_big, h->lbuf1, h->ibuf0};
     launch_piece_plan(A.count, A.gocc, big, shub);
-    ld_note_launch(), k_huge_decide<KIND, WIDE><<<sms * 8, HUGE_THREADS, 0, shub>>>(A, tab_off, big);
+    ld_note_launch(), launch_after(k_huge_decide<KIND, WIDE>, sms * 8, HUGE_THREADS, shub, A, tab_off, big);
   }
   if (fork) {
     for (int k = 0; k < 2; k++) {
@@ -1337,7 +1345,7 @@ int32_t *hs_list(leiden_handle *h) { return (int32_t *)((char *)h->hscratch + (s
 
 void count_sizes(leiden_handle *h, const int32_t *C, int64_t n, int32_t *size) {
   cudaMemsetAsync(size, 0, (size_t)n * sizeof(int32_t), h->stream);
-  ld_note_launch(), k_sizes<<<grid_for(n, 256), 256, 0, h->stream>>>(C, n, size);
+  ld_note_launch(), launch_after(k_sizes, grid_for(n, 256), 256, h->stream, C, n, size);
 }
 
 void lm_iteration(leiden_handle *h, const LevelGraph &g, const uint8_t *in_range, int dynamic, bool dense) {
@@ -1368,7 +1376,7 @@ void lm_iteration(leiden_handle *h, const LevelGraph &g, const uint8_t *in_range
     A.sub = Q.sub;
     launch_bins<KIND_MOVE>(h, g, A);
     if (deferred && g.maxdeg > h->tune.block_max && g.maxdeg > MARK_INLINE)
-      ld_note_launch(), k_mark_hubs<<<h->sm_count * 4, 256, 0, s>>>(A);
+      ld_note_launch(), launch_after(k_mark_hubs, h->sm_count * 4, 256, s, A);
     pending = deferred;
   }
   if (pending) {
@@ -1380,9 +1388,8 @@ void lm_iteration(leiden_handle *h, const LevelGraph &g, const uint8_t *in_range
 void refine_reset(leiden_handle *h, const LevelGraph &g) {
   cudaStream_t s = h->stream;
   cudaMemsetAsync(&h->dcnt->cand_count[0], 0, sizeof(int32_t), s);
-  ld_note_launch(), k_refine_reset<<<grid_for(g.n, APPEND_STEP), 256, 0, s>>>(g.n, h->CB, h->dR2, h->Cp, h->Sp, h->Kc,
-                                                                              h->prop, h->cand, h->dcnt, g.gid,
-                                                                              h->gc.refined);
+  ld_note_launch(), launch_after(k_refine_reset, grid_for(g.n, APPEND_STEP), 256, s, g.n, h->CB, h->dR2, h->Cp, h->Sp,
+                                 h->Kc, h->prop, h->cand, h->dcnt, g.gid, h->gc.refined);
 }
 
 // One round on the candidates of list `slot` (cand + slot*n, count
@@ -1391,15 +1398,16 @@ void refine_round(leiden_handle *h, const LevelGraph &g, int slot) {
   cudaStream_t s = h->stream;
   int32_t *in = h->cand + (int64_t)slot * g.n, *out = h->cand + (int64_t)(1 - slot) * g.n;
   int32_t *cin = &h->dcnt->cand_count[slot], *cout = &h->dcnt->cand_count[1 - slot];
-  static_assert(offsetof(DevCounters, accepted) == offsetof(DevCounters, ref) + sizeof(SubCounters), "cleared together");
+  static_assert(offsetof(DevCounters, accepted) == offsetof(DevCounters, ref) + sizeof(SubCounters),
+                "cleared together");
   cudaMemsetAsync(&h->dcnt->ref, 0, sizeof(SubCounters) + sizeof(int32_t), s);  // bins, accepted
   cudaMemsetAsync(cout, 0, sizeof(int32_t), s);
   ld_note_launch(), launch_after(k_refine_collect, grid_for(g.n, APPEND_STEP), 256, s, in, cin, out, cout, g.n, h->Cp,
                                  h->Sp, h->Kc, g.deg, h->prop, h->bins, &h->dcnt->ref, h->tune);
   Args A = make_args(h, g);
   launch_bins<KIND_REFINE>(h, g, A);
-  ld_note_launch(), launch_after(k_refine_accept, grid_for(g.n, 256, h->sm_count * 4), 256, s, out, cout, h->prop, h->Cp,
-                                 h->Sp, h->Kc, h->dcnt, g.gid, h->gc.accepted);
+  ld_note_launch(), launch_after(k_refine_accept, grid_for(g.n, 256, h->sm_count * 4), 256, s, out, cout, h->prop,
+                                 h->Cp, h->Sp, h->Kc, h->dcnt, g.gid, h->gc.accepted);
 }
 
 LD_CHECK_WORD_READER(check_word_move)

@@ -161,6 +161,7 @@ constexpr int SPLIT_WINDOW = 4;   // arcs loaded at once
 __global__ void __launch_bounds__(256) k_split_find(const int32_t *list, DevCounters *cnt, const int64_t *off,
                                                     const int32_t *deg, const int32_t *col, const int32_t *C,
                                                     int2 *hit) {
+  ld_after_previous();
   int64_t m = cnt->split_count;
   int64_t bytes = 0;  // algorithmic bytes: per vertex 20, per arc read 8
   for (int64_t t = ld_gtid(); t < m; t += ld_gstride()) {
@@ -190,6 +191,7 @@ __global__ void __launch_bounds__(256) k_split_find(const int32_t *list, DevCoun
 }
 __global__ void __launch_bounds__(256) k_split_link(const int32_t *list, const DevCounters *cnt, int32_t *parent,
                                                     const int2 *hit, bool rest) {
+  ld_after_previous();
   int64_t m = cnt->split_count, k = rest ? (m >> 3) * 7 + (m & 7 ? (m & 7) - 1 : 0) : (m + 7) >> 3;
   for (int64_t q = ld_gtid(); q < k; q += ld_gstride()) {
     int64_t t = rest ? q + q / 7 + 1 : q << 3;  // the q-th t with t % 8 != 0, or == 0
@@ -251,6 +253,7 @@ __global__ void k_split_link_rest(const int32_t *list, DevCounters *cnt, const i
 __global__ void __launch_bounds__(1024) k_split_link_big(const int32_t *big, const DevCounters *cnt,
                                                         const int64_t *off, const int32_t *deg, const int32_t *col,
                                                         const int32_t *C, int32_t *parent) {
+  ld_after_previous();
   int64_t m = cnt->big_count;
   for (int64_t t = blockIdx.x; t < m; t += gridDim.x) {
     int32_t i = big[t];
@@ -277,16 +280,19 @@ __global__ void k_split_compress(const int32_t *list, const DevCounters *cnt, in
 // pass are renumbered; the others are mapped to one spare id past the dense
 // range (rank[n]), which aggregation leaves out.
 __global__ void k_used(int64_t n, const int32_t *C, int32_t *used, const int32_t *gid, const uint8_t *cont) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride())
     if (!gid || cont[gid[i]]) used[C[i]] = 1;
 }
 __global__ void k_rank(int64_t n, const int64_t *rank, int32_t *C, const int32_t *gid, const uint8_t *cont) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride())
     C[i] = (int32_t)((!gid || cont[gid[i]]) ? rank[C[i]] : rank[n]);
 }
 // (first: Ctop is the identity, which is not written out)
 __global__ void k_lookup(int64_t N, const int32_t *Cp, int32_t *Ctop, const int32_t *gid0, const uint8_t *cont,
                          bool first) {
+  ld_after_previous();
   for (int64_t v = ld_gtid(); v < N; v += ld_gstride())
     if (!gid0 || cont[gid0[v]]) Ctop[v] = Cp[first ? v : Ctop[v]];
 }
@@ -297,6 +303,7 @@ __global__ void k_lookup(int64_t N, const int32_t *Cp, int32_t *Ctop, const int3
 __global__ void k_break_lookup(int64_t N, const int32_t *Cp, int32_t *Ctop, const int32_t *gid0, const uint8_t *cont,
                                const int64_t *loff, const int64_t *voff, int64_t n, const int32_t *gid,
                                uint8_t *used, bool first) {
+  ld_after_previous();
   for (int64_t v = ld_gtid(); v < N; v += ld_gstride()) {
     int32_t g = gid0[v];
     if (loff[g + 1] > loff[g] && !cont[g]) Ctop[v] = (int32_t)(Cp[first ? v : Ctop[v]] - loff[g] + voff[g]);
@@ -309,10 +316,12 @@ __global__ void k_break_lookup(int64_t N, const int32_t *Cp, int32_t *Ctop, cons
 // Graph of each super-vertex and the graphs' ranges at the next level.
 __global__ void k_level_ids(int64_t n, const int32_t *Cdense, const int32_t *gid, const uint8_t *cont,
                             int32_t *gid_next) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride())
     if (cont[gid[i]]) gid_next[Cdense[i]] = gid[i];
 }
 __global__ void k_level_off(int G, const int64_t *loff, const int64_t *rank, int64_t *loff_next) {
+  ld_after_previous();
   for (int64_t g = ld_gtid(); g <= G; g += ld_gstride()) loff_next[g] = rank[loff[g]];
 }
 // After refinement every community id is one of its members and that
@@ -320,6 +329,7 @@ __global__ void k_level_off(int G, const int64_t *loff, const int64_t *rank, int
 // splitting the smallest vertex of a component, refinement a stationary
 // representative), so the communities are the vertices with C[i] == i.
 __global__ void k_count_roots(int64_t n, const int32_t *C, DevCounters *cnt, const int32_t *gid, int32_t *ncg) {
+  ld_after_previous();
   int32_t local = 0;
   for (int64_t b = (ld_gtid() & ~31ll); b < n; b += ld_gstride()) {  // warp-uniform trip count
     int64_t i = b + (threadIdx.x & 31);
@@ -352,6 +362,7 @@ __device__ __forceinline__ int32_t member_claim(int32_t *hk, int32_t c) {
 }
 
 __global__ void __launch_bounds__(256) k_member_count(int64_t n, const int32_t *C, int32_t *cnt_c) {
+  ld_after_previous();
   __shared__ int32_t hk[MEMBER_SLOTS], hv[MEMBER_SLOTS];
   for (int s = threadIdx.x; s < MEMBER_SLOTS; s += blockDim.x) { hk[s] = -1; hv[s] = 0; }
   __syncthreads();
@@ -380,6 +391,7 @@ __global__ void __launch_bounds__(256) k_member_count(int64_t n, const int32_t *
 // block visit the same vertices.
 __global__ void __launch_bounds__(256) k_member_fill(int64_t n, const int32_t *C, unsigned long long *cursor,
                                                      int32_t *cverts) {
+  ld_after_previous();
   __shared__ int32_t hk[MEMBER_SLOTS], hv[MEMBER_SLOTS];
   __shared__ unsigned long long hb[MEMBER_SLOTS];
   for (int s = threadIdx.x; s < MEMBER_SLOTS; s += blockDim.x) { hk[s] = -1; hv[s] = 0; }
@@ -416,10 +428,12 @@ __global__ void __launch_bounds__(256) k_member_fill(int64_t n, const int32_t *C
   }
 }
 __global__ void k_member_deg(int64_t n, const int32_t *cverts, const int32_t *deg, int32_t *mdeg) {
+  ld_after_previous();
   for (int64_t t = ld_gtid(); t < n; t += ld_gstride()) mdeg[t] = deg[cverts[t]];
 }
 // super-row offsets: yoff[c] = flat offset of the community's first member
 __global__ void k_yoff(int64_t ncomm, const int64_t *coff, const int64_t *cflat, int64_t *yoff, DevCounters *cnt) {
+  ld_after_previous();
   for (int64_t c = ld_gtid(); c <= ncomm; c += ld_gstride()) {
     yoff[c] = cflat[coff[c]];
     if (c < ncomm) {
@@ -489,6 +503,7 @@ constexpr int AGG_WARPS = 8;
 // the sum of the arcs read.
 template <typename W, bool WIDE>
 __global__ void __launch_bounds__(AGG_WARPS * 32) k_agg_warp(AggArgs A) {
+  ld_after_previous();
   __shared__ WarpTable<WIDE> WT[AGG_WARPS];
   const W *w = (const W *)A.w;
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -570,6 +585,7 @@ constexpr int AGG_TINY = 8;
 
 template <typename W>
 __global__ void __launch_bounds__(256) k_agg_tiny(AggArgs A) {
+  ld_after_previous();
   const W *w = (const W *)A.w;
   const int lane = threadIdx.x & 31, g = lane & 7, grp = lane >> 3;
   const uint32_t gmask = 0xffu << (grp * 8);
@@ -632,6 +648,7 @@ __global__ void __launch_bounds__(256) k_agg_tiny(AggArgs A) {
 // above (R-MAT 21, static, level 0: 2748 -> 722 us).
 template <typename W, bool WIDE>
 __global__ void __launch_bounds__(256) k_agg_block(AggArgs A) {
+  ld_after_previous();
   __shared__ STable<WIDE, STAGE_SLOTS, STAGE_FILL, uint16_t> T;
   __shared__ int32_t filled;
   __shared__ unsigned long long self_s, sum_s;
@@ -759,6 +776,7 @@ __device__ __forceinline__ void agg_take(const AggArgs &A, WarpTable<WIDE> &T8, 
 
 template <typename W, bool WIDE>
 __global__ void __launch_bounds__(256, 4) k_agg_chunk_scan(AggArgs A, const int64_t *tab_off, const int64_t *ch_off) {
+  ld_after_previous();
   __shared__ WarpTable<WIDE> WT[8];  // per-warp sums by community
   WarpTable<WIDE> &T8 = WT[threadIdx.x >> 5];
   wt_init(T8);
@@ -859,6 +877,7 @@ constexpr int EMIT_CHUNK = 2048;
 constexpr int EMIT_UNROLL = 4;
 
 __global__ void __launch_bounds__(1024) k_emit_plan(const int32_t *count_p, const int32_t *occ, int64_t *em_off) {
+  ld_after_previous();
   __shared__ int64_t ws[32];
   __shared__ int64_t carry;
   int64_t count = *count_p;
@@ -888,6 +907,7 @@ __global__ void __launch_bounds__(1024) k_emit_plan(const int32_t *count_p, cons
 
 template <bool WIDE>
 __global__ void __launch_bounds__(256) k_agg_list_emit(AggArgs A, const int64_t *tab_off, const int64_t *em_off) {
+  ld_after_previous();
   int64_t count = *A.count;
   int64_t npc = em_off[count];
   for (int64_t t = blockIdx.x; t < npc; t += gridDim.x) {
@@ -923,6 +943,7 @@ __global__ void __launch_bounds__(256) k_agg_list_emit(AggArgs A, const int64_t 
 // Before the chunked scan: empty fill counts, and zero the K of the listed
 // communities (the scan adds its chunks' weight sums into it).
 __global__ void k_zero_occ(const int32_t *count_p, const int32_t *list, int32_t *occ, int64_t *Kout) {
+  ld_after_previous();
   for (int64_t k = ld_gtid(); k < *count_p; k += ld_gstride()) {
     occ[k] = 0;
     Kout[list[k]] = 0;
@@ -930,6 +951,7 @@ __global__ void k_zero_occ(const int32_t *count_p, const int32_t *list, int32_t 
 }
 
 __global__ void k_agg_bin(int64_t ncomm, const int64_t *yoff, const int64_t *coff, int32_t *bins, DevCounters *cnt) {
+  ld_after_previous();
   int lane = threadIdx.x & 31;
   for (int64_t base = (ld_gtid() & ~31ll); base < ncomm; base += ld_gstride()) {
     int64_t c = base + lane;
@@ -955,6 +977,7 @@ __global__ void k_agg_bin(int64_t ncomm, const int64_t *yoff, const int64_t *cof
 // The state of the next level, every super-vertex on its own and unprocessed.
 __global__ void k_next_pass(int64_t nc, const int64_t *Kout, int64_t *Kp, int64_t *Sp, int32_t *Cp, uint8_t *dR,
                             uint8_t *dS, int32_t *size, int32_t *rep, uint32_t *bm) {
+  ld_after_previous();
   for (int64_t c = ld_gtid(); c < nc; c += ld_gstride()) {
     Kp[c] = Kout[c]; Sp[c] = Kout[c]; Cp[c] = (int32_t)c; dR[c] = 1; dS[c] = 0;
     size[c] = 1;
@@ -971,6 +994,7 @@ __global__ void k_next_pass(int64_t nc, const int64_t *Kout, int64_t *Kp, int64_
 __global__ void k_pass_init(int64_t n, const uint8_t *dV, uint32_t *bm, const int32_t *C, int32_t *Cp,
                             const int64_t *Sig, int64_t *Sp, const int32_t *size0, int32_t *size, int32_t *rep,
                             DevCounters *cnt) {
+  ld_after_previous();
   int lane = threadIdx.x & 31;
   int64_t set = 0;
   int64_t nq = (n >> 5) << 3;  // quads of whole 32-vertex words
@@ -1014,6 +1038,7 @@ __global__ void k_pass_init(int64_t n, const uint8_t *dV, uint32_t *bm, const in
 }
 
 __global__ void k_maxdeg(int64_t n, const int32_t *deg, DevCounters *cnt, int block_max) {
+  ld_after_previous();
   int32_t mx = 0;
   int64_t slots = 0, sum = 0;
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) {
@@ -1049,58 +1074,61 @@ void renumber_and_split(leiden_handle *h, const LevelGraph &g) {
   cudaMemsetAsync(&h->dcnt->split_arcs, 0, sizeof(int64_t) + 2 * sizeof(int32_t), s);
   int32_t *list = h->ibuf1;
   ld_note_launch(), launch_after(k_sr_min, grid_for(g.n, TB), TB, s, g.n, h->Cp, h->rep);
-  ld_note_launch(), launch_after(k_remap_list, grid_for(g.n, APPEND_STEP), 256, s, g.n, h->rep, h->dS, h->dR, g.deg, h->Cp,
-                                                                            h->dR2, h->parent, list, h->dcnt,
-                                                                            h->p.split_all);
+  ld_note_launch(), launch_after(k_remap_list, grid_for(g.n, APPEND_STEP), 256, s, g.n, h->rep, h->dS, h->dR, g.deg,
+                                 h->Cp, h->dR2, h->parent, list, h->dcnt, h->p.split_all);
   kt_begin(h, KT_SPLIT_SAMPLE);
   if (g.n <= SPLIT_APART) {
     ld_note_launch(), launch_after(k_split_sample, h->sm_count * 16, TB, s, list, h->dcnt, g.off, g.deg, g.col, h->Cp,
-                                                                     h->parent);
+                                   h->parent);
   } else {
     int2 *hit = (int2 *)h->lbuf0;
-    ld_note_launch(), k_split_find<<<h->sm_count * 8, 256, 0, s>>>(list, h->dcnt, g.off, g.deg, g.col, h->Cp, hit);
-    ld_note_launch(), k_split_link<<<h->sm_count * 4, 256, 0, s>>>(list, h->dcnt, h->parent, hit, false);
+    ld_note_launch(), launch_after(k_split_find, h->sm_count * 8, 256, s, list, h->dcnt, g.off, g.deg, g.col, h->Cp,
+                                   hit);
+    ld_note_launch(), launch_after(k_split_link, h->sm_count * 4, 256, s, list, h->dcnt, h->parent, hit, false);
     ld_note_launch(), launch_after(k_split_flatten, h->sm_count * 8, TB, s, list, h->dcnt, h->parent);
-    ld_note_launch(), k_split_link<<<h->sm_count * 8, 256, 0, s>>>(list, h->dcnt, h->parent, hit, true);
+    ld_note_launch(), launch_after(k_split_link, h->sm_count * 8, 256, s, list, h->dcnt, h->parent, hit, true);
   }
   kt_end(h);
   ld_note_launch(), launch_after(k_split_flatten, h->sm_count * 8, TB, s, list, h->dcnt, h->parent);
-  ld_note_launch(), launch_after(k_split_link_rest, h->sm_count * 8, TB, s, list, h->dcnt, g.off, g.deg, g.col, h->Cp, h->parent, h->ibuf2);
+  ld_note_launch(), launch_after(k_split_link_rest, h->sm_count * 8, TB, s, list, h->dcnt, g.off, g.deg, g.col, h->Cp,
+                                 h->parent, h->ibuf2);
   if (g.maxdeg > SPLIT_BIG)
-    ld_note_launch(), k_split_link_big<<<h->sm_count, 1024, 0, s>>>(h->ibuf2, h->dcnt, g.off, g.deg, g.col, h->Cp, h->parent);
+    ld_note_launch(), launch_after(k_split_link_big, h->sm_count, 1024, s, h->ibuf2, h->dcnt, g.off, g.deg, g.col,
+                                   h->Cp, h->parent);
   ld_note_launch(), launch_after(k_split_compress, h->sm_count * 8, TB, s, list, h->dcnt, h->parent, h->Cp);
 }
 
 void count_communities(leiden_handle *h, int64_t n, const int32_t *gid) {
   cudaStream_t s = h->stream;
   cudaMemsetAsync(&h->dcnt->list_count, 0, sizeof(int32_t), s);
-  ld_note_launch(), k_count_roots<<<grid_for(n, TB), TB, 0, s>>>(n, h->Cp, h->dcnt, gid, h->gc.ncomm);
+  ld_note_launch(), launch_after(k_count_roots, grid_for(n, TB), TB, s, n, h->Cp, h->dcnt, gid, h->gc.ncomm);
 }
 
 void renumber_dense(leiden_handle *h, int64_t n, const int32_t *gid) {
   cudaStream_t s = h->stream;
   const uint8_t *cont = gid ? h->gc.cont : nullptr;
   cudaMemsetAsync(h->ibuf0, 0, (size_t)n * sizeof(int32_t), s);
-  ld_note_launch(), k_used<<<grid_for(n, TB), TB, 0, s>>>(n, h->Cp, h->ibuf0, gid, cont);
+  ld_note_launch(), launch_after(k_used, grid_for(n, TB), TB, s, n, h->Cp, h->ibuf0, gid, cont);
   exclusive_scan_i32_to_i64(h->ibuf0, h->lbuf0, n, h->scan_tmp, s);
-  ld_note_launch(), k_rank<<<grid_for(n, TB), TB, 0, s>>>(n, h->lbuf0, h->Cp, gid, cont);
+  ld_note_launch(), launch_after(k_rank, grid_for(n, TB), TB, s, n, h->lbuf0, h->Cp, gid, cont);
 }
 
 void lookup_dendrogram(leiden_handle *h, bool first) {
   const uint8_t *cont = h->gid0 ? h->gc.cont : nullptr;
-  ld_note_launch(), k_lookup<<<grid_for(h->n, TB), TB, 0, h->stream>>>(h->n, h->Cp, h->Ctop, h->gid0, cont, first);
+  ld_note_launch(), launch_after(k_lookup, grid_for(h->n, TB), TB, h->stream, h->n, h->Cp, h->Ctop, h->gid0, cont,
+                                 first);
 }
 
 void break_lookup(leiden_handle *h, int64_t n, const int32_t *gid, bool first) {
   if (first) cudaMemsetAsync(h->dE, 0, (size_t)h->n, h->stream);
-  ld_note_launch(), k_break_lookup<<<grid_for(h->n, TB), TB, 0, h->stream>>>(
-      h->n, h->Cp, h->Ctop, h->gid0, h->gc.cont, h->d_loff, h->d_voff, n, gid, h->dE, first);
+  ld_note_launch(), launch_after(k_break_lookup, grid_for(h->n, TB), TB, h->stream, h->n, h->Cp, h->Ctop, h->gid0,
+                                 h->gc.cont, h->d_loff, h->d_voff, n, gid, h->dE, first);
 }
 
 void next_level_ids(leiden_handle *h, int64_t n, const int32_t *gid, int32_t *gid_next, int64_t *loff_next) {
   cudaStream_t s = h->stream;
-  ld_note_launch(), k_level_ids<<<grid_for(n, TB), TB, 0, s>>>(n, h->Cp, gid, h->gc.cont, gid_next);
-  ld_note_launch(), k_level_off<<<grid_for(h->G + 1, TB), TB, 0, s>>>(h->G, h->d_loff, h->lbuf0, loff_next);
+  ld_note_launch(), launch_after(k_level_ids, grid_for(n, TB), TB, s, n, h->Cp, gid, h->gc.cont, gid_next);
+  ld_note_launch(), launch_after(k_level_off, grid_for(h->G + 1, TB), TB, s, h->G, h->d_loff, h->lbuf0, loff_next);
 }
 
 // Aggregate level g by its dense membership Cp into slot `out`; K'' goes to
@@ -1112,18 +1140,21 @@ void aggregate(leiden_handle *h, const LevelGraph &g, int64_t ncomm, int out) {
   // vertices in one spare community ncomm, listed last and not aggregated
   int64_t nc = ncomm + (g.gid ? 1 : 0);
   cudaMemsetAsync(h->ibuf0, 0, (size_t)nc * sizeof(int32_t), s);
-  ld_note_launch(), k_member_count<<<grid_for(n, TB), TB, 0, s>>>(n, h->Cp, h->ibuf0);
+  ld_note_launch(), launch_after(k_member_count, grid_for(n, TB), TB, s, n, h->Cp, h->ibuf0);
   exclusive_scan_i32_to_i64(h->ibuf0, h->coff, nc, h->scan_tmp, s);
   cudaMemcpyAsync(h->lbuf0, h->coff, (size_t)nc * sizeof(int64_t), cudaMemcpyDeviceToDevice, s);
-  ld_note_launch(), k_member_fill<<<grid_for(n, TB), TB, 0, s>>>(n, h->Cp, (unsigned long long *)h->lbuf0, h->cverts);
+  ld_note_launch(), launch_after(k_member_fill, grid_for(n, TB), TB, s, n, h->Cp, (unsigned long long *)h->lbuf0,
+                                 h->cverts);
   // flat arc offsets of the members, and the super-row offsets
-  ld_note_launch(), k_member_deg<<<grid_for(n, TB), TB, 0, s>>>(n, h->cverts, g.deg, h->ibuf1);
+  ld_note_launch(), launch_after(k_member_deg, grid_for(n, TB), TB, s, n, h->cverts, g.deg, h->ibuf1);
   exclusive_scan_i32_to_i64(h->ibuf1, h->cflat, n, h->scan_tmp, s);
   cudaMemsetAsync(&h->dcnt->max_count, 0, sizeof(int32_t), s);
   cudaMemsetAsync(&h->dcnt->huge_slots, 0, sizeof(int64_t), s);
-  ld_note_launch(), k_yoff<<<grid_for(ncomm + 1, TB), TB, 0, s>>>(ncomm, h->coff, h->cflat, h->y_off[out], h->dcnt);
+  ld_note_launch(), launch_after(k_yoff, grid_for(ncomm + 1, TB), TB, s, ncomm, h->coff, h->cflat, h->y_off[out],
+                                 h->dcnt);
   cudaMemsetAsync(&h->dcnt->ref, 0, sizeof(SubCounters), s);
-  ld_note_launch(), k_agg_bin<<<grid_for(ncomm, TB), TB, 0, s>>>(ncomm, h->y_off[out], h->coff, h->bins, h->dcnt);
+  ld_note_launch(), launch_after(k_agg_bin, grid_for(ncomm, TB), TB, s, ncomm, h->y_off[out], h->coff, h->bins,
+                                 h->dcnt);
   cudaMemcpyAsync(&h->hcnt->max_count, &h->dcnt->max_count, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
   cudaMemcpyAsync(&h->hcnt->huge_slots, &h->dcnt->huge_slots, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
   cudaStreamSynchronize(s);
@@ -1146,20 +1177,20 @@ void aggregate(leiden_handle *h, const LevelGraph &g, int64_t ncomm, int out) {
   int sms = h->sm_count;
   A.list = h->bins + (int64_t)BIN_TINY * ncomm;
   A.count = &h->dcnt->ref.bin_count[BIN_TINY];
-  if (g.w64) ld_note_launch(), k_agg_tiny<int64_t><<<sms * 8, 256, 0, s>>>(A);
-  else ld_note_launch(), k_agg_tiny<int32_t><<<sms * 8, 256, 0, s>>>(A);
+  if (g.w64) ld_note_launch(), launch_after(k_agg_tiny<int64_t>, sms * 8, 256, s, A);
+  else ld_note_launch(), launch_after(k_agg_tiny<int32_t>, sms * 8, 256, s, A);
   A.list = h->bins;
   A.count = &h->dcnt->ref.bin_count[BIN_WARP];
   const bool wide = wide_sums(h);
   auto agg_warp = wide ? (g.w64 ? k_agg_warp<int64_t, true> : k_agg_warp<int32_t, true>)
                        : (g.w64 ? k_agg_warp<int64_t, false> : k_agg_warp<int32_t, false>);
-  ld_note_launch(), agg_warp<<<sms * 8, AGG_WARPS * 32, 0, s>>>(A);
+  ld_note_launch(), launch_after(agg_warp, sms * 8, AGG_WARPS * 32, s, A);
   if (maxc > BIN_WARP_MAX) {
     A.list = h->bins + ncomm;
     A.count = &h->dcnt->ref.bin_count[BIN_BLOCK];
     auto agg_block = wide ? (g.w64 ? k_agg_block<int64_t, true> : k_agg_block<int32_t, true>)
                           : (g.w64 ? k_agg_block<int64_t, false> : k_agg_block<int32_t, false>);
-    ld_note_launch(), agg_block<<<sms * 8, 256, 0, s>>>(A);
+    ld_note_launch(), launch_after(agg_block, sms * 8, 256, s, A);
   }
   if (maxc > BIN_BLOCK_MAX) {
     // a table per listed community at once: at most huge_slots slots
@@ -1173,31 +1204,31 @@ void aggregate(leiden_handle *h, const LevelGraph &g, int64_t ncomm, int out) {
     int64_t *tab_off = h->lbuf2, *ch_off = h->lbuf3;
     // a community's super-row has at most one key per community
     launch_table_plan(A.list, A.count, nullptr, h->y_off[out], ncomm, tab_off, ch_off, s);
-    ld_note_launch(), k_zero_occ<<<sms, 256, 0, s>>>(A.count, A.list, A.gocc, A.Kout);
+    ld_note_launch(), launch_after(k_zero_occ, sms, 256, s, A.count, A.list, A.gocc, A.Kout);
     A.xk_bytes = &h->dcnt->xk_bytes[1];
     A.tables = h->dcnt->agg_tables;
     kt_begin(h, KT_AGG_CHUNK);
     auto scan = wide ? (g.w64 ? k_agg_chunk_scan<int64_t, true> : k_agg_chunk_scan<int32_t, true>)
                              : (g.w64 ? k_agg_chunk_scan<int64_t, false> : k_agg_chunk_scan<int32_t, false>);
-    ld_note_launch(), scan<<<sms * 16, 256, 0, s>>>(A, tab_off, ch_off);
+    ld_note_launch(), launch_after(scan, sms * 16, 256, s, A, tab_off, ch_off);
     kt_end(h);
     int64_t *em_off = h->lbuf0;  // free again after the member fill
-    ld_note_launch(), k_emit_plan<<<1, 1024, 0, s>>>(A.count, A.gocc, em_off);
+    ld_note_launch(), launch_after(k_emit_plan, 1, 1024, s, A.count, A.gocc, em_off);
     auto emit = wide ? k_agg_list_emit<true> : k_agg_list_emit<false>;
-    ld_note_launch(), emit<<<sms * 8, 256, 0, s>>>(A, tab_off, em_off);
+    ld_note_launch(), launch_after(emit, sms * 8, 256, s, A, tab_off, em_off);
   }
 }
 
 void reset_next_pass(leiden_handle *h, int64_t ncomm, int out) {
   (void)out;
-  ld_note_launch(), k_next_pass<<<grid_for(ncomm, TB), TB, 0, h->stream>>>(ncomm, h->S2, h->Kp, h->Sp, h->Cp, h->dR,
-                                                                           h->dS, h->csize, h->rep, h->unproc);
+  ld_note_launch(), launch_after(k_next_pass, grid_for(ncomm, TB), TB, h->stream, ncomm, h->S2, h->Kp, h->Sp, h->Cp,
+                                 h->dR, h->dS, h->csize, h->rep, h->unproc);
   h->Kc = h->Kp;
 }
 
 void pass_init(leiden_handle *h, bool sizes_kept) {
-  ld_note_launch(), k_pass_init<<<grid_for(h->n, TB), TB, 0, h->stream>>>(
-      h->n, h->dV, h->unproc, h->C, h->Cp, h->Sig, h->Sp, sizes_kept ? h->csize0 : nullptr, h->csize, h->rep, h->dcnt);
+  ld_note_launch(), launch_after(k_pass_init, grid_for(h->n, TB), TB, h->stream, h->n, h->dV, h->unproc, h->C, h->Cp,
+                                 h->Sig, h->Sp, sizes_kept ? h->csize0 : nullptr, h->csize, h->rep, h->dcnt);
   h->Kc = h->K;
 }
 
@@ -1205,7 +1236,7 @@ void level_maxdeg(leiden_handle *h, const int32_t *deg, int64_t n) {
   cudaMemsetAsync(&h->dcnt->max_count, 0, sizeof(int32_t), h->stream);
   cudaMemsetAsync(&h->dcnt->huge_slots, 0, sizeof(int64_t), h->stream);
   cudaMemsetAsync(&h->dcnt->deg_sum, 0, sizeof(int64_t), h->stream);
-  ld_note_launch(), k_maxdeg<<<grid_for(n, TB), TB, 0, h->stream>>>(n, deg, h->dcnt, h->tune.block_max);
+  ld_note_launch(), launch_after(k_maxdeg, grid_for(n, TB), TB, h->stream, n, deg, h->dcnt, h->tune.block_max);
 }
 
 LD_CHECK_WORD_READER(check_word_phases)

@@ -42,6 +42,7 @@ __device__ __forceinline__ int64_t block_excl_scan(int64_t v, int64_t *total) {
 
 template <typename T>
 __global__ void scan_tile_reduce(const T *in, int64_t n, int64_t *tile_sums) {
+  ld_after_previous();
   int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
   int64_t s = 0;
 #pragma unroll
@@ -55,6 +56,7 @@ __global__ void scan_tile_reduce(const T *in, int64_t n, int64_t *tile_sums) {
 // Single block: exclusive scan of the tile sums in place; writes the grand
 // total to *grand.
 __global__ void scan_tile_offsets(int64_t *tile_sums, int64_t ntiles, int64_t *grand) {
+  ld_after_previous();
   int64_t carry = 0;
   for (int64_t base = 0; base < ntiles; base += SCAN_BLOCK) {
     int64_t i = base + threadIdx.x;
@@ -69,6 +71,7 @@ __global__ void scan_tile_offsets(int64_t *tile_sums, int64_t ntiles, int64_t *g
 
 template <typename T>
 __global__ void scan_tile_apply(const T *in, int64_t *out, int64_t n, const int64_t *tile_offs) {
+  ld_after_previous();
   int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
   int64_t v[SCAN_ITEMS];
   int64_t s = 0;
@@ -92,6 +95,7 @@ __global__ void scan_tile_apply(const T *in, int64_t *out, int64_t n, const int6
 constexpr int64_t SCAN_PREFIX_MAX = 4096;
 template <typename T>
 __global__ void scan_tile_apply_prefix(const T *in, int64_t *out, int64_t n, const int64_t *tile_sums) {
+  ld_after_previous();
   __shared__ int64_t red[SCAN_BLOCK / 32];
   int64_t b = blockIdx.x;
   int64_t p = 0;
@@ -125,6 +129,7 @@ __global__ void scan_tile_apply_prefix(const T *in, int64_t *out, int64_t n, con
 // first barrier, so in == out is safe).
 template <typename T>
 __global__ void scan_single_tile(const T *in, int64_t *out, int64_t n) {
+  ld_after_previous();
   int64_t base = (int64_t)threadIdx.x * SCAN_ITEMS;
   int64_t v[SCAN_ITEMS];
   int64_t s = 0;
@@ -152,14 +157,14 @@ cudaError_t scan_impl(const T *in, int64_t *out, int64_t n, void *tmp, cudaStrea
   if (n <= 0) {
     cudaMemsetAsync(out, 0, sizeof(int64_t), s);
   } else if (ntiles == 1) {
-    ld_note_launch(), scan_single_tile<T><<<1, SCAN_BLOCK, 0, s>>>(in, out, n);
+    ld_note_launch(), launch_after(scan_single_tile<T>, 1, SCAN_BLOCK, s, in, out, n);
   } else if (ntiles <= SCAN_PREFIX_MAX) {
-    ld_note_launch(), scan_tile_reduce<T><<<(unsigned)ntiles, SCAN_BLOCK, 0, s>>>(in, n, tile);
-    ld_note_launch(), scan_tile_apply_prefix<T><<<(unsigned)ntiles, SCAN_BLOCK, 0, s>>>(in, out, n, tile);
+    ld_note_launch(), launch_after(scan_tile_reduce<T>, (unsigned)ntiles, SCAN_BLOCK, s, in, n, tile);
+    ld_note_launch(), launch_after(scan_tile_apply_prefix<T>, (unsigned)ntiles, SCAN_BLOCK, s, in, out, n, tile);
   } else {
-    ld_note_launch(), scan_tile_reduce<T><<<(unsigned)ntiles, SCAN_BLOCK, 0, s>>>(in, n, tile);
-    ld_note_launch(), scan_tile_offsets<<<1, SCAN_BLOCK, 0, s>>>(tile, ntiles, out + n);
-    ld_note_launch(), scan_tile_apply<T><<<(unsigned)ntiles, SCAN_BLOCK, 0, s>>>(in, out, n, tile);
+    ld_note_launch(), launch_after(scan_tile_reduce<T>, (unsigned)ntiles, SCAN_BLOCK, s, in, n, tile);
+    ld_note_launch(), launch_after(scan_tile_offsets, 1, SCAN_BLOCK, s, tile, ntiles, out + n);
+    ld_note_launch(), launch_after(scan_tile_apply<T>, (unsigned)ntiles, SCAN_BLOCK, s, in, out, n, tile);
   }
   return cudaGetLastError();
 }
@@ -170,6 +175,7 @@ constexpr int RS_ROUNDS = 4;  // short tiles: a batch of 1e5 keys still spreads 
 constexpr int RS_TILE = RS_BLOCK * RS_ROUNDS;
 
 __global__ void rs_hist(const uint64_t *keys, int64_t n, int shift, int64_t nblocks, int64_t *hist) {
+  ld_after_previous();
   __shared__ int32_t cnt[256];
   cnt[threadIdx.x] = 0;
   __syncthreads();
@@ -187,6 +193,7 @@ __global__ void rs_hist(const uint64_t *keys, int64_t n, int shift, int64_t nblo
 // lane order decides (match_any gives the peers with the same digit).
 __global__ void rs_scatter(const uint64_t *keys, const int64_t *vals, uint64_t *okeys, int64_t *ovals,
                            int64_t n, int shift, int64_t nblocks, const int64_t *offs) {
+  ld_after_previous();
   __shared__ int64_t base_off[256];
   __shared__ int32_t wcnt[RS_BLOCK / 32][256];
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -234,6 +241,7 @@ __global__ void rs_scatter(const uint64_t *keys, const int64_t *vals, uint64_t *
 // the output equals the radix sort's.
 constexpr int SMALL_SORT_MAX = 2048;
 __global__ void __launch_bounds__(1024) k_small_sort(uint64_t *keys, int64_t *vals, int n, uint64_t mask) {
+  ld_after_previous();
   __shared__ uint64_t sk[SMALL_SORT_MAX];
   __shared__ int32_t si[SMALL_SORT_MAX];
   int P = 1;
@@ -294,7 +302,7 @@ cudaError_t radix_sort_u64(uint64_t *keys, uint64_t *keys_alt, int64_t *vals, in
   if (n <= 1) return cudaSuccess;
   if (n <= SMALL_SORT_MAX) {
     uint64_t mask = bits >= 64 ? ~0ull : ((1ull << bits) - 1);
-    ld_note_launch(), k_small_sort<<<1, 1024, 0, s>>>(keys, vals, (int)n, mask);
+    ld_note_launch(), launch_after(k_small_sort, 1, 1024, s, keys, vals, (int)n, mask);
     return cudaGetLastError();
   }
   int64_t nblocks = (n + RS_TILE - 1) / RS_TILE;
@@ -306,10 +314,11 @@ cudaError_t radix_sort_u64(uint64_t *keys, uint64_t *keys_alt, int64_t *vals, in
   int64_t *vsrc = vals, *vdst = vals_alt;
   int passes = 0;
   for (int shift = 0; shift < bits; shift += 8) {
-    ld_note_launch(), rs_hist<<<(unsigned)nblocks, RS_BLOCK, 0, s>>>(src, n, shift, nblocks, hist);
+    ld_note_launch(), launch_after(rs_hist, (unsigned)nblocks, RS_BLOCK, s, src, n, shift, nblocks, hist);
     cudaError_t e = exclusive_scan_i64(hist, offs, hlen, stmp, s);
     if (e != cudaSuccess) return e;
-    ld_note_launch(), rs_scatter<<<(unsigned)nblocks, RS_BLOCK, 0, s>>>(src, vsrc, dst, vdst, n, shift, nblocks, offs);
+    ld_note_launch(), launch_after(rs_scatter, (unsigned)nblocks, RS_BLOCK, s, src, vsrc, dst, vdst, n, shift, nblocks,
+                                   offs);
     uint64_t *t = src; src = dst; dst = t;
     int64_t *tv = vsrc; vsrc = vdst; vdst = tv;
     passes++;
@@ -331,6 +340,7 @@ namespace {
 __global__ void __launch_bounds__(1024) k_table_plan(const int32_t *list, const int32_t *count_p,
                                                       const int32_t *deg32, const int64_t *off64, int64_t key_cap,
                                                       int64_t *tab_off, int64_t *ch_off, int32_t *occ) {
+  ld_after_previous();
   __shared__ int64_t ws[2][32];
   int64_t count = *count_p;
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -376,6 +386,7 @@ __global__ void __launch_bounds__(1024) k_table_plan(const int32_t *list, const 
 // One block: the items whose tables hold more than BIG_KEYS keys, with the
 // offsets of their pieces of BIG_PIECE keys and their tickets zeroed.
 __global__ void __launch_bounds__(1024) k_piece_plan(const int32_t *count_p, const int32_t *occ, BigTables big) {
+  ld_after_previous();
   __shared__ int64_t ws[2][32];
   int64_t count = *count_p;
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -414,12 +425,15 @@ __global__ void __launch_bounds__(1024) k_piece_plan(const int32_t *count_p, con
 }
 
 __global__ void k_fill_i32(int32_t *p, int32_t v, int64_t n) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) p[i] = v;
 }
 __global__ void k_fill_i64(int64_t *p, int64_t v, int64_t n) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) p[i] = v;
 }
 __global__ void k_iota_i32(int32_t *p, int64_t n) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) p[i] = (int32_t)i;
 }
 }  // namespace
@@ -432,19 +446,19 @@ int grid_for(int64_t n, int block, int max_blocks) {
 }
 
 void launch_fill_i32(int32_t *p, int32_t v, int64_t n, cudaStream_t s) {
-  if (n > 0) ld_note_launch(), k_fill_i32<<<grid_for(n, 256), 256, 0, s>>>(p, v, n);
+  if (n > 0) ld_note_launch(), launch_after(k_fill_i32, grid_for(n, 256), 256, s, p, v, n);
 }
 void launch_fill_i64(int64_t *p, int64_t v, int64_t n, cudaStream_t s) {
-  if (n > 0) ld_note_launch(), k_fill_i64<<<grid_for(n, 256), 256, 0, s>>>(p, v, n);
+  if (n > 0) ld_note_launch(), launch_after(k_fill_i64, grid_for(n, 256), 256, s, p, v, n);
 }
 void launch_table_plan(const int32_t *list, const int32_t *count, const int32_t *deg32, const int64_t *off64,
                        int64_t key_cap, int64_t *tab_off, int64_t *ch_off, cudaStream_t s, int32_t *occ) {
-  ld_note_launch(), k_table_plan<<<1, 1024, 0, s>>>(list, count, deg32, off64, key_cap, tab_off, ch_off, occ);
+  ld_note_launch(), launch_after(k_table_plan, 1, 1024, s, list, count, deg32, off64, key_cap, tab_off, ch_off, occ);
 }
 void launch_piece_plan(const int32_t *count, const int32_t *occ, const BigTables &big, cudaStream_t s) {
-  ld_note_launch(), k_piece_plan<<<1, 1024, 0, s>>>(count, occ, big);
+  ld_note_launch(), launch_after(k_piece_plan, 1, 1024, s, count, occ, big);
 }
 
 void launch_iota_i32(int32_t *p, int64_t n, cudaStream_t s) {
-  if (n > 0) ld_note_launch(), k_iota_i32<<<grid_for(n, 256), 256, 0, s>>>(p, n);
+  if (n > 0) ld_note_launch(), launch_after(k_iota_i32, grid_for(n, 256), 256, s, p, n);
 }

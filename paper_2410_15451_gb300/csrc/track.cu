@@ -23,6 +23,7 @@ __device__ __forceinline__ uint64_t hash64(uint64_t k) { return ld_splitmix64(k)
 // candidates -1, use flags and deviant weights 0.
 __global__ void k_tr_init(int64_t N, long long *bw, int32_t *bc, long long *ow, int32_t *ob, int32_t *cand,
                           int32_t *used, int64_t *dev) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < N; i += ld_gstride()) {
     bw[i] = -1;
     bc[i] = INT_MAX;
@@ -34,6 +35,7 @@ __global__ void k_tr_init(int64_t N, long long *bw, int32_t *bc, long long *ow, 
   }
 }
 __global__ void k_trc_cand(int64_t N, const int32_t *Cold, const int32_t *Cnew, int32_t *cand) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < N; i += ld_gstride()) cand[Cold[i]] = Cnew[i];  // any member will do
 }
 // The weight of an old community is Sigma^{t-1} with K^t (the batch kept it
@@ -41,6 +43,7 @@ __global__ void k_trc_cand(int64_t N, const int32_t *Cold, const int32_t *Cnew, 
 // (the deviants) need adding up: ov = tot - deviant weight.
 __global__ void k_trc_deviants(int64_t N, const int32_t *Cold, const int32_t *Cnew, const int64_t *K,
                                const int32_t *cand, int64_t *dev) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < N; i += ld_gstride()) {
     int32_t o = Cold[i];
     if (Cnew[i] != cand[o]) {
@@ -54,6 +57,7 @@ __global__ void k_trc_deviants(int64_t N, const int32_t *Cold, const int32_t *Cn
 // vertices): every pair weighs 0, so the lowest new label of a member wins.
 __global__ void k_trc_majority(int64_t N, const int32_t *cand, const int64_t *tot, const int64_t *dev,
                                long long *bw, int32_t *bc, int32_t *flag) {
+  ld_after_previous();
   for (int64_t o = ld_gtid(); o < N; o += ld_gstride()) {
     int f = 0;
     if (cand[o] >= 0) {
@@ -70,6 +74,7 @@ __global__ void k_trc_majority(int64_t N, const int32_t *cand, const int64_t *to
 __global__ void k_trc_insert(int64_t N, const int32_t *Cold, const int32_t *Cnew, const int64_t *K,
                              const int32_t *flag, int32_t *bc, int64_t cap, uint64_t *keys, int64_t *vals,
                              int32_t *list, int32_t *occ) {
+  ld_after_previous();
   uint64_t mask = (uint64_t)cap - 1;
   int lane = threadIdx.x & 31;
   for (int64_t base = (ld_gtid() & ~31ll); base < N; base += ld_gstride()) {
@@ -117,6 +122,7 @@ __global__ void k_trc_insert(int64_t N, const int32_t *Cold, const int32_t *Cnew
 }
 __global__ void k_trc_best_w(const int32_t *occ, const int32_t *list, const uint64_t *keys, const int64_t *vals,
                              long long *bw) {
+  ld_after_previous();
   int64_t m = *occ;
   for (int64_t t = ld_gtid(); t < m; t += ld_gstride()) {
     int32_t sl = list[t];
@@ -125,6 +131,7 @@ __global__ void k_trc_best_w(const int32_t *occ, const int32_t *list, const uint
 }
 __global__ void k_trc_best_c(const int32_t *occ, const int32_t *list, uint64_t *keys, int64_t *vals,
                              const long long *bw, int32_t *bc) {
+  ld_after_previous();
   int64_t m = *occ;
   for (int64_t t = ld_gtid(); t < m; t += ld_gstride()) {
     int32_t sl = list[t];
@@ -138,25 +145,30 @@ __global__ void k_trc_best_c(const int32_t *occ, const int32_t *list, uint64_t *
 // For each new community: among the old communities that picked it, the
 // largest overlap, then the lowest old id.
 __global__ void k_tr_best_old_w(int64_t N, const int32_t *bc, const long long *bw, long long *ow) {
+  ld_after_previous();
   for (int64_t b = ld_gtid(); b < N; b += ld_gstride())
     if (bc[b] != INT_MAX) atomicMax(&ow[bc[b]], bw[b]);
 }
 __global__ void k_tr_best_old_b(int64_t N, const int32_t *bc, const long long *bw, const long long *ow, int32_t *ob) {
+  ld_after_previous();
   for (int64_t b = ld_gtid(); b < N; b += ld_gstride())
     if (bc[b] != INT_MAX && bw[b] == ow[bc[b]]) atomicMin(&ob[bc[b]], (int32_t)b);
 }
 __global__ void k_tr_new_used(int64_t N, const int32_t *Cnew, int32_t *used) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < N; i += ld_gstride()) used[Cnew[i]] = 1;
 }
 // unmatched[c] (new id used, nobody picked it); free[id] (no old vertex had id)
 __global__ void k_tr_flags(int64_t N, const int32_t *new_used, const int32_t *ob, const int32_t *bc,
                            int32_t *unmatched, int32_t *freef) {
+  ld_after_previous();
   for (int64_t c = ld_gtid(); c < N; c += ld_gstride()) {
     unmatched[c] = (new_used[c] && ob[c] == INT_MAX) ? 1 : 0;
     freef[c] = bc[c] == INT_MAX ? 1 : 0;
   }
 }
 __global__ void k_tr_free_list(int64_t N, const int32_t *freef, const int64_t *frank, int32_t *flist) {
+  ld_after_previous();
   for (int64_t id = ld_gtid(); id < N; id += ld_gstride())
     if (freef[id]) flist[frank[id]] = (int32_t)id;
 }
@@ -165,6 +177,7 @@ __global__ void k_tr_free_list(int64_t N, const int32_t *freef, const int64_t *f
 __global__ void k_tr_map(int64_t N, const int32_t *new_used, const int32_t *ob, const int64_t *urank,
                          const int64_t *frank, const int32_t *flist, int32_t *map, uint8_t *matched,
                          const int32_t *gid0, const int64_t *voff) {
+  ld_after_previous();
   for (int64_t c = ld_gtid(); c < N; c += ld_gstride()) {
     if (!new_used[c]) continue;
     if (ob[c] != INT_MAX) {
@@ -183,6 +196,7 @@ __global__ void k_tr_map(int64_t N, const int32_t *new_used, const int32_t *ob, 
 // nothing).
 __global__ void k_tr_relabel(int64_t N, const int32_t *Cnew, const int32_t *map, const int64_t *K, int32_t *C,
                              int64_t *Sig, int32_t *size) {
+  ld_after_previous();
   for (int64_t i = ld_gtid(); i < N; i += ld_gstride()) {
     int32_t c = map[Cnew[i]], o = C[i];
     if (c == o) continue;
@@ -197,6 +211,7 @@ __global__ void k_tr_relabel(int64_t N, const int32_t *Cnew, const int32_t *map,
   }
 }
 __global__ void k_tr_dsig(int64_t N, const uint8_t *matched, int64_t *dSig) {
+  ld_after_previous();
   for (int64_t id = ld_gtid(); id < N; id += ld_gstride())
     if (!matched[id]) dSig[id] = 0;
 }
@@ -509,6 +524,7 @@ __global__ void __launch_bounds__(256) k_tn_relabel(int64_t N, const int32_t *Cn
 
 // ---- modularity
 __global__ void k_sig_of(int64_t N, const int32_t *C, const int64_t *K, int64_t *Sig) {
+  ld_after_previous();
   int lane = threadIdx.x & 31;
   for (int64_t base = (ld_gtid() & ~31ll); base < N; base += ld_gstride()) {
     int64_t i = base + lane;
@@ -546,6 +562,7 @@ __global__ void __launch_bounds__(256) k_sigma_intra(int64_t N, const int64_t *o
                                                      const int32_t *col, const int32_t *w, const int32_t *C,
                                                      DevCounters *cnt, const int32_t *gid0, int64_t *sigg,
                                                      int32_t *big) {
+  ld_after_previous();
   const int lane = threadIdx.x & 31;
   int64_t warp = ld_gtid() >> 5, nw = ld_gstride() >> 5;
   int64_t acc = 0;
@@ -593,6 +610,7 @@ __global__ void __launch_bounds__(256) k_sigma_intra_big(const int32_t *big, con
                                                          const int32_t *deg, const int32_t *col, const int32_t *w,
                                                          const int32_t *C, DevCounters *cnt, const int32_t *gid0,
                                                          int64_t *sigg) {
+  ld_after_previous();
   const int64_t count = cnt->big_count;
   if (count == 0) return;
   const int64_t nch = ch_off[count];
@@ -616,6 +634,7 @@ __global__ void __launch_bounds__(256) k_sigma_intra_big(const int32_t *big, con
   if ((threadIdx.x & 31) == 0 && acc) atomicAdd((unsigned long long *)&cnt->sigma_intra, (unsigned long long)acc);
 }
 __global__ void k_sq(int64_t N, const int64_t *Sig, DevCounters *cnt, const int32_t *gid0, unsigned long long *sqg) {
+  ld_after_previous();
   i128 acc = 0;
   for (int64_t c0 = (ld_gtid() & ~31ll); c0 < N; c0 += ld_gstride()) {  // warp-uniform trip count
     int64_t c = c0 + (threadIdx.x & 31);
@@ -636,6 +655,7 @@ constexpr int SUM_UNROLL = 8;
 __global__ void __launch_bounds__(256) k_rowsum(int64_t N, const int64_t *off, const int32_t *deg, const int32_t *w,
                                                 int64_t *K, DevCounters *cnt, const int32_t *gid0, int64_t *m2g,
                                                 int32_t *big) {
+  ld_after_previous();
   __shared__ unsigned long long bsum;
   if (threadIdx.x == 0) bsum = 0;
   __syncthreads();
@@ -686,6 +706,7 @@ __global__ void __launch_bounds__(256) k_rowsum(int64_t N, const int64_t *off, c
 __global__ void __launch_bounds__(256) k_rowsum_big(const int32_t *big, const int64_t *ch_off, const int64_t *off,
                                                     const int32_t *deg, const int32_t *w, int64_t *K, DevCounters *cnt,
                                                     const int32_t *gid0, int64_t *m2g) {
+  ld_after_previous();
   const int64_t count = cnt->big_count;
   if (count == 0) return;
   const int64_t nch = ch_off[count];
@@ -721,21 +742,23 @@ static void track_narrow(leiden_handle *h, const int32_t *Cnew, const int32_t *r
   int2 *tiles = (int2 *)h->lbuf2, *granks = (int2 *)h->lbuf3;
   const uint8_t *used = h->G > 1 ? h->dE : nullptr;
   DevCounters *cnt = h->dcnt;
-  ld_note_launch(), launch_after(k_tn_cand, grid_for(N, TB, h->sm_count * 4), TB, s, N, h->C, Cnew, cand, dev, match, cnt);
+  ld_note_launch(), launch_after(k_tn_cand, grid_for(N, TB, h->sm_count * 4), TB, s, N, h->C, Cnew, cand, dev, match,
+                                 cnt);
   ld_note_launch(), launch_after(k_tn_deviants, gN, TB, s, N, h->C, Cnew, h->K, cand, dev);
-  ld_note_launch(), launch_after(k_tn_majority, gN, TB, s, N, h->csize0, cand, h->Sig, dev, choice, match, bits, flagged, best,
-                                                    cnt);
+  ld_note_launch(), launch_after(k_tn_majority, gN, TB, s, N, h->csize0, cand, h->Sig, dev, choice, match, bits,
+                                 flagged, best, cnt);
   ld_note_launch(), launch_after(k_tn_insert, gN, TB, s, N, h->C, Cnew, h->K, h->Sig, bits, best, h->tr_cap, h->tr_keys,
-                                                  h->tr_vals, h->tr_list, cnt);
+                                 h->tr_vals, h->tr_list, cnt);
   ld_note_launch(), launch_after(k_tn_best, h->sm_count * 2, TB, s, cnt, h->tr_list, h->tr_keys, h->tr_vals, best);
   ld_note_launch(), launch_after(k_tn_match, h->sm_count * 2, TB, s, cnt, flagged, best, choice, match);
-  int tile = TR_STEP * (int)std::max<int64_t>(1, (N + (int64_t)TR_STEP * TR_TILES_MAX - 1) / ((int64_t)TR_STEP * TR_TILES_MAX));
+  const int64_t span = (int64_t)TR_STEP * TR_TILES_MAX;
+  int tile = TR_STEP * (int)std::max<int64_t>(1, (N + span - 1) / span);
   int nt = (int)((N + tile - 1) / tile);
   ld_note_launch(), launch_after(k_tn_tiles, nt, TB, s, N, tile, used, root, nroot, match, h->csize0, tiles, cnt);
-  ld_note_launch(), launch_after(k_tn_lists, nt, TB, s, N, tile, used, root, nroot, match, h->csize0, tiles, rank, freel,
-                                                 h->gid0, h->d_voff, granks);
-  ld_note_launch(), launch_after(k_tn_relabel, gN, TB, s, N, Cnew, match, rank, freel, choice, h->K, h->C, h->Sig, h->csize0,
-                                                   h->dSig, h->gid0, granks);
+  ld_note_launch(), launch_after(k_tn_lists, nt, TB, s, N, tile, used, root, nroot, match, h->csize0, tiles, rank,
+                                 freel, h->gid0, h->d_voff, granks);
+  ld_note_launch(), launch_after(k_tn_relabel, gN, TB, s, N, Cnew, match, rank, freel, choice, h->K, h->C, h->Sig,
+                                 h->csize0, h->dSig, h->gid0, granks);
 }
 
 // C^{t-1} = h->C, final top-level membership = Cnew  ->  h->C, h->Sig, h->dSig.
@@ -751,31 +774,32 @@ void track_communities(leiden_handle *h, const int32_t *Cnew, const int32_t *roo
   int32_t *bc = h->ibuf0, *ob = h->ibuf1, *used = h->ibuf2;
   int32_t *cand = h->mtarget, *flag = h->movers;
   int64_t *dev = h->Sp;
-  ld_note_launch(), k_tr_init<<<gN, TB, 0, s>>>(N, bw, bc, ow, ob, cand, used, dev);
+  ld_note_launch(), launch_after(k_tr_init, gN, TB, s, N, bw, bc, ow, ob, cand, used, dev);
   cudaMemsetAsync(&h->dcnt->tr_occ, 0, sizeof(int32_t), s);
-  ld_note_launch(), k_trc_cand<<<gN, TB, 0, s>>>(N, h->C, Cnew, cand);
-  ld_note_launch(), k_trc_deviants<<<gN, TB, 0, s>>>(N, h->C, Cnew, h->K, cand, dev);
-  ld_note_launch(), k_trc_majority<<<gN, TB, 0, s>>>(N, cand, h->Sig, dev, bw, bc, flag);
+  ld_note_launch(), launch_after(k_trc_cand, gN, TB, s, N, h->C, Cnew, cand);
+  ld_note_launch(), launch_after(k_trc_deviants, gN, TB, s, N, h->C, Cnew, h->K, cand, dev);
+  ld_note_launch(), launch_after(k_trc_majority, gN, TB, s, N, cand, h->Sig, dev, bw, bc, flag);
   int32_t *occ = &h->dcnt->tr_occ;
-  ld_note_launch(), k_trc_insert<<<gN, TB, 0, s>>>(N, h->C, Cnew, h->K, flag, bc, h->tr_cap, h->tr_keys, h->tr_vals,
-                                                   h->tr_list, occ);
-  ld_note_launch(), k_trc_best_w<<<h->sm_count * 8, TB, 0, s>>>(occ, h->tr_list, h->tr_keys, h->tr_vals, bw);
-  ld_note_launch(), k_trc_best_c<<<h->sm_count * 8, TB, 0, s>>>(occ, h->tr_list, h->tr_keys, h->tr_vals, bw, bc);
-  ld_note_launch(), k_tr_best_old_w<<<gN, TB, 0, s>>>(N, bc, bw, ow);
-  ld_note_launch(), k_tr_best_old_b<<<gN, TB, 0, s>>>(N, bc, bw, ow, ob);
-  ld_note_launch(), k_tr_new_used<<<gN, TB, 0, s>>>(N, Cnew, used);
+  ld_note_launch(), launch_after(k_trc_insert, gN, TB, s, N, h->C, Cnew, h->K, flag, bc, h->tr_cap, h->tr_keys,
+                                 h->tr_vals, h->tr_list, occ);
+  ld_note_launch(), launch_after(k_trc_best_w, h->sm_count * 8, TB, s, occ, h->tr_list, h->tr_keys, h->tr_vals, bw);
+  ld_note_launch(), launch_after(k_trc_best_c, h->sm_count * 8, TB, s, occ, h->tr_list, h->tr_keys, h->tr_vals, bw, bc);
+  ld_note_launch(), launch_after(k_tr_best_old_w, gN, TB, s, N, bc, bw, ow);
+  ld_note_launch(), launch_after(k_tr_best_old_b, gN, TB, s, N, bc, bw, ow, ob);
+  ld_note_launch(), launch_after(k_tr_new_used, gN, TB, s, N, Cnew, used);
   int32_t *unmatched = h->rep, *freef = h->prop;
-  ld_note_launch(), k_tr_flags<<<gN, TB, 0, s>>>(N, used, ob, bc, unmatched, freef);
+  ld_note_launch(), launch_after(k_tr_flags, gN, TB, s, N, used, ob, bc, unmatched, freef);
   int64_t *urank = h->lbuf2, *frank = h->lbuf3;
   exclusive_scan_i32_to_i64(unmatched, urank, N, h->scan_tmp, s);
   exclusive_scan_i32_to_i64(freef, frank, N, h->scan_tmp, s);
   int32_t *flist = h->parent, *map = h->CB;
-  ld_note_launch(), k_tr_free_list<<<gN, TB, 0, s>>>(N, freef, frank, flist);
+  ld_note_launch(), launch_after(k_tr_free_list, gN, TB, s, N, freef, frank, flist);
   uint8_t *matched = h->dE;
   cudaMemsetAsync(matched, 0, (size_t)N, s);
-  ld_note_launch(), k_tr_map<<<gN, TB, 0, s>>>(N, used, ob, urank, frank, flist, map, matched, h->gid0, h->d_voff);
-  ld_note_launch(), k_tr_relabel<<<gN, TB, 0, s>>>(N, Cnew, map, h->K, h->C, h->Sig, h->csize0);
-  ld_note_launch(), k_tr_dsig<<<gN, TB, 0, s>>>(N, matched, h->dSig);
+  ld_note_launch(), launch_after(k_tr_map, gN, TB, s, N, used, ob, urank, frank, flist, map, matched, h->gid0,
+                                 h->d_voff);
+  ld_note_launch(), launch_after(k_tr_relabel, gN, TB, s, N, Cnew, map, h->K, h->C, h->Sig, h->csize0);
+  ld_note_launch(), launch_after(k_tr_dsig, gN, TB, s, N, matched, h->dSig);
 }
 
 // sigma (intra arcs) and sum Sigma_c^2 of membership C on G^t.
@@ -786,26 +810,26 @@ void modularity_terms(leiden_handle *h, const int32_t *C) {
   cudaMemsetAsync(Sig, 0, (size_t)N * sizeof(int64_t), s);
   cudaMemsetAsync(&h->dcnt->sigma_intra, 0, sizeof(int64_t), s);
   cudaMemsetAsync(&h->dcnt->sq[0], 0, 2 * sizeof(unsigned long long), s);
-  ld_note_launch(), k_sig_of<<<grid_for(N, TB), TB, 0, s>>>(N, C, h->K, Sig);
+  ld_note_launch(), launch_after(k_sig_of, grid_for(N, TB), TB, s, N, C, h->K, Sig);
   if (h->gid0) {
     cudaMemsetAsync(h->gc.sigma, 0, (size_t)h->G * sizeof(int64_t), s);
     cudaMemsetAsync(h->gc.sq, 0, (size_t)h->G * 2 * sizeof(unsigned long long), s);
   }
   int32_t *big = h->ibuf0;
   cudaMemsetAsync(&h->dcnt->big_count, 0, sizeof(int32_t), s);
-  ld_note_launch(), k_sigma_intra<<<grid_for(N, TB), TB, 0, s>>>(N, h->g_off, h->g_deg, h->g_col, h->g_w, C, h->dcnt,
-                                                                 h->gid0, h->gc.sigma, big);
+  ld_note_launch(), launch_after(k_sigma_intra, grid_for(N, TB), TB, s, N, h->g_off, h->g_deg, h->g_col, h->g_w, C,
+                                 h->dcnt, h->gid0, h->gc.sigma, big);
   launch_table_plan(big, &h->dcnt->big_count, h->g_deg, nullptr, 1, h->lbuf2, h->lbuf3, s);
-  ld_note_launch(), k_sigma_intra_big<<<h->sm_count * 8, TB, 0, s>>>(big, h->lbuf3, h->g_off, h->g_deg, h->g_col,
-                                                                     h->g_w, C, h->dcnt, h->gid0, h->gc.sigma);
-  ld_note_launch(), k_sq<<<grid_for(N, TB), TB, 0, s>>>(N, Sig, h->dcnt, h->gid0, h->gc.sq);
+  ld_note_launch(), launch_after(k_sigma_intra_big, h->sm_count * 8, TB, s, big, h->lbuf3, h->g_off, h->g_deg, h->g_col,
+                                 h->g_w, C, h->dcnt, h->gid0, h->gc.sigma);
+  ld_note_launch(), launch_after(k_sq, grid_for(N, TB), TB, s, N, Sig, h->dcnt, h->gid0, h->gc.sq);
 }
 
 // Sigma = per-community sums of K for membership h->C.
 void recompute_sigma(leiden_handle *h) {
   cudaStream_t s = h->stream;
   cudaMemsetAsync(h->Sig, 0, (size_t)h->n * sizeof(int64_t), s);
-  ld_note_launch(), k_sig_of<<<grid_for(h->n, TB), TB, 0, s>>>(h->n, h->C, h->K, h->Sig);
+  ld_note_launch(), launch_after(k_sig_of, grid_for(h->n, TB), TB, s, h->n, h->C, h->K, h->Sig);
 }
 
 // K = row sums of G^t and 2m.
@@ -815,11 +839,11 @@ void recompute_weights(leiden_handle *h) {
   if (h->gid0) cudaMemsetAsync(h->gc.m2, 0, (size_t)h->G * sizeof(int64_t), s);
   int32_t *big = h->ibuf0;
   cudaMemsetAsync(&h->dcnt->big_count, 0, sizeof(int32_t), s);
-  ld_note_launch(), k_rowsum<<<grid_for(h->n, TB), TB, 0, s>>>(h->n, h->g_off, h->g_deg, h->g_w, h->K, h->dcnt,
-                                                               h->gid0, h->gc.m2, big);
+  ld_note_launch(), launch_after(k_rowsum, grid_for(h->n, TB), TB, s, h->n, h->g_off, h->g_deg, h->g_w, h->K, h->dcnt,
+                                 h->gid0, h->gc.m2, big);
   launch_table_plan(big, &h->dcnt->big_count, h->g_deg, nullptr, 1, h->lbuf2, h->lbuf3, s);
-  ld_note_launch(), k_rowsum_big<<<h->sm_count * 8, TB, 0, s>>>(big, h->lbuf3, h->g_off, h->g_deg, h->g_w, h->K,
-                                                                h->dcnt, h->gid0, h->gc.m2);
+  ld_note_launch(), launch_after(k_rowsum_big, h->sm_count * 8, TB, s, big, h->lbuf3, h->g_off, h->g_deg, h->g_w, h->K,
+                                 h->dcnt, h->gid0, h->gc.m2);
 }
 
 LD_CHECK_WORD_READER(check_word_track)
