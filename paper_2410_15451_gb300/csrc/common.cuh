@@ -8,7 +8,6 @@
 typedef __int128 i128;
 typedef unsigned __int128 u128;
 
-#define LD_WARP 32
 #define LD_FULL 0xffffffffu
 #define LD_EMPTY_KEY (-1)
 
@@ -506,12 +505,6 @@ __device__ __forceinline__ bool ld_bit_test(const uint32_t *bm, int64_t i) {
 __device__ __forceinline__ bool ld_bit_set(uint32_t *bm, int64_t i) {
   uint32_t m = 1u << (i & 31);
   return (atomicOr(&bm[i >> 5], m) & m) == 0;
-}
-
-// Weight load for level 0 (int32) and aggregated levels (int64).
-template <typename W>
-__device__ __forceinline__ int64_t ld_w(const W *w, int64_t a) {
-  return (int64_t)w[a];
 }
 
 // ---------------------------------------------------------------- rows by windows

@@ -294,7 +294,6 @@ size_t sort_tmp_bytes(int64_t n);
 cudaError_t radix_sort_u64(uint64_t *keys, uint64_t *keys_alt, int64_t *vals, int64_t *vals_alt, int64_t n,
                            int bits, void *tmp, cudaStream_t s);
 void launch_fill_i32(int32_t *p, int32_t v, int64_t n, cudaStream_t s);
-void launch_fill_i64(int64_t *p, int64_t v, int64_t n, cudaStream_t s);
 void launch_iota_i32(int32_t *p, int64_t n, cudaStream_t s);
 // Per-item global tables and work chunks for the listed items (see prims.cu).
 constexpr int TABLE_CHUNK = 4096;

@@ -428,10 +428,6 @@ __global__ void k_fill_i32(int32_t *p, int32_t v, int64_t n) {
   ld_after_previous();
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) p[i] = v;
 }
-__global__ void k_fill_i64(int64_t *p, int64_t v, int64_t n) {
-  ld_after_previous();
-  for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) p[i] = v;
-}
 __global__ void k_iota_i32(int32_t *p, int64_t n) {
   ld_after_previous();
   for (int64_t i = ld_gtid(); i < n; i += ld_gstride()) p[i] = (int32_t)i;
@@ -447,9 +443,6 @@ int grid_for(int64_t n, int block, int max_blocks) {
 
 void launch_fill_i32(int32_t *p, int32_t v, int64_t n, cudaStream_t s) {
   if (n > 0) ld_note_launch(), launch_after(k_fill_i32, grid_for(n, 256), 256, s, p, v, n);
-}
-void launch_fill_i64(int64_t *p, int64_t v, int64_t n, cudaStream_t s) {
-  if (n > 0) ld_note_launch(), launch_after(k_fill_i64, grid_for(n, 256), 256, s, p, v, n);
 }
 void launch_table_plan(const int32_t *list, const int32_t *count, const int32_t *deg32, const int64_t *off64,
                        int64_t key_cap, int64_t *tab_off, int64_t *ch_off, cudaStream_t s, int32_t *occ) {
