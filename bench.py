@@ -524,11 +524,13 @@ def source_code_sha256(path):
 
 # The timed kernels: name -> (source file, pattern of its timed launches in
 # the ncu launch list).  The local-moving kernels are timed in their move
-# instantiations (template kind 0), the others in all of theirs.
-TIMED_KERNELS = {"k_decide_warp": ("move.cu", r"k_decide_warp<[^,]+, 0>$"),
-                 "k_decide_block": ("move.cu", r"k_decide_block<[^,]+, 0>$"),
-                 "k_huge_scan": ("move.cu", r"k_huge_scan<[^,]+, 0>$"),
-                 "k_split_sample": ("phases.cu", r"k_split_sample$"),
+# instantiations (template kind 0), the others in all of theirs.  Split
+# sampling on a large level is two kernels (neighbours found, then linked)
+# under one timer: its third entry names the launches that begin a span.
+TIMED_KERNELS = {"k_decide_warp": ("move.cu", r"k_decide_warp<[^,]+, 0(, [^,>]+)?>$"),
+                 "k_decide_block": ("move.cu", r"k_decide_block<[^,]+, 0(, [^,>]+)?>$"),
+                 "k_huge_scan": ("move.cu", r"k_huge_scan<[^,]+, 0(, [^,>]+)?>$"),
+                 "k_split_sample": ("phases.cu", r"k_split_(sample|find|link)$", r"k_split_(sample|find)$"),
                  "k_agg_chunk_scan": ("phases.cu", r"k_agg_chunk_scan<[^>]+>$"),
                  "k_merge_mid": ("batch.cu", r"k_merge_mid$")}
 
@@ -540,7 +542,7 @@ def ncu_traffic(kernel):
     capture (comments aside)."""
     import re
 
-    src, pat = TIMED_KERNELS[kernel]
+    src, pat, *begins = TIMED_KERNELS[kernel]
     try:
         d = json.load(open(TRAFFIC_JSON))
         sha = source_code_sha256(os.path.join(CSRC, src))
@@ -549,7 +551,7 @@ def ncu_traffic(kernel):
     if d.get("source_sha256", {}).get(src) != sha:
         return None
     sel = [k for name, k in d.get("kernels", {}).items() if re.match(pat, name)]
-    n = sum(k["launches"] for k in sel)
+    n = sum(k["launches"] for name, k in d.get("kernels", {}).items() if re.match(begins[0] if begins else pat, name))
     return sum(k["dram_read_bytes"] + k["dram_write_bytes"] for k in sel) / n if n else None
 
 
@@ -575,7 +577,7 @@ def ncu_summary(csv_path, command, out_json=TRAFFIC_JSON,
         ent[r["Metric Name"]] = float(v) * scale
 
     def base(name):
-        name = re.sub(r"\(.*$", "", name.replace("void ", "").replace("<unnamed>::", "")
+        name = re.sub(r"\(.*$", "", re.sub(r"\((bool|int)\)", "", name).replace("void ", "").replace("<unnamed>::", "")
                       .replace("(anonymous namespace)::", ""))
         return name.strip()
 
@@ -590,7 +592,7 @@ def ncu_summary(csv_path, command, out_json=TRAFFIC_JSON,
     tot_us = sum(p["us"] for p in per.values())
     lm = {}
     for name in LMK_NAMES:
-        sel = [p for k, p in per.items() if re.match(re.escape(name) + r"<[^,]+, 0>$", k)]
+        sel = [p for k, p in per.items() if re.match(TIMED_KERNELS[name][1], k)]
         n = sum(p["launches"] for p in sel)
         if n:
             rd, wr = sum(p["read"] for p in sel), sum(p["write"] for p in sel)
