@@ -441,7 +441,7 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range,
     if (refine) ph_bytes(h, LEIDEN_PHASE_SPLIT, 24 * (int64_t)h->hcnt->split_count + 8 * h->hcnt->split_arcs);
     split_unread = !refine;
     ph_mark(h, LEIDEN_PHASE_AGGREGATE);
-    ph_bytes(h, LEIDEN_PHASE_AGGREGATE, 4 * n);  // community count
+    ph_bytes(h, LEIDEN_PHASE_AGGREGATE, B ? 4 * n : 8);  // community count
     if (B) {  // (one graph: counted by the renumbering, or by tracking in the last pass)
       CK(cudaMemsetAsync(h->gc.ncomm, 0, (size_t)G * sizeof(int32_t), s));
       count_communities(h, n, g.gid);
@@ -534,7 +534,8 @@ leiden_status run_leiden(leiden_handle *h, int dynamic, const uint8_t *in_range,
     tau /= p.tau_drop;
   }
   ph_mark(h, LEIDEN_PHASE_TRACK);
-  ph_bytes(h, LEIDEN_PHASE_TRACK, (B ? 0 : 12 * N) + 234 * N);  // final lookup; tracking's sweeps
+  // final lookup (of more than one pass); tracking's sweeps
+  ph_bytes(h, LEIDEN_PHASE_TRACK, (B || last_first ? 0 : 12 * N) + (wide_sums(h) ? 234 : 134) * N);
   if (!B && !last_first) lookup_dendrogram(h, false);
   if (B && !looked_up) { h->err = "batched pass loop ended without a final lookup"; return LEIDEN_ERR_STATE; }
   // a call of one pass: the membership is C' itself

@@ -714,14 +714,14 @@ __global__ void __launch_bounds__(256) k_merge_mid(MergeArgs A, const int32_t *m
   __shared__ int32_t scol[MERGE_MID];
   __shared__ int32_t sw[MERGE_MID];
   int64_t count = *count_p;
-  int64_t bytes = 0;  // algorithmic bytes (thread 0): old row read, new row written, the row's batch arcs
+  int64_t bytes = 0;  // algorithmic bytes (thread 0): the moved part of the row, old and new, its batch arcs
   for (int64_t k = blockIdx.x; k < count; k += gridDim.x) {
     int64_t r = mid[k];
     int64_t L = A.len[r];
-    if (threadIdx.x == 0)
-      bytes += 8 * ((int64_t)A.deg[A.rows[r]] + L) + 16 * (A.dhi[r] - A.dlo[r] + A.ihi[r] - A.ilo[r]);
     int first;
     const int32_t u = merge_tail(A, r, threadIdx.x, 256, scol, sw, first);
+    if (threadIdx.x == 0)
+      bytes += 8 * ((int64_t)A.deg[u] + L - 2 * first) + 16 * (A.dhi[r] - A.dlo[r] + A.ihi[r] - A.ilo[r]);
     __syncthreads();
     const int64_t o = A.dst[r] + first;
     const int n = (int)L - first;
