@@ -265,7 +265,9 @@ unsigned int check_selftest(cudaStream_t s);
 
 // Launch of a kernel that begins with ld_after_previous(): its blocks are
 // scheduled while the kernel before it on the stream drains, which hides most of
-// the launch latency in chains of short kernels.
+// the launch latency in chains of short kernels (0.7 us of 2 to 5 us each; a
+// batch of 96 graphs, 60 such kernels: 1066 -> 974 us with the second half of
+// them launched this way; the level loop's half: R-MAT 20, 16 edges, 531 -> 487 us).
 template <typename... P, typename... A>
 inline void launch_after(void (*kernel)(P...), int grid, int block, cudaStream_t s, const A &...args) {
   cudaLaunchAttribute at{};
