@@ -416,6 +416,19 @@ __device__ __forceinline__ void wt_flush(WarpTable<WIDE> &T, const GTable &G) {
   __syncwarp();
 }
 
+// All 32 lanes, before each adds at most one key: room for them.  Every lane reads
+// the fill count between two warp barriers, so all take the same side of the
+// flush, which is a collective; without the second one a lane that runs ahead
+// raises the count by its own key and may send the lanes behind it into a flush
+// that it does not join.
+template <bool WIDE>
+__device__ __forceinline__ void wt_make_room(WarpTable<WIDE> &T, const GTable &G) {
+  __syncwarp();
+  int filled = T.count;
+  __syncwarp();
+  if (filled > WT_LIMIT) wt_flush(T, G);  // warp-uniform
+}
+
 // ---------------------------------------------------------------- block appends
 // A block of 256 threads appends its items to up to CATS lists at once, one
 // atomic per list and step: one atomic per warp on a list's length costs more

@@ -690,13 +690,11 @@ __global__ void __launch_bounds__(256) k_huge_scan(Args A, const int64_t *tab_of
       if (hot < 0) hot = hot_community(valid[0], c[0], d);
 #pragma unroll
       for (int u = 0; u < HUGE_UNROLL; u++) {
-        if (T8.count > WT_LIMIT) wt_flush(T8, G);
-        if (valid[u]) {
-          if (c[u] == d) kd += wa[u];
-          else if (c[u] == hot) kh += wa[u];
-          else st_insert(T8, &T8.count, c[u], wa[u]);
-        }
-        __syncwarp();
+        wt_make_room(T8, G);
+        if (!valid[u]) continue;
+        if (c[u] == d) kd += wa[u];
+        else if (c[u] == hot) kh += wa[u];
+        else st_insert(T8, &T8.count, c[u], wa[u]);
       }
     }
     wt_flush(T8, G);

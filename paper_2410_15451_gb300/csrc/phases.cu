@@ -768,9 +768,8 @@ __device__ __forceinline__ void agg_take(const AggArgs &A, WarpTable<WIDE> &T8, 
     bool own = valid[u] && cc[u] == self;
     ksum += wa[u];
     selfw += own ? wa[u] : 0;
-    if (T8.count > WT_LIMIT) wt_flush(T8, G);
+    wt_make_room(T8, G);
     if (valid[u] && !own) st_insert(T8, &T8.count, cc[u], wa[u]);
-    __syncwarp();
   }
 }
 

@@ -1,0 +1,43 @@
+"""Rules that the CUDA sources keep and that no run on a GPU would show broken:
+they are read as text."""
+from __future__ import annotations
+
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2410_15451_gb300", "csrc")
+
+
+def sources():
+    """File name -> text without comments."""
+    out = {}
+    for f in sorted(os.listdir(CSRC)):
+        if f.endswith((".cu", ".cuh", ".h")):
+            with open(os.path.join(CSRC, f)) as fh:
+                out[f] = re.sub(r"//[^\n]*|/\*.*?\*/", "", fh.read(), flags=re.S)
+    return out
+
+
+def body(text, start):
+    """The braces that open after `start`, with what they hold."""
+    a = text.index("{", start)
+    depth = 0
+    for k in range(a, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[k], 0)
+        if depth == 0:
+            return text[a:k + 1]
+    raise ValueError("unbalanced braces")
+
+
+def test_flush_of_a_warp_table_is_decided_by_the_whole_warp():
+    """wt_flush holds full-warp collectives.  Whether it runs may only depend on a
+    fill count that every lane read before any of them went on to add a key: the
+    read stands between two warp barriers, and nothing else tests the count."""
+    src = sources()
+    room = body(src["common.cuh"], src["common.cuh"].index("void wt_make_room("))
+    assert re.fullmatch(r"\{\s*__syncwarp\(\);\s*int filled = T\.count;\s*__syncwarp\(\);\s*"
+                        r"if \(filled > WT_LIMIT\) wt_flush\(T, G\);\s*\}", room), room
+    for f, text in src.items():
+        text = text.replace(room, "")
+        assert not re.search(r"\bif\s*\([^;{}]*\)\s*\{?\s*wt_flush\(", text), f
+        assert not re.search(r"\bif\s*\([^;{}]*WT_LIMIT", text), f
