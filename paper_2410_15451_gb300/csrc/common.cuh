@@ -416,17 +416,17 @@ __device__ __forceinline__ void wt_flush(WarpTable<WIDE> &T, const GTable &G) {
   __syncwarp();
 }
 
-// All 32 lanes, before each adds at most one key: room for them.  Every lane reads
-// the fill count between two warp barriers, so all take the same side of the
-// flush, which is a collective; without the second one a lane that runs ahead
-// raises the count by its own key and may send the lanes behind it into a flush
-// that it does not join.
+// All 32 lanes, before each adds at most one key: room for them.  The flush is a
+// collective, so all lanes must take the same side: each reads the fill count and
+// then votes, and no lane adds a key before all have voted (a lane that ran ahead
+// on its own reading would send the lanes behind it into a flush that it does not
+// join).  The lane that added last reads the whole count.  A read between two warp
+// barriers decides the same: R-MAT 20, rollback of 0.1 of its edges, 26.6 ms, with
+// the vote 25.7; R-MAT 21 static 53.2 and 52.8.
 template <bool WIDE>
 __device__ __forceinline__ void wt_make_room(WarpTable<WIDE> &T, const GTable &G) {
-  __syncwarp();
-  int filled = T.count;
-  __syncwarp();
-  if (filled > WT_LIMIT) wt_flush(T, G);  // warp-uniform
+  int filled = *(volatile int32_t *)&T.count;
+  if (__any_sync(LD_FULL, filled > WT_LIMIT)) wt_flush(T, G);
 }
 
 // ---------------------------------------------------------------- block appends

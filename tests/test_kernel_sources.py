@@ -30,13 +30,13 @@ def body(text, start):
 
 
 def test_flush_of_a_warp_table_is_decided_by_the_whole_warp():
-    """wt_flush holds full-warp collectives.  Whether it runs may only depend on a
-    fill count that every lane read before any of them went on to add a key: the
-    read stands between two warp barriers, and nothing else tests the count."""
+    """wt_flush holds full-warp collectives.  Whether it runs is voted on by all lanes,
+    each with a fill count that it read before any of them went on to add a key, and
+    nothing else tests the count."""
     src = sources()
     room = body(src["common.cuh"], src["common.cuh"].index("void wt_make_room("))
-    assert re.fullmatch(r"\{\s*__syncwarp\(\);\s*int filled = T\.count;\s*__syncwarp\(\);\s*"
-                        r"if \(filled > WT_LIMIT\) wt_flush\(T, G\);\s*\}", room), room
+    assert re.fullmatch(r"\{\s*int filled = \*\(volatile int32_t \*\)&T\.count;\s*"
+                        r"if \(__any_sync\(LD_FULL, filled > WT_LIMIT\)\) wt_flush\(T, G\);\s*\}", room), room
     for f, text in src.items():
         text = text.replace(room, "")
         assert not re.search(r"\bif\s*\([^;{}]*\)\s*\{?\s*wt_flush\(", text), f
