@@ -101,3 +101,59 @@ def test_hub_tables_of_every_size(weighted):
     dels = [(2 + 3 * k, int(g.col[g.off[2 + 3 * k]]), 1) for k in range(len(HUB_SLOTS))]
     assert np.array_equal(gpu.update(dels, [(0, 5, 1)], L.LEIDEN_ND), ref.update(dels, [(0, 5, 1)], oracle.ND))
     assert gpu.trace() == ref.trace()
+
+
+def two_parts(n, part, degree, last):
+    """Two rings of `part` vertices joined to their `degree` next ones, the first
+    ids and the ids from `last` on; every other id is unused."""
+    step = np.arange(1, degree // 2 + 1)
+    v = np.arange(part)[:, None]
+    row = np.sort(np.concatenate([(v + step) % part, (v - step) % part], 1), 1)
+    off = np.zeros(n + 1, np.int64)
+    off[1:part + 1] = degree
+    off[last + 1:last + part + 1] = degree
+    off = np.cumsum(off)
+    col = np.concatenate([row.ravel(), row.ravel() + last]).astype(np.int32)
+    return synth.Graph(n, off, col, np.ones(len(col), np.int32))
+
+
+def fastest(call, runs=12):
+    """Seconds of the quickest of `runs` calls that end with a wait for the GPU."""
+    import time
+
+    call()
+    best = float("inf")
+    for _ in range(runs):
+        t = time.perf_counter()
+        call()
+        best = min(best, time.perf_counter() - t)
+    return best
+
+
+@pytest.mark.parametrize("unused", [31, 97, 160, 161, 4096, 1_000_000])
+@pytest.mark.parametrize("part,degree", [(5, 2), (777, 30)])
+def test_modularity_across_unused_ids(part, degree, unused):
+    """A run of rows without arcs between two rows that have some."""
+    import torch
+
+    g = two_parts(2 * part + unused + 3, part, degree, part + unused)
+    C = np.random.default_rng(unused).integers(0, 5, g.n).astype(np.int32)
+    q, _ = oracle.modularity(g.off, g.col, g.w.astype(np.int64), C)
+    d = [torch.from_numpy(x).cuda() for x in (g.off, g.col, g.w, C)]
+    assert L.leiden_modularity_noalloc(g.n, d[0], d[1], d[2], d[3]) == q
+    assert L.leiden_modularity_noalloc(g.n, d[0], d[1], None, d[3]) == q
+
+
+def test_unused_ids_cost_no_more_in_the_middle_than_at_the_end():
+    """One warp has the arcs on both sides of the run; at one step per 32 of its
+    ids it would work for some 31,000 steps where the rest of the call has about
+    ten (the bound leaves a factor of five for what else the call does)."""
+    import torch
+
+    part, unused = 20_001, 1_000_000  # (spans are multiples of 32 arcs: none ends between the parts)
+    t = []
+    for last in (part + unused, part):
+        g = two_parts(2 * part + unused, part, 40, last)
+        d = [torch.from_numpy(x).cuda() for x in (g.off, g.col, np.zeros(g.n, np.int32))]
+        t.append(fastest(lambda: L.leiden_modularity_noalloc(g.n, d[0], d[1], None, d[2])))
+    assert t[0] < 5 * t[1], t
