@@ -897,19 +897,19 @@ __global__ void k_ds_best(const uint64_t *pkey, const int64_t *pw, const int64_t
 }
 
 // Neighbours of G^t of the vertices with dE become affected.  Rows by
-// windows of 32 per warp, the flagged ones flattened; flagged rows above
+// windows of up to 32 per warp (see window_rows), the flagged ones flattened; flagged rows above
 // ROWS_BIG arcs are listed for the chunked kernel (a warp per vertex of the
 // graph spent its time on unflagged rows and on the longest hub: R-MAT 20,
 // 15,700 edges: 580 -> 19 us, and 14 us for the hubs' chunks).
 __global__ void __launch_bounds__(256) k_ds_expand_neighbours(const uint8_t *dE, int64_t n, const int64_t *off,
                                                               const int32_t *deg, const int32_t *col, uint8_t *dV,
-                                                              int32_t *big, DevCounters *cnt) {
+                                                              int32_t *big, DevCounters *cnt, int rows) {
   ld_after_previous();
   const int lane = threadIdx.x & 31;
   int64_t warp = ld_gtid() >> 5, nw = ld_gstride() >> 5;
-  for (int64_t r = warp * 32; r < n; r += nw * 32) {  // warp-uniform
+  for (int64_t r = warp * rows; r < n; r += nw * rows) {  // warp-uniform
     int64_t i = r + lane;
-    bool f = i < n && dE[i];
+    bool f = lane < rows && i < n && dE[i];
     if (!__any_sync(LD_FULL, f)) continue;
     int d = f ? deg[i] : 0;
     if (d > ROWS_BIG) {
@@ -1380,8 +1380,9 @@ leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, i
                                        h->Sig, cnt, dV, h->dE, h->dCf, h->gid0, h->gc.m2);
       }
       cudaMemsetAsync(&cnt->big_count, 0, sizeof(int32_t), s);
-      ld_note_launch(), launch_after(k_ds_expand_neighbours, grid_for(n, TB), TB, s, h->dE, n, h->g_off, h->g_deg,
-                                     h->g_col, dV, h->ibuf0, cnt);
+      const int wr = window_rows(h);
+      ld_note_launch(), launch_after(k_ds_expand_neighbours, window_grid(n, wr), TB, s, h->dE, n, h->g_off, h->g_deg,
+                                     h->g_col, dV, h->ibuf0, cnt, wr);
       launch_table_plan(h->ibuf0, &cnt->big_count, h->g_deg, nullptr, 1, h->lbuf0, h->lbuf1, s);
       ld_note_launch(), launch_after(k_ds_expand_big, h->sm_count * 8, TB, s, h->ibuf0, h->lbuf1, h->g_off, h->g_deg,
                                      h->g_col, dV, cnt);

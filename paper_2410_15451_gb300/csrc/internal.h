@@ -315,6 +315,17 @@ void launch_piece_plan(const int32_t *count, const int32_t *occ, const BigTables
 void launch_table_plan(const int32_t *list, const int32_t *count, const int32_t *deg32, const int64_t *off64,
                        int64_t key_cap, int64_t *tab_off, int64_t *ch_off, cudaStream_t s, int32_t *occ = nullptr);
 int grid_for(int64_t n, int block, int max_blocks = 152 * 16);
+// Rows per window (a power of two up to 32) of the kernels that walk the rows of
+// G^t by windows, a warp each, and the blocks of 256 threads for that many.  Above
+// a mean degree of ROWS_LONG one: most steps of a flat walk would cross a row's
+// end and pay for the search, and the row sums and modularity then have a form
+// with half the registers (modularity before the first static call, both sweeps,
+// us in windows and with a warp per row: rings of 400k vertices of degree 100
+// 326 and 242, 100k of 200 188 and 120; degree-corrected partitions of 1.5M
+// vertices, mean 64, 707 and 873, of 300k, mean 115, 293 and 294).
+constexpr int ROWS_LONG = 72;
+int window_rows(const leiden_handle *h);
+inline int window_grid(int64_t n, int rows) { return grid_for((n + rows - 1) / rows * 32, 256); }
 
 // ------------------------------------------------------------ batch.cu
 leiden_status batch_apply_and_mark(leiden_handle *h, const leiden_edge *d_del, int64_t n_del,

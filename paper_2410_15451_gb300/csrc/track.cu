@@ -536,10 +536,11 @@ __global__ void k_sig_of(int64_t N, const int32_t *C, const int64_t *K, int64_t 
   }
 }
 // Batched handles (gid0 non-null) also sum per graph: sigg, sqg, m2g.
-// Intra-community weight and (k_rowsum) row sums, rows by windows of 32 per
-// warp; rows above ROWS_BIG arcs are listed and their chunks summed by the
-// second kernel.  With a warp per row, the longest hub's warp was the kernel's
-// time (R-MAT 21: k_rowsum 412 -> 260 us).
+// Intra-community weight and (k_rowsum) row sums, rows by windows of up to 32 per
+// warp (see window_rows; lanes past a window's rows hold none); rows above
+// ROWS_BIG arcs are listed and their chunks summed by the second kernel (launched
+// where a row can be that long).  With a warp per row, the longest hub's warp was
+// the kernel's time (R-MAT 21: k_rowsum 412 -> 260 us).
 constexpr int ROW_UNROLL = 4;
 
 // The rows of a window: lane i's first flat position s, end e, row start minus
@@ -561,13 +562,13 @@ __device__ __forceinline__ int window_of(int64_t i, int64_t N, const int64_t *of
 __global__ void __launch_bounds__(256) k_sigma_intra(int64_t N, const int64_t *off, const int32_t *deg,
                                                      const int32_t *col, const int32_t *w, const int32_t *C,
                                                      DevCounters *cnt, const int32_t *gid0, int64_t *sigg,
-                                                     int32_t *big) {
+                                                     int32_t *big, int rows) {
   ld_after_previous();
   const int lane = threadIdx.x & 31;
   int64_t warp = ld_gtid() >> 5, nw = ld_gstride() >> 5;
   int64_t acc = 0;
-  for (int64_t r = warp * 32; r < N; r += nw * 32) {  // warp-uniform
-    int64_t i = r + lane, ab;
+  for (int64_t r = warp * rows; r < N; r += nw * rows) {  // warp-uniform
+    int64_t i = lane < rows ? r + lane : N, ab;
     int s, e;
     int total = window_of(i, N, off, deg, big, &cnt->big_count, s, e, ab);
     int32_t c = i < N ? C[i] : -1, g = gid0 && i < N ? gid0[i] : 0;
@@ -600,6 +601,34 @@ __global__ void __launch_bounds__(256) k_sigma_intra(int64_t N, const int64_t *o
     if (gid0 && one) {
       here = ld_warp_sum_i64(here);
       if (lane == 0 && here) atomicAdd((unsigned long long *)&sigg[g0], (unsigned long long)here);
+    }
+  }
+  acc = ld_warp_sum_i64(acc);
+  if (lane == 0 && acc) atomicAdd((unsigned long long *)&cnt->sigma_intra, (unsigned long long)acc);
+}
+
+// The same with a warp per row, for long rows (window_rows == 1): few registers,
+// so that twice as many loads are in flight as in the windows' form.
+__global__ void __launch_bounds__(256) k_sigma_intra_rows(int64_t N, const int64_t *off, const int32_t *deg,
+                                                          const int32_t *col, const int32_t *w, const int32_t *C,
+                                                          DevCounters *cnt, const int32_t *gid0, int64_t *sigg,
+                                                          int32_t *big) {
+  ld_after_previous();
+  const int lane = threadIdx.x & 31;
+  int64_t acc = 0;
+  for (int64_t i = ld_gtid() >> 5; i < N; i += ld_gstride() >> 5) {  // warp-uniform
+    int32_t c = C[i];
+    int64_t b = off[i], d = deg[i], here = 0;
+    if (d > ROWS_BIG) {
+      if (lane == 0) big[atomicAdd(&cnt->big_count, 1)] = (int32_t)i;
+      continue;
+    }
+    for (int64_t a = lane; a < d; a += 32)
+      if (C[col[b + a]] == c) here += w[b + a];
+    acc += here;
+    if (gid0) {
+      here = ld_warp_sum_i64(here);
+      if (lane == 0 && here) atomicAdd((unsigned long long *)&sigg[gid0[i]], (unsigned long long)here);
     }
   }
   acc = ld_warp_sum_i64(acc);
@@ -654,7 +683,7 @@ __global__ void k_sq(int64_t N, const int64_t *Sig, DevCounters *cnt, const int3
 constexpr int SUM_UNROLL = 8;
 __global__ void __launch_bounds__(256) k_rowsum(int64_t N, const int64_t *off, const int32_t *deg, const int32_t *w,
                                                 int64_t *K, DevCounters *cnt, const int32_t *gid0, int64_t *m2g,
-                                                int32_t *big) {
+                                                int32_t *big, int rows) {
   ld_after_previous();
   __shared__ unsigned long long bsum;
   if (threadIdx.x == 0) bsum = 0;
@@ -662,8 +691,8 @@ __global__ void __launch_bounds__(256) k_rowsum(int64_t N, const int64_t *off, c
   const int lane = threadIdx.x & 31;
   int64_t warp = ld_gtid() >> 5, nw = ld_gstride() >> 5;
   int64_t tot = 0;
-  for (int64_t r = warp * 32; r < N; r += nw * 32) {  // warp-uniform
-    int64_t i = r + lane, ab, kw = 0, lacc = 0;
+  for (int64_t r = warp * rows; r < N; r += nw * rows) {  // warp-uniform
+    int64_t i = lane < rows ? r + lane : N, ab, kw = 0, lacc = 0;
     int s, e, cur = 0;
     int total = window_of(i, N, off, deg, big, &cnt->big_count, s, e, ab);
     for (int x0 = 0; x0 < total; x0 += 32 * SUM_UNROLL) {  // warp-uniform
@@ -701,6 +730,30 @@ __global__ void __launch_bounds__(256) k_rowsum(int64_t N, const int64_t *off, c
   if (lane == 0 && tot) atomicAdd(&bsum, (unsigned long long)tot);
   __syncthreads();
   if (threadIdx.x == 0 && bsum) atomicAdd((unsigned long long *)&cnt->m2, bsum);
+}
+
+__global__ void __launch_bounds__(256) k_rowsum_rows(int64_t N, const int64_t *off, const int32_t *deg,
+                                                     const int32_t *w, int64_t *K, DevCounters *cnt,
+                                                     const int32_t *gid0, int64_t *m2g, int32_t *big) {
+  ld_after_previous();
+  const int lane = threadIdx.x & 31;
+  int64_t tot = 0;
+  for (int64_t i = ld_gtid() >> 5; i < N; i += ld_gstride() >> 5) {  // warp-uniform
+    int64_t b = off[i], d = deg[i], acc = 0;
+    if (d > ROWS_BIG) {
+      if (lane == 0) {
+        big[atomicAdd(&cnt->big_count, 1)] = (int32_t)i;
+        K[i] = 0;
+      }
+      continue;
+    }
+    for (int64_t a = lane; a < d; a += 32) acc += w[b + a];
+    acc = ld_warp_sum_i64(acc);
+    if (lane == 0) K[i] = acc;
+    if (lane == 0 && gid0 && acc) atomicAdd((unsigned long long *)&m2g[gid0[i]], (unsigned long long)acc);
+    tot += acc;
+  }
+  if (lane == 0 && tot) atomicAdd((unsigned long long *)&cnt->m2, (unsigned long long)tot);
 }
 
 __global__ void __launch_bounds__(256) k_rowsum_big(const int32_t *big, const int64_t *ch_off, const int64_t *off,
@@ -816,12 +869,20 @@ void modularity_terms(leiden_handle *h, const int32_t *C) {
     cudaMemsetAsync(h->gc.sq, 0, (size_t)h->G * 2 * sizeof(unsigned long long), s);
   }
   int32_t *big = h->ibuf0;
-  cudaMemsetAsync(&h->dcnt->big_count, 0, sizeof(int32_t), s);
-  ld_note_launch(), launch_after(k_sigma_intra, grid_for(N, TB), TB, s, N, h->g_off, h->g_deg, h->g_col, h->g_w, C,
-                                 h->dcnt, h->gid0, h->gc.sigma, big);
-  launch_table_plan(big, &h->dcnt->big_count, h->g_deg, nullptr, 1, h->lbuf2, h->lbuf3, s);
-  ld_note_launch(), launch_after(k_sigma_intra_big, h->sm_count * 8, TB, s, big, h->lbuf3, h->g_off, h->g_deg, h->g_col,
-                                 h->g_w, C, h->dcnt, h->gid0, h->gc.sigma);
+  const bool some_big = h->g_maxdeg > ROWS_BIG;
+  if (some_big) cudaMemsetAsync(&h->dcnt->big_count, 0, sizeof(int32_t), s);
+  const int rows = window_rows(h);
+  if (rows == 1)
+    ld_note_launch(), launch_after(k_sigma_intra_rows, window_grid(N, 1), TB, s, N, h->g_off, h->g_deg, h->g_col,
+                                   h->g_w, C, h->dcnt, h->gid0, h->gc.sigma, big);
+  else
+    ld_note_launch(), launch_after(k_sigma_intra, window_grid(N, rows), TB, s, N, h->g_off, h->g_deg, h->g_col, h->g_w,
+                                   C, h->dcnt, h->gid0, h->gc.sigma, big, rows);
+  if (some_big) {
+    launch_table_plan(big, &h->dcnt->big_count, h->g_deg, nullptr, 1, h->lbuf2, h->lbuf3, s);
+    ld_note_launch(), launch_after(k_sigma_intra_big, h->sm_count * 8, TB, s, big, h->lbuf3, h->g_off, h->g_deg,
+                                   h->g_col, h->g_w, C, h->dcnt, h->gid0, h->gc.sigma);
+  }
   ld_note_launch(), launch_after(k_sq, grid_for(N, TB), TB, s, N, Sig, h->dcnt, h->gid0, h->gc.sq);
 }
 
@@ -838,12 +899,20 @@ void recompute_weights(leiden_handle *h) {
   cudaMemsetAsync(&h->dcnt->m2, 0, sizeof(int64_t), s);
   if (h->gid0) cudaMemsetAsync(h->gc.m2, 0, (size_t)h->G * sizeof(int64_t), s);
   int32_t *big = h->ibuf0;
-  cudaMemsetAsync(&h->dcnt->big_count, 0, sizeof(int32_t), s);
-  ld_note_launch(), launch_after(k_rowsum, grid_for(h->n, TB), TB, s, h->n, h->g_off, h->g_deg, h->g_w, h->K, h->dcnt,
-                                 h->gid0, h->gc.m2, big);
-  launch_table_plan(big, &h->dcnt->big_count, h->g_deg, nullptr, 1, h->lbuf2, h->lbuf3, s);
-  ld_note_launch(), launch_after(k_rowsum_big, h->sm_count * 8, TB, s, big, h->lbuf3, h->g_off, h->g_deg, h->g_w, h->K,
-                                 h->dcnt, h->gid0, h->gc.m2);
+  const bool some_big = h->g_maxdeg > ROWS_BIG;
+  if (some_big) cudaMemsetAsync(&h->dcnt->big_count, 0, sizeof(int32_t), s);
+  const int rows = window_rows(h);
+  if (rows == 1)
+    ld_note_launch(), launch_after(k_rowsum_rows, window_grid(h->n, 1), TB, s, h->n, h->g_off, h->g_deg, h->g_w, h->K,
+                                   h->dcnt, h->gid0, h->gc.m2, big);
+  else
+    ld_note_launch(), launch_after(k_rowsum, window_grid(h->n, rows), TB, s, h->n, h->g_off, h->g_deg, h->g_w, h->K,
+                                   h->dcnt, h->gid0, h->gc.m2, big, rows);
+  if (some_big) {
+    launch_table_plan(big, &h->dcnt->big_count, h->g_deg, nullptr, 1, h->lbuf2, h->lbuf3, s);
+    ld_note_launch(), launch_after(k_rowsum_big, h->sm_count * 8, TB, s, big, h->lbuf3, h->g_off, h->g_deg, h->g_w,
+                                   h->K, h->dcnt, h->gid0, h->gc.m2);
+  }
 }
 
 LD_CHECK_WORD_READER(check_word_track)

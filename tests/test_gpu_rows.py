@@ -157,3 +157,53 @@ def test_unused_ids_cost_no_more_in_the_middle_than_at_the_end():
         d = [torch.from_numpy(x).cuda() for x in (g.off, g.col, np.zeros(g.n, np.int32))]
         t.append(fastest(lambda: L.leiden_modularity_noalloc(g.n, d[0], d[1], None, d[2])))
     assert t[0] < 5 * t[1], t
+
+
+def ring(n, degree, weighted=False):
+    """Every vertex joined to the `degree` nearest ones of a ring."""
+    g = two_parts(2 * n, n, degree, n)
+    off, col = g.off[:n + 1].copy(), g.col[:n * degree].copy()
+    src = np.repeat(np.arange(n), degree)
+    w = 1 + (src + col) % 7 if weighted else np.ones(len(col))
+    return synth.Graph(n, off, col, w.astype(np.int32))
+
+
+@pytest.mark.parametrize("degree", [4, 6, 16, 32, 64, 130, 2048, 2050])
+def test_windows_of_every_size(degree):
+    """Mean degrees at which a small graph's windows have 32, 16, 8, 4 and 2 rows and a
+    warp has one row (of up to 2048 arcs), the last window partly filled; one graph and two graphs whose boundary
+    lies inside a window."""
+    n = 3001
+    g = ring(n, degree, True)
+    w64 = g.w.astype(np.int64)
+    K = np.add.reduceat(w64, g.off[:-1])
+    C = np.random.default_rng(degree).integers(0, 9, n).astype(np.int32)
+    q, _ = oracle.modularity(g.off, g.col, w64, C)
+    h = L.Leiden(g.n, g.off, g.col, g.w)
+    ref = oracle.Oracle(g.n, g.off, g.col, g.w, schedule=oracle.SYNC)
+    assert h.modularity(C) == q
+    assert np.array_equal(h.static(), ref.static())
+    assert np.array_equal(h.state()["K"], K)
+    dels = [(5, 6, 1), (1500, 1501, 1), (0, n - 1, 1)]
+    assert np.array_equal(h.update(dels, [(1, 1600, 3)], L.LEIDEN_DS), ref.update(dels, [(1, 1600, 3)], oracle.DS))
+    assert np.array_equal(h.affected(), ref.affected())
+    two = L.LeidenBatch([(g.n, g.off, g.col, g.w)] * 2)
+    two.static()
+    assert np.array_equal(two.state()["K"], np.concatenate([K, K]))
+    ref = oracle.Oracle(g.n, g.off, g.col, g.w, schedule=oracle.SYNC)
+    ref.static()
+    assert list(two.modularity()) == [ref.modularity()] * 2
+
+
+def test_a_small_dense_graph_fills_the_gpu():
+    """Ten thousand rows of 2000 arcs: modularity on a handle (row sums first, two
+    sweeps over the arcs) beside the call that cuts spans of arcs (one sweep).
+    Windows of 32 rows would leave it to 313 of some 9,700 warps."""
+    import torch
+
+    g = ring(10_000, 2000)
+    C = np.zeros(g.n, np.int32)
+    d = [torch.from_numpy(x).cuda() for x in (g.off, g.col, g.w, C)]
+    h = L.Leiden(g.n, g.off, g.col, g.w)
+    t = fastest(lambda: h.modularity(C)), fastest(lambda: L.leiden_modularity_noalloc(g.n, d[0], d[1], d[2], d[3]))
+    assert t[0] < 4 * t[1], t
