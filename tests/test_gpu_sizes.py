@@ -151,3 +151,129 @@ def test_rows_merged_at_every_class_limit(arcs_each):
             i2 = [(u, v, x) for u, v, x in i]
             assert np.array_equal(gpu.update(i2, [], mode[0]), ref.update(i2, [], mode[1]))  # all taken out again
             same(gpu, ref)
+
+
+def check_stream(gpu, ref, g, steps, seed, modes=MODES, w_hi=1):
+    """Random batches on both, state and trace compared after each."""
+    cur = g
+    for k in range(steps):
+        mode = modes[k % len(modes)]
+        d, i = synth.random_batch(cur, max(4, g.n // 100), seed=seed + k, frac_ins=[0.5, 0.2, 0.8][k % 3], w_lo=1, w_hi=w_hi)
+        assert np.array_equal(gpu.update(d, i, mode[0]), ref.update(d, i, mode[1]))
+        cur = synth.apply_batch_numpy(cur, d, i)
+        same(gpu, ref)
+    return cur
+
+
+@pytest.mark.parametrize("classes", [1, 2, 16, 32, 64])
+def test_any_number_of_classes(classes):
+    """A local-moving iteration has a set of counters for 16 sub-sweeps, used again
+    above that; with hubs (from 65 arcs on) and, as a batch, with two graphs."""
+    gs = [synth.rmat(11, seed=31), synth.planted_partition(1500, 15, 10.0, 0.2, 32)]
+    for g in gs:
+        gpu = L.Leiden(g.n, g.off, g.col, g.w, classes=classes)
+        L.leiden_set_tuning(gpu.h, tiny_max=4, warp_max=32, block_max=64)
+        ref = oracle.Oracle(g.n, g.off, g.col, g.w, schedule=oracle.SYNC, classes=classes)
+        assert np.array_equal(gpu.static(), ref.static())
+        same(gpu, ref)
+        check_stream(gpu, ref, g, 3, 700)
+    batch = L.LeidenBatch([(g.n, g.off, g.col, g.w) for g in gs], classes=classes)
+    got = batch.static()
+    for k, g in enumerate(gs):
+        ref = oracle.Oracle(g.n, g.off, g.col, g.w, schedule=oracle.SYNC, classes=classes)
+        assert np.array_equal(batch.local(got, k), ref.static())
+
+
+@pytest.mark.parametrize("block_max", [64, 1024])
+def test_total_weight_passes_2_to_32_and_returns(block_max):
+    """Sums by community are held in 32 bits while 2m is below 2^32: a handle that
+    heavy insertions take above it and their deletion back, with random batches
+    and a static call on either side; hubs and hub communities of both kinds."""
+    g = synth.rmat(11, seed=44)
+    gpu = L.Leiden(g.n, g.off, g.col, g.w)
+    L.leiden_set_tuning(gpu.h, tiny_max=8, warp_max=64, block_max=block_max)
+    ref = oracle.Oracle(g.n, g.off, g.col, g.w, schedule=oracle.SYNC)
+    gpu.static(), ref.static()
+    cur = check_stream(gpu, ref, g, 3, 400)
+    for step, w in enumerate([(1 << 30) + 3, (1 << 30) + 3, 1 << 31 >> 1]):
+        free = [(u, v) for u in range(5 * step, 5 * step + 3) for v in range(g.n - 1, 0, -1)
+                if v > u and v not in set(cur.col[cur.off[u]:cur.off[u + 1]].tolist())][:3]
+        heavy = np.array([(u, v, w) for u, v in free], np.int32)
+        none = heavy[:0]
+        assert np.array_equal(gpu.update(none, heavy, L.LEIDEN_DF), ref.update(none, heavy, oracle.DF))
+        same(gpu, ref)
+        assert gpu.state()["m2"] > 1 << 32
+        cur = synth.apply_batch_numpy(cur, none, heavy)
+        if step == 1:
+            assert np.array_equal(gpu.static(), ref.static())
+            same(gpu, ref)
+        # (not of the heavy edges: they are deleted below)
+        for k, mode in enumerate(MODES):
+            edges = [(0, 100 + 7 * step + k, 2), (200, 300 + step, 1), (400 + k, 900, 5)]
+            edges = np.array([e for e in edges if not any({e[0], e[1]} == {u, v} for u, v in free)], np.int32)
+            assert np.array_equal(gpu.update(none, edges, mode[0]), ref.update(none, edges, mode[1]))
+            cur = synth.apply_batch_numpy(cur, none, edges)
+            same(gpu, ref)
+        assert np.array_equal(gpu.update(heavy, none, MODES[step][0]), ref.update(heavy, none, MODES[step][1]))
+        same(gpu, ref)
+        assert gpu.state()["m2"] < 1 << 32
+        cur = synth.apply_batch_numpy(cur, heavy, none)
+        cur = check_stream(gpu, ref, cur, 3, 500 + 10 * step)
+    assert np.array_equal(gpu.static(), ref.static())
+    same(gpu, ref)
+
+
+def spread(g, n):
+    """g's vertices on ids spread evenly over [0, n), in order."""
+    ids = (np.arange(g.n, dtype=np.int64) * n) // g.n
+    deg = np.zeros(n, np.int64)
+    deg[ids] = np.diff(g.off)
+    return synth.Graph(n, np.concatenate([[0], np.cumsum(deg)]), ids[g.col].astype(np.int32), g.w)
+
+
+@pytest.mark.parametrize("flags", [{}, dict(split_all=1)], ids=["changed", "all"])
+def test_more_ids_than_one_tile_each(flags):
+    """Above 2^21 vertices the split links in two steps, above 2^22 ids tracking's
+    tiles take several steps: thin communities that deletions take apart, spread
+    over 4,195,341 ids (an odd remainder), all other ids unused."""
+    small = synth.planted_partition(20_000, 900, 5.0, 0.1, 77)
+    g = spread(small, (1 << 22) + 1037)
+    gpu = L.Leiden(g.n, g.off, g.col, g.w, **flags)
+    ref = oracle.Oracle(g.n, g.off, g.col, g.w, schedule=oracle.SYNC, **flags)
+    assert np.array_equal(gpu.static(), ref.static())
+    same(gpu, ref)
+    ids = (np.arange(small.n, dtype=np.int64) * g.n) // small.n
+    for k, mode in enumerate(MODES):
+        d, i = synth.random_batch(small, 2500, seed=60 + k, frac_ins=0.2)
+        small = synth.apply_batch_numpy(small, d, i)
+        d, i = [np.stack([ids[e[:, 0]], ids[e[:, 1]], e[:, 2]], 1).astype(np.int32) for e in (d, i)]
+        assert np.array_equal(gpu.update(d, i, mode[0]), ref.update(d, i, mode[1]))
+        same(gpu, ref)
+
+
+def test_batch_of_graphs_with_more_ids_than_one_tile_each():
+    """The second graph of a batch starts inside a tile of several steps."""
+    parts = [synth.planted_partition(6000, 300, 5.0, 0.1, 78), synth.planted_partition(5000, 200, 5.0, 0.1, 79)]
+    sizes = [(1 << 22) + 517, 70_001]
+    gs = [spread(p, n) for p, n in zip(parts, sizes)]
+    batch = L.LeidenBatch([(g.n, g.off, g.col, g.w) for g in gs])
+    refs = [oracle.Oracle(g.n, g.off, g.col, g.w, schedule=oracle.SYNC) for g in gs]
+    got = batch.static()
+    for k, r in enumerate(refs):
+        assert np.array_equal(batch.local(got, k), r.static())
+    for step in range(2):
+        dels, ins, want = [], [], []
+        for k, r in enumerate(refs):
+            d, i = synth.random_batch(parts[k], 900, seed=80 + 10 * step + k, frac_ins=0.3)
+            parts[k] = synth.apply_batch_numpy(parts[k], d, i)
+            ids = (np.arange(parts[k].n, dtype=np.int64) * sizes[k]) // parts[k].n
+            d, i = [np.stack([ids[e[:, 0]], ids[e[:, 1]], e[:, 2]], 1).astype(np.int32) for e in (d, i)]
+            want.append(r.update(d, i, oracle.DF))
+            dels.append(batch.to_global(d, k))
+            ins.append(batch.to_global(i, k))
+        got = batch.update(np.concatenate(dels), np.concatenate(ins), L.LEIDEN_DF)
+        for k, w in enumerate(want):
+            assert np.array_equal(batch.local(got, k), w)
+            for key in ("K", "Sigma", "dSigma"):
+                a, b = int(batch.voff[k]), int(batch.voff[k + 1])
+                assert np.array_equal(batch.state()[key][a:b], refs[k].state()[key])
