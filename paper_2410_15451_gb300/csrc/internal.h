@@ -213,8 +213,9 @@ struct leiden_handle {
 // that every entry point turns the same exact numerator into the same double.
 double i128_to_double(i128 x);
 
-// Every kernel launch of the library is written `ld_note_launch(), k<<<...>>>(...)`
-// so that leiden_kernel_launches() counts them.
+// Every kernel launch of the library is written `ld_note_launch(), launch_after(k,
+// ...)`, or `ld_note_launch(), k<<<...>>>(...)` where k does not wait for the kernel
+// before it, so that leiden_kernel_launches() counts them.
 void ld_note_launch();
 
 // Kernel timer of the local-moving kernels: begin/end around a launch of

@@ -461,7 +461,6 @@ template <typename W, int KIND, bool WIDE>
 __global__ void __launch_bounds__(WARPS_PER_BLOCK * 32, 4) k_decide_warp(Args A) {
   ld_after_previous();
   __shared__ WarpTable<WIDE> WT[WARPS_PER_BLOCK];
-  ld_after_previous();
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int64_t ntiny = *A.count_tiny, nwarp = *A.count;
   int64_t ngroups = (ntiny + 3) / 4, total = ngroups + nwarp;

@@ -41,3 +41,30 @@ def test_flush_of_a_warp_table_is_decided_by_the_whole_warp():
         text = text.replace(room, "")
         assert not re.search(r"\bif\s*\([^;{}]*\)\s*\{?\s*wt_flush\(", text), f
         assert not re.search(r"\bif\s*\([^;{}]*WT_LIMIT", text), f
+
+
+def test_kernels_launched_early_wait_first():
+    """A kernel launched by launch_after may start while the one before it runs: its
+    first statement waits, once, or it would race with it (and, as a kernel that
+    ends without having waited, so would the one after it)."""
+    src = sources()
+    text = "\n".join(src.values())
+    kernels = {}
+    for m in re.finditer(r"__global__\s+void\s+(?:__launch_bounds__\([^)]*\)\s*)?(\w+)\s*\(", text):
+        kernels[m.group(1)] = body(text, m.end())
+    launched = set()
+    for f, t in src.items():
+        for m in re.finditer(r"\blaunch_after\(\s*(\w+)", t):
+            name = m.group(1)
+            if name in kernels:
+                launched.add(name)
+            elif name != "void":  # a variable: every kernel that it may hold (void: the helper itself)
+                held = re.findall(r"auto\s+%s\s*=([^;]*);" % name, t)
+                assert held, (f, name)
+                names = set(re.findall(r"\bk_\w+", " ".join(held)))
+                assert names and names <= set(kernels), (f, name)
+                launched |= names
+    assert len(launched) > 80
+    for name in sorted(launched):
+        assert re.match(r"\{\s*ld_after_previous\(\);", kernels[name]), name
+        assert kernels[name].count("ld_after_previous()") == 1, name
