@@ -23,7 +23,9 @@ stream (a spawned process, in parallel with the GPU work), SM clocks sampled
 during the timed region, and the large web-like configuration (1B edges,
 20 DF batches of 1e-4|E|, checked at full size) as `large`, and the batched
 configuration (512 planted-partition graphs in one handle against one call
-per graph, memberships compared graph by graph) as `batched`.
+per graph, memberships compared graph by graph) as `batched`.  The main line
+is one JSON line on standard output; steps, modes, sweep, roofs by kernel and
+phase, `large` and `batched` go to standard error as one line before it.
 
 --impl reference times the CPU oracle (plain sequential C, one host thread)
 on the same workload: the same R-MAT scale-22 graph and batch stream, static
@@ -1259,6 +1261,14 @@ def run_serve(args):
     return 0
 
 
+def print_main(line, detail):
+    """The main line on standard output, a few kilobytes so that a log's tail holds
+    all of it; the per-step, per-kernel and per-configuration records, some 20 KB,
+    as one line on standard error before it."""
+    print("detail: " + json.dumps(detail), file=sys.stderr, flush=True)
+    print(json.dumps(line), flush=True)
+
+
 def main():
     args = parse()
     rank = int(os.environ.get("RANK", "0"))
@@ -1316,25 +1326,28 @@ def main():
             "communities": chk["communities"], "disconnected": chk["components"] - chk["communities"],
             "q_df_exact_check": bool(abs(chk["q"] - r["q_df"]) <= 1e-12 * max(1.0, abs(chk["q"]))),
             "quality_ok": bool(r["q_static"] - r["q_df"] <= 0.005 and chk["connected"]),
-            "p50_ms": r["p50"], "p99_ms": r["p99"], "steps_detail": r["steps"],
-            "modes": r["modes"],
+            "p50_ms": r["p50"], "p99_ms": r["p99"],
             "e2e": {"value": r["e2e"], "unit": "edges/s", "h2d_bytes_per_step": r["size"] * 12,
                     "d2h_bytes_per_step": r["n"] * 4, "p99_ms": r["e2e_p99"]},
             "roofline": dom,
+            "gpu_launches": r["gpu_launches"],
+            "cpu_baseline": cb,
+            "clocks": r["clk"],
+        }
+        detail = {
+            "steps_detail": r["steps"],
+            "modes": r["modes"],
             "roofline_kernels": lmk,
             # the same kernels on the following DF steps with the side streams
             # off (one stream, each kernel alone on the GPU)
             "roofline_kernels_isolated": lmk_iso,
             "one_stream": {"steps": ISO_STEPS, "ms_mean": r["iso_ms"], "p50_ms": r["iso_p50"]},
             "roofline_step": roofline_step(r["lm_stats"], r["mean_ms"]),
-            "gpu_launches": r["gpu_launches"],
-            "cpu_baseline": cb,
-            "clocks": r["clk"],
             "sweep": r["sweep"],
             "large": large,
             "batched": batched,
         }
-        print(json.dumps(line), flush=True)
+        print_main(line, detail)
     if world > 1:
         import torch.distributed as dist
 

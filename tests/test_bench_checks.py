@@ -124,3 +124,16 @@ def test_ncu_summary_reads_the_capture_csv(tmp_path):
     assert json.loads((tmp_path / "t.json").read_text())["source_sha256"]["move.cu"] == \
         bench.source_code_sha256(os.path.join(bench.CSRC, "move.cu"))
     assert "| k_expand | 1 |" in (tmp_path / "t.md").read_text()
+
+
+def test_the_main_line_fits_the_tail_of_a_log(capsys):
+    """One short line on standard output whatever the records' length; they go to
+    standard error, whole."""
+    import json
+
+    line = {"metric": bench.METRIC, "value": 1.0, "config": {"workload": "w" * 300}}
+    detail = {"steps_detail": [{"ms": 3.25, "phase_ms": {"move": 1.5}}] * 400}
+    bench.print_main(line, detail)
+    out, err = capsys.readouterr()
+    assert out.count("\n") == 1 and json.loads(out) == line and len(out) < 3000
+    assert err.startswith("detail: ") and json.loads(err[len("detail: "):]) == detail
