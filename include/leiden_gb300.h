@@ -125,8 +125,8 @@ typedef struct {
    * degree; per arc read 8 B: col, C of the neighbour), [1] the chunked scan
    * of communities above 1024 member arcs in aggregation (per arc: col, C of
    * the neighbour and the weight), [2] the block merge of touched rows of
-   * 1025..4096 arcs (per arc: the old row read and the new row written,
-   * 16 B; per batch arc 16 B). */
+   * 1025..4096 arcs (per arc from the row's first change on: 8 B read of the
+   * old row, 8 B written of the new one; per batch arc 16 B). */
   int64_t xk_launches[3];
   int64_t xk_bytes[3];
   double xk_ms[3];
@@ -314,10 +314,12 @@ leiden_status leiden_create_batched(const leiden_params *params, int32_t graphs,
  * hold: the allocations of leiden_create plus an allowance for batch buffers
  * and aggregated-level hash tables that grow on demand.  -1 on bad input.
  * Used by the server below to admit graphs by footprint.  The batch buffers
- * take about 172 B per arc of batch capacity (two arcs per edge, capacity
- * grown geometrically to at most twice the largest batch); the allowance
- * (8 B per vertex plus 32 MB) covers batches up to about 50k edges on a
- * small graph, more on a large one.  Not included: the arcs of the
+ * take 172 B per arc of batch capacity (two arcs per edge, capacity grown
+ * geometrically to at most twice the largest batch) and 64 B per row that
+ * such a batch may touch (at most two per arc, and each vertex once); the
+ * allowance (8 B per vertex plus 32 MB) covers batches up to about 25k edges
+ * on any graph, 45k on one of few vertices.  Not included: the merge buffer
+ * (8 B per arc of the rows a batch changes), the arcs of the
  * aggregated levels, which a call draws from the device's stream-ordered
  * memory pool only while it aggregates (see the next). */
 int64_t leiden_footprint_bytes(const leiden_params *params, int64_t n, const int64_t *offsets);

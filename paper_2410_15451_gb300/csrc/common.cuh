@@ -67,7 +67,7 @@ struct DevCounters {
                                   //   giant-community aggregation scan, block merge of touched rows)
   int64_t agg_tables[2];          // aggregation's per-community global tables: [0] hashed, [1] indexed
                                   //   by the key (the table has a slot per community)
-  int64_t refine_marks;           // batch: communities marked for refinement (counted per arc)
+  int64_t refine_marks;           // batch: not 0 when a community is marked for refinement
   // kept between calls
   int64_t m2;                     // 2m (sum of arc weights), device copy
   int64_t arena_used;             // next free arc slot of G^t (relocated rows go here)

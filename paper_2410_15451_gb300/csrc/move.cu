@@ -6,7 +6,9 @@
 // (Eq. 2 times 2m^2, exact in int128; ties to the lowest community id) and
 // moves when the gain is positive.  Vertices are binned by degree: a warp
 // with a shared-memory table (<= 128 arcs), a block with a shared table
-// (<= 1024 arcs), a block with a table in global scratch (larger).
+// (<= 1024 arcs); larger ones are cut into chunks for all blocks, with a table in
+// global scratch per vertex that a warp, or a block per piece of it, reads to
+// decide.
 //
 // Deterministic mode (snapshot schedule): moves found in a sub-sweep are
 // applied by a separate kernel after all decisions, so every decision reads

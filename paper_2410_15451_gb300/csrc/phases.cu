@@ -31,7 +31,7 @@ __global__ void k_sr_min(int64_t n, const int32_t *C, int32_t *rep) {
 // root is only ever hooked under a smaller root, so every component ends with
 // its smallest vertex as root -- the label a BFS from the lowest vertex gives.
 // One sweep in place of four with one atomic per warp on the list's length
-// (R-MAT 22: 190 -> 59 us with the search for the smallest members).
+// (R-MAT 22: 190 -> 63 us with the search for the smallest members).
 __global__ void __launch_bounds__(256) k_remap_list(int64_t n, const int32_t *rep, const uint8_t *dS,
                                                     const uint8_t *dR, const int32_t *deg, int32_t *C, uint8_t *dR2,
                                                     int32_t *parent, int32_t *list, DevCounters *cnt, int split_all) {
@@ -153,9 +153,11 @@ __global__ void k_split_sample(const int32_t *list, DevCounters *cnt, const int6
 // every eighth listed vertex, a flattening, and the links of the others, which
 // by then mostly find in two loads that their ends agree.  In the form above
 // the lanes of a warp wait for each other's chains of lookups; this one pays
-// two more sweeps and more failed hooks.  Sampling and linking together:
-// R-MAT 22 (2.4M listed) 376 us above, 334 here; R-MAT 20 (650k) 70 and 101, the
-// web-like graph (777k vertices) 101 and 143.
+// two more sweeps and more failed hooks.  What decides is the number of listed
+// vertices; it is on the device here, and the level's vertices stand for it (with
+// few listed the three further launches do next to nothing).  Sampling and
+// linking together: R-MAT 22 (2.4M listed) 376 us above, 334 here; R-MAT 20 (650k)
+// 70 and 101, the web-like graph (777k vertices) 101 and 143.
 constexpr int64_t SPLIT_APART = (int64_t)1 << 21;
 constexpr int SPLIT_WINDOW = 4;   // arcs loaded at once
 __global__ void __launch_bounds__(256) k_split_find(const int32_t *list, DevCounters *cnt, const int64_t *off,
